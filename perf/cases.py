@@ -17,7 +17,7 @@ DIMS = {256: (16, 16), 512: (32, 16), 1024: (32, 32), 2048: (64, 32), 4096: (64,
 
 
 def _conv(name, kind, dtype, dims, mode, B, H, n):
-    return {"name": name, "kind": kind, "dtype": dtype, "dims": "x".join(map(str, dims)), "mode": mode, "B": B, "H": H, "n": n}
+    return {**({"name": name} if name else {}), "kind": kind, "dtype": dtype, "dims": "x".join(map(str, dims)), "mode": mode, "B": B, "H": H, "n": n}
 
 
 def listed():
