@@ -84,8 +84,8 @@ int64_t m2_spectrum_bytes(const m2_plan* plan, int64_t H);
 
 /* k_f = M * pad(k) per channel (Alg. BlockMonarchConv, the line k_f <- M k; Eq. 2's K_1 given in
  * frequency space).  k_dev: [H, n] float32, n <= N, zero padded to N.  kf_dev: m2_spectrum_bytes
- * bytes; the format is private to the plan (complex fp32, plan order, with the 1/N of M^-1 folded
- * in).  Computed in fp32 whatever the plan dtype; meant to run once per weight update. */
+ * bytes; the format is private to the plan (complex fp32, in the order its kernels read, with the 1/N of
+ * M^-1 folded in).  Computed in fp32 whatever the plan dtype; meant to run once per weight update. */
 int32_t m2_kernel_spectrum(const m2_plan* plan, const float* k_dev, int64_t H, int64_t n, void* kf_dev,
                            void* stream);
 

@@ -24,6 +24,7 @@
 // barrier latency is covered by the others' fp32 work.  Units are handed out by a device-wide counter; the kernel is
 // launched with programmatic stream serialization (set-up overlaps the previous kernel's tail).  All waits are bounded.
 #include "conv_umma.h"
+#include "fft_core.cuh"
 
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -1168,13 +1169,15 @@ convwgrad512_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
 }
 
 // spectrum re-layout for this kernel: kfu[h][k2/2][k1] = (re(k2 even), re(k2 odd), im(even), im(odd)) from plan order
-__global__ void relayout_spectrum_kernel(const float2* __restrict__ kf, float4* __restrict__ kfu, long long total) {
+__global__ void relayout_spectrum_kernel(const float* __restrict__ kf, float4* __restrict__ kfu, long long total, float sgn) {
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;   // over H * 8 * 32
     if (i >= total) return;
     const int k1 = (int)(i & 31), q = (int)((i >> 5) & 7);
     const long long h = i >> 8;
-    const float2 a = kf[h * 512 + k1 * 16 + 2 * q], b = kf[h * 512 + k1 * 16 + 2 * q + 1];
-    kfu[i] = make_float4(a.x, b.x, a.y, b.y);
+    const float* row = kf + h * 1024;   // in the order of the fp32 transform kernels; frequency k1 + 32 k2, k2 = 2 q, 2 q + 1
+    const int ka = k1 + 64 * q, kb = ka + 32;
+    kfu[i] = make_float4(row[m2f::spec_index<m2f::Cfg<9>>(ka, false)], row[m2f::spec_index<m2f::Cfg<9>>(kb, false)],
+                         sgn * row[m2f::spec_index<m2f::Cfg<9>>(ka, true)], sgn * row[m2f::spec_index<m2f::Cfg<9>>(kb, true)]);
 }
 
 // ---- host side ---------------------------------------------------------------------------------------
@@ -1521,7 +1524,7 @@ cudaError_t relayout_spectrum(const m2_plan* pl, void* kf, int64_t H, cudaStream
     if (!has_private_spectrum(pl) || H == 0) return cudaSuccess;
     const long long total = H * 256;
     float4* kfu = reinterpret_cast<float4*>(static_cast<unsigned char*>(kf) + (size_t)H * 512 * 8);
-    relayout_spectrum_kernel<<<(unsigned)((total + 255) / 256), 256, 0, stream>>>((const float2*)kf, kfu, total);
+    relayout_spectrum_kernel<<<(unsigned)((total + 255) / 256), 256, 0, stream>>>((const float*)kf, kfu, total, pl->sign >= 0 ? 1.0f : -1.0f);
     return cudaGetLastError();
 }
 

@@ -1,0 +1,131 @@
+// Kernel spectrum and kernel gradient of the fp32 transform path (fft_conv.cu has the convolution).
+#include "fft_conv.h"
+#include "fft_pass.cuh"
+
+namespace m2f {
+
+// k_f of one channel per row: the forward half alone, scaled by 1 / N
+template <class C, bool HALF>
+__global__ void __launch_bounds__(C::THREADS, min_blocks<C>())
+    fft_spectrum_kernel(const float* __restrict__ k, float4* __restrict__ kf, const float4* __restrict__ tab, int H, int n) {
+    extern __shared__ __align__(16) float smem[];
+    const int r = threadIdx.x / C::TP, t = threadIdx.x % C::TP;
+    const long long h = (long long)blockIdx.x * C::ROWS + r;
+    const bool live = h < H;
+    float* sr = smem + r * C::ROWF + (r & 1) * C::PAR;
+    float* si = sr + C::SMEM_FLOATS;
+    u64 re[16], im[16];
+    // rows of k are only as aligned as n floats make them; a pair needs 8 bytes
+    load_row<C, float, HALF>(re, live ? k + h * n : nullptr, t, n, (n & 1) == 0 && (reinterpret_cast<uintptr_t>(k) & 7) == 0);
+    unroll<16>([&](auto j) { im[j.v] = 0ull; });
+    forward<C, HALF>(re, im, sr, si, tab, t, r);
+    if (!live) return;
+    const u64 sc = dup2(1.0f / (float)C::N);
+    float4* out = kf + h * (C::N / 2) + t;
+    unroll<16>([&](auto s) {
+        constexpr int p = brev<4>(s.v);
+        const u64 a = mul2(re[p], sc), c = mul2(im[p], sc);
+        out[s.v * C::TP] = make_float4(lo(a), hi(a), lo(c), hi(c));
+    });
+}
+
+// dk[h] = Re F^-1( sum over row pairs of conj(F z) (.) F w ) / N with z = x_a + i x_b, w = g_a + i g_b: the real part of the product's
+// inverse is corr(x_a, g_a) + corr(x_b, g_b).  One channel per row of threads, the pairs one after the other; the sum stays in
+// registers, F z waits in shared memory in the thread's own slots.
+template <class C>
+constexpr int wgrad_blocks() { return C::THREADS == 128 ? 2 : 1; }
+template <class C, typename IO, bool HALF>
+__global__ void __launch_bounds__(C::THREADS, wgrad_blocks<C>())
+    fft_wgrad_kernel(const IO* __restrict__ x, const IO* __restrict__ g, float* __restrict__ dk, const float4* __restrict__ tab, int B, int H,
+                     int n) {
+    extern __shared__ __align__(16) float smem[];
+    const int r = threadIdx.x / C::TP, t = threadIdx.x % C::TP;
+    const long long h = (long long)blockIdx.x * C::ROWS + r;
+    const bool live = h < H, vec = (n & 1) == 0;
+    float* sr = smem + r * C::ROWF + (r & 1) * C::PAR;
+    float* si = sr + C::SMEM_FLOATS;
+    float4* zs = reinterpret_cast<float4*>(smem + 2 * C::SMEM_FLOATS) + threadIdx.x;
+    u64 re[16], im[16], ar[16], ai[16];
+    unroll<16>([&](auto s) { ar[s.v] = ai[s.v] = 0ull; });
+#pragma unroll 1
+    for (int b = 0; b < B; b += 2) {
+        const long long oa = ((long long)b * H + h) * n, ob = oa + (long long)H * n;
+        const bool has_b = live && b + 1 < B;
+        load_row<C, IO, HALF>(re, live ? x + oa : nullptr, t, n, vec);
+        load_row<C, IO, HALF>(im, has_b ? x + ob : nullptr, t, n, vec);
+        forward<C, HALF>(re, im, sr, si, tab, t, r);
+        unroll<16>([&](auto s) { zs[s.v * C::THREADS] = make_float4(lo(re[s.v]), hi(re[s.v]), lo(im[s.v]), hi(im[s.v])); });
+        load_row<C, IO, HALF>(re, live ? g + oa : nullptr, t, n, vec);
+        load_row<C, IO, HALF>(im, has_b ? g + ob : nullptr, t, n, vec);
+        row_sync<C>(r);
+        forward<C, HALF>(re, im, sr, si, tab, t, r);
+        unroll<16>([&](auto s) {   // += conj(z) w
+            const float4 z = zs[s.v * C::THREADS];
+            const u64 zr = pk(z.x, z.y), zi = pk(z.z, z.w);
+            ar[s.v] = fma2(zr, re[s.v], fma2(zi, im[s.v], ar[s.v]));
+            ai[s.v] = fma2(zr, im[s.v], fma2(neg2(zi), re[s.v], ai[s.v]));
+        });
+        row_sync<C>(r);
+    }
+    inverse<C, HALF>(ar, ai, sr, si, tab, t, r);
+    const u64 sc = dup2(1.0f / (float)C::N);
+    unroll<16>([&](auto s) { ar[s.v] = mul2(ar[s.v], sc); });
+    store_row<C, float, HALF>(ar, live ? dk + h * n : nullptr, t, n, vec);
+}
+
+template <class C>
+constexpr int wgrad_smem() { return conv_smem<C>() + C::THREADS * 16 * 16; }
+
+cudaError_t prepare_gradients(const m2_plan* pl) {
+    return dispatch(pl->N, [&](auto cfg) {
+        using C = decltype(cfg);
+        cudaError_t e = allow_smem(fft_spectrum_kernel<C, false>, conv_smem<C>());
+        if (e == cudaSuccess) e = allow_smem(fft_spectrum_kernel<C, true>, conv_smem<C>());
+        if constexpr (C::N <= 8192) {
+            auto io = [&](auto z) {
+                using IO = decltype(z);
+                if (e == cudaSuccess) e = allow_smem(fft_wgrad_kernel<C, IO, false>, wgrad_smem<C>());
+                if (e == cudaSuccess) e = allow_smem(fft_wgrad_kernel<C, IO, true>, wgrad_smem<C>());
+            };
+            if (pl->dtype == M2_BF16) io(__nv_bfloat16());
+            else io(float());
+        }
+        return e;
+    });
+}
+
+cudaError_t spectrum(const m2_plan* pl, const float* k, int64_t H, int64_t n, void* kf, cudaStream_t stream) {
+    if (H == 0) return cudaSuccess;
+    return dispatch(pl->N, [&](auto cfg) {
+        using C = decltype(cfg);
+        const unsigned grid = (unsigned)((H + C::ROWS - 1) / C::ROWS);
+        if (2 * n <= C::N)
+            fft_spectrum_kernel<C, true><<<grid, C::THREADS, conv_smem<C>(), stream>>>(k, (float4*)kf, pl->d_fft, (int)H, (int)n);
+        else
+            fft_spectrum_kernel<C, false><<<grid, C::THREADS, conv_smem<C>(), stream>>>(k, (float4*)kf, pl->d_fft, (int)H, (int)n);
+        return cudaGetLastError();
+    });
+}
+
+cudaError_t wgrad(const m2_plan* pl, const void* x, const void* g, float* dk, int64_t B, int64_t H, int64_t n, bool causal,
+                  cudaStream_t stream) {
+    if (H == 0) return cudaSuccess;
+    return dispatch(pl->N, [&](auto cfg) {
+        using C = decltype(cfg);
+        if constexpr (C::N > 8192) {
+            return cudaErrorInvalidValue;
+        } else {
+            const unsigned grid = (unsigned)((H + C::ROWS - 1) / C::ROWS);
+            auto go = [&](auto z, auto half) {
+                using IO = decltype(z);
+                fft_wgrad_kernel<C, IO, decltype(half)::v != 0><<<grid, C::THREADS, wgrad_smem<C>(), stream>>>(
+                    (const IO*)x, (const IO*)g, dk, pl->d_fft, (int)B, (int)H, (int)n);
+            };
+            if (pl->dtype == M2_BF16) causal ? go(__nv_bfloat16(), Ic<1>{}) : go(__nv_bfloat16(), Ic<0>{});
+            else causal ? go(float(), Ic<1>{}) : go(float(), Ic<0>{});
+            return cudaGetLastError();
+        }
+    });
+}
+
+}  // namespace m2f

@@ -8,6 +8,7 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "fft_core.cuh"
 #include "generic_kernels.h"
 
 namespace m2g {
@@ -17,7 +18,26 @@ struct Dims {
     int d[3];
     int N;
     float sgn;  // +1 / -1: omega = exp(sgn 2 pi i / M)
+    int spectrum_order;
 };
+
+// plan position (k1, k2, k3) row-major -> natural frequency k = k1 + N1 k2 + N1 N2 k3
+__device__ __forceinline__ int natural_frequency(const Dims& D, int pos) {
+    int k = 0, w = D.N;
+    for (int a = D.p - 1; a >= 0; --a) {
+        w /= D.d[a];
+        k += w * (pos % D.d[a]);
+        pos /= D.d[a];
+    }
+    return k;
+}
+// spectrum value at a plan position, from either order of the buffer (row = N complex values of one channel)
+__device__ __forceinline__ float2 spectrum_at(const float2* row, const Dims& D, int pos) {
+    if (D.spectrum_order == 0) return row[pos];
+    const float* f = reinterpret_cast<const float*>(row);
+    const int k = natural_frequency(D, pos);
+    return make_float2(f[m2f::spec_index_any(D.spectrum_order, k, false)], D.sgn * f[m2f::spec_index_any(D.spectrum_order, k, true)]);
+}
 
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
     return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
@@ -160,7 +180,7 @@ __global__ void __launch_bounds__(1024) conv_row_kernel(const IO* __restrict__ x
     __syncthreads();
     for (int a = 0; a < D.p; ++a) stage<ST, ITEMS, false>(buf, D, a, R.r[a]);
     const float2* kr = kf + (long long)(h / kf_group) * D.N;
-    for (int i = threadIdx.x; i < D.N; i += blockDim.x) Store<ST>::st(buf + i, cmul(Store<ST>::ld(buf + i), kr[i]));
+    for (int i = threadIdx.x; i < D.N; i += blockDim.x) Store<ST>::st(buf + i, cmul(Store<ST>::ld(buf + i), spectrum_at(kr, D, i)));
     __syncthreads();
     for (int a = D.p - 1; a >= 0; --a) stage<ST, ITEMS, true>(buf, D, a, R.r[a]);
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
@@ -233,20 +253,8 @@ __global__ void spectrum_to_natural_kernel(const float2* __restrict__ kf, float2
     if (i >= total) return;
     const int pos = (int)(i % D.N);
     const long long h = i / D.N;
-    // plan position (k1, k2, k3) row-major -> k = k1 + N1 k2 + N1 N2 k3
-    int rem = pos, k = 0;
-    int digits[3] = {0, 0, 0};
-    for (int a = D.p - 1; a >= 0; --a) {
-        digits[a] = rem % D.d[a];
-        rem /= D.d[a];
-    }
-    int w = 1;
-    for (int a = 0; a < D.p; ++a) {
-        k += w * digits[a];
-        w *= D.d[a];
-    }
-    float2 v = kf[i];
-    out[h * D.N + k] = make_float2(v.x * (float)D.N, v.y * (float)D.N);
+    const float2 v = spectrum_at(kf + h * D.N, D, pos);
+    out[h * D.N + natural_frequency(D, pos)] = make_float2(v.x * (float)D.N, v.y * (float)D.N);
 }
 
 // Order-2 Monarch matmul, TT tokens per block, fp32 accumulate (Sec. 3.1):
@@ -362,6 +370,7 @@ static Dims make_dims(const ConvShape& s) {
         D.N *= D.d[a];
     }
     D.sgn = s.sign >= 0 ? 1.f : -1.f;
+    D.spectrum_order = s.spectrum_order;
     return D;
 }
 

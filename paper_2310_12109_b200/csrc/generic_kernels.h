@@ -13,6 +13,7 @@ struct ConvShape {
     long long stride_b, stride_h, stride_e;
     const float2* roots[3];  // device: omega_{Na}^j per stage
     int kf_group = 1;        // channel h is multiplied by spectrum row h / kf_group
+    int spectrum_order = 0;  // log2 N if the spectrum is in the order of fft_core.cuh (exponent sign +), 0 if in plan order
 };
 
 cudaError_t launch_conv(const ConvShape& s, bool bf16_io, const void* x, const void* kf, void* y, const float* gate_w,

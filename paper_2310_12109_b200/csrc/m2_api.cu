@@ -10,6 +10,7 @@
 
 #include "blocky_monarch.h"
 #include "conv_umma.h"
+#include "fft_conv.h"
 #include "generic_kernels.h"
 #include "cols_umma.h"
 #include "matmul_umma.h"
@@ -97,6 +98,7 @@ m2g::ConvShape conv_shape(const m2_plan* pl, int64_t B, int64_t H, int64_t n) {
     s.stride_b = H * n;
     s.stride_h = n;
     s.stride_e = 1;
+    s.spectrum_order = m2f::spectrum_order(pl);
     return s;
 }
 
@@ -152,17 +154,33 @@ int32_t m2_plan_create(m2_plan** out, int64_t N, int32_t p, const int32_t* facto
     if (device >= 0) {
         DeviceGuard g(device);
         bool ok = g.ok;
-        if (ok) ok = cudaMalloc(&pl->d_status, sizeof(int32_t)) == cudaSuccess;
-        if (ok) ok = cudaMemset(pl->d_status, 0, sizeof(int32_t)) == cudaSuccess;
-        for (int a = 0; a < p && ok; ++a) {
+        // one device block, one copy: status word | roots of every factor | twiddle factors of the fp32 transform kernels
+        const std::vector<float4>* fft = m2f::host_table(pl);
+        size_t off_roots[4], bytes = 256;
+        for (int a = 0; a < p; ++a) {
+            off_roots[a] = bytes;
+            bytes += ((size_t)pl->dims[a] * sizeof(float2) + 255) / 256 * 256;
+        }
+        const size_t off_fft = bytes;
+        if (fft) bytes += fft->size() * sizeof(float4);
+        std::vector<unsigned char> block(bytes, 0);
+        for (int a = 0; a < p; ++a) {
             const int Na = pl->dims[a];
-            std::vector<float2> r(Na);
+            float2* r = reinterpret_cast<float2*>(block.data() + off_roots[a]);
             for (int j = 0; j < Na; ++j) {
                 const double ang = 2.0 * M_PI * (double)j / (double)Na;
                 r[j] = make_float2((float)std::cos(ang), (float)(sign * std::sin(ang)));
             }
-            ok = cudaMalloc(&pl->d_roots[a], sizeof(float2) * Na) == cudaSuccess &&
-                 cudaMemcpy(pl->d_roots[a], r.data(), sizeof(float2) * Na, cudaMemcpyHostToDevice) == cudaSuccess;
+        }
+        if (fft) std::memcpy(block.data() + off_fft, fft->data(), fft->size() * sizeof(float4));
+        if (ok) ok = cudaMalloc(&pl->d_block, bytes) == cudaSuccess;
+        if (ok) ok = cudaMemcpy(pl->d_block, block.data(), bytes, cudaMemcpyHostToDevice) == cudaSuccess;
+        if (ok) {
+            unsigned char* base = static_cast<unsigned char*>(pl->d_block);
+            pl->d_status = reinterpret_cast<int32_t*>(base);
+            for (int a = 0; a < p; ++a) pl->d_roots[a] = reinterpret_cast<float2*>(base + off_roots[a]);
+            if (fft) pl->d_fft = reinterpret_cast<float4*>(base + off_fft);
+            ok = m2f::prepare(pl) == cudaSuccess;
         }
         if (ok) ok = m2u::create_tables(pl) == cudaSuccess;
         if (ok) ok = m2u3::create_tables(pl) == cudaSuccess;
@@ -185,9 +203,7 @@ int32_t m2_plan_destroy(m2_plan* plan) {
         cudaDeviceSynchronize();
         m2u::destroy_tables(plan);
         m2u3::destroy_tables(plan);
-        if (plan->d_status) cudaFree(plan->d_status);
-        for (int a = 0; a < 4; ++a)
-            if (plan->d_roots[a]) cudaFree(plan->d_roots[a]);
+        if (plan->d_block) cudaFree(plan->d_block);
     }
     delete plan;
     return M2_OK;
@@ -219,7 +235,8 @@ int32_t m2_kernel_spectrum(const m2_plan* plan, const float* k_dev, int64_t H, i
     DeviceGuard g(plan->device);
     if (!g.ok) return M2_ERR_CUDA;
     m2g::ConvShape s = conv_shape(plan, 1, H, n);
-    cudaError_t e = m2g::launch_spectrum(s, k_dev, kf_dev, (cudaStream_t)stream);
+    const cudaError_t e = m2f::covered(plan) ? m2f::spectrum(plan, k_dev, H, n, kf_dev, (cudaStream_t)stream)
+                                             : m2g::launch_spectrum(s, k_dev, kf_dev, (cudaStream_t)stream);
     if (e == cudaErrorInvalidValue) return M2_ERR_UNSUPPORTED;
     if (e != cudaSuccess) return M2_ERR_CUDA;
     if (m2u::relayout_spectrum(plan, kf_dev, H, (cudaStream_t)stream) != cudaSuccess) return M2_ERR_CUDA;
@@ -274,7 +291,10 @@ int32_t m2_monarch_conv_bwd_kernel(const m2_plan* plan, const void* x_dev, const
         st = m2u3::conv_wgrad(plan, x_dev, g_dev, dk_dev, B, H, n, mode, ws_dev, (cudaStream_t)stream);
         if (st != M2_ERR_UNSUPPORTED) return st;
     }
-    const cudaError_t e = m2g::launch_conv_wgrad(s, plan->dtype == M2_BF16, x_dev, g_dev, dk_dev, ws_dev, ws_bytes, (cudaStream_t)stream);
+    cudaError_t e = cudaErrorInvalidValue;
+    if (m2f::covered(plan)) e = m2f::wgrad(plan, x_dev, g_dev, dk_dev, B, H, n, mode == M2_CAUSAL, (cudaStream_t)stream);
+    if (e == cudaErrorInvalidValue)
+        e = m2g::launch_conv_wgrad(s, plan->dtype == M2_BF16, x_dev, g_dev, dk_dev, ws_dev, ws_bytes, (cudaStream_t)stream);
     if (e == cudaErrorInvalidValue) return M2_ERR_UNSUPPORTED;
     if (e != cudaSuccess) return M2_ERR_CUDA;
     plan->last_kernel = "conv_wgrad_generic";
@@ -290,8 +310,10 @@ int32_t m2_spectrum_conjugate(const m2_plan* plan, const void* kf_in_dev, int64_
     if (!g.ok) return M2_ERR_CUDA;
     const long long values = H * plan->N;   // complex values per layout; N is even for every plan with a device path
     if (plan->N % 2 != 0) return M2_ERR_UNSUPPORTED;
-    if (m2g::launch_spectrum_conj(kf_in_dev, kf_out_dev, values, m2u::has_private_spectrum(plan) ? values : 0, (cudaStream_t)stream) !=
-        cudaSuccess)
+    // values in plan order lie as (re, im), all others as (re, re', im, im')
+    const long long priv = m2u::has_private_spectrum(plan) ? values : 0;
+    const bool fft = m2f::covered(plan);
+    if (m2g::launch_spectrum_conj(kf_in_dev, kf_out_dev, fft ? 0 : values, fft ? values + priv : priv, (cudaStream_t)stream) != cudaSuccess)
         return M2_ERR_CUDA;
     plan->launches += (H > 0);
     return M2_OK;
@@ -313,7 +335,9 @@ static int32_t conv_fwd_grouped(const m2_plan* plan, const void* x_dev, const vo
     if (ust != M2_ERR_UNSUPPORTED) return ust;
     m2g::ConvShape s = conv_shape(plan, B, H, n);
     s.kf_group = (int)kf_group;
-    cudaError_t e = m2g::launch_conv(s, plan->dtype == M2_BF16, x_dev, kf_dev, y_dev, nullptr, (cudaStream_t)stream);
+    const cudaError_t e = m2f::covered(plan)
+                              ? m2f::conv(plan, x_dev, kf_dev, y_dev, B, H, n, mode == M2_CAUSAL, (int)kf_group, (cudaStream_t)stream)
+                              : m2g::launch_conv(s, plan->dtype == M2_BF16, x_dev, kf_dev, y_dev, nullptr, (cudaStream_t)stream);
     if (e == cudaErrorInvalidValue) return M2_ERR_UNSUPPORTED;
     if (e != cudaSuccess) return M2_ERR_CUDA;
     plan->last_kernel = plan->dtype == M2_BF16 ? "conv_generic_bf16io" : "conv_generic_fp32";

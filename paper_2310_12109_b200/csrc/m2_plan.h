@@ -1,5 +1,7 @@
 // Plan object and host-side integer tables of the Monarch library (internal header).
 #pragma once
+#include <cuda_runtime.h>
+
 #include <cstdint>
 #include <vector>
 
@@ -20,9 +22,11 @@ struct m2_plan {
     std::vector<std::vector<int32_t>> tw_exp;  // tw_exp[s-1], s = 1..p-1
 
     // device side
+    void* d_block = nullptr;      // one allocation that holds the status word, the roots and the twiddle factors below
     int32_t* d_status = nullptr;  // error word set by kernels (bounded waits, self checks)
     float2* d_roots[4] = {nullptr, nullptr, nullptr, nullptr};  // omega_{Na}^j, j < Na, per stage
     m2_umma_tables* umma = nullptr;
+    float4* d_fft = nullptr;      // twiddle tables of the fp32 transform kernels (fft_conv.cu); null: the plan has none
 
     mutable const char* last_kernel = "none";
     mutable int64_t launches = 0;

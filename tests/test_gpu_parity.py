@@ -105,6 +105,42 @@ def test_fp32_conv_sign_minus_matches():
     check(y, ref, TOL_FP32, "sign=-1")
 
 
+@pytest.mark.parametrize("dims,n,causal,dtype,B,H,group", [
+    ((16, 16), 256, False, M.M2_BF16, 3, 18, 2), ((16, 16), 77, True, M.M2_FP32, 4, 5, 1), ((32, 16), 233, True, M.M2_BF16, 5, 9, 3),
+    ((32, 32), 1024, False, M.M2_FP32, 1, 5, 1), ((32, 32), 511, True, M.M2_BF16, 2, 6, 1), ((64, 32), 1024, True, M.M2_FP32, 3, 3, 1),
+    ((64, 32), 2048, False, M.M2_BF16, 2, 3, 3), ((64, 64), 2047, True, M.M2_BF16, 3, 4, 2), ((16, 16, 16), 4096, False, M.M2_FP32, 2, 2, 1),
+    ((32, 32, 8), 8192, False, M.M2_BF16, 3, 2, 1), ((32, 32, 8), 3000, True, M.M2_FP32, 2, 3, 1), ((128, 128), 8191, True, M.M2_FP32, 1, 2, 1),
+    ((128, 128), 16384, False, M.M2_BF16, 2, 1, 1)])
+def test_fp32_transform_kernels(dims, n, causal, dtype, B, H, group):
+    """Power-of-two plans from 256 to 16384: every factorisation of the kernels, row pairs with and without a second row, blocks that
+    hold several rows only partly filled, odd lengths.  Forward, spectrum, input gradient, kernel gradient; fp32 arithmetic for both
+    storage types (the bf16 output is rounded once: 2^-8 relative at most, 1.7e-3 in the 2-norm)."""
+    bf, N, Hk = dtype == M.M2_BF16, int(np.prod(dims)), H // group
+    rnd = synth.round_bf16 if bf else (lambda a: a.astype(np.float32))
+    tdt = torch.bfloat16 if bf else torch.float32
+    x, g = rnd(synth.normal(710 + n, (B, H, n))), rnd(synth.normal(711 + n, (B, H, n)))
+    k = (synth.normal(712 + n, (Hk, n)) / np.sqrt(n)).astype(np.float32)
+    plan = M.Plan(dims, dtype=dtype, device=0)
+    mode = M.M2_CAUSAL if causal else M.M2_CIRCULAR
+    xd, gd, kf = dev(x.astype(np.float32), tdt), dev(g.astype(np.float32), tdt), M.m2_kernel_spectrum(plan, dev(k))
+    x64, g64, k64 = x.astype(np.float64), g.astype(np.float64), np.repeat(k.astype(np.float64), group, axis=0)
+    tol = 4e-3 if bf else TOL_FP32
+    y = M.m2_monarch_conv_fwd_grouped(plan, xd, kf, mode, group)
+    fx = np.fft.rfft(x64, N)
+    want = np.fft.irfft(fx * np.fft.rfft(k64, N)[None], N)[..., :n]
+    check(host(y), want, tol, "forward " + plan.last_kernel())
+    dx = M.m2_monarch_conv_fwd_grouped(plan, gd, M.m2_spectrum_conjugate(plan, kf, Hk), mode, group)
+    fg = np.fft.rfft(g64, N)
+    check(host(dx), np.fft.irfft(fg * np.conj(np.fft.rfft(k64, N))[None], N)[..., :n], tol, "input gradient")
+    dk = M.m2_monarch_conv_bwd_kernel(plan, xd, gd, mode)
+    check(host(dk), np.fft.irfft((fg * np.conj(fx)).sum(0), N)[..., :n], TOL_FP32, "kernel gradient")
+    nat = host(M.m2_spectrum_to_natural(plan, kf, Hk))
+    ref = np.conj(np.fft.fft(k.astype(np.float64), N))   # the library's exponent sign is +
+    assert np.linalg.norm(nat[..., 0] + 1j * nat[..., 1] - ref) <= TOL_FP32 * np.linalg.norm(ref)
+    assert plan.device_status() == 0
+    plan.close()
+
+
 # ---- config 2: bf16 circular, N = 512 = 32 x 16 ----------------------------------------------
 
 @pytest.mark.parametrize("B,H", [(4, 24), (3, 5), (1, 1), (32, 9), (9, 5), (16, 3), (19, 6), (40, 150)])
@@ -390,6 +426,7 @@ def test_config5_small():
 
 @pytest.mark.parametrize("T,C,nblk,expand,dims,kernel", [
     (64, 32, 4, 2, (8, 8), "block_generic"),                       # neither tensor-core kernel covers it
+    (256, 32, 4, 2, (16, 16), "block_generic"),                    # the same with the spectrum in the fp32 transform kernels' order
     (512, 128, 4, 2, (32, 16), "block_conv_umma_mlp_generic"),    # tensor-core mixer, CUDA-core MLP
 ])
 def test_block_other_shapes(T, C, nblk, expand, dims, kernel):
