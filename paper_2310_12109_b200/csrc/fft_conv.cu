@@ -4,8 +4,8 @@
 // has the transforms.
 //
 // What bounds it: shared-memory wavefronts (64 KB each way per digit exchange of a 4096-point row) and packed FP32 issue, about equal;
-// with 126 registers four blocks of 128 threads share an SM.  bf16 x[8][768][2000], N = 4096, one B200: 55 us (0.18 of the 9.8 us its
-// bytes take; 59 % of the load/store data pipe, DRAM 11 %), against 6034 us for the kernel before it, which contracted each 64-wide
+// with 126 registers four blocks of 128 threads share an SM.  bf16 x[8][768][2000], N = 4096, one B200: 49 us (0.2 of the roof: its
+// bytes take 9.8 us; 59 % of the load/store data pipe, DRAM 11 %), against 6034 us for the kernel before it, which contracted each 64-wide
 // digit as a dense product in shared memory with a sincos per element.  fp32 x[1][4][256]: 18.4 -> 11.2 us per call, all of it launch
 // and host path.
 #include <atomic>
@@ -33,8 +33,8 @@ __global__ void __launch_bounds__(C::THREADS, min_blocks<C>())
     const long long oa = ((long long)b * H + h) * n, ob = oa + (long long)H * n;
     const bool has_b = live && b + 1 < B;
     u64 re[16], im[16];
-    load_row<C, IO, HALF>(re, live ? x + oa : nullptr, t, n, vec);
-    load_row<C, IO, HALF>(im, has_b ? x + ob : nullptr, t, n, vec);
+    load_row<C, IO, HALF>(re, x + oa, t, n, vec, live);
+    load_row<C, IO, HALF>(im, x + ob, t, n, vec, has_b);
     forward<C, HALF>(re, im, sr, si, tab, t, r);
     const float4* kr = kf + (long long)(h / kf_group) * (C::N / 2) + t;
     unroll<16>([&](auto s) {
@@ -46,8 +46,8 @@ __global__ void __launch_bounds__(C::THREADS, min_blocks<C>())
         re[p] = pr;
     });
     inverse<C, HALF>(re, im, sr, si, tab, t, r);
-    store_row<C, IO, HALF>(re, live ? y + oa : nullptr, t, n, vec);
-    store_row<C, IO, HALF>(im, has_b ? y + ob : nullptr, t, n, vec);
+    store_row<C, IO, HALF>(re, y + oa, t, n, vec, live);
+    store_row<C, IO, HALF>(im, y + ob, t, n, vec, has_b);
 }
 
 // ---- host side -----------------------------------------------------------------------------------------------------------------

@@ -16,7 +16,7 @@ __global__ void __launch_bounds__(C::THREADS, min_blocks<C>())
     float* si = sr + C::SMEM_FLOATS;
     u64 re[16], im[16];
     // rows of k are only as aligned as n floats make them; a pair needs 8 bytes
-    load_row<C, float, HALF>(re, live ? k + h * n : nullptr, t, n, (n & 1) == 0 && (reinterpret_cast<uintptr_t>(k) & 7) == 0);
+    load_row<C, float, HALF>(re, k + h * n, t, n, (n & 1) == 0 && (reinterpret_cast<uintptr_t>(k) & 7) == 0, live);
     unroll<16>([&](auto j) { im[j.v] = 0ull; });
     forward<C, HALF>(re, im, sr, si, tab, t, r);
     if (!live) return;
@@ -30,33 +30,37 @@ __global__ void __launch_bounds__(C::THREADS, min_blocks<C>())
 }
 
 // dk[h] = Re F^-1( sum over row pairs of conj(F z) (.) F w ) / N with z = x_a + i x_b, w = g_a + i g_b: the real part of the product's
-// inverse is corr(x_a, g_a) + corr(x_b, g_b).  One channel per row of threads, the pairs one after the other; the sum stays in
-// registers, F z waits in shared memory in the thread's own slots.
+// inverse is corr(x_a, g_a) + corr(x_b, g_b).  `share` rows of threads (a power of two) take the pairs of one channel in turn; a row's
+// sum stays in registers, F z waits in shared memory in the thread's own slots, and the rows' sums are added in order at the end.
+// (One row per channel left most SMs idle at short lengths: bf16 [64][768][256] 319 -> 35 us, [32][768][512] 176 -> 35 us with the
+// loads of a row in flight together, too.)
 template <class C>
 constexpr int wgrad_blocks() { return C::THREADS == 128 ? 2 : 1; }
 template <class C, typename IO, bool HALF>
 __global__ void __launch_bounds__(C::THREADS, wgrad_blocks<C>())
     fft_wgrad_kernel(const IO* __restrict__ x, const IO* __restrict__ g, float* __restrict__ dk, const float4* __restrict__ tab, int B, int H,
-                     int n) {
+                     int n, int share) {
     extern __shared__ __align__(16) float smem[];
     const int r = threadIdx.x / C::TP, t = threadIdx.x % C::TP;
-    const long long h = (long long)blockIdx.x * C::ROWS + r;
+    const long long h = (long long)blockIdx.x * (C::ROWS / share) + r / share;
     const bool live = h < H, vec = (n & 1) == 0;
     float* sr = smem + r * C::ROWF + (r & 1) * C::PAR;
     float* si = sr + C::SMEM_FLOATS;
-    float4* zs = reinterpret_cast<float4*>(smem + 2 * C::SMEM_FLOATS) + threadIdx.x;
+    float4* zall = reinterpret_cast<float4*>(smem + 2 * C::SMEM_FLOATS);
+    float4* zs = zall + threadIdx.x;
     u64 re[16], im[16], ar[16], ai[16];
     unroll<16>([&](auto s) { ar[s.v] = ai[s.v] = 0ull; });
 #pragma unroll 1
-    for (int b = 0; b < B; b += 2) {
-        const long long oa = ((long long)b * H + h) * n, ob = oa + (long long)H * n;
-        const bool has_b = live && b + 1 < B;
-        load_row<C, IO, HALF>(re, live ? x + oa : nullptr, t, n, vec);
-        load_row<C, IO, HALF>(im, has_b ? x + ob : nullptr, t, n, vec);
+    for (int b0 = 0; b0 < B; b0 += 2 * share) {   // (every row of threads takes every step: the barriers may span several rows)
+        const int b = b0 + 2 * (r % share);
+        const bool has_a = live && b < B, has_b = live && b + 1 < B;
+        const long long oa = has_a ? ((long long)b * H + h) * n : 0, ob = oa + (long long)H * n;
+        load_row<C, IO, HALF>(re, x + oa, t, n, vec, has_a);
+        load_row<C, IO, HALF>(im, x + ob, t, n, vec, has_b);
         forward<C, HALF>(re, im, sr, si, tab, t, r);
         unroll<16>([&](auto s) { zs[s.v * C::THREADS] = make_float4(lo(re[s.v]), hi(re[s.v]), lo(im[s.v]), hi(im[s.v])); });
-        load_row<C, IO, HALF>(re, live ? g + oa : nullptr, t, n, vec);
-        load_row<C, IO, HALF>(im, has_b ? g + ob : nullptr, t, n, vec);
+        load_row<C, IO, HALF>(re, g + oa, t, n, vec, has_a);
+        load_row<C, IO, HALF>(im, g + ob, t, n, vec, has_b);
         row_sync<C>(r);
         forward<C, HALF>(re, im, sr, si, tab, t, r);
         unroll<16>([&](auto s) {   // += conj(z) w
@@ -67,10 +71,34 @@ __global__ void __launch_bounds__(C::THREADS, wgrad_blocks<C>())
         });
         row_sync<C>(r);
     }
+    if (C::ROWS > 1 && share > 1) {   // value (s, t) of a channel = the sum over its rows' threads t; share * TP threads share the work
+        __syncthreads();
+        unroll<16>([&](auto s) { zs[s.v * C::THREADS] = make_float4(lo(ar[s.v]), hi(ar[s.v]), lo(ai[s.v]), hi(ai[s.v])); });
+        __syncthreads();
+        const int first = (r / share) * share * C::TP, lid = threadIdx.x - first, step = share * C::TP;
+        for (int v = lid; v < 16 * C::TP; v += step) {
+            float4* p = zall + (v / C::TP) * C::THREADS + first + v % C::TP;
+            float4 a = *p;
+            for (int q = 1; q < share; ++q) {
+                const float4 w = p[q * C::TP];
+                a.x += w.x;
+                a.y += w.y;
+                a.z += w.z;
+                a.w += w.w;
+            }
+            *p = a;
+        }
+        __syncthreads();
+        unroll<16>([&](auto s) {
+            const float4 a = zall[s.v * C::THREADS + first + t];
+            ar[s.v] = pk(a.x, a.y);
+            ai[s.v] = pk(a.z, a.w);
+        });
+    }
     inverse<C, HALF>(ar, ai, sr, si, tab, t, r);
     const u64 sc = dup2(1.0f / (float)C::N);
     unroll<16>([&](auto s) { ar[s.v] = mul2(ar[s.v], sc); });
-    store_row<C, float, HALF>(ar, live ? dk + h * n : nullptr, t, n, vec);
+    store_row<C, float, HALF>(ar, dk + h * n, t, n, vec, live && r % share == 0);
 }
 
 template <class C>
@@ -115,11 +143,14 @@ cudaError_t wgrad(const m2_plan* pl, const void* x, const void* g, float* dk, in
         if constexpr (C::N > 8192) {
             return cudaErrorInvalidValue;
         } else {
-            const unsigned grid = (unsigned)((H + C::ROWS - 1) / C::ROWS);
+            int share = 1;   // rows of a block per channel: no more than there are pairs
+            while (share < C::ROWS && 2 * share < B) share *= 2;
+            const int64_t per_block = C::ROWS / share;
+            const unsigned grid = (unsigned)((H + per_block - 1) / per_block);
             auto go = [&](auto z, auto half) {
                 using IO = decltype(z);
                 fft_wgrad_kernel<C, IO, decltype(half)::v != 0><<<grid, C::THREADS, wgrad_smem<C>(), stream>>>(
-                    (const IO*)x, (const IO*)g, dk, pl->d_fft, (int)B, (int)H, (int)n);
+                    (const IO*)x, (const IO*)g, dk, pl->d_fft, (int)B, (int)H, (int)n, share);
             };
             if (pl->dtype == M2_BF16) causal ? go(__nv_bfloat16(), Ic<1>{}) : go(__nv_bfloat16(), Ic<0>{});
             else causal ? go(float(), Ic<1>{}) : go(float(), Ic<0>{});
