@@ -18,6 +18,8 @@ int spectrum_order(const m2_plan* pl);
 
 // k_f = F_N pad(k) / N, fp32, in the kernels' own order (fft_core.cuh, spec_index)
 cudaError_t spectrum(const m2_plan* pl, const float* k, int64_t H, int64_t n, void* kf, cudaStream_t stream);
+// the kernel back in the time domain: kt[h][t] = the first n values, fp32 [H][n]
+cudaError_t time_kernel(const m2_plan* pl, const void* kf, int64_t H, int64_t n, float* kt, cudaStream_t stream);
 // y = conv(k[h / kf_group], x[b][h]), x / y [B][H][n] contiguous in the plan dtype
 cudaError_t conv(const m2_plan* pl, const void* x, const void* kf, void* y, int64_t B, int64_t H, int64_t n, bool causal, int kf_group,
                  cudaStream_t stream);

@@ -29,6 +29,28 @@ __global__ void __launch_bounds__(C::THREADS, min_blocks<C>())
     });
 }
 
+// the inverse half alone: real part of the first n positions (the spectrum carries the 1 / N)
+template <class C, bool HALF>
+__global__ void __launch_bounds__(C::THREADS, min_blocks<C>())
+    fft_time_kernel(const float4* __restrict__ kf, float* __restrict__ kt, const float4* __restrict__ tab, int H, int n) {
+    extern __shared__ __align__(16) float smem[];
+    const int r = threadIdx.x / C::TP, t = threadIdx.x % C::TP;
+    const long long h = (long long)blockIdx.x * C::ROWS + r;
+    const bool live = h < H;
+    float* sr = smem + r * C::ROWF + (r & 1) * C::PAR;
+    float* si = sr + C::SMEM_FLOATS;
+    u64 re[16], im[16];
+    const float4* in = kf + (live ? h : 0) * (C::N / 2) + t;
+    unroll<16>([&](auto s) {
+        constexpr int p = brev<4>(s.v);
+        const float4 w = in[s.v * C::TP];
+        re[p] = pk(w.x, w.y);
+        im[p] = pk(w.z, w.w);
+    });
+    inverse<C, HALF>(re, im, sr, si, tab, t, r);
+    store_row<C, float, HALF>(re, kt + h * n, t, n, (n & 1) == 0, live);
+}
+
 // dk[h] = Re F^-1( sum over row pairs of conj(F z) (.) F w ) / N with z = x_a + i x_b, w = g_a + i g_b: the real part of the product's
 // inverse is corr(x_a, g_a) + corr(x_b, g_b).  `share` rows of threads (a power of two) take the pairs of one channel in turn; a row's
 // sum stays in registers, F z waits in shared memory in the thread's own slots, and the rows' sums are added in order at the end.
@@ -109,6 +131,8 @@ cudaError_t prepare_gradients(const m2_plan* pl) {
         using C = decltype(cfg);
         cudaError_t e = allow_smem(fft_spectrum_kernel<C, false>, conv_smem<C>());
         if (e == cudaSuccess) e = allow_smem(fft_spectrum_kernel<C, true>, conv_smem<C>());
+        if (e == cudaSuccess) e = allow_smem(fft_time_kernel<C, false>, conv_smem<C>());
+        if (e == cudaSuccess) e = allow_smem(fft_time_kernel<C, true>, conv_smem<C>());
         if constexpr (C::N <= 8192) {
             auto io = [&](auto z) {
                 using IO = decltype(z);
@@ -131,6 +155,19 @@ cudaError_t spectrum(const m2_plan* pl, const float* k, int64_t H, int64_t n, vo
             fft_spectrum_kernel<C, true><<<grid, C::THREADS, conv_smem<C>(), stream>>>(k, (float4*)kf, pl->d_fft, (int)H, (int)n);
         else
             fft_spectrum_kernel<C, false><<<grid, C::THREADS, conv_smem<C>(), stream>>>(k, (float4*)kf, pl->d_fft, (int)H, (int)n);
+        return cudaGetLastError();
+    });
+}
+
+cudaError_t time_kernel(const m2_plan* pl, const void* kf, int64_t H, int64_t n, float* kt, cudaStream_t stream) {
+    if (H == 0) return cudaSuccess;
+    return dispatch(pl->N, [&](auto cfg) {
+        using C = decltype(cfg);
+        const unsigned grid = (unsigned)((H + C::ROWS - 1) / C::ROWS);
+        if (2 * n <= C::N)
+            fft_time_kernel<C, true><<<grid, C::THREADS, conv_smem<C>(), stream>>>((const float4*)kf, kt, pl->d_fft, (int)H, (int)n);
+        else
+            fft_time_kernel<C, false><<<grid, C::THREADS, conv_smem<C>(), stream>>>((const float4*)kf, kt, pl->d_fft, (int)H, (int)n);
         return cudaGetLastError();
     });
 }

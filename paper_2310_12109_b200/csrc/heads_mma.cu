@@ -1,0 +1,164 @@
+// Head product of the M2 Hyena layer: per (batch entry, head of 16 channels)
+//   O[t][j] = sum_i X1[t][i] ( sum_{s <= t} k[t - s] X2[s][i] V[s][j] ) = sum_{s <= t} k[t - s] (X1[t] . X2[s]) V[s][j],
+// the causal convolution of the 256 sequences of the outer product X2 V^T with the head's kernel, contracted with X1 (App. "GPT Causal
+// Language Modeling").  In the second form the convolution is an n x n Toeplitz factor on the rank-16 scores: two contractions
+// with K = 16 and one product per (t, s), against 256 convolutions of 2 n points.
+//
+// One thread block per (batch entry, head); a warp owns tiles of 16 positions t and walks the tiles of 16 positions s <= t.  A tile pair
+// is four m16n8k16 MMAs on register fragments: the scores' accumulator, times the kernel values and rounded to bf16, IS the second
+// product's B operand (rows of an accumulator fragment = columns of a B fragment), so nothing goes through shared memory between the
+// two products and no warp waits for another.  (tcgen05 would put every tile through tensor memory, shared memory and two barriers for
+// 8 K multiply-adds.)  Kernel values lie reversed in shared memory, in two copies one element apart, so that the two values of a
+// fragment's column pair are one aligned 64-bit load for even and odd rows alike; lags below zero are stored as zeros.
+//
+// Measured, one B200, layer at B = 32, n = 256, d = 768 (1536 heads): 403 -> 163 us with this kernel in place of 24 576 tensor-core
+// convolution units of 16 rows each (about 280 us of the 403).  Bound by instruction issue: 136 tile pairs of about 20 instructions.
+#include <cuda_bf16.h>
+
+#include "fft_conv.h"
+#include "fft_core.cuh"
+#include "heads_mma.h"
+#include "m2_plan.h"
+
+namespace m2h {
+
+constexpr int kThreads = 256, kDh = 16, kMaxN = 1024;
+
+__host__ __device__ constexpr int padded(int n) { return (n + 15) / 16 * 16; }
+__host__ __device__ constexpr int pitch(int n) { return padded(n) + 8; }              // bf16 elements: rows 16 bytes apart mod 128
+__host__ __device__ constexpr int kcopy(int n) { return padded(n) + 32; }             // floats of one reversed copy of the kernel
+__host__ __device__ constexpr int smem_bytes(int n) { return 3 * kDh * pitch(n) * 2 + 2 * kcopy(n) * 4; }
+
+__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void ldsm4(uint32_t* r, uint32_t a) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a));
+}
+__device__ __forceinline__ void ldsm4t(uint32_t* r, uint32_t a) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a));
+}
+__device__ __forceinline__ void mma(float* d, const uint32_t* a, uint32_t b0, uint32_t b1) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ uint32_t bf2(float a, float b) {
+    const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const uint32_t*>(&v);
+}
+// bf16 pair of the products (a, b) * (k.x, k.y)
+__device__ __forceinline__ uint32_t weigh(float a, float b, float2 k) {
+    const m2f::u64 p = m2f::mul2(m2f::pk(a, b), m2f::pk(k.x, k.y));
+    return bf2(m2f::lo(p), m2f::hi(p));
+}
+
+__global__ void __launch_bounds__(kThreads)
+    heads_kernel(const __nv_bfloat16* __restrict__ X1, const __nv_bfloat16* __restrict__ X2, const __nv_bfloat16* __restrict__ V,
+                 const float* __restrict__ kt, __nv_bfloat16* __restrict__ O, int heads, int n) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int np = padded(n), ld = pitch(n), kc = kcopy(n);
+    __nv_bfloat16* xs1 = reinterpret_cast<__nv_bfloat16*>(smem);
+    __nv_bfloat16* xs2 = xs1 + kDh * ld;
+    __nv_bfloat16* vs = xs2 + kDh * ld;
+    float* ks = reinterpret_cast<float*>(vs + kDh * ld);
+    const int h = blockIdx.x % heads;
+    const size_t base = (size_t)blockIdx.x * kDh * n;   // the 16 channels of a head are consecutive rows
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // copy p (p = 0, 1): the kernel value of a lag lies at np + 14 + p - lag
+    for (int i = tid; i < 2 * kc; i += kThreads) {
+        const int p = i >= kc, lag = np + 14 + p - (i - p * kc);
+        ks[i] = lag >= 0 && lag < n ? kt[(size_t)h * n + lag] : 0.f;
+    }
+    const __nv_bfloat16* src[3] = {X1 + base, X2 + base, V + base};
+    if (n % 8 == 0) {   // 16-byte pieces never straddle a row
+        const int per_row = n / 8;
+        for (int i = tid; i < kDh * per_row; i += kThreads) {
+            const int r = i / per_row, c = (i % per_row) * 8;
+#pragma unroll
+            for (int q = 0; q < 3; ++q)
+                *reinterpret_cast<uint4*>(xs1 + q * kDh * ld + r * ld + c) = __ldg(reinterpret_cast<const uint4*>(src[q]) + i);
+        }
+        if (np != n && tid < 3 * kDh) *reinterpret_cast<uint4*>(xs1 + tid * ld + n) = make_uint4(0u, 0u, 0u, 0u);
+    } else {
+        for (int i = tid; i < kDh * np; i += kThreads) {
+            const int r = i / np, c = i % np;
+#pragma unroll
+            for (int q = 0; q < 3; ++q) xs1[q * kDh * ld + r * ld + c] = c < n ? src[q][(size_t)r * n + c] : __float2bfloat16_rn(0.f);
+        }
+    }
+    __syncthreads();
+    const int m = lane >> 3, r8 = lane & 7, g = lane >> 2, c2 = 2 * (lane & 3);
+    // ldmatrix row addresses: A of the scores (X1, transposed on load), B of the scores (X2, transposed), A of the output (V)
+    const uint32_t a1 = smem_addr(xs1 + ((m >> 1) * 8 + r8) * ld + (m & 1) * 8);
+    const uint32_t b2 = smem_addr(xs2 + ((m & 1) * 8 + r8) * ld + (m >> 1) * 8);
+    const uint32_t av = smem_addr(vs + ((m & 1) * 8 + r8) * ld + (m >> 1) * 8);
+    const float* kp = ks + (g & 1) * kc + np + 14 + (g & 1) - g + c2;   // lag g - c2; minus the tile distance
+    const int tiles = np / 16, nw = kThreads / 32;
+    const int front = nw * ((tiles + 2 * nw - 1) / (2 * nw));   // the first half of a warp's tiles in order, the second from the far end:
+    for (int it = warp; it < tiles; it += nw) {                 // every warp gets as many short tiles as long ones
+        const int ti = it < front ? it : tiles - 1 - (it - front);
+        uint32_t fa[4];
+        ldsm4t(fa, a1 + ti * 32);
+        float o[2][4] = {};
+        for (int si = 0; si <= ti; ++si) {
+            uint32_t fb[4], fv[4];
+            ldsm4t(fb, b2 + si * 32);
+            ldsm4(fv, av + si * 32);
+            const float* kq = kp - (ti - si) * 16;
+            const float2 k0 = *reinterpret_cast<const float2*>(kq), k8 = *reinterpret_cast<const float2*>(kq - 8),
+                         km = *reinterpret_cast<const float2*>(kq + 8);   // lags u, u + 8, u - 8 and the one below each
+            float s0[4] = {}, s1[4] = {};
+            mma(s0, fa, fb[0], fb[1]);
+            mma(s1, fa, fb[2], fb[3]);
+            mma(o[0], fv, weigh(s0[0], s0[1], k0), weigh(s1[0], s1[1], km));
+            mma(o[1], fv, weigh(s0[2], s0[3], k8), weigh(s1[2], s1[3], k0));
+        }
+        __syncwarp();   // this tile's columns of X1 are read by this warp only: the result takes their place
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+            *reinterpret_cast<uint32_t*>(xs1 + g * ld + ti * 16 + x * 8 + c2) = bf2(o[x][0], o[x][1]);
+            *reinterpret_cast<uint32_t*>(xs1 + (g + 8) * ld + ti * 16 + x * 8 + c2) = bf2(o[x][2], o[x][3]);
+        }
+    }
+    __syncthreads();
+    if (n % 8 == 0) {
+        const int per_row = n / 8;
+        for (int i = tid; i < kDh * per_row; i += kThreads)
+            reinterpret_cast<uint4*>(O + base)[i] = *reinterpret_cast<const uint4*>(xs1 + (i / per_row) * ld + (i % per_row) * 8);
+    } else {
+        for (int i = tid; i < kDh * n; i += kThreads) O[base + i] = xs1[(i / n) * ld + i % n];
+    }
+}
+
+bool covered(const m2_plan* pl, int64_t n, int64_t d, int64_t dh) {
+    return pl->dtype == M2_BF16 && m2f::covered(pl) && dh == kDh && d % kDh == 0 && n > 0 && n <= kMaxN;
+}
+
+int32_t heads_fwd(const m2_plan* pl, const void* X1, const void* X2, const void* V, const float* kt, void* O, int64_t B, int64_t d, int64_t n,
+                  cudaStream_t stream) {
+    const int64_t blocks = B * (d / kDh);
+    if (blocks == 0) return M2_OK;
+    if (blocks > 0x7fffffffLL) return M2_ERR_UNSUPPORTED;
+    const int smem = smem_bytes((int)n);
+    if (smem > 48 * 1024 && cudaFuncSetAttribute(heads_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(kMaxN)) != cudaSuccess)
+        return M2_ERR_CUDA;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, heads_kernel, (const __nv_bfloat16*)X1, (const __nv_bfloat16*)X2, (const __nv_bfloat16*)V, kt,
+                           (__nv_bfloat16*)O, (int)(d / kDh), (int)n) != cudaSuccess)
+        return M2_ERR_CUDA;
+    pl->launches += 1;
+    return M2_OK;
+}
+
+}  // namespace m2h

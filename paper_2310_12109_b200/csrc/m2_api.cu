@@ -12,6 +12,7 @@
 #include "conv_umma.h"
 #include "fft_conv.h"
 #include "generic_kernels.h"
+#include "heads_mma.h"
 #include "cols_umma.h"
 #include "matmul_umma.h"
 #include "mlp_umma.h"
@@ -630,12 +631,8 @@ int32_t m2_bert_mixer_fwd(const m2_plan* plan, const void* x_dev, const void* co
     return M2_OK;
 }
 
-// heads of 16 channels on the N = 512 tensor-core plan: outer product, long convolution and contraction are one kernel and the
-// dh-times larger tensors do not exist
-static bool hyena_heads_fused(const m2_plan* plan, int64_t n, int64_t d, int64_t dh) {
-    return plan->dtype == M2_BF16 && m2u::has_private_spectrum(plan) && !m2u3::covered(plan) && dh == 16 && d % 16 == 0 && n % 16 == 0 &&
-           n <= 256;
-}
+// heads of 16 channels (bf16): outer product, long convolution and contraction are one kernel and the dh-times larger tensors do not exist
+static bool hyena_heads_fused(const m2_plan* plan, int64_t n, int64_t d, int64_t dh) { return m2h::covered(plan, n, d, dh); }
 
 int64_t m2_hyena_scratch_bytes(const m2_plan* plan, int64_t B, int64_t n, int64_t d, int64_t dh) {
     if (!plan || B < 0 || n < 0 || d < 0 || dh <= 0) return -1;
@@ -673,6 +670,12 @@ int32_t m2_hyena_heads_fwd(const m2_plan* plan, const void* u_dev, const void* c
         plan->launches += 1;
         return M2_OK;
     };
+    // the fused head product wants the long kernels in the time domain, [d / dh][n] fp32: they wait in y, which is written last
+    float* kt = static_cast<float*>(y_dev);
+    if (hyena_heads_fused(plan, n, d, dh)) {
+        if (m2f::time_kernel(plan, kf_long_dev, d / dh, n, kt, st) != cudaSuccess) return M2_ERR_CUDA;
+        plan->launches += 1;
+    }
     // channel-first from here on: every projection, convolution and head product works on rows of n positions
     if (m2g::launch_transpose_any(u_dev, uT, B, (int)n, (int)d, bf, st) != cudaSuccess) return M2_ERR_CUDA;
     int32_t rc = dense(W[0], uT, P1);
@@ -683,7 +686,7 @@ int32_t m2_hyena_heads_fwd(const m2_plan* plan, const void* u_dev, const void* c
     if (rc == M2_OK) rc = m2_monarch_conv_fwd(plan, P3, kf3_dev, C3, B, d, n, M2_CAUSAL, stream);
     if (rc != M2_OK) return rc;
     if (hyena_heads_fused(plan, n, d, dh)) {
-        rc = m2u::conv_heads_fwd(plan, C1, C2, C3, kf_long_dev, P1, B, d, dh, n, st);
+        rc = m2h::heads_fwd(plan, C1, C2, C3, kt, P1, B, d, n, st);
         if (rc != M2_OK) return rc;
     } else {
         if (m2g::launch_heads_outer(C2, C3, XV, B, (int)d, (int)dh, (int)n, bf, st) != cudaSuccess) return M2_ERR_CUDA;

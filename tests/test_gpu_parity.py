@@ -765,6 +765,32 @@ def test_m2_hyena_heads_fwd(B, n, d, dh, dims, dtype):
     plan.close()
 
 
+@pytest.mark.parametrize("B,n,d,dims", [(1, 8, 16, (32, 16)), (2, 200, 64, (32, 16)), (2, 77, 64, (32, 16)), (1, 512, 32, (32, 32))])
+def test_hyena_head_product_tiles(B, n, d, dims):
+    """The fused head product (heads of 16) where its tiles of 16 positions can go wrong: one half-empty tile, 13 tiles (warps with one
+    and with two), rows that are not whole 16-byte pieces, four tiles per warp on the 1024-point plan.  Identity projections and
+    pass-through short kernels leave O[t] = sum_{s <= t} k[t - s] (u[t] . u[s]) u[s] per head, computed here as written."""
+    u = synth.round_bf16(synth.normal(synth.stream_id(18, n), (B, n, d)))
+    k = (synth.normal(synth.stream_id(18, n + 1), (d // 16, n)) * np.exp(-0.05 * np.arange(n))[None] / 4).astype(np.float32)
+    delta = np.zeros((d, n), dtype=np.float32)
+    delta[:, 0] = 1.0
+    plan = M.Plan(dims, dtype=M.M2_BF16, device=0)
+    kfd, kfl = M.m2_kernel_spectrum(plan, dev(delta)), M.m2_kernel_spectrum(plan, dev(k))
+    eye = torch.eye(d, dtype=torch.bfloat16, device="cuda")
+    y = M.m2_hyena_heads_fwd(plan, dev(u.astype(np.float32), torch.bfloat16), [eye] * 4, kfd, kfd, kfd, kfl, 16)
+    torch.cuda.synchronize()
+    assert plan.device_status() == 0 and plan.last_kernel() == "hyena_heads_fwd_fused"
+    uh = u.astype(np.float64).reshape(B, n, d // 16, 16)
+    lag = np.arange(n)[:, None] - np.arange(n)[None]
+    T = np.where(lag >= 0, k.astype(np.float64)[:, np.maximum(lag, 0)], 0.0)          # [heads, t, s]
+    want = np.einsum("hts,bthi,bshi,bshj->bthj", T, uh, uh, uh, optimize=True).reshape(B, n, d)
+    got = host(y)
+    # weighed scores and the result are rounded to bf16 (2^-9 each at most, independent), the unit-kernel convolutions round too
+    assert np.linalg.norm(got - want) <= TOL_BF16 / 2 * np.linalg.norm(want)
+    assert np.abs(got - want).max() <= 8 * TOL_BF16 * np.sqrt(np.mean(want ** 2)) + 2 * TOL_BF16 * np.abs(want).max()
+    plan.close()
+
+
 def test_m2_hyena_heads_full_size_sampled():
     """The layer at the benchmark shape (B = 32, n = 256, d = 768, heads of 16: 24 576 units of the fused kernel, many rounds per
     pipeline); batch entries are independent, so the first and the last one are compared with the oracle run on them alone."""
