@@ -24,7 +24,6 @@
 // barrier latency is covered by the others' fp32 work.  Units are handed out by a device-wide counter; the kernel is
 // launched with programmatic stream serialization (set-up overlaps the previous kernel's tail).  All waits are bounded.
 #include "conv_umma.h"
-#include "fft_core.cuh"
 
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -832,38 +831,42 @@ conv512p_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
 //
 //   dk[h] = M^-1 ( sum_b conj(M x_b) (.) M g_b ) [0:n)          (the transpose of Eq. 2 with respect to k)
 //
-// The forward half of the pipeline above (S1, twiddle, S2) runs on the x tile and on the g tile of a unit (8 batch
-// entries of one channel) side by side: 128 TMEM columns per pipeline, 4 pipelines per CTA.  Each thread then holds the
-// two spectra of its rows at the same (k1, k2), forms conj(X) G in fp32, adds its two rows, the four warps' sums are
-// added through shared memory, and the unit's [k1][k2] sum goes to partial[b group][h] in plan order.  A CUDA-core
-// kernel adds the b groups in order and applies M^-1 in fp32 (one block per channel).
+// The forward half of the row-pair pipeline above (S1, twiddle, S2) runs on the x tile and on the g tile of a unit (16 batch rows of
+// one channel) side by side: with z = x_a + i x_b and w = g_a + i g_b the real part of M^-1(conj(M z) (.) M w) is the sum of the two
+// rows' correlations, so a pair costs what a row would.  128 TMEM columns per pipeline, 4 pipelines per CTA; two issuing threads, one
+// per tile.  Each thread then holds the two spectra of its rows at the same (k1, k2), forms conj(Z) W in fp32, adds its two rows, the
+// four warps' sums are added through shared memory, and the unit's sum goes to partial[b group][h] in the order of the fp32
+// transform kernels (fft_core.cuh), which add the b groups in order and apply M^-1 (m2f::time_kernel).
+// Shared memory per pipeline: x tile | A2 of x | g tile; A2 of g takes the place of the x tile.  Bound by the hand-offs' latency (as
+// the forward kernel): x, g [32][768][512]: 30 -> 20 us against one row per lane, and 14.6 -> 6 us for the sum and M^-1.
 constexpr int kGroupsW = 4;
 constexpr int kThreadsW = 128 * kGroupsW;
-constexpr int WG_X = 0;              // x tile 8192 | g tile 8192 (one box [r][n1][16 n2] each, 32-byte swizzled)
-constexpr int WG_A = 16384;          // A2 of x 16384 | A2 of g 16384; afterwards the four warps' sums [warp][k2][33 k1] float2
+constexpr int WG_X = 0;              // re tile 8192 | im tile 8192 (one box [r][n1][16 n2] each, 32-byte swizzled); later A2 of g
+constexpr int WG_A = 16384;          // A2 of x; afterwards the four warps' sums [warp][k2][k1] float2
+constexpr int WG_G = 32768;          // as WG_X
 constexpr int W_GROUP_BYTES = 49152;
-constexpr int W_SMEM_BYTES = OFF_GROUP + kGroupsW * W_GROUP_BYTES;
-static_assert(W_SMEM_BYTES <= 232448 && 4 * 16 * 33 * 8 <= 32768, "per-CTA budgets");
+constexpr int W_SMEM_BYTES = P_OFF_GROUP + kGroupsW * W_GROUP_BYTES;
+static_assert(W_SMEM_BYTES <= 232448 && 4 * 16 * 32 * 8 <= 16384 && 128 * kGroupsW <= kTmemCols, "per-CTA budgets");
 
 __global__ void __launch_bounds__(kThreadsW, 1)
-convwgrad512_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_g, float2* __restrict__ partial,
-                    const uint4* __restrict__ consts, int B, int H, int n, int32_t* __restrict__ status) {
+convwgrad512_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_g, float4* __restrict__ partial,
+                    const uint4* __restrict__ consts, int B, int H, int n, float sgn, int32_t* __restrict__ status) {
     extern __shared__ __align__(1024) unsigned char smem_all[];
     const int wg = threadIdx.x >> 7, tid = threadIdx.x & 127, warp = tid >> 5;
-    const bool leader = tid == 32 * (wg & 3);
+    const bool leader = tid == 32 * (wg & 3), leader2 = tid == 32 * ((wg + 2) & 3);   // issue for the x tile and for the g tile
     const uint32_t s_all = smem_u32(smem_all);
-    unsigned char* smem = smem_all + OFF_GROUP + wg * W_GROUP_BYTES;
-    const uint32_t s_base = s_all + OFF_GROUP + wg * W_GROUP_BYTES;
-    const uint32_t bar_x = s_all + OFF_BAR + wg * 32, bar_mma = bar_x + 8;
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_all + OFF_BAR + wg * 32 + 24);
-    const uint32_t s_tptr = s_all + OFF_BAR + 512;
-    const int bgroups = (B + kRows - 1) / kRows;
-    const int units = H * bgroups;
+    unsigned char* smem = smem_all + P_OFF_GROUP + wg * W_GROUP_BYTES;
+    const uint32_t s_base = s_all + P_OFF_GROUP + wg * W_GROUP_BYTES;
+    const uint32_t bar_x = s_all + P_OFF_BAR + wg * 32, bar_mma = bar_x + 8, bar_g = bar_x + 16;
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_all + P_OFF_BAR + wg * 32 + 24);
+    const uint32_t s_tptr = s_all + P_OFF_BAR + 512;
+    const int units = H * ((B + 2 * kRows - 1) / (2 * kRows));
     const int ustride = gridDim.x * kGroupsW;
     int u = wg * gridDim.x + blockIdx.x;   // pipeline-major: a partial last round spreads over all CTAs
     if (leader) {
         mbar_init(bar_x, 1);
-        mbar_init(bar_mma, 1);
+        mbar_init(bar_g, 1);
+        mbar_init(bar_mma, 2);   // both issuing threads commit in every stage
         *abort_flag = 0;
         fence_barrier_init();
         prefetch_tensormap(&map_x);
@@ -871,25 +874,28 @@ convwgrad512_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
     }
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     {
-        uint4* dst = reinterpret_cast<uint4*>(smem_all + OFF_CONST);
-        for (int i = threadIdx.x; i < CONST_BYTES / 16; i += kThreadsW) dst[i] = consts[i];
+        uint4* dst = reinterpret_cast<uint4*>(smem_all);
+        for (int i = threadIdx.x; i < P_CONST_BYTES / 16; i += kThreadsW) dst[i] = consts[i];
     }
     if (threadIdx.x < 32) tmem_alloc(s_tptr, kTmemCols);
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    bool x_pending = false;
-    auto load_unit = [&](int v) {   // both tiles of unit v, one barrier phase
-        mbar_expect_tx(bar_x, 16384);
-        const int hh = v % H, bb = (v / H) * kRows;
-        tma_load_4d(s_base + WG_X, &map_x, 0, 0, hh, bb, bar_x);          // boxes [8 rows][32 n1][16 n2], 32-byte swizzled
-        tma_load_4d(s_base + WG_X + 8192, &map_g, 0, 0, hh, bb, bar_x);
-        x_pending = true;
+    bool x_pending = false, g_pending = false;   // copies in flight (leader)
+    auto load_tile = [&](const CUtensorMap* map, int off, uint32_t bar, int v) {   // the two boxes [8 rows][32 n1][16 n2] of unit v
+        const int hh = v % H, bb = (v / H) * 2 * kRows;
+        mbar_expect_tx(bar, 16384);
+        tma_load_4d(s_base + off, map, 0, 0, hh, bb, bar);
+        tma_load_4d(s_base + off + 8192, map, 0, 0, hh, bb + kRows, bar);
     };
-    if (leader && u < units) load_unit(u);
+    if (leader && u < units) {
+        load_tile(&map_x, WG_X, bar_x, u);
+        load_tile(&map_g, WG_G, bar_g, u);
+        x_pending = g_pending = true;
+    }
     fence_proxy_async();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_cta = *reinterpret_cast<volatile uint32_t*>(smem_all + OFF_BAR + 512);
+    const uint32_t tmem_cta = *reinterpret_cast<volatile uint32_t*>(smem_all + P_OFF_BAR + 512);
     const uint32_t tmem = tmem_cta + wg * 128;
     const uint32_t t_lane = tmem + ((uint32_t)(warp * 32) << 16);
     constexpr uint32_t ID_S1 = instr_desc_bf16(128, 64, true, false);
@@ -900,18 +906,18 @@ convwgrad512_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
     while (u < units) {
         const int h = u % H, bg = u / H;
         const int un = u + ustride;
-        // ---- S1 on both tiles -----------------------------------------------------------------------
-        if (leader) {
-            ok = mbar_wait(bar_x, ph_x);
-            x_pending = false;
+        // ---- S1: one issuing thread per tile ----------------------------------------------------------------
+        if (leader || leader2) {
+            const int off = leader ? WG_X : WG_G, col = leader ? 0 : 64;
+            ok = mbar_wait(leader ? bar_x : bar_g, ph_x);
             if (ok) {
                 tc_fence_after();
 #pragma unroll
-                for (int tt = 0; tt < 2; ++tt)
+                for (int c = 0; c < 2; ++c)   // K = (re | im part of the input) x n1
 #pragma unroll 1
                     for (int s = 0; s < k1steps; ++s)
-                        umma_f16(tmem + 64 * tt, smem_desc_sw32(s_base + WG_X + tt * 8192 + s * 512, 1024, 256),
-                                 smem_desc(s_all + OFF_B1 + s * 256, 128, 512), ID_S1, s > 0);
+                        umma_f16(tmem + col, smem_desc_sw32(s_base + off + c * 8192 + s * 512, 1024, 256),
+                                 smem_desc(s_all + P_OFF_B1 + (2 * c + s) * 256, 128, 1024), ID_S1, (c | s) > 0);
                 umma_commit(bar_mma);
             }
         }
@@ -919,11 +925,17 @@ convwgrad512_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
         ok = ok && mbar_wait(bar_mma, ph_m);
         ph_m ^= 1;
         tc_fence_after();
-        if (leader && ok && un < units) load_unit(un);   // the tiles are free
+        if (leader && ok) {   // both tiles have landed and been read
+            x_pending = g_pending = false;
+            if (un < units) {
+                load_tile(&map_g, WG_G, bar_g, un);
+                g_pending = true;
+            }
+        }
         // ---- h1: twiddle, A2 of x and of g ---------------------------------------------------------------
         if (ok) {
             const int r = tid >> 4, n2 = tid & 15, n2hi = n2 >> 3, n2lo = n2 & 7;   // lane = r * 16 + n2: the row order of the input boxes
-            const float4* twA = reinterpret_cast<const float4*>(smem_all + OFF_TWA) + n2;
+            const float4* twA = reinterpret_cast<const float4*>(smem_all + P_OFF_TWA) + n2;
 #pragma unroll 1
             for (int tt = 0; tt < 2; ++tt)
 #pragma unroll
@@ -948,7 +960,7 @@ convwgrad512_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
                         for (int q = 0; q < 4; ++q) w[q] = twA[(4 * j + q) * 16];
                         uint4 pr, pi;
                         cmul_pack8(re + 8 * jj, im + 8 * jj, w, pr, pi);
-                        unsigned char* base = smem + WG_A + tt * 16384 + (r * 4 + j) * 512 + n2lo * 16;
+                        unsigned char* base = smem + (tt ? WG_X : WG_A) + (r * 4 + j) * 512 + n2lo * 16;
                         *reinterpret_cast<uint4*>(base + (0 + n2hi) * 128) = pr;
                         *reinterpret_cast<uint4*>(base + (2 + n2hi) * 128) = pi;
                     }
@@ -960,24 +972,27 @@ convwgrad512_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
             aborted = true;
             break;
         }
-        // ---- S2 on both ---------------------------------------------------------------------------------
-        if (leader) {
+        // ---- S2: likewise ---------------------------------------------------------------------------------
+        if (leader || leader2) {
             tc_fence_after();
+            const int off = leader ? WG_A : WG_X, col = leader ? 0 : 64;
 #pragma unroll
-            for (int tt = 0; tt < 2; ++tt)
+            for (int hf = 0; hf < 2; ++hf)
 #pragma unroll
-                for (int hf = 0; hf < 2; ++hf)
-#pragma unroll
-                    for (int s = 0; s < 2; ++s)
-                        umma_f16(tmem + 64 * tt + hf * 32, smem_desc(s_base + WG_A + tt * 16384 + hf * 8192 + s * 256, 128, 512),
-                                 smem_desc(s_all + OFF_B2 + s * 256, 128, 512), ID_S2, s > 0);
+                for (int s = 0; s < 2; ++s)
+                    umma_f16(tmem + col + hf * 32, smem_desc(s_base + off + hf * 8192 + s * 256, 128, 512),
+                             smem_desc(s_all + P_OFF_B2 + s * 256, 128, 512), ID_S2, s > 0);
             umma_commit(bar_mma);
         }
         ok = mbar_wait(bar_mma, ph_m);
         ph_m ^= 1;
         tc_fence_after();
-        // ---- conj(X) G, summed over this thread's two rows, then over the four warps ------------------------------
-        float2* red = reinterpret_cast<float2*>(smem + WG_A);   // [warp][k2][33]: both A2 buffers are free now
+        if (leader && ok && un < units) {   // A2 of g has been read
+            load_tile(&map_x, WG_X, bar_x, un);
+            x_pending = true;
+        }
+        // ---- conj(Z) W, summed over this thread's two rows, then over the four warps ------------------------------
+        float2* red = reinterpret_cast<float2*>(smem + WG_A);   // [warp][k2][k1]: A2 of x is free now
         if (ok) {
             const int k1 = tid & 31;
 #pragma unroll
@@ -1004,7 +1019,7 @@ convwgrad512_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
                     }
                 }
 #pragma unroll
-                for (int q = 0; q < 8; ++q) red[(warp * 16 + 8 * g + q) * 33 + k1] = make_float2(sr[q], si[q]);
+                for (int q = 0; q < 8; ++q) red[(warp * 16 + 8 * g + q) * 32 + k1] = make_float2(sr[q], si[q]);
             }
         }
         tc_fence_before();
@@ -1012,19 +1027,21 @@ convwgrad512_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
             aborted = true;
             break;
         }
-        {
-            float2* dst = partial + ((size_t)bg * H + h) * 512;
+        {   // frequencies k1 + 32 k2 and k1 + 32 (k2 + 8) are one quad of the transform kernels' order (exponent sign +)
+            float4* dst = partial + ((size_t)bg * H + h) * 256;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int p = tid + 128 * i, k1 = p >> 4, k2 = p & 15;   // plan order
-                float2 a = red[(0 * 16 + k2) * 33 + k1];
+            for (int i = 0; i < 2; ++i) {
+                const int p = tid + 128 * i;   // k2 * 32 + k1, k2 < 8
+                float2 a = red[p], b = red[p + 256];
 #pragma unroll
                 for (int w = 1; w < 4; ++w) {
-                    const float2 b = red[(w * 16 + k2) * 33 + k1];
-                    a.x += b.x;
-                    a.y += b.y;
+                    const float2 c = red[w * 512 + p], d = red[w * 512 + p + 256];
+                    a.x += c.x;
+                    a.y += c.y;
+                    b.x += d.x;
+                    b.y += d.y;
                 }
-                dst[p] = a;
+                dst[p] = make_float4(a.x, b.x, sgn * a.y, sgn * b.y);
             }
         }
         if (group_sync_or(wg, false, abort_flag)) {   // the sums are read: the next unit's h1 may overwrite them
@@ -1036,22 +1053,11 @@ convwgrad512_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
     if (leader) {
         if (aborted) atomicExch(status, (int32_t)M2_ERR_TIMEOUT);
         if (x_pending) mbar_wait(bar_x, ph_x);
+        if (g_pending) mbar_wait(bar_g, ph_x);
     }
     tc_fence_before();
     __syncthreads();
     if (threadIdx.x < 32) tmem_dealloc(tmem_cta, kTmemCols);
-}
-
-// spectrum re-layout for this kernel: kfu[h][k2/2][k1] = (re(k2 even), re(k2 odd), im(even), im(odd)) from plan order
-__global__ void relayout_spectrum_kernel(const float* __restrict__ kf, float4* __restrict__ kfu, long long total, float sgn) {
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;   // over H * 8 * 32
-    if (i >= total) return;
-    const int k1 = (int)(i & 31), q = (int)((i >> 5) & 7);
-    const long long h = i >> 8;
-    const float* row = kf + h * 1024;   // in the order of the fp32 transform kernels; frequency k1 + 32 k2, k2 = 2 q, 2 q + 1
-    const int ka = k1 + 64 * q, kb = ka + 32;
-    kfu[i] = make_float4(row[m2f::spec_index<m2f::Cfg<9>>(ka, false)], row[m2f::spec_index<m2f::Cfg<9>>(kb, false)],
-                         sgn * row[m2f::spec_index<m2f::Cfg<9>>(ka, true)], sgn * row[m2f::spec_index<m2f::Cfg<9>>(kb, true)]);
 }
 
 // ---- host side ---------------------------------------------------------------------------------------
@@ -1260,57 +1266,11 @@ int32_t conv_fwd_wait_selftest(const m2_plan* pl, const void* x, const void* kf,
     return conv_fwd_impl(pl, x, kf, y, B, H, n, mode, stream, 1, 1);
 }
 
-// dk[h] = Re M^-1 ( sum_p partial[p][h][:] ) [0:n) / 512 for N = 512 = 32 x 16: the parts added in index order, then the two
-// inverse stages in fp32 (conj F_16 over k2 with the conjugated twiddle, conj F_32 over k1, real part); one block per channel
-__global__ void __launch_bounds__(256) wgrad512_finish_kernel(const float2* __restrict__ partial, int parts, float* __restrict__ dk,
-                                                              const float2* __restrict__ roots32, const float2* __restrict__ roots16, int H, int n,
-                                                              float sgn) {
-    __shared__ float2 a[512], bb[512], r32[32], r16[16];
-    const int h = blockIdx.x, tid = threadIdx.x;
-    if (tid < 32) r32[tid] = roots32[tid];
-    if (tid < 16) r16[tid] = roots16[tid];
-    for (int i = tid; i < 512; i += 256) {
-        float2 v = make_float2(0.f, 0.f);
-        for (int p = 0; p < parts; ++p) {
-            const float2 w = partial[((size_t)p * H + h) * 512 + i];
-            v.x += w.x;
-            v.y += w.y;
-        }
-        a[i] = v;
-    }
-    __syncthreads();
-    for (int o = tid; o < 512; o += 256) {   // (k1, n2) = sum_k2 conj(w_16^{k2 n2}) a[k1][k2], times conj(w_512^{n2 k1})
-        const int k1 = o >> 4, n2 = o & 15;
-        float sr = 0.f, si = 0.f;
-#pragma unroll
-        for (int k2 = 0; k2 < 16; ++k2) {
-            const float2 w = r16[(k2 * n2) & 15], v = a[k1 * 16 + k2];   // conj(w) v = (wx vx + wy vy) + i (wx vy - wy vx)
-            sr = fmaf(w.x, v.x, fmaf(w.y, v.y, sr));
-            si = fmaf(w.x, v.y, fmaf(-w.y, v.x, si));
-        }
-        float ts, tc;
-        sincospif(2.0f * (float)((n2 * k1) & 511) / 512.0f, &ts, &tc);
-        ts *= sgn;   // w_512^{n2 k1} = tc + i ts; multiply by its conjugate
-        bb[o] = make_float2(sr * tc + si * ts, si * tc - sr * ts);
-    }
-    __syncthreads();
-    for (int t = tid; t < 512; t += 256) {   // y[n1*16 + n2] = Re sum_k1 conj(w_32^{k1 n1}) bb[k1][n2]
-        const int n1 = t >> 4, n2 = t & 15;
-        float acc = 0.f;
-#pragma unroll
-        for (int k1 = 0; k1 < 32; ++k1) {
-            const float2 w = r32[(k1 * n1) & 31], v = bb[k1 * 16 + n2];
-            acc = fmaf(w.x, v.x, fmaf(w.y, v.y, acc));
-        }
-        if (t < n) dk[(size_t)h * n + t] = acc * (1.0f / 512.0f);
-    }
-}
-
 int64_t conv_wgrad_workspace_bytes(const m2_plan* pl, int64_t B, int64_t H) {
-    return pl->umma && covered(pl) ? ((B + kRows - 1) / kRows) * H * 512 * 8 : 0;
+    return pl->umma && covered(pl) ? ((B + 2 * kRows - 1) / (2 * kRows)) * H * 512 * 8 : 0;
 }
 
-// partial[b group][h][512] (plan order) = sum over the group's rows of conj(M x) (.) M g; returns the number of b groups in *parts
+// partial[b group][h][512] (transform kernels' order) = sum over the group's 16 rows of conj(M x) (.) M g; returns the number of b groups in *parts
 int32_t conv_wgrad_partials(const m2_plan* pl, const void* x, const void* g, void* partial, int64_t B, int64_t H, int64_t n, int32_t mode,
                             int* parts, cudaStream_t stream) {
     if (!pl->umma || !covered(pl)) return M2_ERR_UNSUPPORTED;
@@ -1321,7 +1281,7 @@ int32_t conv_wgrad_partials(const m2_plan* pl, const void* x, const void* g, voi
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const long long bgroups = (B + kRows - 1) / kRows, units = H * bgroups;
+    const long long bgroups = (B + 2 * kRows - 1) / (2 * kRows), units = H * bgroups;
     const long long ctas = (units + kGroupsW - 1) / kGroupsW;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(ctas < sms ? ctas : sms));
@@ -1333,21 +1293,10 @@ int32_t conv_wgrad_partials(const m2_plan* pl, const void* x, const void* g, voi
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, convwgrad512_kernel, mx, mg, (float2*)partial, (const uint4*)t->d_const, (int)B, (int)H, (int)n,
-                           pl->d_status) != cudaSuccess)
+    if (cudaLaunchKernelEx(&cfg, convwgrad512_kernel, mx, mg, (float4*)partial, (const uint4*)t->d_const_p, (int)B, (int)H, (int)n,
+                           pl->sign >= 0 ? 1.0f : -1.0f, pl->d_status) != cudaSuccess)
         return M2_ERR_CUDA;
     *parts = (int)bgroups;
-    pl->launches += 1;
-    return M2_OK;
-}
-
-// the second launch of the kernel gradient: dk from the partial sums
-int32_t conv_wgrad_finish(const m2_plan* pl, const void* partial, int parts, float* dk, int64_t H, int64_t n, cudaStream_t stream) {
-    if (!pl->umma || !covered(pl)) return M2_ERR_UNSUPPORTED;
-    if (H == 0) return M2_OK;
-    wgrad512_finish_kernel<<<(unsigned)H, 256, 0, stream>>>((const float2*)partial, parts, dk, pl->d_roots[0], pl->d_roots[1], (int)H, (int)n,
-                                                            pl->sign >= 0 ? 1.0f : -1.0f);
-    if (cudaGetLastError() != cudaSuccess) return M2_ERR_CUDA;
     pl->launches += 1;
     return M2_OK;
 }
@@ -1355,13 +1304,7 @@ int32_t conv_wgrad_finish(const m2_plan* pl, const void* partial, int parts, flo
 bool has_private_spectrum(const m2_plan* pl) { return pl->umma != nullptr && (covered(pl) || m2u3::covered(pl)); }
 
 cudaError_t relayout_spectrum(const m2_plan* pl, void* kf, int64_t H, cudaStream_t stream) {
-    if (m2u3::covered(pl)) return m2u3::relayout_spectrum(pl, kf, H, stream);
-    if (!has_private_spectrum(pl) || H == 0) return cudaSuccess;
-    const long long total = H * 256;
-    float4* kfu = reinterpret_cast<float4*>(static_cast<unsigned char*>(kf) + (size_t)H * 512 * 8);
-    relayout_spectrum_kernel<<<(unsigned)((total + 255) / 256), 256, 0, stream>>>((const float*)kf, kfu, total, pl->sign >= 0 ? 1.0f : -1.0f);
-    return cudaGetLastError();
+    return m2u3::covered(pl) ? m2u3::relayout_spectrum(pl, kf, H, stream) : cudaSuccess;   // (N = 512: m2f::spectrum writes both orders)
 }
-
 
 }  // namespace m2u

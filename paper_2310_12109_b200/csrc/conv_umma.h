@@ -25,13 +25,12 @@ int32_t conv_gate_fwd(const m2_plan* plan, const void* x, const void* kf, const 
 int32_t conv_fwd_wait_selftest(const m2_plan* plan, const void* x, const void* kf, void* y, int64_t B, int64_t H, int64_t n,
                                int32_t mode, cudaStream_t stream);
 
-// Kernel gradient, tensor-core part: partial[b group][h][512] = sum over the group's 8 rows of conj(M x) (.) M g in plan
-// order (complex fp32, conv_wgrad_workspace_bytes(plan, B, H) bytes); *parts = number of b groups.
+// Kernel gradient, tensor-core part: partial[b group][h][512] = sum over the group's 16 rows of conj(M z) (.) M w, z and w the row pairs
+// of x and g as complex rows, in the order of the fp32 transform kernels (complex fp32, conv_wgrad_workspace_bytes(plan, B, H)
+// bytes); *parts = number of b groups.
 int64_t conv_wgrad_workspace_bytes(const m2_plan* plan, int64_t B, int64_t H);
 int32_t conv_wgrad_partials(const m2_plan* plan, const void* x, const void* g, void* partial, int64_t B, int64_t H, int64_t n,
                             int32_t mode, int* parts, cudaStream_t stream);
-// ... and dk[H][n] (fp32) = Re M^-1(sum of the parts)[0:n) / N from them (CUDA cores, fp32)
-int32_t conv_wgrad_finish(const m2_plan* plan, const void* partial, int parts, float* dk, int64_t H, int64_t n, cudaStream_t stream);
 
 }  // namespace m2u
 

@@ -7,7 +7,8 @@ namespace m2f {
 // k_f of one channel per row: the forward half alone, scaled by 1 / N
 template <class C, bool HALF>
 __global__ void __launch_bounds__(C::THREADS, min_blocks<C>())
-    fft_spectrum_kernel(const float* __restrict__ k, float4* __restrict__ kf, const float4* __restrict__ tab, int H, int n) {
+    fft_spectrum_kernel(const float* __restrict__ k, float4* __restrict__ kf, float4* __restrict__ kfu, float sgn,
+                        const float4* __restrict__ tab, int H, int n) {
     extern __shared__ __align__(16) float smem[];
     const int r = threadIdx.x / C::TP, t = threadIdx.x % C::TP;
     const long long h = (long long)blockIdx.x * C::ROWS + r;
@@ -24,16 +25,31 @@ __global__ void __launch_bounds__(C::THREADS, min_blocks<C>())
     float4* out = kf + h * (C::N / 2) + t;
     unroll<16>([&](auto s) {
         constexpr int p = brev<4>(s.v);
-        const u64 a = mul2(re[p], sc), c = mul2(im[p], sc);
-        out[s.v * C::TP] = make_float4(lo(a), hi(a), lo(c), hi(c));
+        re[p] = mul2(re[p], sc);
+        im[p] = mul2(im[p], sc);
+        out[s.v * C::TP] = make_float4(lo(re[p]), hi(re[p]), lo(im[p]), hi(im[p]));
     });
+    if constexpr (C::N == 512) {
+        // thread t = q1 holds the frequencies q1 + 16 q2, q2 in the low halves of slots 0 .. 15, then in the high ones: k1 = q1 + 16 c,
+        // k2 = 2 q, 2 q + 1 is q2 = 4 q + c, 4 q + 2 + c
+        if (kfu != nullptr) {
+            float4* priv = kfu + h * 256 + t;
+            unroll<16>([&](auto s) {
+                constexpr int q = s.v / 2, c = s.v % 2, qa = 4 * q + c, qb = qa + 2, pa = brev<4>(qa & 15), pb = brev<4>(qb & 15);
+                priv[q * 32 + c * 16] = qa < 16 ? make_float4(lo(re[pa]), lo(re[pb]), sgn * lo(im[pa]), sgn * lo(im[pb]))
+                                                : make_float4(hi(re[pa]), hi(re[pb]), sgn * hi(im[pa]), sgn * hi(im[pb]));
+            });
+        }
+    }
 }
 
-// the inverse half alone: real part of the first n positions (the spectrum carries the 1 / N)
+// the inverse half alone, of the sum of `parts` spectra in order: scale times the real part of the first n positions
 template <class C, bool HALF>
 __global__ void __launch_bounds__(C::THREADS, min_blocks<C>())
-    fft_time_kernel(const float4* __restrict__ kf, float* __restrict__ kt, const float4* __restrict__ tab, int H, int n) {
+    fft_time_kernel(const float4* __restrict__ kf, int parts, float scale, float* __restrict__ kt, const float4* __restrict__ tab, int H,
+                    int n) {
     extern __shared__ __align__(16) float smem[];
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int r = threadIdx.x / C::TP, t = threadIdx.x % C::TP;
     const long long h = (long long)blockIdx.x * C::ROWS + r;
     const bool live = h < H;
@@ -41,11 +57,27 @@ __global__ void __launch_bounds__(C::THREADS, min_blocks<C>())
     float* si = sr + C::SMEM_FLOATS;
     u64 re[16], im[16];
     const float4* in = kf + (live ? h : 0) * (C::N / 2) + t;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     unroll<16>([&](auto s) {
         constexpr int p = brev<4>(s.v);
         const float4 w = in[s.v * C::TP];
         re[p] = pk(w.x, w.y);
         im[p] = pk(w.z, w.w);
+    });
+#pragma unroll 1
+    for (int q = 1; q < parts; ++q) {
+        in += (long long)H * (C::N / 2);
+        unroll<16>([&](auto s) {
+            constexpr int p = brev<4>(s.v);
+            const float4 w = in[s.v * C::TP];
+            re[p] = add2(re[p], pk(w.x, w.y));
+            im[p] = add2(im[p], pk(w.z, w.w));
+        });
+    }
+    const u64 sc = dup2(scale);
+    unroll<16>([&](auto s) {
+        re[s.v] = mul2(re[s.v], sc);
+        im[s.v] = mul2(im[s.v], sc);
     });
     inverse<C, HALF>(re, im, sr, si, tab, t, r);
     store_row<C, float, HALF>(re, kt + h * n, t, n, (n & 1) == 0, live);
@@ -146,29 +178,30 @@ cudaError_t prepare_gradients(const m2_plan* pl) {
     });
 }
 
-cudaError_t spectrum(const m2_plan* pl, const float* k, int64_t H, int64_t n, void* kf, cudaStream_t stream) {
+cudaError_t spectrum(const m2_plan* pl, const float* k, int64_t H, int64_t n, void* kf, void* kfu, cudaStream_t stream) {
     if (H == 0) return cudaSuccess;
     return dispatch(pl->N, [&](auto cfg) {
         using C = decltype(cfg);
         const unsigned grid = (unsigned)((H + C::ROWS - 1) / C::ROWS);
+        const float sgn = pl->sign >= 0 ? 1.0f : -1.0f;
         if (2 * n <= C::N)
-            fft_spectrum_kernel<C, true><<<grid, C::THREADS, conv_smem<C>(), stream>>>(k, (float4*)kf, pl->d_fft, (int)H, (int)n);
+            fft_spectrum_kernel<C, true><<<grid, C::THREADS, conv_smem<C>(), stream>>>(k, (float4*)kf, (float4*)kfu, sgn, pl->d_fft, (int)H, (int)n);
         else
-            fft_spectrum_kernel<C, false><<<grid, C::THREADS, conv_smem<C>(), stream>>>(k, (float4*)kf, pl->d_fft, (int)H, (int)n);
+            fft_spectrum_kernel<C, false><<<grid, C::THREADS, conv_smem<C>(), stream>>>(k, (float4*)kf, (float4*)kfu, sgn, pl->d_fft, (int)H, (int)n);
         return cudaGetLastError();
     });
 }
 
-cudaError_t time_kernel(const m2_plan* pl, const void* kf, int64_t H, int64_t n, float* kt, cudaStream_t stream) {
+cudaError_t time_kernel(const m2_plan* pl, const void* kf, int parts, float scale, int64_t H, int64_t n, float* kt, cudaStream_t stream) {
     if (H == 0) return cudaSuccess;
     return dispatch(pl->N, [&](auto cfg) {
         using C = decltype(cfg);
         const unsigned grid = (unsigned)((H + C::ROWS - 1) / C::ROWS);
-        if (2 * n <= C::N)
-            fft_time_kernel<C, true><<<grid, C::THREADS, conv_smem<C>(), stream>>>((const float4*)kf, kt, pl->d_fft, (int)H, (int)n);
-        else
-            fft_time_kernel<C, false><<<grid, C::THREADS, conv_smem<C>(), stream>>>((const float4*)kf, kt, pl->d_fft, (int)H, (int)n);
-        return cudaGetLastError();
+        auto go = [&](auto half) {
+            return launch_early(fft_time_kernel<C, decltype(half)::v != 0>, grid, C::THREADS, conv_smem<C>(), stream, (const float4*)kf, parts,
+                                scale, kt, (const float4*)pl->d_fft, (int)H, (int)n);
+        };
+        return 2 * n <= C::N ? go(Ic<1>{}) : go(Ic<0>{});
     });
 }
 

@@ -236,13 +236,15 @@ int32_t m2_kernel_spectrum(const m2_plan* plan, const float* k_dev, int64_t H, i
     DeviceGuard g(plan->device);
     if (!g.ok) return M2_ERR_CUDA;
     m2g::ConvShape s = conv_shape(plan, 1, H, n);
-    const cudaError_t e = m2f::covered(plan) ? m2f::spectrum(plan, k_dev, H, n, kf_dev, (cudaStream_t)stream)
+    const bool priv512 = plan->N == 512 && m2u::has_private_spectrum(plan);   // the second copy is written by the same kernel
+    void* kfu = priv512 ? static_cast<unsigned char*>(kf_dev) + (size_t)H * 512 * sizeof(float2) : nullptr;
+    const cudaError_t e = m2f::covered(plan) ? m2f::spectrum(plan, k_dev, H, n, kf_dev, kfu, (cudaStream_t)stream)
                                              : m2g::launch_spectrum(s, k_dev, kf_dev, (cudaStream_t)stream);
     if (e == cudaErrorInvalidValue) return M2_ERR_UNSUPPORTED;
     if (e != cudaSuccess) return M2_ERR_CUDA;
     if (m2u::relayout_spectrum(plan, kf_dev, H, (cudaStream_t)stream) != cudaSuccess) return M2_ERR_CUDA;
     plan->last_kernel = "spectrum_generic_fp32";
-    plan->launches += (H > 0) * (m2u::has_private_spectrum(plan) ? 2 : 1);
+    plan->launches += (H > 0) * (m2u::has_private_spectrum(plan) && !priv512 ? 2 : 1);
     return M2_OK;
 }
 
@@ -280,8 +282,9 @@ int32_t m2_monarch_conv_bwd_kernel(const m2_plan* plan, const void* x_dev, const
         int parts = 0;
         st = m2u::conv_wgrad_partials(plan, x_dev, g_dev, ws_dev, B, H, n, mode, &parts, (cudaStream_t)stream);
         if (st == M2_OK) {
-            st = m2u::conv_wgrad_finish(plan, ws_dev, parts, dk_dev, H, n, (cudaStream_t)stream);
-            if (st != M2_OK) return st;
+            if (m2f::time_kernel(plan, ws_dev, parts, 1.0f / (float)plan->N, H, n, dk_dev, (cudaStream_t)stream) != cudaSuccess)
+                return M2_ERR_CUDA;
+            plan->launches += 1;
             plan->last_kernel = "conv_wgrad_umma_o2_512";
             return M2_OK;
         }
@@ -673,7 +676,7 @@ int32_t m2_hyena_heads_fwd(const m2_plan* plan, const void* u_dev, const void* c
     // the fused head product wants the long kernels in the time domain, [d / dh][n] fp32: they wait in y, which is written last
     float* kt = static_cast<float*>(y_dev);
     if (hyena_heads_fused(plan, n, d, dh)) {
-        if (m2f::time_kernel(plan, kf_long_dev, d / dh, n, kt, st) != cudaSuccess) return M2_ERR_CUDA;
+        if (m2f::time_kernel(plan, kf_long_dev, 1, 1.0f, d / dh, n, kt, st) != cudaSuccess) return M2_ERR_CUDA;
         plan->launches += 1;
     }
     // channel-first from here on: every projection, convolution and head product works on rows of n positions
