@@ -14,7 +14,7 @@
 // the epilogue applies the optional factor K (.) and ReLU in fp32, rounds to bf16, stages the tile in the swizzled image of
 // the TMA store boxes and stores it to its rows.  One persistent CTA per SM with a producer warp, an issuing warp
 // and four epilogue warps; two accumulators in TMEM, so a tile's epilogue overlaps the next tile's UMMAs.  Block sizes are
-// multiples of 64 (an output tile past the end of a block is clipped by the store's tensor map), d a multiple of 8 (a ragged
+// 64 and 128 here, larger multiples of 64 in gemm_pair.cu (whose tile of 256 rows they fill), d a multiple of 8 (a ragged
 // last column tile is zero-filled on the way in and clipped on the way out).  All waits are bounded.
 #include <cuda.h>
 
@@ -24,6 +24,7 @@
 #include <cstring>
 
 #include "cols_umma.h"
+#include "gemm_pair.h"
 #include "ptx_sm100.cuh"
 #include "tma_host.h"
 
@@ -266,6 +267,20 @@ cudaError_t prepare() {
 // one stage: nb blocks of b x b; out rows o*so + j = W[j] applied to the rows i*si + j*sj of V (N = rows per matrix of the batch)
 static int32_t stage(const m2_plan* pl, int64_t N, const void* W, const void* V, void* O, const void* Kmul, int relu, int64_t Bt, int64_t d,
                      int b, int nb, int64_t si, int64_t sj, int64_t so, cudaStream_t stream) {
+    if (b > 128) {   // a block fills both halves of a pair's tile (at 128 half of it would be padding)
+        PairGemm g;
+        g.a[0] = {W, b, b, b, nb, (int64_t)b * b, 1, 0};
+        g.b = {V, d, b, si * d, nb, sj * d, Bt, N * d};
+        g.o[0] = {O, d, b, so * d, nb, d, Bt, N * d};
+        g.rows = b;
+        g.cols = d;
+        g.k = b;
+        g.kmul = Kmul;
+        g.krs = so;
+        g.relu = relu;
+        pl->launches -= 1;   // (the caller counts its stages)
+        return gemm_pair(pl, g, stream);
+    }
     const int m = b == 64 ? 64 : 128;
     const int nc = d > 128 ? 256 : d > 64 ? 128 : 64;   // columns per tile
     alignas(64) CUtensorMap mw, mv, mo;
@@ -323,19 +338,40 @@ int32_t apply(const m2_plan* pl, const void* X, const void* L, const void* R, co
     return M2_OK;
 }
 
-// A dense matrix is a block-diagonal one with a single block: O[bt] = W V[bt] for Bt matrices V [c][cols] (cols contiguous),
-// W: [c][c] row-major (outputs x inputs).  pl only lends its status word and launch counter.
-bool dense_covered(const m2_plan* pl, int64_t c, int64_t cols) {
-    return pl->dtype == M2_BF16 && c >= 64 && c <= 4096 && c % 64 == 0 && cols > 0 && cols % 8 == 0;
+bool dense_covered(const m2_plan* pl, int64_t c, int64_t n) {
+    return pl->dtype == M2_BF16 && c >= 64 && c <= 4096 && c % 64 == 0 && n > 0 && n % 8 == 0;
 }
 
-int32_t dense(const m2_plan* pl, const void* W, const void* V, void* O, int64_t Bt, int64_t c, int64_t cols, cudaStream_t stream) {
-    if (!dense_covered(pl, c, cols) || Bt > 65535) return M2_ERR_UNSUPPORTED;
-    if (Bt == 0) return M2_OK;
-    if (prepare() != cudaSuccess) return M2_ERR_CUDA;
-    const int32_t st = stage(pl, c, W, V, O, nullptr, 0, Bt, cols, (int)c, 1, 1, c, 1, stream);   // (the block stride is never used: one block)
-    if (st == M2_OK) pl->launches += 1;
-    return st;
+int32_t project(const m2_plan* pl, int weights, const void* const* W, const void* x, void* const* out, int64_t Bt, int64_t c, int64_t n,
+                cudaStream_t stream) {
+    if (!dense_covered(pl, c, n) || Bt > 65535) return M2_ERR_UNSUPPORTED;
+    PairGemm g;
+    g.weights = weights;
+    for (int w = 0; w < weights; ++w) {
+        g.a[w] = {W[w], c, c, c, 1, 0, 1, 0};
+        g.o[w] = {out[w], n, c, n, 1, 0, Bt, c * n};
+    }
+    g.b = {x, c, n, c, 1, 0, Bt, c * n};
+    g.rows = c;
+    g.cols = n;
+    g.k = c;
+    g.b_kmajor = 1;
+    return gemm_pair(pl, g, stream);
+}
+
+int32_t project_back(const m2_plan* pl, const void* W, const void* z, void* y, int64_t Bt, int64_t c, int64_t n, cudaStream_t stream) {
+    if (!dense_covered(pl, c, n) || Bt > 65535) return M2_ERR_UNSUPPORTED;
+    PairGemm g;
+    g.a[0] = {z, n, c, n, 1, 0, Bt, c * n};
+    g.b = {W, c, c, c, 1, 0, 1, 0};
+    g.o[0] = {y, c, n, c, 1, 0, Bt, c * n};
+    g.rows = n;
+    g.cols = c;
+    g.k = c;
+    g.a_mmajor = 1;
+    g.b_kmajor = 1;
+    g.a_batched = 1;
+    return gemm_pair(pl, g, stream);
 }
 
 }  // namespace m2c

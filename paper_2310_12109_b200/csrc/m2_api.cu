@@ -569,6 +569,36 @@ int32_t m2_layer_fwd(const m2_plan* plan_n, const m2_plan* plan_d, const void* x
     return M2_OK;
 }
 
+// Projections of the Hyena layer and the M2-BERT mixer.  in: [B][n][d] -> out[i]: [B][d][n] (channel-first), i < count; xT receives x
+// channel-first where the tensor-core kernel, which reads x as it lies, does not cover the shape (or want_xT).
+static int32_t project_in(const m2_plan* plan, int count, const void* const* W, const void* x, void* xT, bool want_xT, void* const* out,
+                          int64_t B, int64_t d, int64_t n, cudaStream_t st) {
+    const bool bf = plan->dtype == M2_BF16, tc = m2c::dense_covered(plan, d, n);
+    if (!tc || want_xT) {
+        if (m2g::launch_transpose_any(x, xT, B, (int)n, (int)d, bf, st) != cudaSuccess) return M2_ERR_CUDA;
+        plan->launches += 1;
+    }
+    if (tc) return m2c::project(plan, count, W, x, out, B, d, n, st);
+    for (int i = 0; i < count; ++i) {
+        const cudaError_t e = m2g::launch_dense_cols(W[i], xT, out[i], B, (int)d, (int)n, bf, st);
+        if (e == cudaErrorInvalidValue) return M2_ERR_UNSUPPORTED;
+        if (e != cudaSuccess) return M2_ERR_CUDA;
+        plan->launches += 1;
+    }
+    return M2_OK;
+}
+// z: [B][d][n] -> y: [B][n][d]; tmp: a tensor of scratch
+static int32_t project_out(const m2_plan* plan, const void* W, const void* z, void* tmp, void* y, int64_t B, int64_t d, int64_t n,
+                           cudaStream_t st) {
+    if (m2c::dense_covered(plan, d, n)) return m2c::project_back(plan, W, z, y, B, d, n, st);
+    const bool bf = plan->dtype == M2_BF16;
+    const cudaError_t e = m2g::launch_dense_cols(W, z, tmp, B, (int)d, (int)n, bf, st);
+    if (e == cudaErrorInvalidValue) return M2_ERR_UNSUPPORTED;
+    if (e != cudaSuccess || m2g::launch_transpose_any(tmp, y, B, (int)d, (int)n, bf, st) != cudaSuccess) return M2_ERR_CUDA;
+    plan->launches += 2;
+    return M2_OK;
+}
+
 int64_t m2_bert_mixer_scratch_bytes(const m2_plan* plan, int64_t B, int64_t d) {
     if (!plan || B < 0 || d < 0) return -1;
     return 8 * round256(B * d * plan->N * (plan->dtype == M2_BF16 ? 2 : 4));
@@ -595,19 +625,8 @@ int32_t m2_bert_mixer_fwd(const m2_plan* plan, const void* x_dev, const void* co
     const int64_t tb = round256(B * d * n * (bf ? 2 : 4));
     unsigned char* sc = static_cast<unsigned char*>(scratch_dev);
     void *xT = sc, *Pq = sc + tb, *Pk = sc + 2 * tb, *Pv = sc + 3 * tb, *QK = sc + 4 * tb, *C = sc + 5 * tb, *Cr = sc + 6 * tb, *Z = sc + 7 * tb;
-    auto dense = [&](const void* Wm, const void* V, void* O) -> int32_t {   // O[b] = Wm V[b] on [B][d][n]
-        int32_t rc = m2c::dense(plan, Wm, V, O, B, d, n, st);
-        if (rc != M2_ERR_UNSUPPORTED) return rc;
-        const cudaError_t e = m2g::launch_dense_cols(Wm, V, O, B, (int)d, (int)n, bf, st);
-        if (e == cudaErrorInvalidValue) return M2_ERR_UNSUPPORTED;
-        if (e != cudaSuccess) return M2_ERR_CUDA;
-        plan->launches += 1;
-        return M2_OK;
-    };
-    if (m2g::launch_transpose_any(x_dev, xT, B, (int)n, (int)d, bf, st) != cudaSuccess) return M2_ERR_CUDA;   // channel-first from here on
-    int32_t rc = dense(W[0], xT, Pq);
-    if (rc == M2_OK) rc = dense(W[1], xT, Pk);
-    if (rc == M2_OK) rc = dense(W[2], xT, Pv);
+    void* const proj[3] = {Pq, Pk, Pv};
+    int32_t rc = project_in(plan, 3, W, x_dev, xT, true, proj, B, d, n, st);   // channel-first from here on
     if (rc != M2_OK) return rc;
     if (m2g::launch_gate_in(Pq, Pk, w_short[0], w_short[1], QK, B, (int)d, (int)n, bf, st) != cudaSuccess) return M2_ERR_CUDA;
     // the residual convolution first; on the N = 512 tensor-core plan the main convolution then applies the gate and adds the
@@ -626,10 +645,9 @@ int32_t m2_bert_mixer_fwd(const m2_plan* plan, const void* x_dev, const void* co
         if (m2g::launch_gate_out(Pv, w_short[2], C, Cr, Z, B, (int)d, (int)n, bf, st) != cudaSuccess) return M2_ERR_CUDA;
         plan->launches += 1;
     }
-    rc = dense(W[3], Z, Pq);
+    rc = project_out(plan, W[3], Z, Pq, y_dev, B, d, n, st);
     if (rc != M2_OK) return rc;
-    if (m2g::launch_transpose_any(Pq, y_dev, B, (int)d, (int)n, bf, st) != cudaSuccess) return M2_ERR_CUDA;
-    plan->launches += 3;   // the two transposes and the input gate (the products, convolutions and the output gate count themselves)
+    plan->launches += 1;   // the input gate (everything else counts itself)
     plan->last_kernel = fused_out ? "bert_mixer_fwd_fused_gate" : "bert_mixer_fwd";
     return M2_OK;
 }
@@ -664,15 +682,6 @@ int32_t m2_hyena_heads_fwd(const m2_plan* plan, const void* u_dev, const void* c
     unsigned char* sc = static_cast<unsigned char*>(scratch_dev);
     void *uT = sc, *P1 = sc + tb, *P2 = sc + 2 * tb, *P3 = sc + 3 * tb, *C1 = sc + 4 * tb, *C2 = sc + 5 * tb, *C3 = sc + 6 * tb;
     void *XV = sc + 7 * tb, *XVc = sc + (7 + dh) * tb;
-    auto dense = [&](const void* Wm, const void* V, void* O) -> int32_t {   // O[b] = Wm V[b] on [B][d][n]
-        int32_t rc = m2c::dense(plan, Wm, V, O, B, d, n, st);
-        if (rc != M2_ERR_UNSUPPORTED) return rc;
-        const cudaError_t e = m2g::launch_dense_cols(Wm, V, O, B, (int)d, (int)n, bf, st);
-        if (e == cudaErrorInvalidValue) return M2_ERR_UNSUPPORTED;
-        if (e != cudaSuccess) return M2_ERR_CUDA;
-        plan->launches += 1;
-        return M2_OK;
-    };
     // the fused head product wants the long kernels in the time domain, [d / dh][n] fp32: they wait in y, which is written last
     float* kt = static_cast<float*>(y_dev);
     if (hyena_heads_fused(plan, n, d, dh)) {
@@ -680,10 +689,8 @@ int32_t m2_hyena_heads_fwd(const m2_plan* plan, const void* u_dev, const void* c
         plan->launches += 1;
     }
     // channel-first from here on: every projection, convolution and head product works on rows of n positions
-    if (m2g::launch_transpose_any(u_dev, uT, B, (int)n, (int)d, bf, st) != cudaSuccess) return M2_ERR_CUDA;
-    int32_t rc = dense(W[0], uT, P1);
-    if (rc == M2_OK) rc = dense(W[1], uT, P2);
-    if (rc == M2_OK) rc = dense(W[2], uT, P3);
+    void* const proj[3] = {P1, P2, P3};
+    int32_t rc = project_in(plan, 3, W, u_dev, uT, false, proj, B, d, n, st);
     if (rc == M2_OK) rc = m2_monarch_conv_fwd(plan, P1, kf1_dev, C1, B, d, n, M2_CAUSAL, stream);
     if (rc == M2_OK) rc = m2_monarch_conv_fwd(plan, P2, kf2_dev, C2, B, d, n, M2_CAUSAL, stream);
     if (rc == M2_OK) rc = m2_monarch_conv_fwd(plan, P3, kf3_dev, C3, B, d, n, M2_CAUSAL, stream);
@@ -698,10 +705,8 @@ int32_t m2_hyena_heads_fwd(const m2_plan* plan, const void* u_dev, const void* c
         if (m2g::launch_heads_reduce(C1, XVc, P1, B, (int)d, (int)dh, (int)n, bf, st) != cudaSuccess) return M2_ERR_CUDA;
         plan->launches += 2;
     }
-    rc = dense(W[3], P1, P2);
+    rc = project_out(plan, W[3], P1, P2, y_dev, B, d, n, st);
     if (rc != M2_OK) return rc;
-    if (m2g::launch_transpose_any(P2, y_dev, B, (int)d, (int)n, bf, st) != cudaSuccess) return M2_ERR_CUDA;
-    plan->launches += 2;   // the two transposes (the products, convolutions and head kernels count themselves)
     plan->last_kernel = hyena_heads_fused(plan, n, d, dh) ? "hyena_heads_fwd_fused" : "hyena_heads_fwd";
     return M2_OK;
 }
