@@ -275,8 +275,7 @@ static int32_t stage(const m2_plan* pl, int64_t N, const void* W, const void* V,
         g.rows = b;
         g.cols = d;
         g.k = b;
-        g.kmul = Kmul;
-        g.krs = so;
+        g.kmul = {Kmul, d, b, so * d, nb, d, 1, 0};
         g.relu = relu;
         pl->launches -= 1;   // (the caller counts its stages)
         return gemm_pair(pl, g, stream);

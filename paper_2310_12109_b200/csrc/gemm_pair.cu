@@ -14,7 +14,8 @@
 //
 // Measured, one B200 (per launch, cold): three projections 768 x 768 of 32 x 512 positions in one launch 52 us (58 GFLOP) where three
 // launches took 27 us each, the output projection 25 us where it took 27 and a 10 us transposition; a stage of the 65536 x 768
-// operator (256 blocks of 256 x 256, 233 MB) 50 -> 42 us.  Bound by the operands' way from L2 (12 TB/s over all SMs), the operator by
+// operator (256 blocks of 256 x 256, 233 MB) 50 -> 42 us, the one with the factor (335 MB) 72 -> 57 us once its rows came by TMA
+// into the staging area instead of 16 bytes per lane from strided rows.  Bound by the operands' way from L2 (12 TB/s over all SMs), the operator by
 // DRAM (5.5 TB/s).
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -34,12 +35,12 @@ constexpr int kEpilogueWarps = 8, kPairThreads = 32 * (kEpilogueWarps + 2);
 constexpr int kPairStages = 5;
 constexpr int P_STAGE = 32768;                        // A [128][64] 16384 | B [64][128] 16384
 constexpr int P_OUT = kPairStages * P_STAGE;          // staging: 8 KB per epilogue warp, two boxes [32 rows][64 columns]
-constexpr int P_BAR = P_OUT + kEpilogueWarps * 8192;  // full[5], empty[5], acc_full[2], acc_empty[2], tmem ptr, abort flag
-constexpr int P_SMEM = P_BAR + 128;
+constexpr int P_BAR = P_OUT + kEpilogueWarps * 8192;  // full[5], empty[5], acc_full[2], acc_empty[2], tmem ptr, abort flag, factor[8]
+constexpr int P_SMEM = P_BAR + 192;
 static_assert(P_SMEM <= 232448, "shared memory budget");
 
 struct PairMaps {
-    CUtensorMap a[3], b, o[3];
+    CUtensorMap a[3], b, o[3], k;
 };
 
 __device__ __forceinline__ uint32_t map_to_even(uint32_t addr) {   // the same shared-memory offset in the pair's even CTA
@@ -87,19 +88,18 @@ struct PairShape {
     int nb, tiles;         // blocks per matrix; tiles in all
     int nc;                // columns per tile: 256 or 128
     int a_mmajor, b_kmajor, a_batched;
-    int krs, relu;         // K (.): row of an output = o * krs + j
+    int kmul, relu;        // factor K (.) on the result (its rows are those of one output matrix), then ReLU
 };
 
 // tile index = ((bt * nb + j) * otiles + ot) * ctiles + ct: pairs running at the same time share a block's operands in L2
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
-gemm_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constant__ PairShape S, const __nv_bfloat16* __restrict__ Kmul,
-                 int32_t* __restrict__ status) {
+gemm_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constant__ PairShape S, int32_t* __restrict__ status) {
     extern __shared__ __align__(1024) unsigned char smem[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int rank = blockIdx.x & 1, pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
     const uint32_t s_base = smem_u32(smem);
     const uint32_t bar_full = s_base + P_BAR, bar_empty = bar_full + 8 * kPairStages, bar_accf = bar_empty + 8 * kPairStages,
-                   bar_acce = bar_accf + 16, s_tptr = bar_acce + 16;
+                   bar_acce = bar_accf + 16, s_tptr = bar_acce + 16, bar_k = s_tptr + 16;
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + P_BAR + 16 * kPairStages + 40);
     if (tid == 0) {
         for (int s = 0; s < kPairStages; ++s) {
@@ -110,6 +110,7 @@ gemm_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constant__ 
             mbar_init(bar_accf + 8 * a, 1);
             mbar_init(bar_acce + 8 * a, 2 * kEpilogueWarps);   // one arrival per epilogue warp of the pair
         }
+        for (int w = 0; w < kEpilogueWarps; ++w) mbar_init(bar_k + 8 * w, 1);
         *abort_flag = 0;
         fence_barrier_init();
     }
@@ -211,17 +212,17 @@ gemm_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constant__ 
         for (int t = pair; t < S.tiles && ok; t += pairs, ++it) {
             const int ct = t % S.ctiles, ot = (t / S.ctiles) % S.otiles, j = (t / (S.ctiles * S.otiles)) % S.nb,
                       bt = t / (S.ctiles * S.otiles * S.nb);
-            const int acc = it & 1, o0 = (ot % S.otiles_w) * 256 + rank * 128 + q * 32, o = o0 + lane, c0 = ct * S.nc + hc * half;
-            // the factor K (.) for this thread's row, requested while the tile's UMMAs still run
-            uint4 kreg[16];
-            if (Kmul != nullptr) {
-                const uint4* krow = reinterpret_cast<const uint4*>(Kmul + ((size_t)o * S.krs + j) * S.cols + c0);   // K is shared by the batch
-#pragma unroll
-                for (int e = 0; e < 16; ++e)   // (the row length is a multiple of 8)
-                    kreg[e] = e < half / 8 && o < S.rows && c0 + 8 * e < S.cols ? __ldg(krow + e) : make_uint4(0u, 0u, 0u, 0u);
+            const int acc = it & 1, o0 = (ot % S.otiles_w) * 256 + rank * 128 + q * 32, c0 = ct * S.nc + hc * half;
+            if (lane == 0) {
+                tma_store_wait_read0();   // this warp's previous stores have read the staging area
+                if (S.kmul) {             // the factor's boxes wait there while the tile's UMMAs run
+                    mbar_expect_tx(bar_k + 8 * warp, (uint32_t)nbox * 4096u);
+                    for (int bx = 0; bx < nbox; ++bx)
+                        tma_load_4d(s_base + P_OUT + warp * 8192 + bx * 4096, &maps.k, c0 + 64 * bx, o0, j, 0, bar_k + 8 * warp);
+                }
             }
             ok = mbar_wait(bar_accf + 8 * acc, (it >> 1) & 1);
-            if (lane == 0) tma_store_wait_read0();   // this warp's previous stores have read the staging area
+            if (ok && S.kmul) ok = mbar_wait(bar_k + 8 * warp, it & 1);
             ok = __all_sync(0xffffffffu, ok && *abort_flag == 0);
             if (!ok) break;
             tc_fence_after();
@@ -239,8 +240,9 @@ gemm_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constant__ 
 #pragma unroll
                     for (int c8 = 0; c8 < 4; ++c8) {
                         float* w = v + 8 * c8;
-                        if (Kmul != nullptr) {
-                            const uint4 kp = kreg[bx * 8 + hq * 4 + c8];
+                        uint4* cell = reinterpret_cast<uint4*>(stg + bx * 4096 + lane * 128 + (((hq * 4 + c8) ^ (lane & 7)) << 4));
+                        if (S.kmul) {
+                            const uint4 kp = *cell;
                             const uint32_t kw[4] = {kp.x, kp.y, kp.z, kp.w};
 #pragma unroll
                             for (int e = 0; e < 4; ++e) {
@@ -252,8 +254,7 @@ gemm_pair_kernel(const __grid_constant__ PairMaps maps, const __grid_constant__ 
                                 for (int e = 0; e < 8; ++e) w[e] = fmaxf(w[e], 0.f);
                             }
                         }
-                        *reinterpret_cast<uint4*>(stg + bx * 4096 + lane * 128 + (((hq * 4 + c8) ^ (lane & 7)) << 4)) =
-                            make_uint4(pack2(w[0], w[1]), pack2(w[2], w[3]), pack2(w[4], w[5]), pack2(w[6], w[7]));
+                        *cell = make_uint4(pack2(w[0], w[1]), pack2(w[2], w[3]), pack2(w[4], w[5]), pack2(w[6], w[7]));
                     }
                 }
             }
@@ -316,7 +317,7 @@ int32_t gemm_pair(const m2_plan* pl, const PairGemm& g, cudaStream_t stream) {
     S.a_mmajor = g.a_mmajor;
     S.b_kmajor = g.b_kmajor;
     S.a_batched = g.a_batched;
-    S.krs = (int)g.krs;
+    S.kmul = g.kmul.p != nullptr;
     S.relu = g.relu;
     const int64_t tiles = g.o[0].nbt * S.nb * S.otiles * S.ctiles;
     if (tiles > 0x7fffffffLL) return M2_ERR_UNSUPPORTED;
@@ -327,6 +328,7 @@ int32_t gemm_pair(const m2_plan* pl, const PairGemm& g, cudaStream_t stream) {
         const int v = w < g.weights ? w : 0;
         if (!map4(&maps.a[w], g.a[v], 64, g.a_mmajor ? 64 : 128) || !map4(&maps.o[w], g.o[v], 64, 32)) return M2_ERR_UNSUPPORTED;
     }
+    if (!map4(&maps.k, g.kmul.p ? g.kmul : g.o[0], 64, 32)) return M2_ERR_UNSUPPORTED;
     if (!map4(&maps.b, g.b, 64, g.b_kmajor ? (uint32_t)(S.nc / 2) : 64)) return M2_ERR_UNSUPPORTED;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
@@ -342,7 +344,7 @@ int32_t gemm_pair(const m2_plan* pl, const PairGemm& g, cudaStream_t stream) {
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, gemm_pair_kernel, maps, S, (const __nv_bfloat16*)g.kmul, pl->d_status) != cudaSuccess) return M2_ERR_CUDA;
+    if (cudaLaunchKernelEx(&cfg, gemm_pair_kernel, maps, S, pl->d_status) != cudaSuccess) return M2_ERR_CUDA;
     pl->launches += 1;
     return M2_OK;
 }

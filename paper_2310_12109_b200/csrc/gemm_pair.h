@@ -20,8 +20,7 @@ struct PairGemm {
     PairTensor a[3], b, o[3];
     int64_t rows = 0, cols = 0, k = 0;
     int a_mmajor = 0, b_kmajor = 0, a_batched = 0;
-    const void* kmul = nullptr;  // bf16 factor on the result: row o of block j is row o * krs + j of [..][cols]
-    int64_t krs = 0;
+    PairTensor kmul = {};        // factor on the result, shared by the batch: n0 = column, n1 = row; p == nullptr: none
     int relu = 0;                // after the factor
 };
 int32_t gemm_pair(const m2_plan* pl, const PairGemm& g, cudaStream_t stream);
