@@ -1261,6 +1261,8 @@ int32_t conv_gate_fwd(const m2_plan* pl, const void* x, const void* kf, const fl
     return conv_fwd_impl(pl, x, kf, y, B, H, 512, M2_CIRCULAR, stream, 0, 1, w_gate, gate_rows, addend);
 }
 
+bool covers_rows(const m2_plan* pl, int64_t n) { return pl->umma && covered(pl) && n % 16 == 0 && n <= 512; }
+
 int32_t conv_fwd_wait_selftest(const m2_plan* pl, const void* x, const void* kf, void* y, int64_t B, int64_t H, int64_t n, int32_t mode,
                                cudaStream_t stream) {
     return conv_fwd_impl(pl, x, kf, y, B, H, n, mode, stream, 1, 1);

@@ -22,6 +22,7 @@ int32_t conv_fwd(const m2_plan* plan, const void* x, const void* kf, void* y, in
 // after the gate, y = conv(x, k) * gate + addend (neither may be y).
 int32_t conv_gate_fwd(const m2_plan* plan, const void* x, const void* kf, const float* w_gate, void* y, int64_t B, int64_t H,
                       cudaStream_t stream, const void* gate_rows = nullptr, const void* addend = nullptr);
+bool covers_rows(const m2_plan* plan, int64_t n);   // conv_fwd has a kernel for rows of n values
 int32_t conv_fwd_wait_selftest(const m2_plan* plan, const void* x, const void* kf, void* y, int64_t B, int64_t H, int64_t n,
                                int32_t mode, cudaStream_t stream);
 

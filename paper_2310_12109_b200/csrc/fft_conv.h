@@ -17,8 +17,9 @@ cudaError_t prepare_gradients(const m2_plan* pl);   // (part of prepare)
 int spectrum_order(const m2_plan* pl);
 
 // k_f = F_N pad(k) / N, fp32, in the kernels' own order (fft_core.cuh, spec_index); kfu != nullptr (N = 512 only): also in the order of
-// the tensor-core kernels, kfu[h][k2 / 2][k1] = (re, re', im, im') of the frequencies k1 + 32 k2, k1 + 32 (k2 + 1)
-cudaError_t spectrum(const m2_plan* pl, const float* k, int64_t H, int64_t n, void* kf, void* kfu, cudaStream_t stream);
+// the tensor-core kernels, kfu[h][k2 / 2][k1] = (re, re', im, im') of the frequencies k1 + 32 k2, k1 + 32 (k2 + 1); kt != nullptr: k
+// itself, zero padded, fp32 [H][N]
+cudaError_t spectrum(const m2_plan* pl, const float* k, int64_t H, int64_t n, void* kf, void* kfu, float* kt, cudaStream_t stream);
 // back to the time domain: kt[h][t] = scale times the first n values of F^-1 of the sum of `parts` buffers [H][N], fp32 [H][n]; a
 // spectrum carries its 1 / N already (scale 1 gives the kernel)
 cudaError_t time_kernel(const m2_plan* pl, const void* kf, int parts, float scale, int64_t H, int64_t n, float* kt, cudaStream_t stream);

@@ -7,8 +7,8 @@ namespace m2f {
 // k_f of one channel per row: the forward half alone, scaled by 1 / N
 template <class C, bool HALF>
 __global__ void __launch_bounds__(C::THREADS, min_blocks<C>())
-    fft_spectrum_kernel(const float* __restrict__ k, float4* __restrict__ kf, float4* __restrict__ kfu, float sgn,
-                        const float4* __restrict__ tab, int H, int n) {
+    fft_spectrum_kernel(const float* __restrict__ k, float4* __restrict__ kf, float4* __restrict__ kfu, float* __restrict__ kt,
+                        float sgn, const float4* __restrict__ tab, int H, int n) {
     extern __shared__ __align__(16) float smem[];
     const int r = threadIdx.x / C::TP, t = threadIdx.x % C::TP;
     const long long h = (long long)blockIdx.x * C::ROWS + r;
@@ -19,6 +19,8 @@ __global__ void __launch_bounds__(C::THREADS, min_blocks<C>())
     // rows of k are only as aligned as n floats make them; a pair needs 8 bytes
     load_row<C, float, HALF>(re, k + h * n, t, n, (n & 1) == 0 && (reinterpret_cast<uintptr_t>(k) & 7) == 0, live);
     unroll<16>([&](auto j) { im[j.v] = 0ull; });
+    if (kt != nullptr && live)
+        for (int i = t; i < C::N; i += C::TP) kt[h * C::N + i] = i < n ? k[h * n + i] : 0.f;
     forward<C, HALF>(re, im, sr, si, tab, t, r);
     if (!live) return;
     const u64 sc = dup2(1.0f / (float)C::N);
@@ -178,16 +180,16 @@ cudaError_t prepare_gradients(const m2_plan* pl) {
     });
 }
 
-cudaError_t spectrum(const m2_plan* pl, const float* k, int64_t H, int64_t n, void* kf, void* kfu, cudaStream_t stream) {
+cudaError_t spectrum(const m2_plan* pl, const float* k, int64_t H, int64_t n, void* kf, void* kfu, float* kt, cudaStream_t stream) {
     if (H == 0) return cudaSuccess;
     return dispatch(pl->N, [&](auto cfg) {
         using C = decltype(cfg);
         const unsigned grid = (unsigned)((H + C::ROWS - 1) / C::ROWS);
         const float sgn = pl->sign >= 0 ? 1.0f : -1.0f;
         if (2 * n <= C::N)
-            fft_spectrum_kernel<C, true><<<grid, C::THREADS, conv_smem<C>(), stream>>>(k, (float4*)kf, (float4*)kfu, sgn, pl->d_fft, (int)H, (int)n);
+            fft_spectrum_kernel<C, true><<<grid, C::THREADS, conv_smem<C>(), stream>>>(k, (float4*)kf, (float4*)kfu, kt, sgn, pl->d_fft, (int)H, (int)n);
         else
-            fft_spectrum_kernel<C, false><<<grid, C::THREADS, conv_smem<C>(), stream>>>(k, (float4*)kf, (float4*)kfu, sgn, pl->d_fft, (int)H, (int)n);
+            fft_spectrum_kernel<C, false><<<grid, C::THREADS, conv_smem<C>(), stream>>>(k, (float4*)kf, (float4*)kfu, kt, sgn, pl->d_fft, (int)H, (int)n);
         return cudaGetLastError();
     });
 }

@@ -738,18 +738,33 @@ cudaError_t launch_gate_transpose(const void* x, const void* vT, const float* w,
 
 // conj of a spectrum buffer: `pairs` interleaved complex values (re, im), then `quads` values of the tensor-core
 // kernels' layouts (re, re', im, im')
-__global__ void spectrum_conj_kernel(const float4* __restrict__ in, float4* __restrict__ out, long long pair_quads, long long total) {
+// quads [0, pair_quads): (re, im, re', im'); [pair_quads, total): (re, re', im, im'); then the kernel in the time domain, rows of N
+// values, whose lags change sign: one thread per pair of lags u, N - u (in place is fine)
+__global__ void spectrum_conj_kernel(const float4* __restrict__ in, float4* __restrict__ out, long long pair_quads, long long total, int N,
+                                     long long time_pairs) {
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i >= total) return;
-    const float4 v = in[i];
-    out[i] = i < pair_quads ? make_float4(v.x, -v.y, v.z, -v.w) : make_float4(v.x, v.y, -v.z, -v.w);
+    if (i < total) {
+        const float4 v = in[i];
+        out[i] = i < pair_quads ? make_float4(v.x, -v.y, v.z, -v.w) : make_float4(v.x, v.y, -v.z, -v.w);
+    } else if (i - total < time_pairs) {
+        const int per_row = N / 2 + 1;
+        const long long p = i - total, row = p / per_row;
+        const int u = (int)(p % per_row), v = (N - u) % N;
+        const float* a = reinterpret_cast<const float*>(in + total) + row * N;
+        float* b = reinterpret_cast<float*>(out + total) + row * N;
+        const float x = a[u], y = a[v];
+        b[v] = x;
+        b[u] = y;
+    }
 }
 
-cudaError_t launch_spectrum_conj(const void* in, void* out, long long plan_order_values, long long private_values, cudaStream_t st) {
-    // plan_order_values complex values (even); private_values complex values stored as (re, re', im, im') quads
-    const long long pair_quads = plan_order_values / 2, total = pair_quads + private_values / 2;
+cudaError_t launch_spectrum_conj(const void* in, void* out, long long plan_order_values, long long private_values, int N, long long time_rows,
+                                 cudaStream_t st) {
+    // plan_order_values complex values (even); private_values complex values stored as (re, re', im, im') quads; time_rows rows of N
+    const long long pair_quads = plan_order_values / 2, total = pair_quads + private_values / 2, time_pairs = time_rows * (N / 2 + 1);
     if (total == 0) return cudaSuccess;
-    spectrum_conj_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>((const float4*)in, (float4*)out, pair_quads, total);
+    spectrum_conj_kernel<<<(unsigned)((total + time_pairs + 255) / 256), 256, 0, st>>>((const float4*)in, (float4*)out, pair_quads, total, N,
+                                                                                      time_pairs);
     return cudaGetLastError();
 }
 

@@ -63,6 +63,7 @@ cudaError_t launch_gate_in(const void* Pq, const void* Pk, const float* wq, cons
 cudaError_t launch_gate_out(const void* Pv, const float* wv, const void* C, const void* Cr, void* Z, long long B, int d, int n, bool bf16,
                             cudaStream_t st);
 // conjugates a spectrum buffer: plan-order part (interleaved re, im) followed by the tensor-core kernels' private part
-cudaError_t launch_spectrum_conj(const void* in, void* out, long long plan_order_values, long long private_values, cudaStream_t st);
+cudaError_t launch_spectrum_conj(const void* in, void* out, long long plan_order_values, long long private_values, int N, long long time_rows,
+                                 cudaStream_t st);
 
 }  // namespace m2g

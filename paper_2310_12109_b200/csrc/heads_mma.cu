@@ -13,12 +13,11 @@
 //
 // Measured, one B200, layer at B = 32, n = 256, d = 768 (1536 heads): 403 -> 163 us with this kernel in place of 24 576 tensor-core
 // convolution units of 16 rows each (about 280 us of the 403).  Bound by instruction issue: 136 tile pairs of about 20 instructions.
-#include <cuda_bf16.h>
-
 #include "fft_conv.h"
 #include "fft_core.cuh"
 #include "heads_mma.h"
 #include "m2_plan.h"
+#include "mma_sync.cuh"
 
 namespace m2h {
 
@@ -29,23 +28,12 @@ __host__ __device__ constexpr int pitch(int n) { return padded(n) + 8; }        
 __host__ __device__ constexpr int kcopy(int n) { return padded(n) + 32; }             // floats of one reversed copy of the kernel
 __host__ __device__ constexpr int smem_bytes(int n) { return 3 * kDh * pitch(n) * 2 + 2 * kcopy(n) * 4; }
 
-__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void ldsm4(uint32_t* r, uint32_t a) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a));
-}
-__device__ __forceinline__ void ldsm4t(uint32_t* r, uint32_t a) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a));
-}
-__device__ __forceinline__ void mma(float* d, const uint32_t* a, uint32_t b0, uint32_t b1) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-__device__ __forceinline__ uint32_t bf2(float a, float b) {
-    const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
-    return *reinterpret_cast<const uint32_t*>(&v);
-}
+using m2t::bf2;
+using m2t::ldsm4;
+using m2t::ldsm4t;
+using m2t::mma;
+using m2t::smem_addr;
+
 // bf16 pair of the products (a, b) * (k.x, k.y)
 __device__ __forceinline__ uint32_t weigh(float a, float b, float2 k) {
     const m2f::u64 p = m2f::mul2(m2f::pk(a, b), m2f::pk(k.x, k.y));

@@ -16,6 +16,7 @@
 #include "cols_umma.h"
 #include "matmul_umma.h"
 #include "mlp_umma.h"
+#include "toeplitz_mma.h"
 #include "m2_plan.h"
 
 // Scratch of m2_block_fwd_static: the intermediate z of the block forward for callers that cannot
@@ -224,7 +225,7 @@ int32_t m2_plan_get_table(const m2_plan* plan, int32_t which, int32_t* host_out,
 
 int64_t m2_spectrum_bytes(const m2_plan* plan, int64_t H) {
     if (!plan || H < 0) return -1;
-    return H * plan->N * (int64_t)sizeof(float2) * (m2u::has_private_spectrum(plan) ? 2 : 1);
+    return H * plan->N * ((int64_t)sizeof(float2) * (m2u::has_private_spectrum(plan) ? 2 : 1) + (m2t::has_time_kernel(plan) ? (int64_t)sizeof(float) : 0));
 }
 
 int32_t m2_kernel_spectrum(const m2_plan* plan, const float* k_dev, int64_t H, int64_t n, void* kf_dev, void* stream) {
@@ -238,7 +239,8 @@ int32_t m2_kernel_spectrum(const m2_plan* plan, const float* k_dev, int64_t H, i
     m2g::ConvShape s = conv_shape(plan, 1, H, n);
     const bool priv512 = plan->N == 512 && m2u::has_private_spectrum(plan);   // the second copy is written by the same kernel
     void* kfu = priv512 ? static_cast<unsigned char*>(kf_dev) + (size_t)H * 512 * sizeof(float2) : nullptr;
-    const cudaError_t e = m2f::covered(plan) ? m2f::spectrum(plan, k_dev, H, n, kf_dev, kfu, (cudaStream_t)stream)
+    float* kt = m2t::has_time_kernel(plan) ? const_cast<float*>(m2t::time_kernel(plan, kf_dev, H)) : nullptr;
+    const cudaError_t e = m2f::covered(plan) ? m2f::spectrum(plan, k_dev, H, n, kf_dev, kfu, kt, (cudaStream_t)stream)
                                              : m2g::launch_spectrum(s, k_dev, kf_dev, (cudaStream_t)stream);
     if (e == cudaErrorInvalidValue) return M2_ERR_UNSUPPORTED;
     if (e != cudaSuccess) return M2_ERR_CUDA;
@@ -317,7 +319,8 @@ int32_t m2_spectrum_conjugate(const m2_plan* plan, const void* kf_in_dev, int64_
     // values in plan order lie as (re, im), all others as (re, re', im, im')
     const long long priv = m2u::has_private_spectrum(plan) ? values : 0;
     const bool fft = m2f::covered(plan);
-    if (m2g::launch_spectrum_conj(kf_in_dev, kf_out_dev, fft ? 0 : values, fft ? values + priv : priv, (cudaStream_t)stream) != cudaSuccess)
+    if (m2g::launch_spectrum_conj(kf_in_dev, kf_out_dev, fft ? 0 : values, fft ? values + priv : priv, (int)plan->N,
+                                  m2t::has_time_kernel(plan) ? H : 0, (cudaStream_t)stream) != cudaSuccess)
         return M2_ERR_CUDA;
     plan->launches += (H > 0);
     return M2_OK;
@@ -332,6 +335,14 @@ static int32_t conv_fwd_grouped(const m2_plan* plan, const void* x_dev, const vo
     DeviceGuard g(plan->device);
     if (!g.ok) return M2_ERR_CUDA;
     if (B * H == 0) return M2_OK;
+    // Short causal rows: Toeplitz products, from 9 rows a channel on (half of a tile of 16; up to 8 rows the 32 x 16 plan has a
+    // tensor-core kernel of its own).
+    if (mode == M2_CAUSAL && n <= m2t::kMaxN && m2t::has_time_kernel(plan) && x_dev != y_dev && (B > 8 || !m2u::covers_rows(plan, n))) {
+        const m2t::Rows rows = {x_dev, m2t::time_kernel(plan, kf_dev, H / kf_group), y_dev};
+        const int32_t tst = m2t::conv(plan, &rows, 1, B, H, n, (int)kf_group, (cudaStream_t)stream);
+        if (tst == M2_OK) plan->last_kernel = "conv_toeplitz_mma";
+        if (tst != M2_ERR_UNSUPPORTED) return tst;
+    }
     // tensor-core path where a kernel exists for the shape, CUDA-core path otherwise
     int32_t ust = m2u::conv_fwd(plan, x_dev, kf_dev, y_dev, B, H, n, mode, (cudaStream_t)stream, (int)kf_group);
     if (ust == M2_ERR_UNSUPPORTED && kf_group == 1) ust = m2u3::conv_fwd(plan, x_dev, kf_dev, y_dev, B, H, n, mode, (cudaStream_t)stream);
@@ -691,9 +702,18 @@ int32_t m2_hyena_heads_fwd(const m2_plan* plan, const void* u_dev, const void* c
     // channel-first from here on: every projection, convolution and head product works on rows of n positions
     void* const proj[3] = {P1, P2, P3};
     int32_t rc = project_in(plan, 3, W, u_dev, uT, false, proj, B, d, n, st);
-    if (rc == M2_OK) rc = m2_monarch_conv_fwd(plan, P1, kf1_dev, C1, B, d, n, M2_CAUSAL, stream);
-    if (rc == M2_OK) rc = m2_monarch_conv_fwd(plan, P2, kf2_dev, C2, B, d, n, M2_CAUSAL, stream);
-    if (rc == M2_OK) rc = m2_monarch_conv_fwd(plan, P3, kf3_dev, C3, B, d, n, M2_CAUSAL, stream);
+    if (rc != M2_OK) return rc;
+    rc = M2_ERR_UNSUPPORTED;
+    if (m2t::has_time_kernel(plan)) {   // the three convolutions in one launch
+        const m2t::Rows rows[3] = {{P1, m2t::time_kernel(plan, kf1_dev, d), C1}, {P2, m2t::time_kernel(plan, kf2_dev, d), C2},
+                                   {P3, m2t::time_kernel(plan, kf3_dev, d), C3}};
+        rc = m2t::conv(plan, rows, 3, B, d, n, 1, st);
+    }
+    if (rc == M2_ERR_UNSUPPORTED) {
+        rc = m2_monarch_conv_fwd(plan, P1, kf1_dev, C1, B, d, n, M2_CAUSAL, stream);
+        if (rc == M2_OK) rc = m2_monarch_conv_fwd(plan, P2, kf2_dev, C2, B, d, n, M2_CAUSAL, stream);
+        if (rc == M2_OK) rc = m2_monarch_conv_fwd(plan, P3, kf3_dev, C3, B, d, n, M2_CAUSAL, stream);
+    }
     if (rc != M2_OK) return rc;
     if (hyena_heads_fused(plan, n, d, dh)) {
         rc = m2h::heads_fwd(plan, C1, C2, C3, kt, P1, B, d, n, st);

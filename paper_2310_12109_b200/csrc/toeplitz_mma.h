@@ -1,0 +1,25 @@
+// Short causal convolutions as Toeplitz products (internal header).
+#pragma once
+#include <cuda_runtime.h>
+
+#include <cstdint>
+
+struct m2_plan;
+
+namespace m2t {
+
+constexpr int kMaxN = 512;   // longest row
+// bf16 plans whose spectrum buffers carry the kernel in the time domain as well (m2f::spectrum): N = 256, 512, 1024
+bool has_time_kernel(const m2_plan* pl);
+// device address of that part of a spectrum buffer for H channels: fp32 [H][N], lag u at u mod N
+const float* time_kernel(const m2_plan* pl, const void* kf, int64_t H);
+
+struct Rows {
+    const void* x;    // [B][H][n]
+    const float* kt;  // [H / kf_group][N]
+    void* y;          // [B][H][n]; must not be x
+};
+// y = the first n values of the circular convolution of the zero-padded rows (2 n <= N), up to three sets of rows in one launch
+int32_t conv(const m2_plan* pl, const Rows* sets, int count, int64_t B, int64_t H, int64_t n, int kf_group, cudaStream_t stream);
+
+}  // namespace m2t
