@@ -11,8 +11,9 @@
 // 8 K multiply-adds.)  Kernel values lie reversed in shared memory, in two copies one element apart, so that the two values of a
 // fragment's column pair are one aligned 64-bit load for even and odd rows alike; lags below zero are stored as zeros.
 //
-// Measured, one B200, layer at B = 32, n = 256, d = 768 (1536 heads): 403 -> 163 us with this kernel in place of 24 576 tensor-core
-// convolution units of 16 rows each (about 280 us of the 403).  Bound by instruction issue: 136 tile pairs of about 20 instructions.
+// Measured, one B200, 1536 heads of n = 256: 21.6 us (28.6 with index divisions in the copies and the two copies of the kernel in the
+// same banks) where 24 576 tensor-core convolution units of 16 rows took about 280 us.  Bound by instruction issue and the fragments'
+// latency: 136 tile pairs of about 20 instructions.
 #include "fft_conv.h"
 #include "fft_core.cuh"
 #include "heads_mma.h"
@@ -25,7 +26,7 @@ constexpr int kThreads = 256, kDh = 16, kMaxN = 1024;
 
 __host__ __device__ constexpr int padded(int n) { return (n + 15) / 16 * 16; }
 __host__ __device__ constexpr int pitch(int n) { return padded(n) + 8; }              // bf16 elements: rows 16 bytes apart mod 128
-__host__ __device__ constexpr int kcopy(int n) { return padded(n) + 32; }             // floats of one reversed copy of the kernel
+__host__ __device__ constexpr int kcopy(int n) { return (padded(n) + 31) / 32 * 32 + 48; }   // floats of one reversed copy; copies 16 banks apart
 __host__ __device__ constexpr int smem_bytes(int n) { return 3 * kDh * pitch(n) * 2 + 2 * kcopy(n) * 4; }
 
 using m2t::bf2;
@@ -55,26 +56,28 @@ __global__ void __launch_bounds__(kThreads)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     // copy p (p = 0, 1): the kernel value of a lag lies at np + 14 + p - lag
-    for (int i = tid; i < 2 * kc; i += kThreads) {
-        const int p = i >= kc, lag = np + 14 + p - (i - p * kc);
-        ks[i] = lag >= 0 && lag < n ? kt[(size_t)h * n + lag] : 0.f;
+    for (int i = tid; i < kc; i += kThreads) {
+        const int lag = np + 14 - i;
+        const float a = lag >= 0 && lag < n ? __ldg(kt + (size_t)h * n + lag) : 0.f;
+        ks[i] = a;
+        if (i + 1 < kc) ks[kc + i + 1] = a;
     }
+    if (tid == 0) ks[kc] = 0.f;   // (lag np + 15)
     const __nv_bfloat16* src[3] = {X1 + base, X2 + base, V + base};
     if (n % 8 == 0) {   // 16-byte pieces never straddle a row
-        const int per_row = n / 8;
-        for (int i = tid; i < kDh * per_row; i += kThreads) {
-            const int r = i / per_row, c = (i % per_row) * 8;
+        for (int c = lane * 8; c < n; c += 256) {   // two rows of each tensor per warp, all six loads in flight
+            uint4 v[6];
 #pragma unroll
-            for (int q = 0; q < 3; ++q)
-                *reinterpret_cast<uint4*>(xs1 + q * kDh * ld + r * ld + c) = __ldg(reinterpret_cast<const uint4*>(src[q]) + i);
+            for (int q = 0; q < 6; ++q) v[q] = __ldg(reinterpret_cast<const uint4*>(src[q >> 1] + (size_t)(warp + 8 * (q & 1)) * n + c));
+#pragma unroll
+            for (int q = 0; q < 6; ++q) *reinterpret_cast<uint4*>(xs1 + ((q >> 1) * kDh + warp + 8 * (q & 1)) * ld + c) = v[q];
         }
         if (np != n && tid < 3 * kDh) *reinterpret_cast<uint4*>(xs1 + tid * ld + n) = make_uint4(0u, 0u, 0u, 0u);
     } else {
-        for (int i = tid; i < kDh * np; i += kThreads) {
-            const int r = i / np, c = i % np;
+        for (int r = warp; r < kDh; r += 8)
+            for (int c = lane; c < np; c += 32)
 #pragma unroll
-            for (int q = 0; q < 3; ++q) xs1[q * kDh * ld + r * ld + c] = c < n ? src[q][(size_t)r * n + c] : __float2bfloat16_rn(0.f);
-        }
+                for (int q = 0; q < 3; ++q) xs1[q * kDh * ld + r * ld + c] = c < n ? src[q][(size_t)r * n + c] : __float2bfloat16_rn(0.f);
     }
     __syncthreads();
     const int m = lane >> 3, r8 = lane & 7, g = lane >> 2, c2 = 2 * (lane & 3);
@@ -112,11 +115,12 @@ __global__ void __launch_bounds__(kThreads)
     }
     __syncthreads();
     if (n % 8 == 0) {
-        const int per_row = n / 8;
-        for (int i = tid; i < kDh * per_row; i += kThreads)
-            reinterpret_cast<uint4*>(O + base)[i] = *reinterpret_cast<const uint4*>(xs1 + (i / per_row) * ld + (i % per_row) * 8);
+        for (int r = warp; r < kDh; r += 8)
+            for (int c = lane * 8; c < n; c += 256)
+                *reinterpret_cast<uint4*>(O + base + (size_t)r * n + c) = *reinterpret_cast<const uint4*>(xs1 + r * ld + c);
     } else {
-        for (int i = tid; i < kDh * n; i += kThreads) O[base + i] = xs1[(i / n) * ld + i % n];
+        for (int r = warp; r < kDh; r += 8)
+            for (int c = lane; c < n; c += 32) O[base + (size_t)r * n + c] = xs1[r * ld + c];
     }
 }
 

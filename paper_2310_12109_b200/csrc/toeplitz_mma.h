@@ -8,8 +8,8 @@ struct m2_plan;
 
 namespace m2t {
 
-constexpr int kMaxN = 512;   // longest row
-// bf16 plans whose spectrum buffers carry the kernel in the time domain as well (m2f::spectrum): N = 256, 512, 1024
+constexpr int kMaxN = 256;   // longest row
+// bf16 plans whose spectrum buffers carry the kernel in the time domain as well (m2f::spectrum): N = 256 and 512
 bool has_time_kernel(const m2_plan* pl);
 // device address of that part of a spectrum buffer for H channels: fp32 [H][N], lag u at u mod N
 const float* time_kernel(const m2_plan* pl, const void* kf, int64_t H);

@@ -192,6 +192,28 @@ def test_conv_with_a_kernel_shared_by_channel_groups(B, dims, n, causal, dtype, 
     plan.close()
 
 
+@pytest.mark.parametrize("B,H,n,dims,group", [(9, 3, 1, (32, 16), 1), (17, 4, 15, (32, 16), 2), (16, 2, 31, (16, 16), 1), (33, 3, 34, (16, 16), 1),
+                                              (1, 700, 128, (16, 16), 1), (32, 150, 200, (32, 16), 5), (40, 3, 255, (32, 16), 1), (9, 300, 256, (32, 16), 1)])
+def test_short_causal_convolution_as_toeplitz_product(B, H, n, dims, group):
+    """The Toeplitz kernel at the edges of its tiles: one and two tiles of 16, a half-empty tile of 32 positions, 1 / 16 / 17 / 33 / 40
+    batch rows, odd and even row lengths, more items than blocks, channel groups; forward and with the conjugated spectrum (lags
+    reversed).  The kernel's values keep 16 bits, the output is rounded once to bf16 (1.7e-3 in the 2-norm)."""
+    Hk, N = H // group, int(np.prod(dims))
+    x = synth.round_bf16(synth.normal(720 + n, (B, H, n)))
+    k = (synth.normal(721 + n, (Hk, n)) / np.sqrt(n)).astype(np.float32)
+    plan = M.Plan(dims, dtype=M.M2_BF16, device=0)
+    kf = M.m2_kernel_spectrum(plan, dev(k))
+    xd = dev(x.astype(np.float32), torch.bfloat16)
+    fx = np.fft.rfft(x.astype(np.float64), N)
+    fk = np.repeat(np.fft.rfft(k.astype(np.float64), N), group, axis=0)[None]
+    y = M.m2_monarch_conv_fwd_grouped(plan, xd, kf, M.M2_CAUSAL, group)
+    assert plan.last_kernel() == "conv_toeplitz_mma"
+    check(host(y), np.fft.irfft(fx * fk, N)[..., :n], 4e-3, "Toeplitz product")
+    g = M.m2_monarch_conv_fwd_grouped(plan, xd, M.m2_spectrum_conjugate(plan, kf, Hk), M.M2_CAUSAL, group)
+    check(host(g), np.fft.irfft(fx * np.conj(fk), N)[..., :n], 4e-3, "transposed Toeplitz product")
+    plan.close()
+
+
 @pytest.mark.parametrize("B", [5, 19])
 def test_bf16_causal_order2_and_ragged(B):
     for n in (256, 100, 48):
