@@ -251,6 +251,12 @@ int32_t m2_hyena_heads_fwd(const m2_plan* plan, const void* u_dev, const void* c
 int32_t m2_blocks_transpose(const m2_plan* plan, const void* W_in_dev, void* W_out_dev, int64_t nblocks, int64_t rows,
                             int64_t cols, void* stream);
 
+/* The same gradient in one call, dX = M^T G, for plans whose tensor-core kernels use the blocks of L and R transposed as they lie (bf16, 64 x 64
+ * blocks, with a workspace of m2_matmul_workspace_bytes(plan, T) bytes and G_dev on a 32-byte boundary); M2_ERR_UNSUPPORTED
+ * otherwise: transpose the blocks and call m2_monarch_matmul. */
+int32_t m2_monarch_matmul_bwd_input(const m2_plan* plan, const void* G_dev, const void* L_dev, const void* R_dev, void* dX_dev, int64_t T,
+                                    void* ws_dev, int64_t ws_bytes, void* stream);
+
 /* Order-p Monarch product Y_t = M X_t in the direct form (Eq. 1; App. D.6, "p-variate Monarch") for a plan of any order
  * p = 1..3 with arbitrary (learnable) blocks.  With the input index n = (n_1, .., n_p), n_1 most significant, stage
  * a = 1..p contracts the digit n_a into the output digit k_a with the block chosen by (k_1, .., k_{a-1}, n_{a+1}, .., n_p);

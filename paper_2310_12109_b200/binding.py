@@ -58,6 +58,7 @@ SIGNATURES = {
     "m2_blocky_monarch_conv_fwd": (_i32, [_vp, _vp, _vp, _vp, _vp, _i64, _i64, _i64, _vp]),
     "m2_selftest_bounded_wait": (_i32, [_vp, _vp, _vp, _vp, _i64, _i64, _i64, _i32, _vp]),
     "m2_selftest_bounded_wait_matmul": (_i32, [_vp, _vp, _vp, _vp, _vp, _i64, _vp, _i64, _vp]),
+    "m2_monarch_matmul_bwd_input": (_i32, [_vp, _vp, _vp, _vp, _vp, _i64, _vp, _i64, _vp]),
     "m2_monarch_apply_order_p": (_i32, [_vp, _vp, ctypes.POINTER(ctypes.c_void_p), _vp, _i64, _vp]),
     "m2_status_string": (ctypes.c_char_p, [_i32]),
     "m2_last_device_status": (_i32, [_vp, ctypes.POINTER(_i32)]),
@@ -414,6 +415,19 @@ def m2_blocks_transpose(plan: Plan, W: torch.Tensor) -> torch.Tensor:
 def m2_monarch_matmul_bwd_input(plan_t: Plan, G: torch.Tensor, L: torch.Tensor, R: torch.Tensor, ws: torch.Tensor | None = None):
     """dX = M^T G for M = P L P^T R P: the forward call with the block-wise transposed factors in swapped roles.
     plan_t: a plan with the factors (N2, N1) (the forward plan itself when N1 == N2)."""
+    if plan_t.dims[0] == plan_t.dims[1]:   # plan_t is the forward plan: kernels that take the blocks as they lie, if it has them
+        for t in (G, L, R):
+            assert t.is_cuda and t.dtype == plan_t.torch_dtype and t.is_contiguous()
+        n1 = plan_t.dims[0]
+        assert G.dim() == 2 and G.shape[1] == plan_t.N and tuple(L.shape) == (n1, n1, n1) and tuple(R.shape) == (n1, n1, n1)
+        if ws is None:
+            ws = m2_matmul_workspace(plan_t, G.shape[0], G.device)
+        dX = torch.empty_like(G)
+        st = lib().m2_monarch_matmul_bwd_input(plan_t.handle, _ptr(G), _ptr(L), _ptr(R), _ptr(dX), G.shape[0], _ptr(ws),
+                                               0 if ws is None else ws.numel(), _stream())
+        if st != M2_ERR_UNSUPPORTED:
+            _check(st, "m2_monarch_matmul_bwd_input")
+            return dX
     return m2_monarch_matmul(plan_t, G, m2_blocks_transpose(plan_t, R), m2_blocks_transpose(plan_t, L), ws=ws)
 
 

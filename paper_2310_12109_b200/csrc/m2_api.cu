@@ -747,6 +747,17 @@ int32_t m2_blocks_transpose(const m2_plan* plan, const void* W_in_dev, void* W_o
     return M2_OK;
 }
 
+int32_t m2_monarch_matmul_bwd_input(const m2_plan* plan, const void* G_dev, const void* L_dev, const void* R_dev, void* dX_dev, int64_t T,
+                                    void* ws_dev, int64_t ws_bytes, void* stream) {
+    const int32_t st = check_matmul_args(plan, G_dev, L_dev, R_dev, dX_dev, T);
+    if (st != M2_OK) return st;
+    if (ws_dev && !aligned16(ws_dev)) return M2_ERR_ALIGNMENT;
+    if (!m2mm::covered(plan) || !ws_dev || ws_bytes < m2mm::workspace_bytes(plan, T)) return M2_ERR_UNSUPPORTED;
+    DeviceGuard g(plan->device);
+    if (!g.ok) return M2_ERR_CUDA;
+    return m2mm::matmul_bwd_input(plan, G_dev, L_dev, R_dev, dX_dev, T, ws_dev, (cudaStream_t)stream);
+}
+
 int64_t m2_matmul_bwd_workspace_bytes(const m2_plan* plan, int64_t T) {
     if (!plan || plan->p != 2 || T < 0) return -1;
     const int64_t generic = T * plan->N * 4, umma = m2mm::wgrad_workspace_bytes(plan, T);

@@ -58,6 +58,11 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, uint32_t sr
                  "r"(c1), "r"(c2)
                  : "memory");
 }
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, uint32_t bar) {
+    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
+                 "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(bar)
+                 : "memory");
+}
 __device__ __forceinline__ void bulk_store(void* gdst, uint32_t ssrc, uint32_t bytes) {
     asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(gdst), "r"(ssrc), "r"(bytes) : "memory");
 }
@@ -268,8 +273,48 @@ constexpr int kFwdThreads = 32 * (kLoadWarps + kDrainWarps + kIssueWarps);
 constexpr size_t kTileBytes = (size_t)kTok * 8192;    // a tile of x, z or y
 static_assert(F_SMEM_BYTES <= 232448, "shared-memory budget of the forward passes");
 
+// 8 pieces of 16 consecutive block indices, one per 128-byte line; cached in L2 only: the rest of every line belongs to other SMs.
+// Rows that are only 16-byte aligned come as two halves.
+__device__ __forceinline__ void load_pieces(uint32_t (&w)[8][8], const unsigned char* src, bool live) {
+    const bool whole = (reinterpret_cast<uintptr_t>(src) & 31u) == 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        if (live && whole) {
+            asm volatile("ld.global.cg.v8.u32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                         : "=r"(w[i][0]), "=r"(w[i][1]), "=r"(w[i][2]), "=r"(w[i][3]), "=r"(w[i][4]), "=r"(w[i][5]), "=r"(w[i][6]), "=r"(w[i][7])
+                         : "l"(src + i * 128));
+        } else if (live) {
+#pragma unroll
+            for (int m = 0; m < 8; m += 4)
+                asm volatile("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];"
+                             : "=r"(w[i][m]), "=r"(w[i][m + 1]), "=r"(w[i][m + 2]), "=r"(w[i][m + 3])
+                             : "l"(src + i * 128 + m * 4));
+        } else {
+#pragma unroll
+            for (int m = 0; m < 8; ++m) w[i][m] = 0u;
+        }
+    }
+}
+// the 16 x 8 transpose in registers (this is P): 16 bytes = 8 consecutive values of the contracted index of one (token, block), into
+// the swizzled operands [token][64] of 16 blocks, 4 KB apart
+__device__ __forceinline__ void store_pieces(const uint32_t (&w)[8][8], unsigned char* dst) {
+#pragma unroll
+    for (int m = 0; m < 8; ++m) {
+        uint4 lo, hi;
+        lo.x = prmt(w[0][m], w[1][m], 0x5410); hi.x = prmt(w[0][m], w[1][m], 0x7632);
+        lo.y = prmt(w[2][m], w[3][m], 0x5410); hi.y = prmt(w[2][m], w[3][m], 0x7632);
+        lo.z = prmt(w[4][m], w[5][m], 0x5410); hi.z = prmt(w[4][m], w[5][m], 0x7632);
+        lo.w = prmt(w[6][m], w[7][m], 0x5410); hi.w = prmt(w[6][m], w[7][m], 0x7632);
+        *reinterpret_cast<uint4*>(dst + (2 * m) * 4096) = lo;
+        *reinterpret_cast<uint4*>(dst + (2 * m + 1) * 4096) = hi;
+    }
+}
+
 // PASS 1: in = x[T][64 n1][64 n2], weights R[n2][k1][n1], out = workspace z
 // PASS 2: in = workspace z, weights L[k1][k2][n2], out = y[T][64 k2][64 k1] (optionally sigma(K (.) y))
+//
+// wt: every weight block is used transposed (the products of the backward pass): the block as it lies in shared memory is then an
+// M-major operand instead of a K-major one, nothing is moved.
 //
 // Persistent: CTA c of a grid that is a multiple of 4 walks the items c, c + grid, .. of (token tile, block group) pairs numbered
 // group-fastest, so its block group is c % 4 for good (the weights stay) and the 4 CTAs that share a tile's lines work on it at
@@ -283,7 +328,7 @@ template <int PASS>
 __global__ void __launch_bounds__(kFwdThreads, 1)
 monarch64_fwd_kernel(const __nv_bfloat16* __restrict__ in, const __grid_constant__ CUtensorMap map_w,
                      const __grid_constant__ CUtensorMap map_y, __nv_bfloat16* __restrict__ out, long long T,
-                     int32_t* __restrict__ status, const __nv_bfloat16* __restrict__ Kmul, long long Hk, int relu, int selftest) {
+                     int32_t* __restrict__ status, const __nv_bfloat16* __restrict__ Kmul, long long Hk, int relu, int selftest, int wt) {
     extern __shared__ __align__(1024) unsigned char smem[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t s_base = smem_u32(smem);
@@ -356,17 +401,7 @@ monarch64_fwd_kernel(const __nv_bfloat16* __restrict__ in, const __grid_constant
                 const bool live = tile * kTok + t_in < T;
                 const unsigned char* src =
                     reinterpret_cast<const unsigned char*>(in) + (size_t)(tile * kTok + t_in) * 8192 + (size_t)(8 * sub) * 128 + grp * 32;
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {   // cached in L2 only: the rest of every line belongs to other SMs
-                    if (live) {
-                        asm volatile("ld.global.cg.v8.u32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                                     : "=r"(w[i][0]), "=r"(w[i][1]), "=r"(w[i][2]), "=r"(w[i][3]), "=r"(w[i][4]), "=r"(w[i][5]), "=r"(w[i][6]), "=r"(w[i][7])
-                                     : "l"(src + i * 128));
-                    } else {
-#pragma unroll
-                        for (int m = 0; m < 8; ++m) w[i][m] = 0u;
-                    }
-                }
+                load_pieces(w, src, live);
             } else {   // whole tiles of the workspace were written
                 const unsigned char* src =
                     reinterpret_cast<const unsigned char*>(in) + (size_t)tile * kTileBytes + (size_t)t_in * 2048 + (size_t)(16 * grp + sub) * 32;
@@ -378,18 +413,8 @@ monarch64_fwd_kernel(const __nv_bfloat16* __restrict__ in, const __grid_constant
             }
         };
         auto store_opnd = [&]() {
-            if (PASS == 1) {   // the 16 x 8 transpose in registers (this is P): 16 bytes = 8 consecutive n1 of one (t, n2)
-                unsigned char* dst = smem + F_OFF_A + sw_off(t_in, sub);
-#pragma unroll
-                for (int m = 0; m < 8; ++m) {
-                    uint4 lo, hi;
-                    lo.x = prmt(w[0][m], w[1][m], 0x5410); hi.x = prmt(w[0][m], w[1][m], 0x7632);
-                    lo.y = prmt(w[2][m], w[3][m], 0x5410); hi.y = prmt(w[2][m], w[3][m], 0x7632);
-                    lo.z = prmt(w[4][m], w[5][m], 0x5410); hi.z = prmt(w[4][m], w[5][m], 0x7632);
-                    lo.w = prmt(w[6][m], w[7][m], 0x5410); hi.w = prmt(w[6][m], w[7][m], 0x7632);
-                    *reinterpret_cast<uint4*>(dst + (2 * m) * 4096) = lo;
-                    *reinterpret_cast<uint4*>(dst + (2 * m + 1) * 4096) = hi;
-                }
+            if (PASS == 1) {
+                store_pieces(w, smem + F_OFF_A + sw_off(t_in, sub));
             } else {           // a piece is 32 bytes of row t of block k1's operand as it lies
                 unsigned char* dst = smem + F_OFF_A + sub * 4096;
 #pragma unroll
@@ -494,7 +519,8 @@ monarch64_fwd_kernel(const __nv_bfloat16* __restrict__ in, const __grid_constant
         if (!ok && lane == 0) timed_out();
     } else if (lane == 0) {
         // ---- issuing threads ----
-        constexpr uint32_t IDESC = instr_desc_bf16(64, kTok, false, false);
+        const uint32_t idesc = instr_desc_bf16(64, kTok, wt != 0, false);
+        const uint64_t wstep = wt ? 2048 >> 4 : 32 >> 4;   // 16 inputs: rows of the block as it lies, or 32 bytes of a row
         constexpr int kPer = kGroup2 / kIssueWarps;
         const int b0 = (warp - kLoadWarps - kDrainWarps) * kPer;
         ok = mbar_wait(bar_w, 0);
@@ -512,7 +538,7 @@ monarch64_fwd_kernel(const __nv_bfloat16* __restrict__ in, const __grid_constant
                 const uint64_t ad = smem_desc_sw128(s_base + F_OFF_W + b * 8192, 16, 1024);
                 const uint64_t bd = smem_desc_sw128(s_base + F_OFF_A + b * 4096, 16, 1024);
 #pragma unroll
-                for (int s = 0; s < 4; ++s) umma_f16(d, ad + s * 2, bd + s * 2, IDESC, s > 0);   // K step of 16: 32 bytes of a swizzled row
+                for (int s = 0; s < 4; ++s) umma_f16(d, ad + s * wstep, bd + s * 2, idesc, s > 0);   // K step of 16: 32 bytes of a swizzled row
             }
             umma_commit(bar_mma + 8 * p);
         }
@@ -533,191 +559,213 @@ monarch64_fwd_kernel(const __nv_bfloat16* __restrict__ in, const __grid_constant
 // Z = the intermediate in the workspace layout [token tile][m / 8][b][t % 128][m % 8] that pass 1 writes:
 //   dR[n2][k1][n1] = sum_t dv[t][n2][k1] x[t][n1][n2]:  V = x (b = n2, a = n1),  Z = pass 1 of (g, L^T) (m = k1)
 //   dL[k1][k2][n2] = sum_t g[t][k2][k1] v[t][n2][k1]:   V = g (b = k1, a = k2),  Z = pass 1 of (x, R)   (m = n2), D = dL[k1]^T
-// With the tokens as the K dimension both operands lie in shared memory as the forward kernels already produce them: the
-// 128-byte-swizzled tile [t][a] that pass 1 builds from 16-byte pieces of V is an N-major B operand (a row = one t), and a
-// workspace block [t][8 m] is a column of M-major core matrices (8 consecutive t x 16 bytes) of the A operand.
-// A CTA owns 8 consecutive blocks and one share of the 64-token half tiles, accumulates its 8 [64 x 64] partial results in
-// TMEM (M = 64: rows in lanes 0..15 of every lane quarter) over its whole share and writes them once; a second kernel adds
-// the shares in a fixed order.
-constexpr int WG_OFF_X = 0;           // 8 operands [64 t][64 a] bf16, swizzled rows of 128 bytes            65536
-constexpr int WG_OFF_Z = 65536;       // [m / 8][block 8][64 t][16 B]                                         65536
-constexpr int WG_OFF_BAR = 131072;
-constexpr int WG_SMEM = WG_OFF_BAR + 64;
-constexpr int kWgSplits = 18;         // 8 block groups x 18 shares = 144 CTAs
-constexpr size_t kWgPartialBytes = (size_t)kWgSplits * 64 * 4096 * 4;
+// With the tokens as the K dimension both operands lie in shared memory as the forward passes already produce them: the swizzled
+// tile [t][a] that pass 1 builds from 32-byte pieces of V is an MN-major operand (a row = one t), and a piece of the workspace,
+// 16 values of m of one (t, b), is a row of a 32-byte-swizzled MN-major operand, so the copy engine brings Z as boxes
+// [16 blocks][32 t][32 B].  Either may be the A operand: dL and dR leave as they are stored.
+// A CTA owns 16 consecutive blocks and every (grid / 4)-th 32-token tile, accumulates its 16 [64 x 64] partial results in TMEM (M = 64:
+// blocks 8 .. 15 at lane offset 16) and writes them once; a second kernel adds the shares in a fixed order.  Roles: warps 0..7 load V
+// (the next tile's pieces are in flight while this one is multiplied), lane 0 of warp 8 copies Z (two buffers), lane 0 of warps 9 and
+// 10 issue for 8 blocks each.  Bound, as the forward passes, by the requests for V's pieces (about 0.46 per cycle and SM).
+// GRADTIME
+constexpr int G_OFF_V = 0;            // 16 operands [32 t][64 a] bf16, swizzled rows of 128 bytes                        65536
+constexpr int G_OFF_Z = 65536;        // two buffers [m / 16][16 blocks][32 t][32 B]                                     131072
+constexpr int G_OFF_BAR = 196608;     // bar_v, bar_mma[2], bar_z[2], tmem ptr, abort flag
+constexpr int G_SMEM = G_OFF_BAR + 64;
+constexpr int kGradLoadWarps = 8, kGradThreads = 32 * (kGradLoadWarps + 3);
+constexpr int kGradShares = 37;       // 4 block groups x 37 = 148 CTAs
+constexpr size_t kGradPartialBytes = (size_t)kGradShares * 64 * 4096 * 4;
+static_assert(G_SMEM <= 232448, "shared-memory budget of the gradient kernel");
 
-__global__ void __launch_bounds__(kThreads, 1)
-monarch64_wgrad_kernel(const __nv_bfloat16* __restrict__ in, const __nv_bfloat16* __restrict__ zin, float* __restrict__ partial,
-                       long long T, int units, int32_t* __restrict__ status) {
+template <bool Z_IS_A>
+__global__ void __launch_bounds__(kGradThreads, 1)
+monarch64_wgrad_kernel(const __nv_bfloat16* __restrict__ in, const __grid_constant__ CUtensorMap map_z, float* __restrict__ partial,
+                       long long T, int32_t* __restrict__ status) {
     extern __shared__ __align__(1024) unsigned char smem[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t s_base = smem_u32(smem);
-    const uint32_t bar_mma = s_base + WG_OFF_BAR, s_tptr = s_base + WG_OFF_BAR + 16, bar_in = s_base + WG_OFF_BAR + 24;
-    const int grp = blockIdx.x, split = blockIdx.y, nsplit = gridDim.y;
+    const uint32_t bar_v = s_base + G_OFF_BAR, bar_mma = bar_v + 8, bar_z = bar_v + 24, s_tptr = bar_v + 40;
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + G_OFF_BAR + 48);
+    const int grp = blockIdx.x & 3, share = blockIdx.x >> 2, nshare = gridDim.x >> 2;
+    const int ntiles = (int)((T + kTok - 1) / kTok);
     if (tid == 0) {
-        mbar_init(bar_mma, 1);
-        mbar_init(bar_in, 1);
+        mbar_init(bar_v, kGradLoadWarps);
+        mbar_init(bar_mma, 2);         // both issuing threads; tile n uses barrier n % 2, so that a wait for tile n - 2 cannot miss it
+        mbar_init(bar_mma + 8, 2);
+        mbar_init(bar_z, 1);
+        mbar_init(bar_z + 8, 1);
+        *abort_flag = 0;
         fence_barrier_init();
+        prefetch_tensormap(&map_z);
     }
-    if (tid < 32) tmem_alloc(s_tptr, 512);
+    if (warp == 8) tmem_alloc(s_tptr, 512);
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");   // the workspace was written by the kernel before this one
-    tc_fence_before();
     __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(smem + WG_OFF_BAR + 16);
-    constexpr uint32_t IDESC = instr_desc_bf16(64, 64, true, true);
-    uint32_t ph = 0;
+    asm volatile("griddepcontrol.wait;" ::: "memory");   // the workspace was written by the kernel before this one
+    const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(smem + G_OFF_BAR + 40);
     bool ok = true;
-    int it = 0;
+    uint32_t n = 0;   // tiles begun
+    if (warp < kGradLoadWarps) {
+        const int t_in = tid >> 3, sub = tid & 7;   // (token, 8 consecutive a), as in pass 1
+        uint32_t w[8][8];
+        auto load_in = [&](int tile) {
+            const long long t = (long long)tile * kTok + t_in;
+            load_pieces(w, reinterpret_cast<const unsigned char*>(in) + (size_t)t * 8192 + (size_t)(8 * sub) * 128 + grp * 32, t < T);
+        };
+        if (share < ntiles) load_in(share);
 #pragma unroll 1
-    for (int u = split; u < units; u += nsplit, ++it) {
-        const int tile = u >> 1, half = u & 1;
-        const long long t0 = (long long)tile * kTileT + half * 64;
-        if (tid == 0) {   // 64 tokens of the 8 blocks' workspace columns: 64 pieces of 1 KB
-            mbar_expect_tx(bar_in, 65536);
-            const unsigned char* zb = reinterpret_cast<const unsigned char*>(zin) + (size_t)tile * (8 * 131072) + (size_t)grp * 16384 + half * 1024;
-            for (int kc = 0; kc < 8; ++kc)
-                for (int bl = 0; bl < 8; ++bl)
-                    bulk_load(s_base + WG_OFF_Z + kc * 8192 + bl * 1024, zb + (size_t)kc * 131072 + bl * 2048, 1024, bar_in);
+        for (int tile = share; tile < ntiles; tile += nshare, ++n) {
+            if (__any_sync(~0u, *abort_flag != 0)) break;
+            if (n > 0) ok = __all_sync(~0u, mbar_wait(bar_mma + 8 * ((n - 1) & 1), ((n - 1) >> 1) & 1));   // the UMMAs have read the operands
+            if (!ok) break;
+            store_pieces(w, smem + G_OFF_V + sw_off(t_in, sub));
+            fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_v);
+            if (tile + nshare < ntiles) load_in(tile + nshare);
         }
-        {   // one (token, group of 8 a) per thread: 8 pieces of 16 bytes, 8 x 8 transpose, 8 stores (see pass 1)
-            const int g = tid & 7, tt = tid >> 3;
-            uint4 v[8];
-            const bool live = t0 + tt < T;
-            const uint4* src = reinterpret_cast<const uint4*>(in + (size_t)(t0 + tt) * 4096 + (size_t)(8 * g) * 64 + grp * 8);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                v[i] = make_uint4(0u, 0u, 0u, 0u);
-                if (live)
-                    asm volatile("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v[i].x), "=r"(v[i].y), "=r"(v[i].z), "=r"(v[i].w) : "l"(src + i * 8));
-            }
-            const uint32_t* w = reinterpret_cast<const uint32_t*>(v);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                uint4 lo, hi;
-                lo.x = prmt(w[0 * 4 + j], w[1 * 4 + j], 0x5410); hi.x = prmt(w[0 * 4 + j], w[1 * 4 + j], 0x7632);
-                lo.y = prmt(w[2 * 4 + j], w[3 * 4 + j], 0x5410); hi.y = prmt(w[2 * 4 + j], w[3 * 4 + j], 0x7632);
-                lo.z = prmt(w[4 * 4 + j], w[5 * 4 + j], 0x5410); hi.z = prmt(w[4 * 4 + j], w[5 * 4 + j], 0x7632);
-                lo.w = prmt(w[6 * 4 + j], w[7 * 4 + j], 0x5410); hi.w = prmt(w[6 * 4 + j], w[7 * 4 + j], 0x7632);
-                *reinterpret_cast<uint4*>(smem + WG_OFF_X + (2 * j) * 8192 + sw_off(tt, g)) = lo;
-                *reinterpret_cast<uint4*>(smem + WG_OFF_X + (2 * j + 1) * 8192 + sw_off(tt, g)) = hi;
-            }
-        }
-        fence_proxy_async();
-        tc_fence_before();
-        __syncthreads();
-        if (tid == 0) {
+        // the 16 accumulators: row r of block b sits in lane (r % 16) + 16 (b / 8) of lane quarter r / 16, columns 64 (b % 8) ..
+        if (ok && n > 0) ok = __all_sync(~0u, mbar_wait(bar_mma + 8 * ((n - 1) & 1), ((n - 1) >> 1) & 1) && *abort_flag == 0);
+        if (ok && n > 0) {
             tc_fence_after();
-            const bool in_ok = mbar_wait(bar_in, ph);
-            if (in_ok) {
+            const int q = warp & 3, r = 16 * q + (lane & 15), set = lane >> 4;
+            const uint32_t t_lane = tmem + ((uint32_t)(q * 32) << 16);
 #pragma unroll 1
-                for (int bl = 0; bl < kGroup; ++bl)
+            for (int cb = 4 * (warp >> 2); cb < 4 * (warp >> 2) + 4; ++cb) {
+                float* dst = partial + (((size_t)share * 64 + grp * 16 + cb + 8 * set) * 64 + r) * 64;
+#pragma unroll 1
+                for (int c0 = 0; c0 < 64; c0 += 32) {
+                    float v[32];
 #pragma unroll
-                    for (int s = 0; s < 4; ++s)   // 16 tokens per instruction
-                        umma_f16(tmem + bl * 64, smem_desc(s_base + WG_OFF_Z + bl * 1024 + s * 256, 128, 8192),
-                                 smem_desc_sw128(s_base + WG_OFF_X + bl * 8192 + s * 2048, 8192, 1024), IDESC, (it > 0 || s > 0) ? 1u : 0u);
-            }
-            umma_commit(bar_mma);
-            if (!in_ok) atomicExch(status, (int32_t)M2_ERR_TIMEOUT);
-        }
-        ok = mbar_wait(bar_mma, ph);   // both operand buffers are free again
-        ph ^= 1;
-        tc_fence_after();
-        if (!__syncthreads_and(ok)) {
-            ok = false;
-            break;
-        }
-    }
-    // the 8 accumulators: row r of a block sits in lane (r % 16) of lane quarter r / 16; warpgroup wg takes blocks 2 wg, 2 wg + 1
-    if (ok && it > 0) {
-        const int q = warp & 3, wg = warp >> 2, r = 16 * q + lane;
-        const uint32_t t_lane = tmem + ((uint32_t)(q * 32) << 16);
-#pragma unroll 1
-        for (int bb = 0; bb < 2; ++bb) {
-            const int bl = 2 * wg + bb;
-            float* dst = partial + (((size_t)split * 64 + grp * 8 + bl) * 64 + r) * 64;
-#pragma unroll 1
-            for (int c0 = 0; c0 < 64; c0 += 8) {
-                float v[8];
-                tmem_ld8(t_lane + bl * 64 + c0, v);
-                tmem_ld_wait();
-                tmem_ld_fence8(v);
-                if (lane < 16) {
-                    *reinterpret_cast<float4*>(dst + c0) = make_float4(v[0], v[1], v[2], v[3]);
-                    *reinterpret_cast<float4*>(dst + c0 + 4) = make_float4(v[4], v[5], v[6], v[7]);
+                    for (int c = 0; c < 4; ++c) tmem_ld8(t_lane + cb * 64 + c0 + 8 * c, v + 8 * c);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) tmem_ld_fence8(v + 8 * c);
+#pragma unroll
+                    for (int c = 0; c < 32; c += 4) *reinterpret_cast<float4*>(dst + c0 + c) = make_float4(v[c], v[c + 1], v[c + 2], v[c + 3]);
                 }
             }
         }
+    } else if (lane == 0 && warp == 8) {
+        for (int tile = share; tile < ntiles && ok && *abort_flag == 0; tile += nshare, ++n) {
+            const uint32_t z = s_base + G_OFF_Z + (n & 1) * 65536, bz = bar_z + 8 * (n & 1);
+            if (n >= 2) ok = mbar_wait(bar_mma + 8 * (n & 1), ((n - 2) >> 1) & 1);   // the buffer's previous tile has been multiplied
+            if (!ok) break;
+            mbar_expect_tx(bz, 65536);
+            for (int c = 0; c < 4; ++c) tma_load_3d(z + c * 16384, &map_z, 0, (tile * 4 + c) * kTok, 16 * grp, bz);
+        }
+        for (uint32_t i = n > 2 ? n - 2 : 0; i < n; ++i) mbar_wait(bar_z + 8 * (i & 1), (i >> 1) & 1);   // nothing is left in flight
+    } else if (lane == 0) {
+        const uint32_t idesc = instr_desc_bf16(64, 64, true, true);
+        const int b0 = (warp - 9) * 8;
+        for (int tile = share; tile < ntiles && ok && *abort_flag == 0; tile += nshare, ++n) {
+            ok = mbar_wait(bar_v, n & 1) && mbar_wait(bar_z + 8 * (n & 1), (n >> 1) & 1);
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t z = s_base + G_OFF_Z + (n & 1) * 65536;
+#pragma unroll 1
+            for (int b = b0; b < b0 + 8; ++b) {
+                const uint32_t d = tmem + ((uint32_t)(16 * (b >> 3)) << 16) + (uint32_t)(b & 7) * 64;
+                const uint64_t zd = smem_desc_sw32(z + b * 1024, 16384, 256), vd = smem_desc_sw128(s_base + G_OFF_V + b * 4096, 8192, 1024);
+#pragma unroll
+                for (int k = 0; k < 2; ++k)   // 16 tokens per instruction
+                    umma_f16(d, Z_IS_A ? zd + k * 32 : vd + k * 128, Z_IS_A ? vd + k * 128 : zd + k * 32, idesc, (n > 0 || k > 0) ? 1u : 0u);
+            }
+            umma_commit(bar_mma + 8 * (n & 1));
+        }
     }
-    if (!ok && tid == 0) atomicExch(status, (int32_t)M2_ERR_TIMEOUT);
+    if (!ok && lane == 0) {
+        atomicExch(status, (int32_t)M2_ERR_TIMEOUT);
+        *abort_flag = 1;
+    }
     tc_fence_before();
     __syncthreads();
-    if (tid < 32) tmem_dealloc(tmem, 512);
+    if (warp == 8) tmem_dealloc(tmem, 512);
 }
 
-// out[b][i][j] = sum_s partial[s][b][i][j]  (transposed: partial[s][b][j][i]), shares added in index order
-__global__ void wgrad_reduce_kernel(const float* __restrict__ partial, float* __restrict__ out, int nsplit, int transposed) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;   // < 64 * 4096
-    const int b = e >> 12, i = (e >> 6) & 63, j = e & 63;
-    const int src = transposed ? (b << 12) + (j << 6) + i : e;
-    float acc = 0.f;
-    for (int s = 0; s < nsplit; ++s) acc += partial[(size_t)s * (64 * 4096) + src];
+// out = the sum of the shares in index order, four values per thread (nshare = 0: zeros)
+__global__ void __launch_bounds__(256) wgrad_reduce_kernel(const float4* __restrict__ partial, float4* __restrict__ out, int nshare) {
+    const int e = blockIdx.x * 256 + threadIdx.x;   // < 64 * 4096 / 4
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
+    for (int s = 0; s < nshare; ++s) {
+        const float4 v = partial[(size_t)s * 65536 + e];
+        acc.x += v.x;
+        acc.y += v.y;
+        acc.z += v.z;
+        acc.w += v.w;
+    }
     out[e] = acc;
 }
 
-int64_t wgrad_workspace_bytes(const m2_plan* pl, int64_t T) {
-    return covered(pl) ? workspace_bytes(pl, T) + (int64_t)kWgPartialBytes + 64 * 4096 * 2 : 0;
+int64_t wgrad_workspace_bytes(const m2_plan* pl, int64_t T) { return covered(pl) ? workspace_bytes(pl, T) + (int64_t)kGradPartialBytes : 0; }
+
+static cudaLaunchConfig_t early_launch(unsigned grid, int threads, size_t smem, cudaStream_t stream, cudaLaunchAttribute* attr) {
+    attr->id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr->val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3(grid);
+    c.blockDim = dim3((unsigned)threads);
+    c.dynamicSmemBytes = smem;
+    c.stream = stream;
+    c.attrs = attr;
+    c.numAttrs = 1;
+    return c;
+}
+static unsigned fwd_grid(int64_t T) {
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const long long nitems = 4 * ((T + kTok - 1) / kTok);
+    const long long ctas = (sms / 4) * 4 > 4 ? (sms / 4) * 4 : 4;   // a multiple of 4: a CTA keeps its block group
+    return (unsigned)(nitems < ctas ? nitems : ctas);
+}
+// weight blocks as TMA tiles: [64 blocks x 64 rows][64] bf16, one box = one block, 128-byte swizzle
+static bool weight_map(CUtensorMap* m, const void* W) {
+    const cuuint64_t gdim[2] = {64, 64 * 64}, gstr[1] = {128};
+    const cuuint32_t box[2] = {64, 64};
+    return tma_host::encode_sw128_bf16(m, W, 2, gdim, gstr, box);
 }
 
 int32_t wgrad(const m2_plan* pl, const void* X, const void* G, const void* L, const void* R, float* dL, float* dR, int64_t T, void* ws,
               cudaStream_t stream) {
     if (!covered(pl)) return M2_ERR_UNSUPPORTED;
-    const int units = (int)(2 * ((T + kTileT - 1) / kTileT));
-    const int nsplit = units < kWgSplits ? units : kWgSplits;
     unsigned char* zws = static_cast<unsigned char*>(ws);
     float* partial = reinterpret_cast<float*>(zws + workspace_bytes(pl, T));
-    __nv_bfloat16* Lt = reinterpret_cast<__nv_bfloat16*>(zws + workspace_bytes(pl, T) + kWgPartialBytes);
+    const int64_t ntiles = (T + kTok - 1) / kTok;
+    unsigned shares = fwd_grid(T) / 4;
+    if (shares > kGradShares) shares = kGradShares;
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t red = early_launch(256, 256, 0, stream, &attr);
     if (T == 0) {
-        wgrad_reduce_kernel<<<1024, 256, 0, stream>>>(partial, dL, 0, 0);
-        wgrad_reduce_kernel<<<1024, 256, 0, stream>>>(partial, dR, 0, 0);
+        if (cudaLaunchKernelEx(&red, wgrad_reduce_kernel, (const float4*)partial, (float4*)dL, 0) != cudaSuccess ||
+            cudaLaunchKernelEx(&red, wgrad_reduce_kernel, (const float4*)partial, (float4*)dR, 0) != cudaSuccess)
+            return M2_ERR_CUDA;
         pl->launches += 2;
-        return cudaGetLastError() == cudaSuccess ? M2_OK : M2_ERR_CUDA;
+        return M2_OK;
     }
-    alignas(64) CUtensorMap unused;
-    memset(&unused, 0, sizeof(unused));   // pass 1 never touches its map
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t p1 = {};
-    p1.gridDim = dim3(8, (unsigned)((T + kTileT - 1) / kTileT));
-    p1.blockDim = dim3(kThreads);
-    p1.dynamicSmemBytes = SMEM_BYTES;
-    p1.stream = stream;
-    p1.attrs = attr;
-    p1.numAttrs = 1;
-    cudaLaunchConfig_t wg = p1;
-    wg.gridDim = dim3(8, (unsigned)nsplit);
-    wg.dynamicSmemBytes = WG_SMEM;
-    const __nv_bfloat16 *x = (const __nv_bfloat16*)X, *g = (const __nv_bfloat16*)G;
-    // dL: v = R-stage of x, then sum_t v (x) g per block k1
-    if (cudaLaunchKernelEx(&p1, monarch64_pass_kernel<1>, x, (const __nv_bfloat16*)R, unused, (__nv_bfloat16*)zws, (long long)T, pl->d_status,
-                           (const __nv_bfloat16*)nullptr, 1LL, 0) != cudaSuccess)
+    if (ntiles > 0x1000000) return M2_ERR_UNSUPPORTED;   // (row index of the workspace map)
+    // the workspace as (16 values of m | (tile, m / 16, t), 2 KB apart | block, 32 B apart): a box lands block by block
+    alignas(64) CUtensorMap mr, ml, mz;
+    const cuuint64_t zdim[3] = {16, (cuuint64_t)ntiles * 4 * kTok, 64}, zstr[2] = {2048, 32};
+    const cuuint32_t zbox[3] = {16, (cuuint32_t)kTok, 16};
+    if (!weight_map(&mr, R) || !weight_map(&ml, L) || !tma_host::encode_sw32_bf16(&mz, zws, 3, zdim, zstr, zbox)) return M2_ERR_UNSUPPORTED;
+    const cudaLaunchConfig_t p1 = early_launch(fwd_grid(T), kFwdThreads, F_SMEM_BYTES, stream, &attr);
+    const cudaLaunchConfig_t wg = early_launch(4 * shares, kGradThreads, G_SMEM, stream, &attr);
+    const __nv_bfloat16 *x = (const __nv_bfloat16*)X, *g = (const __nv_bfloat16*)G, *none = nullptr;
+    __nv_bfloat16* z = (__nv_bfloat16*)zws;
+    // dL: v = R-stage of x, then sum_t g (x) v per block k1;  dR: dv = L^T-stage of g, then sum_t dv (x) x per block n2
+    if (cudaLaunchKernelEx(&p1, monarch64_fwd_kernel<1>, x, mr, mr, z, (long long)T, pl->d_status, none, 1LL, 0, 0, 0) != cudaSuccess ||
+        cudaLaunchKernelEx(&wg, monarch64_wgrad_kernel<false>, g, mz, partial, (long long)T, pl->d_status) != cudaSuccess ||
+        cudaLaunchKernelEx(&red, wgrad_reduce_kernel, (const float4*)partial, (float4*)dL, (int)shares) != cudaSuccess ||
+        cudaLaunchKernelEx(&p1, monarch64_fwd_kernel<1>, g, ml, ml, z, (long long)T, pl->d_status, none, 1LL, 0, 0, 1) != cudaSuccess ||
+        cudaLaunchKernelEx(&wg, monarch64_wgrad_kernel<true>, x, mz, partial, (long long)T, pl->d_status) != cudaSuccess ||
+        cudaLaunchKernelEx(&red, wgrad_reduce_kernel, (const float4*)partial, (float4*)dR, (int)shares) != cudaSuccess)
         return M2_ERR_CUDA;
-    if (cudaLaunchKernelEx(&wg, monarch64_wgrad_kernel, g, (const __nv_bfloat16*)zws, partial, (long long)T, units, pl->d_status) != cudaSuccess)
-        return M2_ERR_CUDA;
-    wgrad_reduce_kernel<<<1024, 256, 0, stream>>>(partial, dL, nsplit, 1);
-    // dR: dv = L^T-stage of g, then sum_t dv (x) x per block n2
-    if (m2g::launch_blocks_transpose(L, Lt, 64, 64, 64, true, stream) != cudaSuccess) return M2_ERR_CUDA;
-    if (cudaLaunchKernelEx(&p1, monarch64_pass_kernel<1>, g, (const __nv_bfloat16*)Lt, unused, (__nv_bfloat16*)zws, (long long)T, pl->d_status,
-                           (const __nv_bfloat16*)nullptr, 1LL, 0) != cudaSuccess)
-        return M2_ERR_CUDA;
-    if (cudaLaunchKernelEx(&wg, monarch64_wgrad_kernel, x, (const __nv_bfloat16*)zws, partial, (long long)T, units, pl->d_status) != cudaSuccess)
-        return M2_ERR_CUDA;
-    wgrad_reduce_kernel<<<1024, 256, 0, stream>>>(partial, dR, nsplit, 0);
-    if (cudaGetLastError() != cudaSuccess) return M2_ERR_CUDA;
     pl->last_kernel = "matmul_wgrad_umma_64x64";
-    pl->launches += 7;
+    pl->launches += 6;
     return M2_OK;
 }
 
@@ -730,7 +778,8 @@ cudaError_t prepare(const m2_plan* pl) {
     if (!covered(pl)) return cudaSuccess;
     cudaError_t e = cudaFuncSetAttribute(monarch64_pass_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(monarch64_pass_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(monarch64_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, WG_SMEM);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(monarch64_wgrad_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, G_SMEM);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(monarch64_wgrad_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, G_SMEM);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(monarch64_fwd_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, F_SMEM_BYTES);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(monarch64_fwd_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, F_SMEM_BYTES);
     return e;
@@ -770,42 +819,25 @@ static int32_t matmul_g8(const m2_plan* pl, const void* X, const void* L, const 
 }
 
 static int32_t matmul_impl(const m2_plan* pl, const void* X, const void* L, const void* R, void* Y, int64_t T, void* ws, const void* Kmul,
-                           int64_t Hk, int relu, int selftest, cudaStream_t stream) {
+                           int64_t Hk, int relu, int selftest, int wt, cudaStream_t stream) {
     if (!covered(pl)) return M2_ERR_UNSUPPORTED;
     if (T == 0) return selftest ? M2_ERR_UNSUPPORTED : M2_OK;
-    // the 32-byte loads of pass 1 want x on a 32-byte boundary (torch allocations are; a view need not be)
+    // the loads of pass 1 want x on a 32-byte boundary (torch allocations are; a view need not be)
     if ((reinterpret_cast<uintptr_t>(X) & 31u) != 0)
-        return selftest ? M2_ERR_UNSUPPORTED : matmul_g8(pl, X, L, R, Y, T, ws, Kmul, Hk, relu, stream);
-    // weight blocks as TMA tiles: [64 blocks x 64 rows][64] bf16, one box = one block, 128-byte swizzle
+        return selftest || wt ? M2_ERR_UNSUPPORTED : matmul_g8(pl, X, L, R, Y, T, ws, Kmul, Hk, relu, stream);
     alignas(64) CUtensorMap mr, ml, my;
-    const cuuint64_t gdim[2] = {64, 64 * 64}, gstr[1] = {128};
-    const cuuint32_t box[2] = {64, 64};
-    if (!tma_host::encode_sw128_bf16(&mr, R, 2, gdim, gstr, box) || !tma_host::encode_sw128_bf16(&ml, L, 2, gdim, gstr, box))
-        return M2_ERR_UNSUPPORTED;
+    if (!weight_map(&mr, R) || !weight_map(&ml, L)) return M2_ERR_UNSUPPORTED;
     // y[t][k2][k1] seen as (k1 64 | k2, stride 128 B | t, stride 8 KB); box = 16 k1 x 16 k2 x 4 tokens, 32-byte swizzle
     const cuuint64_t ydim[3] = {64, 64, (cuuint64_t)T}, ystr[2] = {128, 8192};
     const cuuint32_t ybox[3] = {16, 16, 4};
     if (!tma_host::encode_sw32_bf16(&my, Y, 3, ydim, ystr, ybox)) return M2_ERR_UNSUPPORTED;
-    cudaLaunchConfig_t cfg = {};
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const long long nitems = 4 * ((T + kTok - 1) / kTok);
-    const long long ctas = (sms / 4) * 4 > 4 ? (sms / 4) * 4 : 4;   // a multiple of 4: a CTA keeps its block group
-    cfg.gridDim = dim3((unsigned)(nitems < ctas ? nitems : ctas));
-    cfg.blockDim = dim3(kFwdThreads);
-    cfg.dynamicSmemBytes = F_SMEM_BYTES;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = early_launch(fwd_grid(T), kFwdThreads, F_SMEM_BYTES, stream, &attr);
     if (cudaLaunchKernelEx(&cfg, monarch64_fwd_kernel<1>, (const __nv_bfloat16*)X, mr, my, (__nv_bfloat16*)ws, (long long)T, pl->d_status,
-                           (const __nv_bfloat16*)nullptr, 1LL, 0, selftest) != cudaSuccess)
+                           (const __nv_bfloat16*)nullptr, 1LL, 0, selftest, wt) != cudaSuccess)
         return M2_ERR_CUDA;
     if (cudaLaunchKernelEx(&cfg, monarch64_fwd_kernel<2>, (const __nv_bfloat16*)ws, ml, my, (__nv_bfloat16*)Y, (long long)T, pl->d_status,
-                           (const __nv_bfloat16*)Kmul, (long long)(Hk > 0 ? Hk : 1), relu, selftest) != cudaSuccess)
+                           (const __nv_bfloat16*)Kmul, (long long)(Hk > 0 ? Hk : 1), relu, selftest, wt) != cudaSuccess)
         return M2_ERR_CUDA;
     pl->last_kernel = "matmul_umma_64x64";
     pl->launches += 2;
@@ -814,12 +846,16 @@ static int32_t matmul_impl(const m2_plan* pl, const void* X, const void* L, cons
 
 int32_t matmul(const m2_plan* pl, const void* X, const void* L, const void* R, void* Y, int64_t T, void* ws, const void* Kmul,
                int64_t Hk, int relu, cudaStream_t stream) {
-    return matmul_impl(pl, X, L, R, Y, T, ws, Kmul, Hk, relu, 0, stream);
+    return matmul_impl(pl, X, L, R, Y, T, ws, Kmul, Hk, relu, 0, 0, stream);
+}
+
+int32_t matmul_bwd_input(const m2_plan* pl, const void* G, const void* L, const void* R, void* dX, int64_t T, void* ws, cudaStream_t stream) {
+    return matmul_impl(pl, G, R, L, dX, T, ws, nullptr, 1, 0, 0, 1, stream);   // M^T: the factors in the opposite order, blocks transposed
 }
 
 int32_t matmul_wait_selftest(const m2_plan* pl, const void* X, const void* L, const void* R, void* Y, int64_t T, void* ws,
                              cudaStream_t stream) {
-    return matmul_impl(pl, X, L, R, Y, T, ws, nullptr, 1, 0, 1, stream);
+    return matmul_impl(pl, X, L, R, Y, T, ws, nullptr, 1, 0, 1, 0, stream);
 }
 
 }  // namespace m2mm
