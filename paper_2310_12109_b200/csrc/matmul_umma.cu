@@ -274,9 +274,10 @@ constexpr size_t kTileBytes = (size_t)kTok * 8192;    // a tile of x, z or y
 static_assert(F_SMEM_BYTES <= 232448, "shared-memory budget of the forward passes");
 
 // 8 pieces of 16 consecutive block indices, one per 128-byte line; cached in L2 only: the rest of every line belongs to other SMs.
-// Rows that are only 16-byte aligned come as two halves.
+// HALVES: rows that are only 16-byte aligned come as two halves.
+template <bool HALVES>
 __device__ __forceinline__ void load_pieces(uint32_t (&w)[8][8], const unsigned char* src, bool live) {
-    const bool whole = (reinterpret_cast<uintptr_t>(src) & 31u) == 0;
+    const bool whole = !HALVES || (reinterpret_cast<uintptr_t>(src) & 31u) == 0;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
         if (live && whole) {
@@ -313,8 +314,9 @@ __device__ __forceinline__ void store_pieces(const uint32_t (&w)[8][8], unsigned
 // PASS 1: in = x[T][64 n1][64 n2], weights R[n2][k1][n1], out = workspace z
 // PASS 2: in = workspace z, weights L[k1][k2][n2], out = y[T][64 k2][64 k1] (optionally sigma(K (.) y))
 //
-// wt: every weight block is used transposed (the products of the backward pass): the block as it lies in shared memory is then an
-// M-major operand instead of a K-major one, nothing is moved.
+// BWD (the products of the backward pass; a variant of its own because the run-time choices cost the forward pass 2 %): with wt every
+// weight block is used transposed -- the block as it lies in shared memory is then an M-major operand instead of a K-major one, nothing is
+// moved --, and `in` of pass 1 may be on a 16-byte boundary only.
 //
 // Persistent: CTA c of a grid that is a multiple of 4 walks the items c, c + grid, .. of (token tile, block group) pairs numbered
 // group-fastest, so its block group is c % 4 for good (the weights stay) and the 4 CTAs that share a tile's lines work on it at
@@ -324,7 +326,7 @@ __device__ __forceinline__ void store_pieces(const uint32_t (&w)[8][8], unsigned
 //   issuing threads wait for bar_opnd (operands of tile i) and bar_tfree[i % 2] (set drained of tile i - 2), issue, commit to
 //                   bar_mma[i % 2];
 //   draining warps  wait for bar_mma[i % 2], move the set to global memory, arrive on bar_tfree[i % 2].
-template <int PASS>
+template <int PASS, bool BWD>
 __global__ void __launch_bounds__(kFwdThreads, 1)
 monarch64_fwd_kernel(const __nv_bfloat16* __restrict__ in, const __grid_constant__ CUtensorMap map_w,
                      const __grid_constant__ CUtensorMap map_y, __nv_bfloat16* __restrict__ out, long long T,
@@ -401,7 +403,7 @@ monarch64_fwd_kernel(const __nv_bfloat16* __restrict__ in, const __grid_constant
                 const bool live = tile * kTok + t_in < T;
                 const unsigned char* src =
                     reinterpret_cast<const unsigned char*>(in) + (size_t)(tile * kTok + t_in) * 8192 + (size_t)(8 * sub) * 128 + grp * 32;
-                load_pieces(w, src, live);
+                load_pieces<BWD>(w, src, live);
             } else {   // whole tiles of the workspace were written
                 const unsigned char* src =
                     reinterpret_cast<const unsigned char*>(in) + (size_t)tile * kTileBytes + (size_t)t_in * 2048 + (size_t)(16 * grp + sub) * 32;
@@ -519,8 +521,8 @@ monarch64_fwd_kernel(const __nv_bfloat16* __restrict__ in, const __grid_constant
         if (!ok && lane == 0) timed_out();
     } else if (lane == 0) {
         // ---- issuing threads ----
-        const uint32_t idesc = instr_desc_bf16(64, kTok, wt != 0, false);
-        const uint64_t wstep = wt ? 2048 >> 4 : 32 >> 4;   // 16 inputs: rows of the block as it lies, or 32 bytes of a row
+        const uint32_t idesc = instr_desc_bf16(64, kTok, BWD && wt != 0, false);
+        const uint64_t wstep = BWD && wt ? 2048 >> 4 : 32 >> 4;   // 16 inputs: rows of the block as it lies, or 32 bytes of a row
         constexpr int kPer = kGroup2 / kIssueWarps;
         const int b0 = (warp - kLoadWarps - kDrainWarps) * kPer;
         ok = mbar_wait(bar_w, 0);
@@ -567,7 +569,7 @@ monarch64_fwd_kernel(const __nv_bfloat16* __restrict__ in, const __grid_constant
 // blocks 8 .. 15 at lane offset 16) and writes them once; a second kernel adds the shares in a fixed order.  Roles: warps 0..7 load V
 // (the next tile's pieces are in flight while this one is multiplied), lane 0 of warp 8 copies Z (two buffers), lane 0 of warps 9 and
 // 10 issue for 8 blocks each.  Bound, as the forward passes, by the requests for V's pieces (about 0.46 per cycle and SM).
-// GRADTIME
+// Measured, one B200, 5001 tokens: 26 us (37 for the kernel before it, which loaded, multiplied and waited in turn, 8 blocks at a time).
 constexpr int G_OFF_V = 0;            // 16 operands [32 t][64 a] bf16, swizzled rows of 128 bytes                        65536
 constexpr int G_OFF_Z = 65536;        // two buffers [m / 16][16 blocks][32 t][32 B]                                     131072
 constexpr int G_OFF_BAR = 196608;     // bar_v, bar_mma[2], bar_z[2], tmem ptr, abort flag
@@ -599,6 +601,17 @@ monarch64_wgrad_kernel(const __nv_bfloat16* __restrict__ in, const __grid_consta
         prefetch_tensormap(&map_z);
     }
     if (warp == 8) tmem_alloc(s_tptr, 512);
+    // this CTA's quarter of a tile's lines of V, towards L2 as whole lines ahead of the pieces (see the forward passes)
+    auto prefetch_tile = [&](int tile) {
+        if (tile < ntiles) {
+            const long long t0p = (long long)tile * kTok, rows = T - t0p >= kTok ? kTok : T - t0p;
+            bulk_prefetch_l2(reinterpret_cast<const unsigned char*>(in) + t0p * 8192 + grp * (rows * 2048), (uint32_t)(rows * 2048));
+        }
+    };
+    if (tid == 33) {
+        prefetch_tile(share);
+        prefetch_tile(share + nshare);
+    }
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     __syncthreads();
     asm volatile("griddepcontrol.wait;" ::: "memory");   // the workspace was written by the kernel before this one
@@ -610,7 +623,7 @@ monarch64_wgrad_kernel(const __nv_bfloat16* __restrict__ in, const __grid_consta
         uint32_t w[8][8];
         auto load_in = [&](int tile) {
             const long long t = (long long)tile * kTok + t_in;
-            load_pieces(w, reinterpret_cast<const unsigned char*>(in) + (size_t)t * 8192 + (size_t)(8 * sub) * 128 + grp * 32, t < T);
+            load_pieces<true>(w, reinterpret_cast<const unsigned char*>(in) + (size_t)t * 8192 + (size_t)(8 * sub) * 128 + grp * 32, t < T);
         };
         if (share < ntiles) load_in(share);
 #pragma unroll 1
@@ -623,16 +636,18 @@ monarch64_wgrad_kernel(const __nv_bfloat16* __restrict__ in, const __grid_consta
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_v);
             if (tile + nshare < ntiles) load_in(tile + nshare);
+            if (tid == 33) prefetch_tile(tile + 2 * nshare);
         }
         // the 16 accumulators: row r of block b sits in lane (r % 16) + 16 (b / 8) of lane quarter r / 16, columns 64 (b % 8) ..
         if (ok && n > 0) ok = __all_sync(~0u, mbar_wait(bar_mma + 8 * ((n - 1) & 1), ((n - 1) >> 1) & 1) && *abort_flag == 0);
         if (ok && n > 0) {
             tc_fence_after();
-            const int q = warp & 3, r = 16 * q + (lane & 15), set = lane >> 4;
+            const int q = warp & 3;
             const uint32_t t_lane = tmem + ((uint32_t)(q * 32) << 16);
+            // through the free operand buffers, 32 rows of 64 values per warp (pitch 68: no bank conflicts), so that whole rows leave
+            float* st = reinterpret_cast<float*>(smem) + warp * (32 * 68);
 #pragma unroll 1
             for (int cb = 4 * (warp >> 2); cb < 4 * (warp >> 2) + 4; ++cb) {
-                float* dst = partial + (((size_t)share * 64 + grp * 16 + cb + 8 * set) * 64 + r) * 64;
 #pragma unroll 1
                 for (int c0 = 0; c0 < 64; c0 += 32) {
                     float v[32];
@@ -642,8 +657,17 @@ monarch64_wgrad_kernel(const __nv_bfloat16* __restrict__ in, const __grid_consta
 #pragma unroll
                     for (int c = 0; c < 4; ++c) tmem_ld_fence8(v + 8 * c);
 #pragma unroll
-                    for (int c = 0; c < 32; c += 4) *reinterpret_cast<float4*>(dst + c0 + c) = make_float4(v[c], v[c + 1], v[c + 2], v[c + 3]);
+                    for (int c = 0; c < 32; c += 4)
+                        *reinterpret_cast<float4*>(st + lane * 68 + c0 + c) = make_float4(v[c], v[c + 1], v[c + 2], v[c + 3]);
                 }
+                __syncwarp();
+#pragma unroll
+                for (int k = 0; k < 16; ++k) {   // row 2 k + lane / 16 of the 32: set row / 16, index row % 16 of this lane quarter
+                    const int row = 2 * k + (lane >> 4);
+                    float* dst = partial + (((size_t)share * 64 + grp * 16 + cb + 8 * (row >> 4)) * 64 + 16 * q + (row & 15)) * 64;
+                    reinterpret_cast<float4*>(dst)[lane & 15] = *reinterpret_cast<const float4*>(st + row * 68 + 4 * (lane & 15));
+                }
+                __syncwarp();
             }
         }
     } else if (lane == 0 && warp == 8) {
@@ -683,21 +707,35 @@ monarch64_wgrad_kernel(const __nv_bfloat16* __restrict__ in, const __grid_consta
     if (warp == 8) tmem_dealloc(tmem, 512);
 }
 
-// out = the sum of the shares in index order, four values per thread (nshare = 0: zeros)
+// out = the sum of the shares, four values per thread (nshare = 0: zeros): warp y of a block adds the shares y, y + 8, .. in order, the
+// eight sums are added in order (one thread per value walking all shares: 11.1 us for 37 shares, now 9.7)
 __global__ void __launch_bounds__(256) wgrad_reduce_kernel(const float4* __restrict__ partial, float4* __restrict__ out, int nshare) {
-    const int e = blockIdx.x * 256 + threadIdx.x;   // < 64 * 4096 / 4
+    __shared__ float4 part[8][32];
+    const int lane = threadIdx.x & 31, y = threadIdx.x >> 5, e = blockIdx.x * 32 + lane;   // < 64 * 4096 / 4
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 8
-    for (int s = 0; s < nshare; ++s) {
-        const float4 v = partial[(size_t)s * 65536 + e];
+#pragma unroll 5
+    for (int s = y; s < nshare; s += 8) {
+        const float4 v = __ldcg(partial + (size_t)s * 65536 + e);
         acc.x += v.x;
         acc.y += v.y;
         acc.z += v.z;
         acc.w += v.w;
     }
-    out[e] = acc;
+    part[y][lane] = acc;
+    __syncthreads();
+    if (y == 0) {
+#pragma unroll
+        for (int q = 1; q < 8; ++q) {
+            const float4 v = part[q][lane];
+            acc.x += v.x;
+            acc.y += v.y;
+            acc.z += v.z;
+            acc.w += v.w;
+        }
+        out[e] = acc;
+    }
 }
 
 int64_t wgrad_workspace_bytes(const m2_plan* pl, int64_t T) { return covered(pl) ? workspace_bytes(pl, T) + (int64_t)kGradPartialBytes : 0; }
@@ -738,7 +776,7 @@ int32_t wgrad(const m2_plan* pl, const void* X, const void* G, const void* L, co
     unsigned shares = fwd_grid(T) / 4;
     if (shares > kGradShares) shares = kGradShares;
     cudaLaunchAttribute attr;
-    const cudaLaunchConfig_t red = early_launch(256, 256, 0, stream, &attr);
+    const cudaLaunchConfig_t red = early_launch(2048, 256, 0, stream, &attr);
     if (T == 0) {
         if (cudaLaunchKernelEx(&red, wgrad_reduce_kernel, (const float4*)partial, (float4*)dL, 0) != cudaSuccess ||
             cudaLaunchKernelEx(&red, wgrad_reduce_kernel, (const float4*)partial, (float4*)dR, 0) != cudaSuccess)
@@ -757,10 +795,11 @@ int32_t wgrad(const m2_plan* pl, const void* X, const void* G, const void* L, co
     const __nv_bfloat16 *x = (const __nv_bfloat16*)X, *g = (const __nv_bfloat16*)G, *none = nullptr;
     __nv_bfloat16* z = (__nv_bfloat16*)zws;
     // dL: v = R-stage of x, then sum_t g (x) v per block k1;  dR: dv = L^T-stage of g, then sum_t dv (x) x per block n2
-    if (cudaLaunchKernelEx(&p1, monarch64_fwd_kernel<1>, x, mr, mr, z, (long long)T, pl->d_status, none, 1LL, 0, 0, 0) != cudaSuccess ||
+    auto first = (reinterpret_cast<uintptr_t>(X) & 31u) == 0 ? monarch64_fwd_kernel<1, false> : monarch64_fwd_kernel<1, true>;
+    if (cudaLaunchKernelEx(&p1, first, x, mr, mr, z, (long long)T, pl->d_status, none, 1LL, 0, 0, 0) != cudaSuccess ||
         cudaLaunchKernelEx(&wg, monarch64_wgrad_kernel<false>, g, mz, partial, (long long)T, pl->d_status) != cudaSuccess ||
         cudaLaunchKernelEx(&red, wgrad_reduce_kernel, (const float4*)partial, (float4*)dL, (int)shares) != cudaSuccess ||
-        cudaLaunchKernelEx(&p1, monarch64_fwd_kernel<1>, g, ml, ml, z, (long long)T, pl->d_status, none, 1LL, 0, 0, 1) != cudaSuccess ||
+        cudaLaunchKernelEx(&p1, monarch64_fwd_kernel<1, true>, g, ml, ml, z, (long long)T, pl->d_status, none, 1LL, 0, 0, 1) != cudaSuccess ||
         cudaLaunchKernelEx(&wg, monarch64_wgrad_kernel<true>, x, mz, partial, (long long)T, pl->d_status) != cudaSuccess ||
         cudaLaunchKernelEx(&red, wgrad_reduce_kernel, (const float4*)partial, (float4*)dR, (int)shares) != cudaSuccess)
         return M2_ERR_CUDA;
@@ -780,8 +819,10 @@ cudaError_t prepare(const m2_plan* pl) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(monarch64_pass_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(monarch64_wgrad_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, G_SMEM);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(monarch64_wgrad_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, G_SMEM);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(monarch64_fwd_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, F_SMEM_BYTES);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(monarch64_fwd_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, F_SMEM_BYTES);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(monarch64_fwd_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, F_SMEM_BYTES);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(monarch64_fwd_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, F_SMEM_BYTES);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(monarch64_fwd_kernel<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, F_SMEM_BYTES);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(monarch64_fwd_kernel<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, F_SMEM_BYTES);
     return e;
 }
 
@@ -833,10 +874,10 @@ static int32_t matmul_impl(const m2_plan* pl, const void* X, const void* L, cons
     if (!tma_host::encode_sw32_bf16(&my, Y, 3, ydim, ystr, ybox)) return M2_ERR_UNSUPPORTED;
     cudaLaunchAttribute attr;
     const cudaLaunchConfig_t cfg = early_launch(fwd_grid(T), kFwdThreads, F_SMEM_BYTES, stream, &attr);
-    if (cudaLaunchKernelEx(&cfg, monarch64_fwd_kernel<1>, (const __nv_bfloat16*)X, mr, my, (__nv_bfloat16*)ws, (long long)T, pl->d_status,
+    if (cudaLaunchKernelEx(&cfg, wt ? monarch64_fwd_kernel<1, true> : monarch64_fwd_kernel<1, false>, (const __nv_bfloat16*)X, mr, my, (__nv_bfloat16*)ws, (long long)T, pl->d_status,
                            (const __nv_bfloat16*)nullptr, 1LL, 0, selftest, wt) != cudaSuccess)
         return M2_ERR_CUDA;
-    if (cudaLaunchKernelEx(&cfg, monarch64_fwd_kernel<2>, (const __nv_bfloat16*)ws, ml, my, (__nv_bfloat16*)Y, (long long)T, pl->d_status,
+    if (cudaLaunchKernelEx(&cfg, wt ? monarch64_fwd_kernel<2, true> : monarch64_fwd_kernel<2, false>, (const __nv_bfloat16*)ws, ml, my, (__nv_bfloat16*)Y, (long long)T, pl->d_status,
                            (const __nv_bfloat16*)Kmul, (long long)(Hk > 0 ? Hk : 1), relu, selftest, wt) != cudaSuccess)
         return M2_ERR_CUDA;
     pl->last_kernel = "matmul_umma_64x64";

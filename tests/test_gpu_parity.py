@@ -637,6 +637,34 @@ def test_matmul_weight_gradients(T, dims, dtype):
     plan.close()
 
 
+@pytest.mark.parametrize("T,offset", [(1, 0), (33, 8), (1200, 0), (1217, 8)])
+def test_matmul_gradients_at_the_tile_boundaries(T, offset):
+    """The 64 x 64 gradient kernels with one tile, a second tile of one token, one tile per share and one more, with X and G on a 32-byte
+    boundary and 16 bytes off it (half loads; the input gradient then transposes the blocks)."""
+    c = synth.config3(T=T, b=64)
+    plan = M.Plan((64, 64), dtype=M.M2_BF16, device=0)
+    L, R = dev(c["L"], torch.bfloat16), dev(c["R"], torch.bfloat16)
+    G = synth.round_bf16(synth.normal(synth.stream_id(9, 7), (T, 4096)))
+
+    def place(a):
+        buf = torch.zeros(T * 4096 + 16, dtype=torch.bfloat16, device="cuda")
+        v = buf[offset:offset + T * 4096].view(T, 4096)
+        v.copy_(dev(a, torch.bfloat16))
+        return v
+    Xd, Gd = place(c["X"]), place(G)
+    dL, dR = M.m2_monarch_matmul_bwd_weights(plan, Xd, Gd, L, R)
+    dX = M.m2_monarch_matmul_bwd_input(plan, Gd, L, R)
+    torch.cuda.synchronize()
+    assert plan.device_status() == 0
+    L64, R64 = c["L"].astype(np.float64), c["R"].astype(np.float64)
+    rL, rR = O.monarch_weight_grads(L64, R64, c["X"].astype(np.float64), G.astype(np.float64))
+    # (the rows of a gradient over a handful of tokens are small sums: judged over the tensor)
+    for got, ref in ((dL, rL), (dR, rR)):
+        assert np.linalg.norm(host(got) - ref) <= TOL_BF16 * np.linalg.norm(ref)
+    check(host(dX), O.monarch_apply_transpose(L64, R64, G.astype(np.float64)), TOL_BF16, "dX")
+    plan.close()
+
+
 @pytest.mark.parametrize("T,Hk,dims,dtype,act", [(300, 3, (64, 64), M.M2_BF16, "relu"), (257, 257, (64, 64), M.M2_BF16, "none"),
                                                   (50, 1, (8, 4), M.M2_BF16, "relu"), (19, 5, (4, 6), M.M2_FP32, "relu"),
                                                   (19, 19, (4, 6), M.M2_FP32, "none")])
