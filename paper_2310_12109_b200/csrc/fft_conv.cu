@@ -4,7 +4,7 @@
 // has the transforms.
 //
 // What bounds it: shared-memory wavefronts (64 KB each way per digit exchange of a 4096-point row) and packed FP32 issue, about equal;
-// with 126 registers four blocks of 128 threads share an SM.  bf16 x[8][768][2000], N = 4096, one B200: 49 us (0.2 of the roof: its
+// with 126 registers four blocks of 128 threads share an SM.  bf16 x[8][768][2000], N = 4096, one B200: 47 us (0.2 of the roof: its
 // bytes take 9.8 us; 59 % of the load/store data pipe, DRAM 11 %), against 6034 us for the kernel before it, which contracted each 64-wide
 // digit as a dense product in shared memory with a sincos per element.  fp32 x[1][4][256]: 18.4 -> 11.2 us per call, all of it launch
 // and host path.
@@ -22,6 +22,7 @@ __global__ void __launch_bounds__(C::THREADS, min_blocks<C>())
     fft_conv_kernel(const IO* __restrict__ x, const float4* __restrict__ kf, IO* __restrict__ y, const float4* __restrict__ tab, int B, int H,
                     int n, long long npairs, int kf_group) {
     extern __shared__ __align__(16) float smem[];
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int r = threadIdx.x / C::TP, t = threadIdx.x % C::TP;
     const long long pair = (long long)blockIdx.x * C::ROWS + r;
     const int per_h = (B + 1) / 2;
@@ -33,6 +34,7 @@ __global__ void __launch_bounds__(C::THREADS, min_blocks<C>())
     const long long oa = ((long long)b * H + h) * n, ob = oa + (long long)H * n;
     const bool has_b = live && b + 1 < B;
     u64 re[16], im[16];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     load_row<C, IO, HALF>(re, x + oa, t, n, vec, live);
     load_row<C, IO, HALF>(im, x + ob, t, n, vec, has_b);
     forward<C, HALF>(re, im, sr, si, tab, t, r);
@@ -145,12 +147,11 @@ cudaError_t conv(const m2_plan* pl, const void* x, const void* kf, void* y, int6
         const unsigned grid = (unsigned)((npairs + C::ROWS - 1) / C::ROWS);
         auto go = [&](auto z, auto half) {
             using IO = decltype(z);
-            fft_conv_kernel<C, IO, decltype(half)::v != 0><<<grid, C::THREADS, conv_smem<C>(), stream>>>(
-                (const IO*)x, (const float4*)kf, (IO*)y, pl->d_fft, (int)B, (int)H, (int)n, npairs, kf_group);
+            return launch_early(fft_conv_kernel<C, IO, decltype(half)::v != 0>, grid, C::THREADS, conv_smem<C>(), stream, (const IO*)x,
+                                (const float4*)kf, (IO*)y, (const float4*)pl->d_fft, (int)B, (int)H, (int)n, npairs, kf_group);
         };
-        if (pl->dtype == M2_BF16) causal ? go(__nv_bfloat16(), Ic<1>{}) : go(__nv_bfloat16(), Ic<0>{});
-        else causal ? go(float(), Ic<1>{}) : go(float(), Ic<0>{});
-        return cudaGetLastError();
+        if (pl->dtype == M2_BF16) return causal ? go(__nv_bfloat16(), Ic<1>{}) : go(__nv_bfloat16(), Ic<0>{});
+        return causal ? go(float(), Ic<1>{}) : go(float(), Ic<0>{});
     });
 }
 

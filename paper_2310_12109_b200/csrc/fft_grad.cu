@@ -10,12 +10,14 @@ __global__ void __launch_bounds__(C::THREADS, min_blocks<C>())
     fft_spectrum_kernel(const float* __restrict__ k, float4* __restrict__ kf, float4* __restrict__ kfu, float* __restrict__ kt,
                         float sgn, const float4* __restrict__ tab, int H, int n) {
     extern __shared__ __align__(16) float smem[];
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int r = threadIdx.x / C::TP, t = threadIdx.x % C::TP;
     const long long h = (long long)blockIdx.x * C::ROWS + r;
     const bool live = h < H;
     float* sr = smem + r * C::ROWF + (r & 1) * C::PAR;
     float* si = sr + C::SMEM_FLOATS;
     u64 re[16], im[16];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     // rows of k are only as aligned as n floats make them; a pair needs 8 bytes
     load_row<C, float, HALF>(re, k + h * n, t, n, (n & 1) == 0 && (reinterpret_cast<uintptr_t>(k) & 7) == 0, live);
     unroll<16>([&](auto j) { im[j.v] = 0ull; });
@@ -97,6 +99,7 @@ __global__ void __launch_bounds__(C::THREADS, wgrad_blocks<C>())
     fft_wgrad_kernel(const IO* __restrict__ x, const IO* __restrict__ g, float* __restrict__ dk, const float4* __restrict__ tab, int B, int H,
                      int n, int share) {
     extern __shared__ __align__(16) float smem[];
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int r = threadIdx.x / C::TP, t = threadIdx.x % C::TP;
     const long long h = (long long)blockIdx.x * (C::ROWS / share) + r / share;
     const bool live = h < H, vec = (n & 1) == 0;
@@ -106,6 +109,7 @@ __global__ void __launch_bounds__(C::THREADS, wgrad_blocks<C>())
     float4* zs = zall + threadIdx.x;
     u64 re[16], im[16], ar[16], ai[16];
     unroll<16>([&](auto s) { ar[s.v] = ai[s.v] = 0ull; });
+    asm volatile("griddepcontrol.wait;" ::: "memory");
 #pragma unroll 1
     for (int b0 = 0; b0 < B; b0 += 2 * share) {   // (every row of threads takes every step: the barriers may span several rows)
         const int b = b0 + 2 * (r % share);
@@ -186,11 +190,11 @@ cudaError_t spectrum(const m2_plan* pl, const float* k, int64_t H, int64_t n, vo
         using C = decltype(cfg);
         const unsigned grid = (unsigned)((H + C::ROWS - 1) / C::ROWS);
         const float sgn = pl->sign >= 0 ? 1.0f : -1.0f;
-        if (2 * n <= C::N)
-            fft_spectrum_kernel<C, true><<<grid, C::THREADS, conv_smem<C>(), stream>>>(k, (float4*)kf, (float4*)kfu, kt, sgn, pl->d_fft, (int)H, (int)n);
-        else
-            fft_spectrum_kernel<C, false><<<grid, C::THREADS, conv_smem<C>(), stream>>>(k, (float4*)kf, (float4*)kfu, kt, sgn, pl->d_fft, (int)H, (int)n);
-        return cudaGetLastError();
+        auto go = [&](auto half) {
+            return launch_early(fft_spectrum_kernel<C, decltype(half)::v != 0>, grid, C::THREADS, conv_smem<C>(), stream, k, (float4*)kf,
+                                (float4*)kfu, kt, sgn, (const float4*)pl->d_fft, (int)H, (int)n);
+        };
+        return 2 * n <= C::N ? go(Ic<1>{}) : go(Ic<0>{});
     });
 }
 
@@ -221,12 +225,11 @@ cudaError_t wgrad(const m2_plan* pl, const void* x, const void* g, float* dk, in
             const unsigned grid = (unsigned)((H + per_block - 1) / per_block);
             auto go = [&](auto z, auto half) {
                 using IO = decltype(z);
-                fft_wgrad_kernel<C, IO, decltype(half)::v != 0><<<grid, C::THREADS, wgrad_smem<C>(), stream>>>(
-                    (const IO*)x, (const IO*)g, dk, pl->d_fft, (int)B, (int)H, (int)n, share);
+                return launch_early(fft_wgrad_kernel<C, IO, decltype(half)::v != 0>, grid, C::THREADS, wgrad_smem<C>(), stream, (const IO*)x,
+                                    (const IO*)g, dk, (const float4*)pl->d_fft, (int)B, (int)H, (int)n, share);
             };
-            if (pl->dtype == M2_BF16) causal ? go(__nv_bfloat16(), Ic<1>{}) : go(__nv_bfloat16(), Ic<0>{});
-            else causal ? go(float(), Ic<1>{}) : go(float(), Ic<0>{});
-            return cudaGetLastError();
+            if (pl->dtype == M2_BF16) return causal ? go(__nv_bfloat16(), Ic<1>{}) : go(__nv_bfloat16(), Ic<0>{});
+            return causal ? go(float(), Ic<1>{}) : go(float(), Ic<0>{});
         }
     });
 }

@@ -743,6 +743,7 @@ cudaError_t launch_gate_transpose(const void* x, const void* vT, const float* w,
 __global__ void spectrum_conj_kernel(const float4* __restrict__ in, float4* __restrict__ out, long long pair_quads, long long total, int N,
                                      long long time_pairs) {
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    pdl_prologue();
     if (i < total) {
         const float4 v = in[i];
         out[i] = i < pair_quads ? make_float4(v.x, -v.y, v.z, -v.w) : make_float4(v.x, v.y, -v.z, -v.w);
@@ -763,9 +764,8 @@ cudaError_t launch_spectrum_conj(const void* in, void* out, long long plan_order
     // plan_order_values complex values (even); private_values complex values stored as (re, re', im, im') quads; time_rows rows of N
     const long long pair_quads = plan_order_values / 2, total = pair_quads + private_values / 2, time_pairs = time_rows * (N / 2 + 1);
     if (total == 0) return cudaSuccess;
-    spectrum_conj_kernel<<<(unsigned)((total + time_pairs + 255) / 256), 256, 0, st>>>((const float4*)in, (float4*)out, pair_quads, total, N,
-                                                                                      time_pairs);
-    return cudaGetLastError();
+    return launch_pdl(spectrum_conj_kernel, dim3((unsigned)((total + time_pairs + 255) / 256)), dim3(256), st, (const float4*)in, (float4*)out,
+                      pair_quads, total, N, time_pairs);
 }
 
 long long conv_wgrad_scratch_bytes(long long N, long long H) {
