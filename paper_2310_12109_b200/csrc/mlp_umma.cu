@@ -5,18 +5,21 @@
 //
 // An item = 128 tokens x one block.  The hidden dimension is walked in 6 chunks of 128:
 //   S1(c)  D1[c % 2][128 tok][128 hid] = Z[128][192] * W_up[j][chunk c]^T        12 UMMAs (M128 N128 K16)
-//   E1(c)  TMEM -> registers -> GELU -> bf16 -> back into TMEM, over the first 64 columns of the D1 buffer it came from
+//   E1(c)  TMEM -> registers -> GELU -> bf16 -> back into TMEM, over columns of the D1 buffer that the same warp has read
 //          (two values per column): G[128 tok][128 hid] is the A operand of S2 and never touches shared memory
 //   S2(c)  D2[128 tok][192 out] += G * W_down[j][:, chunk c]^T                     8 UMMAs (M128 N192 K16, A from TMEM)
 // and at the end of an item D2 -> bf16 -> staging -> TMA stores.
 //
 // Persistent: one CTA per SM walks the items c, c + grid, ..; all barriers count chunks across items, so the weight
-// chunks, the activations and the first UMMAs of the next item are under way while the GELU warps finish and store the
-// current one (a CTA per item spent a third of its time launching, setting up and draining).  Warp roles: warp 0 feeds
-// the activation tiles and the weight chunks by TMA (W_up chunks double-buffered), warp 1 issues the UMMAs and runs
-// S1(c + 1) ahead of E1(c) (two D1 buffers), warps 2..17 are the GELU warps (lane quarter = warp % 4, 32 of the 128
-// chunk columns each).  Shared-memory operands are K-major with the 128-byte swizzle, written by TMA.  Every wait is
-// bounded; a role that gave up keeps arriving at the GELU warps' block barriers so that nobody is left behind.
+// chunks, the activations and the first UMMAs of the next item are under way while the current one finishes.  Warp roles: warp 0
+// feeds the activation tiles and the weight chunks by TMA (W_up chunks double-buffered), warp 1 issues the UMMAs and runs
+// S1(c + 1) ahead of E1(c) (two D1 buffers), warps 2..17 are the GELU warps, warps 18..21 store the items' results.
+// What bounds it: the GELU arithmetic (13 packed operations a pair: 1.7 K cycles of the FMA pipe a chunk) and the issue of the
+// UMMAs (2.1 K cycles a chunk).  The GELU warps are two groups of eight that take the chunks in turn, each with its own D1
+// buffer, so that the latencies of one (accumulator, tensor-memory loads and stores, hand-over) pass under the arithmetic of the
+// other; no GELU warp takes part in the output.  All 16 warps on one chunk at a time, with a barrier between reading D1 and
+// writing G and the output as a phase of their own, took 58 us for 16384 tokens x 4 blocks; this form takes 52 us.
+// Shared-memory operands are K-major with the 128-byte swizzle, written by TMA.  Every wait is bounded.
 #include <cuda.h>
 
 #include <atomic>
@@ -31,16 +34,17 @@ namespace m2mlp {
 using namespace sm100;
 
 constexpr int kCI = 192, kHID = 768, kCO = 192, kChunk = 128, kChunks = kHID / kChunk, kTileT = 128;
-constexpr int kEpiWarps = 16, kThreads = 64 + 32 * kEpiWarps;
+constexpr int kGrpWarps = 8, kDrainWarps = 4, kThreads = 64 + 32 * (2 * kGrpWarps + kDrainWarps);
+static_assert(kChunks % 2 == 0, "a chunk's parity is its GELU group");
 constexpr int OFF_Z = 0;                    // 3 K-blocks [128][64] bf16                               49152
 constexpr int OFF_W1 = 49152;               // 2 buffers x 3 K-blocks [128 hid][64]                   98304
 constexpr int OFF_W2 = 147456;              // 2 K-blocks [192 out][64]                               49152
-constexpr int OFF_ST = 196608;              // output staging: 2 buffers [128 tok][64]                32768
+constexpr int OFF_ST = 196608;              // output staging: per drain warp 2 buffers [32 tok][64]   32768
 constexpr int OFF_BAR = 229376;
 constexpr int SMEM_BYTES = OFF_BAR + 192;
 static_assert(SMEM_BYTES <= 232448, "shared memory budget");
 // mbarriers (8 bytes each) from OFF_BAR
-enum { B_Z = 0, B_W1F = 1, B_W1E = 3, B_W2F = 5, B_W2E = 6, B_D1F = 7, B_D1E = 9, B_GF = 11, B_ZE = 12, B_D2F = 13, B_D2E = 14, B_COUNT = 15 };
+enum { B_Z = 0, B_W1F = 1, B_W1E = 3, B_W2F = 5, B_W2E = 6, B_D1F = 7, B_GF = 9, B_ZE = 11, B_D2F = 12, B_D2E = 13, B_COUNT = 14 };
 
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint32_t bar) {
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
@@ -112,13 +116,12 @@ mlp_umma_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant
             mbar_init(bar(B_W1F + i), 1);
             mbar_init(bar(B_W1E + i), 1);
             mbar_init(bar(B_D1F + i), 1);
-            mbar_init(bar(B_D1E + i), kEpiWarps);   // one arrival per GELU warp
+            mbar_init(bar(B_GF + i), kGrpWarps);   // one arrival per warp of the GELU group
         }
         mbar_init(bar(B_W2F), 1);
         mbar_init(bar(B_W2E), 1);
-        mbar_init(bar(B_GF), kEpiWarps);
         mbar_init(bar(B_D2F), 1);
-        mbar_init(bar(B_D2E), kEpiWarps);
+        mbar_init(bar(B_D2E), kDrainWarps);
         fence_barrier_init();
         prefetch_tensormap(&map_z);
         prefetch_tensormap(&map_w1);
@@ -182,9 +185,9 @@ mlp_umma_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant
             constexpr uint32_t ID1 = instr_desc_bf16(128, 128, ZCF, false), ID2 = instr_desc_bf16(128, 192, false, false);
             auto s1 = [&](int g) {   // D1[g % 2] = Z * W_up chunk g
                 const int b = g & 1;
-                ok = mbar_wait(bar(B_W1F + b), (g >> 1) & 1);
-                if (ok && g >= 2) ok = mbar_wait(bar(B_D1E + b), ((g >> 1) - 1) & 1);   // the GELU warps have read D1[b]
-                if (!ok) return;
+                if (g % kChunks == 0) ok = mbar_wait(bar(B_Z), (g / kChunks) & 1);       // the item's activation tile
+                if (ok) ok = mbar_wait(bar(B_W1F + b), (g >> 1) & 1);
+                if (!ok) return;                                                        // D1[b] is free: S2(g - 2), issued before, reads it last
                 tc_fence_after();
 #pragma unroll 1
                 for (int kb = 0; kb < 3; ++kb)
@@ -198,128 +201,103 @@ mlp_umma_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant
                 umma_commit(bar(B_W1E + b));
                 if (g % kChunks == kChunks - 1) umma_commit(bar(B_ZE));   // the item's last S1: its activation tile is free after it
             };
-            if (total > 0) {
-                ok = mbar_wait(bar(B_Z), 0);
-                if (ok) s1(0);
-            }
+            if (total > 0) s1(0);
             for (int g = 0; g < total && ok; ++g) {
                 const int c = g % kChunks, q = g / kChunks;
-                if (c + 1 < kChunks) s1(g + 1);
+                if (g + 1 < total) s1(g + 1);
                 if (!ok) break;
-                ok = mbar_wait(bar(B_GF), g & 1) && mbar_wait(bar(B_W2F), g & 1);
+                ok = mbar_wait(bar(B_GF + (g & 1)), (g >> 1) & 1) && mbar_wait(bar(B_W2F), g & 1);
                 if (ok && c == 0 && q > 0) ok = mbar_wait(bar(B_D2E), (q - 1) & 1);   // the previous item's D2 has been read
                 if (!ok) break;
                 tc_fence_after();
-                // A = G in tensor memory: the first 64 columns of D1[g % 2], 8 columns per K step of 16
+                // A = G in tensor memory, 8 columns per K step of 16: columns 0..31 (hidden 0..63) and 64..95 (64..127) of D1[g % 2]
 #pragma unroll 1
                 for (int kb = 0; kb < 2; ++kb)
 #pragma unroll
                     for (int s = 0; s < 4; ++s)
-                        umma_f16_ta(D2, D1 + (g & 1) * 128 + (kb * 4 + s) * 8,
+                        umma_f16_ta(D2, D1 + (g & 1) * 128 + kb * 64 + s * 8,
                                     smem_desc_sw128(s_base + OFF_W2 + kb * 24576 + s * 32, 16, 1024), ID2, (c | kb | s) != 0);
                 umma_commit(bar(B_W2E));
-                if (c == kChunks - 1) {
-                    umma_commit(bar(B_D2F));
-                    if (g + 1 < total) {   // the next item's first S1 follows this item's last S2
-                        ok = mbar_wait(bar(B_Z), (q + 1) & 1);
-                        if (ok) s1(g + 1);
-                    }
-                }
+                if (c == kChunks - 1) umma_commit(bar(B_D2F));
             }
         }
-    } else {
-        // ---- GELU warps: lane quarter qq = warp % 4 (a TMEM rule), column slice sl = 32 of the chunk's 128 columns ----
-        const int ew = warp - 2, qq = warp & 3, sl = ew >> 2;
-        const int row = qq * 32 + lane;                                   // token within the tile
-        const uint32_t t_lane = tmem + ((uint32_t)(qq * 32) << 16);
-        const bool storer = ew == 0 && lane == 0;                         // issues the output stores
-        for (int g = 0; g < total; ++g) {
-            const int b = g & 1, c = g % kChunks, q = g / kChunks;
-            if (ok) ok = mbar_wait(bar(B_D1F + b), (g >> 1) & 1);
-            if (ok) {
-                tc_fence_after();
+    } else if (warp < 2 + 2 * kGrpWarps) {
+        // ---- GELU warps: two groups of eight take the chunks in turn, so that one computes while the other's accumulator is on its
+        //      way.  Lane quarter qq = warp % 4 (a TMEM rule), column half sl = 64 of the chunk's 128 columns.  G lies over the
+        //      columns that this warp itself has read: no warp waits for another ----
+        const int ew = warp - 2, grp = ew >> 3, qq = warp & 3, sl = (ew >> 2) & 1;
+        const uint32_t t_half = tmem + ((uint32_t)(qq * 32) << 16) + grp * 128 + sl * 64;
+        for (int g = grp; g < total && ok; g += 2) {
+            ok = mbar_wait(bar(B_D1F + grp), (g >> 1) & 1);
+            if (!ok) break;
+            tc_fence_after();
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
                 float v[32];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) tmem_ld8(t_lane + b * 128 + sl * 32 + 8 * i, v + 8 * i);
+                for (int i = 0; i < 4; ++i) tmem_ld8(t_half + h * 32 + 8 * i, v + 8 * i);
                 tmem_ld_wait();
 #pragma unroll
                 for (int i = 0; i < 4; ++i) tmem_ld_fence8(v + 8 * i);
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bar(B_D1E + b));                  // this warp has read its part of D1[b]
                 uint32_t pk[16];
 #pragma unroll
                 for (int i = 0; i < 16; ++i) pk[i] = gelu2_pack(v[2 * i], v[2 * i + 1]);
-                // G goes back into tensor memory over the first 64 columns of D1[b]: every GELU warp must have read the buffer
-                ok = mbar_wait(bar(B_D1E + b), (g >> 1) & 1);
-                if (ok) {
-                    tc_fence_after();
-                    tmem_st8(t_lane + b * 128 + sl * 16, pk);
-                    tmem_st8(t_lane + b * 128 + sl * 16 + 8, pk + 8);
-                    tmem_st_wait();
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(bar(B_GF));
-                }
+                tmem_st8(t_half + h * 16, pk);
+                tmem_st8(t_half + h * 16 + 8, pk + 8);
             }
-            if (c != kChunks - 1) continue;
-            // ---- output of item q: D2 -> bf16 -> staging -> TMA stores.  The 24 chunks (16 bytes) of a 192-column row
-            //      belong to three K-blocks of 64 columns; K-blocks 0 and 1 are staged in the two 16 KB buffers and sent,
-            //      K-block 2 follows in the first buffer once its store has read it.  The block barriers are passed by
-            //      every GELU warp whatever happened before. ----
-            if (ok) ok = mbar_wait(bar(B_D2F), q & 1);
-            uint4 keep[6];
-            if (ok) {
-                tc_fence_after();
+            tmem_st_wait();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(B_GF + grp));
+        }
+    } else {
+        // ---- output warps, one per lane quarter: D2 -> bf16 -> two staging boxes of the warp's own -> TMA stores, while the GELU
+        //      warps are at the next item.  K-blocks 0 and 1 of the row (64 columns each) go out through the two boxes, K-block 2
+        //      waits in registers, so that D2 is given back early, and follows through the first box ----
+        const int qq = warp & 3;
+        const uint32_t t_d2 = tmem + ((uint32_t)(qq * 32) << 16) + 256, st_off = OFF_ST + qq * 8192;
+        for (int q = 0; q < nq && ok; ++q) {
+            ok = mbar_wait(bar(B_D2F), q & 1);
+            if (!ok) break;
+            tc_fence_after();
+            if (lane == 0) tma_store_wait_read0();                           // the previous item's stores have read the boxes
+            __syncwarp();
+#pragma unroll 1
+            for (int kb = 0; kb < 3; ++kb) {
+                uint32_t pk[32];
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {                                // 48 of the 192 output columns per slice: 6 chunks
-                    float w[24];
+                for (int h = 0; h < 2; ++h) {
+                    float w[32];
 #pragma unroll
-                    for (int i = 0; i < 3; ++i) tmem_ld8(t_lane + 256 + sl * 48 + h * 24 + 8 * i, w + 8 * i);
+                    for (int i = 0; i < 4; ++i) tmem_ld8(t_d2 + kb * 64 + h * 32 + 8 * i, w + 8 * i);
                     tmem_ld_wait();
 #pragma unroll
-                    for (int i = 0; i < 3; ++i) tmem_ld_fence8(w + 8 * i);
+                    for (int i = 0; i < 4; ++i) tmem_ld_fence8(w + 8 * i);
 #pragma unroll
-                    for (int i = 0; i < 3; ++i)
-                        keep[h * 3 + i] = make_uint4(pack_bf16(w[8 * i], w[8 * i + 1]), pack_bf16(w[8 * i + 2], w[8 * i + 3]),
-                                                     pack_bf16(w[8 * i + 4], w[8 * i + 5]), pack_bf16(w[8 * i + 6], w[8 * i + 7]));
+                    for (int i = 0; i < 16; ++i) pk[h * 16 + i] = pack_bf16(w[2 * i], w[2 * i + 1]);
                 }
-                tc_fence_before();
+                if (kb == 2) {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) {
+                        mbar_arrive(bar(B_D2E));                             // D2 may be overwritten by the next item
+                        tma_store_wait_read0();
+                    }
+                    __syncwarp();
+                }
+                const uint32_t box = st_off + (kb & 1) * 4096;
+#pragma unroll
+                for (int kc = 0; kc < 8; ++kc)
+                    *reinterpret_cast<uint4*>(smem + box + sw_off(lane, kc)) = make_uint4(pk[4 * kc], pk[4 * kc + 1], pk[4 * kc + 2], pk[4 * kc + 3]);
+                fence_proxy_async();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(bar(B_D2E));                      // D2 may be overwritten by the next item
-            }
-            if (storer) tma_store_wait_read0();                              // the previous item's stores have read the staging buffers
-            asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory");
-            if (ok) {
-#pragma unroll
-                for (int i = 0; i < 6; ++i) {
-                    const int kc = sl * 6 + i;                               // 16-byte chunk of the 192-column row
-                    if (kc < 16) *reinterpret_cast<uint4*>(smem + OFF_ST + (kc >> 3) * 16384 + sw_off(row, kc & 7)) = keep[i];
+                if (lane == 0) {
+                    tma_store_2d(&map_y, s_base + box, item_j(q) * kCO + kb * 64, item_t0(q) + qq * 32);
+                    tma_store_commit();
                 }
-                fence_proxy_async();
-            }
-            asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory");
-            if (storer && ok) {
-                for (int kb = 0; kb < 2; ++kb) tma_store_2d(&map_y, s_base + OFF_ST + kb * 16384, item_j(q) * kCO + kb * 64, item_t0(q));
-                tma_store_commit();
-                tma_store_wait_read0();
-            }
-            asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory");
-            if (ok) {
-#pragma unroll
-                for (int i = 0; i < 6; ++i) {
-                    const int kc = sl * 6 + i;
-                    if (kc >= 16) *reinterpret_cast<uint4*>(smem + OFF_ST + sw_off(row, kc & 7)) = keep[i];
-                }
-                fence_proxy_async();
-            }
-            asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory");
-            if (storer && ok) {
-                tma_store_2d(&map_y, s_base + OFF_ST, item_j(q) * kCO + 128, item_t0(q));
-                tma_store_commit();
             }
         }
-        if (storer) tma_store_wait_all0();                                   // complete before shared memory goes away
+        if (lane == 0) tma_store_wait_all0();                                // complete before shared memory goes away
     }
     if (!ok) atomicExch(status, (int32_t)M2_ERR_TIMEOUT);
     tc_fence_before();
@@ -354,8 +332,8 @@ int32_t launch(const void* z, const void* Wup, const void* Wdn, void* y, int C, 
     alignas(64) CUtensorMap mz, mw1, mw2, my;
     {   // activations [tokens][C]: box = 64 columns x 128 tokens, 128B swizzle (rows past the end: zero-filled / clipped)
         const cuuint64_t gdim[2] = {(cuuint64_t)C, (cuuint64_t)tokens}, gstr[1] = {(cuuint64_t)C * 2};
-        const cuuint32_t box[2] = {64, (cuuint32_t)kTileT};
-        if (!tma_host::encode_sw128_bf16(&my, y, 2, gdim, gstr, box)) return M2_ERR_UNSUPPORTED;
+        const cuuint32_t box[2] = {64, (cuuint32_t)kTileT}, ybox[2] = {64, 32};
+        if (!tma_host::encode_sw128_bf16(&my, y, 2, gdim, gstr, ybox)) return M2_ERR_UNSUPPORTED;
         if (T == 0) {
             if (!tma_host::encode_sw128_bf16(&mz, z, 2, gdim, gstr, box)) return M2_ERR_UNSUPPORTED;
         } else {   // z[b][c][t]: box = 64 tokens x the block's 192 channels of one batch entry
