@@ -108,7 +108,7 @@ conv512_kernel(const __grid_constant__ CUtensorMap map_x, __nv_bfloat16* __restr
     const int warp = tid >> 5;                // warp within the group = TMEM lane quarter
     // the thread that issues this pipeline's UMMAs and copies; its warp differs from group to group so that
     // the extra work spreads over the SM's four schedulers
-    const bool leader = tid == 32 * (wg & 3);
+    const bool lead_warp = warp == (wg & 3), leader = lead_warp && elect_one();
     const uint32_t s_all = smem_u32(smem_all);
     unsigned char* smem = smem_all + OFF_GROUP + wg * GROUP_BYTES;   // this group's slice
     const uint32_t s_base = s_all + OFF_GROUP + wg * GROUP_BYTES;
@@ -177,7 +177,7 @@ conv512_kernel(const __grid_constant__ CUtensorMap map_x, __nv_bfloat16* __restr
         const int h = u % H;
         const int b0 = (u / H) * kRows;
         // ---- S1 ---------------------------------------------------------------------------------
-        if (leader) {
+        if (lead_warp && elect_one()) {
             ok = mbar_wait(bar_x, ph_x);
             x_pending = false;
             if (ok) {
@@ -238,7 +238,7 @@ conv512_kernel(const __grid_constant__ CUtensorMap map_x, __nv_bfloat16* __restr
             break;
         }
         // ---- S2 ---------------------------------------------------------------------------------
-        if (leader) {
+        if (lead_warp && elect_one()) {
             tc_fence_after();
 #pragma unroll
             for (int hf = 0; hf < 2; ++hf)
@@ -294,7 +294,7 @@ conv512_kernel(const __grid_constant__ CUtensorMap map_x, __nv_bfloat16* __restr
             break;
         }
         // ---- S2' --------------------------------------------------------------------------------
-        if (leader) {
+        if (lead_warp && elect_one()) {
             tc_fence_after();
 #pragma unroll
             for (int hf = 0; hf < 2; ++hf)
@@ -351,7 +351,7 @@ conv512_kernel(const __grid_constant__ CUtensorMap map_x, __nv_bfloat16* __restr
             break;
         }
         // ---- S1' --------------------------------------------------------------------------------
-        if (leader) {
+        if (lead_warp && elect_one()) {
             tc_fence_after();
 #pragma unroll
             for (int s = 0; s < 4; ++s)
@@ -445,9 +445,9 @@ conv512p_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
     const int warp = tid >> 5;                // warp within the group = TMEM lane quarter
     // the thread that issues this pipeline's UMMAs and copies; its warp differs from group to group so that
     // the extra work spreads over the SM's four schedulers
-    const bool leader = tid == 32 * (wg & 3);
+    const bool lead_warp = warp == (wg & 3), leader = lead_warp && elect_one();
     // a second issuing thread, two schedulers further on, takes the second half of the stages that have two independent halves
-    const bool leader2 = tid == 32 * ((wg + 2) & 3);
+    const bool lead_warp2 = warp == ((wg + 2) & 3);
     const uint32_t s_all = smem_u32(smem_all);
     unsigned char* smem = smem_all + P_OFF_GROUP + wg * P_GROUP_BYTES;   // this group's slice
     const uint32_t s_base = s_all + P_OFF_GROUP + wg * P_GROUP_BYTES;
@@ -536,7 +536,7 @@ conv512p_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
         const int h = u % H;
         const int b0 = (u / H) * 2 * kRows;
         // ---- S1 ---------------------------------------------------------------------------------
-        if (leader) {
+        if (lead_warp && elect_one()) {
             ok = mbar_wait(bar_x, ph_x, wlim);
             x_pending = false;
             if (ok) {
@@ -553,7 +553,7 @@ conv512p_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
                 umma_commit(bar_mma);
             }
         }
-        if (leader2) umma_commit(bar_mma);   // (nothing of its own to track in this stage)
+        if (lead_warp2 && elect_one()) umma_commit(bar_mma);   // (nothing of its own to track in this stage)
         ph_x ^= 1;
         // ---- h1: twiddle, A2 ---------------------------------------------------------------------
         ok = ok && mbar_wait(bar_mma, ph_m, wlim);
@@ -601,9 +601,9 @@ conv512p_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
             break;
         }
         // ---- S2 ---------------------------------------------------------------------------------
-        if (leader || leader2) {
+        if ((lead_warp || lead_warp2) && elect_one()) {
             tc_fence_after();
-            const int hf = leader ? 0 : 1;
+            const int hf = lead_warp ? 0 : 1;
 #pragma unroll
             for (int s = 0; s < 2; ++s)
                 umma_f16(tmem + T2 + hf * 32, smem_desc(s_base + P_G_A + hf * 8192 + s * 256, 128, 512),
@@ -654,9 +654,9 @@ conv512p_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
             break;
         }
         // ---- S2' --------------------------------------------------------------------------------
-        if (leader || leader2) {
+        if ((lead_warp || lead_warp2) && elect_one()) {
             tc_fence_after();
-            const int hf = leader ? 0 : 1;
+            const int hf = lead_warp ? 0 : 1;
 #pragma unroll
             for (int s = 0; s < 2; ++s)
                 umma_f16(tmem + T1 + hf * 32, smem_desc(s_base + P_G_A + hf * 8192 + s * 256, 128, 512),
@@ -705,12 +705,12 @@ conv512p_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
             break;
         }
         // ---- S1' --------------------------------------------------------------------------------
-        if (leader || leader2) {
+        if ((lead_warp || lead_warp2) && elect_one()) {
             tc_fence_after();
             // the conjugated F_32 image is the A operand here (M = (re | im) x n1 = 64) and the data the B operand (N = 4 rows x 16 n2),
             // so that a thread of the last hand-off owns whole 32-byte runs of the output; the second half of the rows goes to
             // lanes 16..31 of every lane quarter (an M = 64 accumulator keeps row m in lane m % 16 + 32 (m / 16))
-            const int hf = leader ? 0 : 1;
+            const int hf = lead_warp ? 0 : 1;
 #pragma unroll
             for (int s = 0; s < 4; ++s)
                 umma_f16(tmem + T2 + ((uint32_t)(16 * hf) << 16), smem_desc(s_all + P_OFF_B4 + s * 256, 128, 1024),
@@ -853,7 +853,8 @@ convwgrad512_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
                     const uint4* __restrict__ consts, int B, int H, int n, float sgn, int32_t* __restrict__ status) {
     extern __shared__ __align__(1024) unsigned char smem_all[];
     const int wg = threadIdx.x >> 7, tid = threadIdx.x & 127, warp = tid >> 5;
-    const bool leader = tid == 32 * (wg & 3), leader2 = tid == 32 * ((wg + 2) & 3);   // issue for the x tile and for the g tile
+    // issue for the x tile and for the g tile
+    const bool lead_warp = warp == (wg & 3), lead_warp2 = warp == ((wg + 2) & 3), leader = lead_warp && elect_one();
     const uint32_t s_all = smem_u32(smem_all);
     unsigned char* smem = smem_all + P_OFF_GROUP + wg * W_GROUP_BYTES;
     const uint32_t s_base = s_all + P_OFF_GROUP + wg * W_GROUP_BYTES;
@@ -907,9 +908,9 @@ convwgrad512_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
         const int h = u % H, bg = u / H;
         const int un = u + ustride;
         // ---- S1: one issuing thread per tile ----------------------------------------------------------------
-        if (leader || leader2) {
-            const int off = leader ? WG_X : WG_G, col = leader ? 0 : 64;
-            ok = mbar_wait(leader ? bar_x : bar_g, ph_x);
+        if ((lead_warp || lead_warp2) && elect_one()) {
+            const int off = lead_warp ? WG_X : WG_G, col = lead_warp ? 0 : 64;
+            ok = mbar_wait(lead_warp ? bar_x : bar_g, ph_x);
             if (ok) {
                 tc_fence_after();
 #pragma unroll
@@ -973,9 +974,9 @@ convwgrad512_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
             break;
         }
         // ---- S2: likewise ---------------------------------------------------------------------------------
-        if (leader || leader2) {
+        if ((lead_warp || lead_warp2) && elect_one()) {
             tc_fence_after();
-            const int off = leader ? WG_A : WG_X, col = leader ? 0 : 64;
+            const int off = lead_warp ? WG_A : WG_X, col = lead_warp ? 0 : 64;
 #pragma unroll
             for (int hf = 0; hf < 2; ++hf)
 #pragma unroll

@@ -152,7 +152,7 @@ monarch64_pass_kernel(const __nv_bfloat16* __restrict__ in, const __nv_bfloat16*
     tc_fence_after();
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(smem + OFF_BAR + 16);
 
-    if (tid == 0) {
+    if (tid < 32 && elect_one()) {
         constexpr uint32_t IDESC = instr_desc_bf16(128, 64, false, false);
         bool in_ok = true;
         if (PASS == 2) in_ok = mbar_wait(bar_in, 0);
@@ -519,7 +519,7 @@ monarch64_fwd_kernel(const __nv_bfloat16* __restrict__ in, const __grid_constant
         }
         if (PASS == 2 && lane == 0) tma_store_wait_all0();   // this thread's stores are complete before shared memory goes away
         if (!ok && lane == 0) timed_out();
-    } else if (lane == 0) {
+    } else if (elect_one()) {
         // ---- issuing threads ----
         const uint32_t idesc = instr_desc_bf16(64, kTok, BWD && wt != 0, false);
         const uint64_t wstep = BWD && wt ? 2048 >> 4 : 32 >> 4;   // 16 inputs: rows of the block as it lies, or 32 bytes of a row
@@ -670,16 +670,18 @@ monarch64_wgrad_kernel(const __nv_bfloat16* __restrict__ in, const __grid_consta
                 __syncwarp();
             }
         }
-    } else if (lane == 0 && warp == 8) {
-        for (int tile = share; tile < ntiles && ok && *abort_flag == 0; tile += nshare, ++n) {
-            const uint32_t z = s_base + G_OFF_Z + (n & 1) * 65536, bz = bar_z + 8 * (n & 1);
-            if (n >= 2) ok = mbar_wait(bar_mma + 8 * (n & 1), ((n - 2) >> 1) & 1);   // the buffer's previous tile has been multiplied
-            if (!ok) break;
-            mbar_expect_tx(bz, 65536);
-            for (int c = 0; c < 4; ++c) tma_load_3d(z + c * 16384, &map_z, 0, (tile * 4 + c) * kTok, 16 * grp, bz);
+    } else if (warp == 8) {
+        if (lane == 0) {
+            for (int tile = share; tile < ntiles && ok && *abort_flag == 0; tile += nshare, ++n) {
+                const uint32_t z = s_base + G_OFF_Z + (n & 1) * 65536, bz = bar_z + 8 * (n & 1);
+                if (n >= 2) ok = mbar_wait(bar_mma + 8 * (n & 1), ((n - 2) >> 1) & 1);   // the buffer's previous tile has been multiplied
+                if (!ok) break;
+                mbar_expect_tx(bz, 65536);
+                for (int c = 0; c < 4; ++c) tma_load_3d(z + c * 16384, &map_z, 0, (tile * 4 + c) * kTok, 16 * grp, bz);
+            }
+            for (uint32_t i = n > 2 ? n - 2 : 0; i < n; ++i) mbar_wait(bar_z + 8 * (i & 1), (i >> 1) & 1);   // nothing is left in flight
         }
-        for (uint32_t i = n > 2 ? n - 2 : 0; i < n; ++i) mbar_wait(bar_z + 8 * (i & 1), (i >> 1) & 1);   // nothing is left in flight
-    } else if (lane == 0) {
+    } else if (elect_one()) {
         const uint32_t idesc = instr_desc_bf16(64, 64, true, true);
         const int b0 = (warp - 9) * 8;
         for (int tile = share; tile < ntiles && ok && *abort_flag == 0; tile += nshare, ++n) {
@@ -698,7 +700,7 @@ monarch64_wgrad_kernel(const __nv_bfloat16* __restrict__ in, const __grid_consta
             umma_commit(bar_mma + 8 * (n & 1));
         }
     }
-    if (!ok && lane == 0) {
+    if (!ok) {
         atomicExch(status, (int32_t)M2_ERR_TIMEOUT);
         *abort_flag = 1;
     }
