@@ -14,11 +14,14 @@
 // chunks, the activations and the first UMMAs of the next item are under way while the current one finishes.  Warp roles: warp 0
 // feeds the activation tiles and the weight chunks by TMA (W_up chunks double-buffered), warp 1 issues the UMMAs and runs
 // S1(c + 1) ahead of E1(c) (two D1 buffers), warps 2..17 are the GELU warps, warps 18..21 store the items' results.
-// What bounds it: the GELU arithmetic (13 packed operations a pair: 1.7 K cycles of the FMA pipe a chunk) and the issue of the
-// UMMAs (2.1 K cycles a chunk).  The GELU warps are two groups of eight that take the chunks in turn, each with its own D1
-// buffer, so that the latencies of one (accumulator, tensor-memory loads and stores, hand-over) pass under the arithmetic of the
-// other; no GELU warp takes part in the output.  All 16 warps on one chunk at a time, with a barrier between reading D1 and
-// writing G and the output as a phase of their own, took 58 us for 16384 tokens x 4 blocks; this form takes 52 us.
+// The GELU warps are two groups of eight that take the chunks in turn, each with its own D1 buffer, so that the latencies of one
+// (accumulator, tensor-memory loads and stores, hand-over) pass under the arithmetic of the other; no GELU warp takes part in the
+// output.  G is handed over in two halves, and the issuing thread looks at the next barriers together.
+// What bounds it: the issuing thread, whose UMMAs, waits (~200 cycles each even on a completed barrier) and commits follow one
+// another: 2.4 K cycles a chunk against 1.5 K of tensor work and 1.7 K of GELU arithmetic (clock stamps; leaving out the weight
+// loads does not change the time).  16384 tokens x 4 blocks: 58 us with all 16 warps on one chunk at a time, a barrier between
+// reading D1 and writing G and the output as a phase of their own; 52 with two groups and output warps; 48 with the UMMAs issued
+// from uniform registers; 46 with the two-part hand-over and the joint polling.
 // Shared-memory operands are K-major with the 128-byte swizzle, written by TMA.  Every wait is bounded.
 #include <cuda.h>
 
@@ -44,7 +47,7 @@ constexpr int OFF_BAR = 229376;
 constexpr int SMEM_BYTES = OFF_BAR + 192;
 static_assert(SMEM_BYTES <= 232448, "shared memory budget");
 // mbarriers (8 bytes each) from OFF_BAR
-enum { B_Z = 0, B_W1F = 1, B_W1E = 3, B_W2F = 5, B_W2E = 6, B_D1F = 7, B_GF = 9, B_ZE = 11, B_D2F = 12, B_D2E = 13, B_COUNT = 14 };
+enum { B_Z = 0, B_W1F = 1, B_W1E = 3, B_W2F = 5, B_W2E = 6, B_D1F = 7, B_GF = 9, B_ZE = 11, B_D2F = 12, B_D2E = 13, B_GH = 14, B_COUNT = 16 };
 
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint32_t bar) {
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
@@ -116,6 +119,7 @@ mlp_umma_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant
             mbar_init(bar(B_W1F + i), 1);
             mbar_init(bar(B_W1E + i), 1);
             mbar_init(bar(B_D1F + i), 1);
+            mbar_init(bar(B_GH + i), kGrpWarps);
             mbar_init(bar(B_GF + i), kGrpWarps);   // one arrival per warp of the GELU group
         }
         mbar_init(bar(B_W2F), 1);
@@ -181,15 +185,15 @@ mlp_umma_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant
         }
     } else if (warp == 1) {
         // ---- UMMA issuer ---------------------------------------------------------------------------------------------
-        if (lane == 0) {
+        if (elect_one()) {
             constexpr uint32_t ID1 = instr_desc_bf16(128, 128, ZCF, false), ID2 = instr_desc_bf16(128, 192, false, false);
             auto s1 = [&](int g) {   // D1[g % 2] = Z * W_up chunk g
                 const int b = g & 1;
                 if (g % kChunks == 0) ok = mbar_wait(bar(B_Z), (g / kChunks) & 1);       // the item's activation tile
-                if (ok) ok = mbar_wait(bar(B_W1F + b), (g >> 1) & 1);
+                if (ok && g < 2) ok = mbar_wait(bar(B_W1F + b), 0);
                 if (!ok) return;                                                        // D1[b] is free: S2(g - 2), issued before, reads it last
                 tc_fence_after();
-#pragma unroll 1
+#pragma unroll
                 for (int kb = 0; kb < 3; ++kb)
 #pragma unroll
                     for (int s = 0; s < 4; ++s)
@@ -206,17 +210,32 @@ mlp_umma_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant
                 const int c = g % kChunks, q = g / kChunks;
                 if (g + 1 < total) s1(g + 1);
                 if (!ok) break;
-                ok = mbar_wait(bar(B_GF + (g & 1)), (g >> 1) & 1) && mbar_wait(bar(B_W2F), g & 1);
+                {   // polled together: G of this chunk, its W_down chunk, and the W_up chunk that the next S1 reads
+                    const uint32_t bg = bar(B_GH + (g & 1)), bw = bar(B_W2F), bu = bar(B_W1F + (g & 1));
+                    const uint32_t pg = (g >> 1) & 1;
+                    const bool more = g + 2 < total;
+                    const bool tg = mbar_try_wait(bg, pg), tw = mbar_try_wait(bw, g & 1), tu = !more || mbar_try_wait(bu, pg ^ 1);
+                    ok = (tg || mbar_wait(bg, pg)) && (tw || mbar_wait(bw, g & 1)) && (tu || mbar_wait(bu, pg ^ 1));
+                }
                 if (ok && c == 0 && q > 0) ok = mbar_wait(bar(B_D2E), (q - 1) & 1);   // the previous item's D2 has been read
                 if (!ok) break;
                 tc_fence_after();
                 // A = G in tensor memory, 8 columns per K step of 16: columns 0..31 (hidden 0..63) and 64..95 (64..127) of D1[g % 2]
-#pragma unroll 1
-                for (int kb = 0; kb < 2; ++kb)
 #pragma unroll
-                    for (int s = 0; s < 4; ++s)
-                        umma_f16_ta(D2, D1 + (g & 1) * 128 + kb * 64 + s * 8,
-                                    smem_desc_sw128(s_base + OFF_W2 + kb * 24576 + s * 32, 16, 1024), ID2, (c | kb | s) != 0);
+                for (int h = 0; h < 2; ++h) {
+                    if (h == 1) {
+                        ok = mbar_wait(bar(B_GF + (g & 1)), (g >> 1) & 1);
+                        if (!ok) break;
+                        tc_fence_after();
+                    }
+#pragma unroll
+                    for (int kb = 0; kb < 2; ++kb)
+#pragma unroll
+                        for (int s = 2 * h; s < 2 * h + 2; ++s)
+                            umma_f16_ta(D2, D1 + (g & 1) * 128 + kb * 64 + s * 8,
+                                        smem_desc_sw128(s_base + OFF_W2 + kb * 24576 + s * 32, 16, 1024), ID2, c != 0 || (h | kb | (s & 1)) != 0);
+                }
+                if (!ok) break;
                 umma_commit(bar(B_W2E));
                 if (c == kChunks - 1) umma_commit(bar(B_D2F));
             }
@@ -244,11 +263,11 @@ mlp_umma_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant
                 for (int i = 0; i < 16; ++i) pk[i] = gelu2_pack(v[2 * i], v[2 * i + 1]);
                 tmem_st8(t_half + h * 16, pk);
                 tmem_st8(t_half + h * 16 + 8, pk + 8);
+                tmem_st_wait();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar((h == 0 ? B_GH : B_GF) + grp));
             }
-            tmem_st_wait();
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar(B_GF + grp));
         }
     } else {
         // ---- output warps, one per lane quarter: D2 -> bf16 -> two staging boxes of the warp's own -> TMA stores, while the GELU
