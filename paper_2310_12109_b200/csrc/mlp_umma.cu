@@ -17,9 +17,10 @@
 // The GELU warps are two groups of eight that take the chunks in turn, each with its own D1 buffer, so that the latencies of one
 // (accumulator, tensor-memory loads and stores, hand-over) pass under the arithmetic of the other; no GELU warp takes part in the
 // output.  G is handed over in two halves, and the issuing thread looks at the next barriers together.
-// What bounds it: the issuing thread, whose UMMAs, waits (~200 cycles each even on a completed barrier) and commits follow one
-// another: 2.4 K cycles a chunk against 1.5 K of tensor work and 1.7 K of GELU arithmetic (clock stamps; leaving out the weight
-// loads does not change the time).  16384 tokens x 4 blocks: 58 us with all 16 warps on one chunk at a time, a barrier between
+// What bounds it: the UMMAs and what separates them.  S1 reads 8 KB of operands from shared memory per 64 cycles of tensor work, all
+// of its bandwidth, and takes ~85 cycles an instruction; with the waits of the issuing thread (~200 cycles each even on a completed
+// barrier) a chunk takes 2.4 K cycles against 1.5 K of tensor work and 1.7 K of GELU arithmetic (clock stamps; neither leaving out the
+// weight loads nor one commit less a chunk changes the time).  16384 tokens x 4 blocks: 58 us with all 16 warps on one chunk at a time, a barrier between
 // reading D1 and writing G and the output as a phase of their own; 52 with two groups and output warps; 48 with the UMMAs issued
 // from uniform registers; 46 with the two-part hand-over and the joint polling.
 // Shared-memory operands are K-major with the 128-byte swizzle, written by TMA.  Every wait is bounded.
