@@ -460,6 +460,18 @@ def test_block_other_shapes(T, C, nblk, expand, dims, kernel):
     check(y.reshape(-1, C), yr.reshape(-1, C), TOL_BF16, "block y")
 
 
+@pytest.mark.parametrize("B,T,C,nblk,dims", [(1, 64, 192, 1, (8, 8)), (3, 64, 192, 1, (8, 8)), (161, 64, 384, 2, (8, 8)), (5, 36, 192, 1, (6, 6))])
+def test_tensor_core_mlp_on_ragged_token_counts(B, T, C, nblk, dims):
+    """Tensor-core MLP on channel-last activations: less than one tile of 128 tokens, a last tile whose store boxes of 32 tokens lie
+    partly or wholly past the end, one item per CTA and more than one."""
+    c = synth.config5(B=B, T=T, C=C, nblk=nblk)
+    c["dims"] = dims
+    y, z = run_block(c, "block_conv_generic_mlp_umma")
+    yr, zr = block_ref(c)
+    check(z.reshape(-1, C), zr.reshape(-1, C), TOL_BF16, f"block z {B}x{T}x{C}")
+    check(y.reshape(-1, C), yr.reshape(-1, C), TOL_BF16, f"block y {B}x{T}x{C}")
+
+
 @pytest.mark.parametrize("B", [1, 9, 17])
 def test_config5_ragged_batches(B):
     """Batch sizes that leave the last 16-row unit of the gated convolution partly empty (rows past B are never read or written)."""
