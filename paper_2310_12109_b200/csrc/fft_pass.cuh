@@ -66,11 +66,17 @@ __device__ __forceinline__ void load_row(u64* v, const IO* row, int t, int n, bo
     } else {
         raw w[32];
         constexpr int L = C::R1 == 16 ? 2 * JN : JN;
-        unroll<L>([&](auto j) {
-            const int i = C::R1 == 16 ? (j.v / 2) * STEP + 2 * t + (j.v & 1) : j.v * STEP + t;
-            w[j.v] = 0;
-            if (i < lim) w[j.v] = __ldg(reinterpret_cast<const raw*>(row + i));
-        });
+        // A whole row needs no bound per load: with 32 of them per row and four rows the bounds kept bf16 loads of the kernel gradient
+        // from being in flight together (N = 1024, 16 rows of 768 channels: 76.9 us with
+        // them, 39.2 without; fp32 40; the convolution 29.6 -> 23.7, causal 23.0 -> 20.5).
+        if (sizeof(IO) == 2 && C::R1 == 32 && lim >= L * STEP)
+            unroll<L>([&](auto j) { w[j.v] = __ldg(reinterpret_cast<const raw*>(row + j.v * STEP + t)); });
+        else
+            unroll<L>([&](auto j) {
+                const int i = C::R1 == 16 ? (j.v / 2) * STEP + 2 * t + (j.v & 1) : j.v * STEP + t;
+                w[j.v] = 0;
+                if (i < lim) w[j.v] = __ldg(reinterpret_cast<const raw*>(row + i));
+            });
         unroll<L / 2>([&](auto j) { v[j.v] = pk(Io<IO>::cvt(w[2 * j.v]), Io<IO>::cvt(w[2 * j.v + 1])); });
     }
 }
