@@ -141,6 +141,12 @@ def test_fp32_transform_kernels(dims, n, causal, dtype, B, H, group):
     plan.close()
 
 
+@pytest.mark.parametrize("n,causal,B", [(1024, False, 3), (1024, False, 2), (512, True, 5), (510, True, 3)])
+def test_bf16_rows_of_32_point_columns(n, causal, B):
+    """N = 1024 in bf16: whole rows (loaded without a bound) and shorter ones, batches with and without a second row in the last pair."""
+    test_fp32_transform_kernels((32, 32), n, causal, M.M2_BF16, B, 6, 1)
+
+
 # ---- config 2: bf16 circular, N = 512 = 32 x 16 ----------------------------------------------
 
 @pytest.mark.parametrize("B,H", [(4, 24), (3, 5), (1, 1), (32, 9), (9, 5), (16, 3), (19, 6), (40, 150)])
