@@ -1,6 +1,6 @@
 // Convolution in fp32 (fft_grad.cu: kernel spectrum and kernel gradient) for every plan whose length is a power of two from 256 to 16384: the fp32
 // path, and the bf16 shapes the tensor-core kernels do not cover.  A complex row (two real batch rows of one channel: the kernel is
-// real, so F^-1(k_f (.) F(x_a + i x_b)) = y_a + i y_b) stays in registers and shared memory from the load to the store; fft_core.cuh
+// real, so F^-1(k_f (.) F(x_a + i x_b)) = y_a + i y_b; balance_pair keeps them apart) stays in registers and shared memory from the load to the store; fft_core.cuh
 // has the transforms.
 //
 // What bounds it: shared-memory wavefronts (64 KB each way per digit exchange of a 4096-point row) and packed FP32 issue, about equal;
@@ -37,6 +37,8 @@ __global__ void __launch_bounds__(C::THREADS, min_blocks<C>())
     asm volatile("griddepcontrol.wait;" ::: "memory");
     load_row<C, IO, HALF>(re, x + oa, t, n, vec, live);
     load_row<C, IO, HALF>(im, x + ob, t, n, vec, has_b);
+    uint32_t* slot = reinterpret_cast<uint32_t*>(smem + 2 * C::SMEM_FLOATS) + r * scale_words<C>();
+    balance_pair<C, HALF>(re, im, slot, t, r);
     forward<C, HALF>(re, im, sr, si, tab, t, r);
     const float4* kr = kf + (long long)(h / kf_group) * (C::N / 2) + t;
     unroll<16>([&](auto s) {
@@ -48,6 +50,7 @@ __global__ void __launch_bounds__(C::THREADS, min_blocks<C>())
         re[p] = pr;
     });
     inverse<C, HALF>(re, im, sr, si, tab, t, r);
+    unbalance_pair<C>(re, im, slot);
     store_row<C, IO, HALF>(re, y + oa, t, n, vec, live);
     store_row<C, IO, HALF>(im, y + ob, t, n, vec, has_b);
 }

@@ -108,6 +108,84 @@ __device__ __forceinline__ void store_row(const u64* v, IO* row, int t, int n, b
     }
 }
 
+// ---- two real rows as one complex row ----
+// The rounding error of a transform is relative to the norm of the complex row, and a value that is not finite reaches all of it, so the
+// two rows are made alike first: each is brought to a largest magnitude in [1, 2) by a power of two, which is exact and is taken back
+// when the row leaves (without the factors a row beside one 1e4 times as large is about 1e-3 off).  One B200, without and with them: bf16
+// x[8][768][2000] 44.9 and 46.3 us, [16][768][1024] 21.3 and 23.4, fp32 [4][768][2048] 26.2 and 26.9.
+template <class C>
+__host__ __device__ constexpr int scale_words() { return 2 * (C::TP > 32 ? C::TP / 32 + 1 : 1); }   // per row pair: its warps' maxima, the factors
+template <class C>
+__host__ __device__ constexpr int scale_bytes() { return (C::ROWS * scale_words<C>() * 4 + 15) / 16 * 16; }
+constexpr uint32_t kInfBits = 0x7f800000u;
+
+// largest magnitudes of the pair's rows as bits, NaN above infinity above everything else; each thread brings its part of both.  Ends
+// with a barrier of the row's threads where they are in several warps
+template <class C, bool HALF>
+__device__ __forceinline__ void pair_tops(const u64* re, const u64* im, uint32_t* slot, int t, int r, uint32_t& ta, uint32_t& tb) {
+    auto top = [](const u64* v) {
+        float m = 0.f;
+        unroll<(HALF ? 8 : 16)>([&](auto j) { asm("max.NaN.abs.f32 %0, %0, %1, %2;" : "+f"(m) : "f"(lo(v[j.v])), "f"(hi(v[j.v]))); });
+        return __float_as_uint(m);
+    };
+    ta = top(re);
+    tb = top(im);
+    if constexpr (C::TP >= 32) {
+        ta = __reduce_max_sync(0xffffffffu, ta);
+        tb = __reduce_max_sync(0xffffffffu, tb);
+    } else {
+#pragma unroll
+        for (int o = C::TP / 2; o > 0; o /= 2) {
+            ta = max(ta, __shfl_xor_sync(0xffffffffu, ta, o));
+            tb = max(tb, __shfl_xor_sync(0xffffffffu, tb, o));
+        }
+    }
+    if constexpr (C::TP > 32) {
+        if (t % 32 == 0) {
+            slot[t / 32 * 2] = ta;
+            slot[t / 32 * 2 + 1] = tb;
+        }
+        row_sync<C>(r);
+#pragma unroll
+        for (int w = 0; w < C::TP / 32; ++w) {
+            ta = max(ta, slot[2 * w]);
+            tb = max(tb, slot[2 * w + 1]);
+        }
+    }
+}
+// 2^e for a largest magnitude in [2^e, 2^(e+1)), and its inverse; both normal numbers
+__device__ __forceinline__ uint32_t top_exponent(uint32_t top) { return min(max(top >> 23, 1u), 253u); }
+__device__ __forceinline__ float scale_up(uint32_t top) { return __uint_as_float(top_exponent(top) << 23); }
+__device__ __forceinline__ float scale_down(uint32_t top) { return __uint_as_float((254u - top_exponent(top)) << 23); }
+template <bool HALF>
+__device__ __forceinline__ void scale_row(u64* v, float f) {   // as load_row leaves it
+    const u64 w = dup2(f);
+    unroll<(HALF ? 8 : 16)>([&](auto j) { v[j.v] = mul2(v[j.v], w); });
+}
+// Makes a pair's rows alike for a convolution.  A row with a value that is not finite takes no part (zeros) and leaves as NaN, a row of
+// zeros leaves as zeros.
+template <class C, bool HALF>
+__device__ __forceinline__ void balance_pair(u64* re, u64* im, uint32_t* slot, int t, int r) {
+    uint32_t ta, tb;
+    pair_tops<C, HALF>(re, im, slot, t, r, ta, tb);
+    auto one = [&](u64* v, uint32_t top, uint32_t* back) {
+        if (top >= kInfBits) unroll<(HALF ? 8 : 16)>([&](auto j) { v[j.v] = 0ull; });
+        else scale_row<HALF>(v, scale_down(top));
+        if (t == 0) *back = top >= kInfBits ? 0x7fffffffu : top == 0 ? 0u : __float_as_uint(scale_up(top));
+    };
+    one(re, ta, slot + scale_words<C>() - 2);
+    one(im, tb, slot + scale_words<C>() - 1);
+}
+// (the row's threads have met since)
+template <class C>
+__device__ __forceinline__ void unbalance_pair(u64* re, u64* im, const uint32_t* slot) {
+    const u64 fa = dup2(__uint_as_float(slot[scale_words<C>() - 2])), fb = dup2(__uint_as_float(slot[scale_words<C>() - 1]));
+    unroll<16>([&](auto s) {
+        re[s.v] = mul2(re[s.v], fa);
+        im[s.v] = mul2(im[s.v], fb);
+    });
+}
+
 // registers (input digit of the first pass) -> registers (output of the last digit: q in slot brev(q); R = 32: q, q + 16).
 // The row's shared memory must be free on entry; afterwards other threads may still be reading it.
 template <class C, bool HALF>
@@ -187,7 +265,7 @@ cudaError_t dispatch(int64_t N, F&& f) {
 }
 
 template <class C>
-constexpr int conv_smem() { return 2 * C::SMEM_FLOATS * 4; }
+constexpr int conv_smem() { return 2 * C::SMEM_FLOATS * 4 + scale_bytes<C>(); }
 template <class K>
 cudaError_t allow_smem(K kern, int bytes) {
     return bytes > 48 * 1024 ? cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) : cudaSuccess;

@@ -141,6 +141,34 @@ def test_fp32_transform_kernels(dims, n, causal, dtype, B, H, group):
     plan.close()
 
 
+@pytest.mark.parametrize("dims,n,causal,dtype", [
+    ((16, 16), 256, False, M.M2_BF16), ((32, 16), 200, True, M.M2_FP32), ((32, 32), 511, True, M.M2_BF16), ((64, 32), 2048, False, M.M2_FP32),
+    ((64, 64), 2000, True, M.M2_BF16), ((16, 16, 16), 1001, True, M.M2_FP32), ((32, 32, 8), 8192, False, M.M2_FP32), ((128, 128), 8192, True, M.M2_BF16)])
+def test_rows_that_share_a_transform_do_not_mix(dims, n, causal, dtype):
+    """Batch rows 2 b and 2 b + 1 go through the transform kernels as one complex row: a small row beside a large one is as accurate as
+    alone, a row of zeros stays zero, a value that is not finite stays in its row."""
+    bf, N, H = dtype == M.M2_BF16, int(np.prod(dims)), 3
+    scale = np.array([1e4, 1.0, 0.0, 1e6, 1e-12, 1.0, 1e3, 1.0, 1e-3])
+    bad = {5: np.nan, 6: np.inf}
+    rnd = synth.round_bf16 if bf else (lambda a: a.astype(np.float32))
+    x = rnd(synth.normal(730 + n, (len(scale), H, n)) * scale[:, None, None]).astype(np.float32)
+    k = (synth.normal(731 + n, (H, n)) / np.sqrt(n)).astype(np.float32)
+    want = np.fft.irfft(np.fft.rfft(x.astype(np.float64), N) * np.fft.rfft(k.astype(np.float64), N)[None], N)[..., :n]
+    for b, v in bad.items():
+        x[b, :, n // 3] = v
+    plan = M.Plan(dims, dtype=dtype, device=0)
+    y = host(M.m2_monarch_conv_fwd(plan, dev(x, torch.bfloat16 if bf else torch.float32), M.m2_kernel_spectrum(plan, dev(k)),
+                                   M.M2_CAUSAL if causal else M.M2_CIRCULAR))
+    assert plan.device_status() == 0
+    plan.close()
+    good = [b for b in range(len(scale)) if b not in bad and scale[b] != 0]
+    for b in good:
+        check(y[b], want[b], 4e-3 if bf else TOL_FP32, f"row {b} of scale {scale[b]}")
+    assert (y[scale == 0] == 0).all()
+    for b in bad:
+        assert np.isnan(y[b]).all()
+
+
 @pytest.mark.parametrize("n,causal,B", [(1024, False, 3), (1024, False, 2), (512, True, 5), (510, True, 3)])
 def test_bf16_rows_of_32_point_columns(n, causal, B):
     """N = 1024 in bf16: whole rows (loaded without a bound) and shorter ones, batches with and without a second row in the last pair."""
