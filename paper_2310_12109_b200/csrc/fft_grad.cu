@@ -107,6 +107,7 @@ __global__ void __launch_bounds__(C::THREADS, wgrad_blocks<C>())
     float* si = sr + C::SMEM_FLOATS;
     float4* zall = reinterpret_cast<float4*>(smem + 2 * C::SMEM_FLOATS);
     float4* zs = zall + threadIdx.x;
+    uint32_t* slot = reinterpret_cast<uint32_t*>(zall + C::THREADS * 16) + r * scale_words<C>();
     u64 re[16], im[16], ar[16], ai[16];
     unroll<16>([&](auto s) { ar[s.v] = ai[s.v] = 0ull; });
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -117,10 +118,16 @@ __global__ void __launch_bounds__(C::THREADS, wgrad_blocks<C>())
         const long long oa = has_a ? ((long long)b * H + h) * n : 0, ob = oa + (long long)H * n;
         load_row<C, IO, HALF>(re, x + oa, t, n, vec, has_a);
         load_row<C, IO, HALF>(im, x + ob, t, n, vec, has_b);
+        uint32_t ta, tb;   // x / 2^e and 2^e g: the cross terms of a pair are then no larger than the pair's share of the sum
+        pair_tops<C, HALF>(re, im, slot, t, r, ta, tb);
+        scale_row<HALF>(re, scale_down(ta));
+        scale_row<HALF>(im, scale_down(tb));
         forward<C, HALF>(re, im, sr, si, tab, t, r);
         unroll<16>([&](auto s) { zs[s.v * C::THREADS] = make_float4(lo(re[s.v]), hi(re[s.v]), lo(im[s.v]), hi(im[s.v])); });
         load_row<C, IO, HALF>(re, g + oa, t, n, vec, has_a);
         load_row<C, IO, HALF>(im, g + ob, t, n, vec, has_b);
+        scale_row<HALF>(re, scale_up(ta));
+        scale_row<HALF>(im, scale_up(tb));
         row_sync<C>(r);
         forward<C, HALF>(re, im, sr, si, tab, t, r);
         unroll<16>([&](auto s) {   // += conj(z) w
