@@ -831,20 +831,20 @@ conv512p_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
 //
 //   dk[h] = M^-1 ( sum_b conj(M x_b) (.) M g_b ) [0:n)          (the transpose of Eq. 2 with respect to k)
 //
-// The forward half of the row-pair pipeline above (S1, twiddle, S2) runs on the x tile and on the g tile of a unit (16 batch rows of
-// one channel) side by side: with z = x_a + i x_b and w = g_a + i g_b the real part of M^-1(conj(M z) (.) M w) is the sum of the two
-// rows' correlations, so a pair costs what a row would.  128 TMEM columns per pipeline, 4 pipelines per CTA; two issuing threads, one
-// per tile.  Each thread then holds the two spectra of its rows at the same (k1, k2), forms conj(Z) W in fp32, adds its two rows, the
-// four warps' sums are added through shared memory, and the unit's sum goes to partial[b group][h] in the order of the fp32
-// transform kernels (fft_core.cuh), which add the b groups in order and apply M^-1 (m2f::time_kernel).
-// Shared memory per pipeline: x tile | A2 of x | g tile; A2 of g takes the place of the x tile.  Bound by the hand-offs' latency (as
-// the forward kernel): x, g [32][768][512]: 30 -> 20 us against one row per lane, and 14.6 -> 6 us for the sum and M^-1.
+// The forward half of the pipeline above (S1, twiddle, S2) runs on the x tile and on the g tile of a unit (8 batch rows of one channel,
+// real rows: packed in pairs the products' cross terms cancel only up to the bf16 rounding of the hand-off, 3.1e-3 from the exact
+// gradient at 9 rows of N(0, 1) against 2.96e-3, and without bound where a pair's rows differ in scale) side by side.  128 TMEM columns per pipeline, 4
+// pipelines per CTA; two issuing threads, one per tile.  Each thread then holds the two spectra of its rows at the same (k1, k2), forms
+// conj(X) G in fp32, adds its two rows, the four warps' sums are added through shared memory, and the unit's sum goes to
+// partial[b group][h] in the order of the fp32 transform kernels (fft_core.cuh), which add the b groups and apply M^-1
+// (m2f::time_kernel).
+// Shared memory per pipeline: x tile, later A2 of g | A2 of x | g tile.  Bound by the hand-offs' latency (as the forward kernel).
 constexpr int kGroupsW = 4;
 constexpr int kThreadsW = 128 * kGroupsW;
-constexpr int WG_X = 0;              // re tile 8192 | im tile 8192 (one box [r][n1][16 n2] each, 32-byte swizzled); later A2 of g
+constexpr int WG_X = 0;              // x tile 8192 (one box [r][n1][16 n2], 32-byte swizzled); later A2 of g 16384
 constexpr int WG_A = 16384;          // A2 of x; afterwards the four warps' sums [warp][k2][k1] float2
-constexpr int WG_G = 32768;          // as WG_X
-constexpr int W_GROUP_BYTES = 49152;
+constexpr int WG_G = 32768;          // g tile 8192
+constexpr int W_GROUP_BYTES = 40960;
 constexpr int W_SMEM_BYTES = P_OFF_GROUP + kGroupsW * W_GROUP_BYTES;
 static_assert(W_SMEM_BYTES <= 232448 && 4 * 16 * 32 * 8 <= 16384 && 128 * kGroupsW <= kTmemCols, "per-CTA budgets");
 
@@ -861,7 +861,7 @@ convwgrad512_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
     const uint32_t bar_x = s_all + P_OFF_BAR + wg * 32, bar_mma = bar_x + 8, bar_g = bar_x + 16;
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_all + P_OFF_BAR + wg * 32 + 24);
     const uint32_t s_tptr = s_all + P_OFF_BAR + 512;
-    const int units = H * ((B + 2 * kRows - 1) / (2 * kRows));
+    const int units = H * ((B + kRows - 1) / kRows);
     const int ustride = gridDim.x * kGroupsW;
     int u = wg * gridDim.x + blockIdx.x;   // pipeline-major: a partial last round spreads over all CTAs
     if (leader) {
@@ -881,11 +881,9 @@ convwgrad512_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
     if (threadIdx.x < 32) tmem_alloc(s_tptr, kTmemCols);
     asm volatile("griddepcontrol.wait;" ::: "memory");
     bool x_pending = false, g_pending = false;   // copies in flight (leader)
-    auto load_tile = [&](const CUtensorMap* map, int off, uint32_t bar, int v) {   // the two boxes [8 rows][32 n1][16 n2] of unit v
-        const int hh = v % H, bb = (v / H) * 2 * kRows;
-        mbar_expect_tx(bar, 16384);
-        tma_load_4d(s_base + off, map, 0, 0, hh, bb, bar);
-        tma_load_4d(s_base + off + 8192, map, 0, 0, hh, bb + kRows, bar);
+    auto load_tile = [&](const CUtensorMap* map, int off, uint32_t bar, int v) {   // the box [8 rows][32 n1][16 n2] of unit v
+        mbar_expect_tx(bar, 8192);
+        tma_load_4d(s_base + off, map, 0, 0, v % H, (v / H) * kRows, bar);
     };
     if (leader && u < units) {
         load_tile(&map_x, WG_X, bar_x, u);
@@ -913,12 +911,10 @@ convwgrad512_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
             ok = mbar_wait(lead_warp ? bar_x : bar_g, ph_x);
             if (ok) {
                 tc_fence_after();
-#pragma unroll
-                for (int c = 0; c < 2; ++c)   // K = (re | im part of the input) x n1
 #pragma unroll 1
-                    for (int s = 0; s < k1steps; ++s)
-                        umma_f16(tmem + col, smem_desc_sw32(s_base + off + c * 8192 + s * 512, 1024, 256),
-                                 smem_desc(s_all + P_OFF_B1 + (2 * c + s) * 256, 128, 1024), ID_S1, (c | s) > 0);
+                for (int s = 0; s < k1steps; ++s)   // K = n1: the rows of the F_32 image that belong to the real part of the input
+                    umma_f16(tmem + col, smem_desc_sw32(s_base + off + s * 512, 1024, 256), smem_desc(s_all + P_OFF_B1 + s * 256, 128, 1024),
+                             ID_S1, s > 0);
                 umma_commit(bar_mma);
             }
         }
@@ -992,7 +988,7 @@ convwgrad512_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
             load_tile(&map_x, WG_X, bar_x, un);
             x_pending = true;
         }
-        // ---- conj(Z) W, summed over this thread's two rows, then over the four warps ------------------------------
+        // ---- conj(X) G, summed over this thread's two rows, then over the four warps ------------------------------
         float2* red = reinterpret_cast<float2*>(smem + WG_A);   // [warp][k2][k1]: A2 of x is free now
         if (ok) {
             const int k1 = tid & 31;
@@ -1270,10 +1266,10 @@ int32_t conv_fwd_wait_selftest(const m2_plan* pl, const void* x, const void* kf,
 }
 
 int64_t conv_wgrad_workspace_bytes(const m2_plan* pl, int64_t B, int64_t H) {
-    return pl->umma && covered(pl) ? ((B + 2 * kRows - 1) / (2 * kRows)) * H * 512 * 8 : 0;
+    return pl->umma && covered(pl) ? ((B + kRows - 1) / kRows) * H * 512 * 8 : 0;
 }
 
-// partial[b group][h][512] (transform kernels' order) = sum over the group's 16 rows of conj(M x) (.) M g; returns the number of b groups in *parts
+// partial[b group][h][512] (transform kernels' order) = sum over the group's 8 rows of conj(M x) (.) M g; returns the number of b groups in *parts
 int32_t conv_wgrad_partials(const m2_plan* pl, const void* x, const void* g, void* partial, int64_t B, int64_t H, int64_t n, int32_t mode,
                             int* parts, cudaStream_t stream) {
     if (!pl->umma || !covered(pl)) return M2_ERR_UNSUPPORTED;
@@ -1284,7 +1280,7 @@ int32_t conv_wgrad_partials(const m2_plan* pl, const void* x, const void* g, voi
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const long long bgroups = (B + 2 * kRows - 1) / (2 * kRows), units = H * bgroups;
+    const long long bgroups = (B + kRows - 1) / kRows, units = H * bgroups;
     const long long ctas = (units + kGroupsW - 1) / kGroupsW;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(ctas < sms ? ctas : sms));

@@ -23,12 +23,14 @@ int32_t conv_fwd(const m2_plan* plan, const void* x, const void* kf, void* y, in
 int32_t conv_gate_fwd(const m2_plan* plan, const void* x, const void* kf, const float* w_gate, void* y, int64_t B, int64_t H,
                       cudaStream_t stream, const void* gate_rows = nullptr, const void* addend = nullptr);
 bool covers_rows(const m2_plan* plan, int64_t n);   // conv_fwd has a kernel for rows of n values
+// The row-pair kernel launched so that every pipeline's first bounded wait runs out with nothing in flight (no copy is
+// issued, a few polls per wait): the kernel leaves through its abort path, sets M2_ERR_TIMEOUT in the plan's status
+// word, writes nothing to y.  Needs B > 8 (the row-pair kernel); M2_ERR_UNSUPPORTED otherwise.
 int32_t conv_fwd_wait_selftest(const m2_plan* plan, const void* x, const void* kf, void* y, int64_t B, int64_t H, int64_t n,
                                int32_t mode, cudaStream_t stream);
 
-// Kernel gradient, tensor-core part: partial[b group][h][512] = sum over the group's 16 rows of conj(M z) (.) M w, z and w the row pairs
-// of x and g as complex rows, in the order of the fp32 transform kernels (complex fp32, conv_wgrad_workspace_bytes(plan, B, H)
-// bytes); *parts = number of b groups.
+// Kernel gradient, tensor-core part: partial[b group][h][512] = sum over the group's 8 rows of conj(M x) (.) M g in the order of the
+// fp32 transform kernels (complex fp32, conv_wgrad_workspace_bytes(plan, B, H) bytes); *parts = number of b groups.
 int64_t conv_wgrad_workspace_bytes(const m2_plan* plan, int64_t B, int64_t H);
 int32_t conv_wgrad_partials(const m2_plan* plan, const void* x, const void* g, void* partial, int64_t B, int64_t H, int64_t n,
                             int32_t mode, int* parts, cudaStream_t stream);
