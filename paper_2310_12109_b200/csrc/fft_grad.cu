@@ -47,20 +47,52 @@ __global__ void __launch_bounds__(C::THREADS, min_blocks<C>())
     }
 }
 
-// the inverse half alone, of the sum of `parts` spectra in order: scale times the real part of the first n positions
+// Values of `share` neighbouring rows of threads added in order: value (s, t) of a channel = the sum over its rows' threads t; share * TP
+// threads share the work.  all: 16 float4 per thread of the block; other rows may still be reading it on return
+template <class C>
+__device__ __forceinline__ void add_shares(u64* re, u64* im, float4* all, int share, int r, int t) {
+    float4* own = all + threadIdx.x;
+    __syncthreads();
+    unroll<16>([&](auto s) { own[s.v * C::THREADS] = make_float4(lo(re[s.v]), hi(re[s.v]), lo(im[s.v]), hi(im[s.v])); });
+    __syncthreads();
+    const int first = (r / share) * share * C::TP, lid = threadIdx.x - first, step = share * C::TP;
+    for (int v = lid; v < 16 * C::TP; v += step) {
+        float4* p = all + (v / C::TP) * C::THREADS + first + v % C::TP;
+        float4 a = *p;
+        for (int q = 1; q < share; ++q) {
+            const float4 w = p[q * C::TP];
+            a.x += w.x;
+            a.y += w.y;
+            a.z += w.z;
+            a.w += w.w;
+        }
+        *p = a;
+    }
+    __syncthreads();
+    unroll<16>([&](auto s) {
+        const float4 a = all[s.v * C::THREADS + first + t];
+        re[s.v] = pk(a.x, a.y);
+        im[s.v] = pk(a.z, a.w);
+    });
+}
+
+// the inverse half alone, of the sum of `parts` spectra: scale times the real part of the first n positions.  `share` rows of threads
+// (a power of two) take the parts of one channel in turn, as in fft_wgrad_kernel: a part is a round trip to memory, and few channels with
+// many parts waited for one after the other (x, g [4096][1][256], the whole gradient: 136 us with 256 parts added by one row of threads,
+// 30 by eight).
 template <class C, bool HALF>
 __global__ void __launch_bounds__(C::THREADS, min_blocks<C>())
     fft_time_kernel(const float4* __restrict__ kf, int parts, float scale, float* __restrict__ kt, const float4* __restrict__ tab, int H,
-                    int n) {
+                    int n, int share) {
     extern __shared__ __align__(16) float smem[];
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int r = threadIdx.x / C::TP, t = threadIdx.x % C::TP;
-    const long long h = (long long)blockIdx.x * C::ROWS + r;
+    const long long h = (long long)blockIdx.x * (C::ROWS / share) + r / share;
     const bool live = h < H;
     float* sr = smem + r * C::ROWF + (r & 1) * C::PAR;
     float* si = sr + C::SMEM_FLOATS;
     u64 re[16], im[16];
-    const float4* in = kf + (live ? h : 0) * (C::N / 2) + t;
+    const float4* in = kf + ((long long)(r % share) * H + (live ? h : 0)) * (C::N / 2) + t;   // (share <= parts)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     unroll<16>([&](auto s) {
         constexpr int p = brev<4>(s.v);
@@ -69,8 +101,8 @@ __global__ void __launch_bounds__(C::THREADS, min_blocks<C>())
         im[p] = pk(w.z, w.w);
     });
 #pragma unroll 1
-    for (int q = 1; q < parts; ++q) {
-        in += (long long)H * (C::N / 2);
+    for (int q = r % share + share; q < parts; q += share) {
+        in += (long long)share * H * (C::N / 2);
         unroll<16>([&](auto s) {
             constexpr int p = brev<4>(s.v);
             const float4 w = in[s.v * C::TP];
@@ -78,13 +110,20 @@ __global__ void __launch_bounds__(C::THREADS, min_blocks<C>())
             im[p] = add2(im[p], pk(w.z, w.w));
         });
     }
+    if constexpr (C::ROWS > 1) {
+        static_assert(2 * C::SMEM_FLOATS * 4 >= C::THREADS * 256, "the rows' values fit where the transform exchanges its digits");
+        if (share > 1) {
+            add_shares<C>(re, im, reinterpret_cast<float4*>(smem), share, r, t);
+            __syncthreads();
+        }
+    }
     const u64 sc = dup2(scale);
     unroll<16>([&](auto s) {
         re[s.v] = mul2(re[s.v], sc);
         im[s.v] = mul2(im[s.v], sc);
     });
     inverse<C, HALF>(re, im, sr, si, tab, t, r);
-    store_row<C, float, HALF>(re, kt + h * n, t, n, (n & 1) == 0, live);
+    store_row<C, float, HALF>(re, kt + h * n, t, n, (n & 1) == 0, live && r % share == 0);
 }
 
 // dk[h] = Re F^-1( sum over row pairs of conj(F z) (.) F w ) / N with z = x_a + i x_b, w = g_a + i g_b: the real part of the product's
@@ -138,30 +177,7 @@ __global__ void __launch_bounds__(C::THREADS, wgrad_blocks<C>())
         });
         row_sync<C>(r);
     }
-    if (C::ROWS > 1 && share > 1) {   // value (s, t) of a channel = the sum over its rows' threads t; share * TP threads share the work
-        __syncthreads();
-        unroll<16>([&](auto s) { zs[s.v * C::THREADS] = make_float4(lo(ar[s.v]), hi(ar[s.v]), lo(ai[s.v]), hi(ai[s.v])); });
-        __syncthreads();
-        const int first = (r / share) * share * C::TP, lid = threadIdx.x - first, step = share * C::TP;
-        for (int v = lid; v < 16 * C::TP; v += step) {
-            float4* p = zall + (v / C::TP) * C::THREADS + first + v % C::TP;
-            float4 a = *p;
-            for (int q = 1; q < share; ++q) {
-                const float4 w = p[q * C::TP];
-                a.x += w.x;
-                a.y += w.y;
-                a.z += w.z;
-                a.w += w.w;
-            }
-            *p = a;
-        }
-        __syncthreads();
-        unroll<16>([&](auto s) {
-            const float4 a = zall[s.v * C::THREADS + first + t];
-            ar[s.v] = pk(a.x, a.y);
-            ai[s.v] = pk(a.z, a.w);
-        });
-    }
+    if (C::ROWS > 1 && share > 1) add_shares<C>(ar, ai, zall, share, r, t);
     inverse<C, HALF>(ar, ai, sr, si, tab, t, r);
     const u64 sc = dup2(1.0f / (float)C::N);
     unroll<16>([&](auto s) { ar[s.v] = mul2(ar[s.v], sc); });
@@ -209,10 +225,13 @@ cudaError_t time_kernel(const m2_plan* pl, const void* kf, int parts, float scal
     if (H == 0) return cudaSuccess;
     return dispatch(pl->N, [&](auto cfg) {
         using C = decltype(cfg);
-        const unsigned grid = (unsigned)((H + C::ROWS - 1) / C::ROWS);
+        int share = 1;   // rows of a block per channel: no more than there are parts
+        while (share < C::ROWS && 2 * share <= parts) share *= 2;
+        const int64_t per_block = C::ROWS / share;
+        const unsigned grid = (unsigned)((H + per_block - 1) / per_block);
         auto go = [&](auto half) {
             return launch_early(fft_time_kernel<C, decltype(half)::v != 0>, grid, C::THREADS, conv_smem<C>(), stream, (const float4*)kf, parts,
-                                scale, kt, (const float4*)pl->d_fft, (int)H, (int)n);
+                                scale, kt, (const float4*)pl->d_fft, (int)H, (int)n, share);
         };
         return 2 * n <= C::N ? go(Ic<1>{}) : go(Ic<0>{});
     });

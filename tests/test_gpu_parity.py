@@ -189,6 +189,17 @@ def test_kernel_gradient_of_rows_of_different_scale(dims, n, causal, dtype):
     plan.close()
 
 
+@pytest.mark.parametrize("B,H,n,causal", [(9, 9, 512, False), (40, 5, 256, True), (137, 1, 512, False)])
+def test_kernel_gradient_adds_its_parts(B, H, n, causal):
+    """N = 512: 2, 5 and 18 partial sums of 8 batch rows, added by 2, 4 and 8 rows of threads per channel; blocks with channels to spare."""
+    x, g = synth.round_bf16(synth.normal(750 + B, (B, H, n))).astype(np.float64), synth.round_bf16(synth.normal(751 + B, (B, H, n))).astype(np.float64)
+    plan = M.Plan((32, 16), dtype=M.M2_BF16, device=0)
+    dk = M.m2_monarch_conv_bwd_kernel(plan, dev(x, torch.bfloat16), dev(g, torch.bfloat16), M.M2_CAUSAL if causal else M.M2_CIRCULAR)
+    assert plan.device_status() == 0 and plan.last_kernel() == "conv_wgrad_umma_o2_512"
+    check(host(dk), np.fft.irfft((np.fft.rfft(g, 512) * np.conj(np.fft.rfft(x, 512))).sum(0), 512)[..., :n], TOL_BF16, "kernel gradient")
+    plan.close()
+
+
 @pytest.mark.parametrize("n,causal,B", [(1024, False, 3), (1024, False, 2), (512, True, 5), (510, True, 3)])
 def test_bf16_rows_of_32_point_columns(n, causal, B):
     """N = 1024 in bf16: whole rows (loaded without a bound) and shorter ones, batches with and without a second row in the last pair."""
