@@ -21,8 +21,10 @@ int spectrum_order(const m2_plan* pl);
 // itself, zero padded, fp32 [H][N]
 cudaError_t spectrum(const m2_plan* pl, const float* k, int64_t H, int64_t n, void* kf, void* kfu, float* kt, cudaStream_t stream);
 // back to the time domain: kt[h][t] = scale times the first n values of F^-1 of the sum of `parts` buffers [H][N], fp32 [H][n]; a
-// spectrum carries its 1 / N already (scale 1 gives the kernel)
-cudaError_t time_kernel(const m2_plan* pl, const void* kf, int parts, float scale, int64_t H, int64_t n, float* kt, cudaStream_t stream);
+// spectrum carries its 1 / N already (scale 1 gives the kernel).  both (2 n <= N): kt is [H][2 n], lag u at u mod 2 n for -n <= u < n, lags
+// below zero that are rounding only are zero
+cudaError_t time_kernel(const m2_plan* pl, const void* kf, int parts, float scale, int64_t H, int64_t n, bool both, float* kt,
+                        cudaStream_t stream);
 // y = conv(k[h / kf_group], x[b][h]), x / y [B][H][n] contiguous in the plan dtype
 cudaError_t conv(const m2_plan* pl, const void* x, const void* kf, void* y, int64_t B, int64_t H, int64_t n, bool causal, int kf_group,
                  cudaStream_t stream);

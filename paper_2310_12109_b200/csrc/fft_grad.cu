@@ -79,11 +79,12 @@ __device__ __forceinline__ void add_shares(u64* re, u64* im, float4* all, int sh
 // the inverse half alone, of the sum of `parts` spectra: scale times the real part of the first n positions.  `share` rows of threads
 // (a power of two) take the parts of one channel in turn, as in fft_wgrad_kernel: a part is a round trip to memory, and few channels with
 // many parts waited for one after the other (x, g [4096][1][256], the whole gradient: 136 us with 256 parts added by one row of threads,
-// 30 by eight).
+// 30 by eight).  both: rows of 2 n values, the first n positions and the last n (2 n <= N), where what is below 2^-20 of the row's largest
+// value -- the transforms' rounding, if the kernel has no such lags -- is written as zero.
 template <class C, bool HALF>
 __global__ void __launch_bounds__(C::THREADS, min_blocks<C>())
     fft_time_kernel(const float4* __restrict__ kf, int parts, float scale, float* __restrict__ kt, const float4* __restrict__ tab, int H,
-                    int n, int share) {
+                    int n, int share, int both) {
     extern __shared__ __align__(16) float smem[];
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int r = threadIdx.x / C::TP, t = threadIdx.x % C::TP;
@@ -123,6 +124,22 @@ __global__ void __launch_bounds__(C::THREADS, min_blocks<C>())
         im[s.v] = mul2(im[s.v], sc);
     });
     inverse<C, HALF>(re, im, sr, si, tab, t, r);
+    if (!HALF && both) {   // (one launch-wide choice: the threads of a row meet)
+        uint32_t top, same;
+        pair_tops<C, false>(re, re, reinterpret_cast<uint32_t*>(smem + 2 * C::SMEM_FLOATS) + r * scale_words<C>(), t, r, top, same);
+        const float least = __uint_as_float(top) * 0x1p-20f;
+        auto put = [&](int i, float v) {
+            if (i < n) kt[h * 2 * n + i] = v;
+            else if (i >= C::N - n) kt[h * 2 * n + i - (C::N - 2 * n)] = fabsf(v) <= least ? 0.f : v;
+        };
+        if (live && r % share == 0)
+            unroll<16>([&](auto q) {
+                constexpr int p = brev<4>(q.v), STEP = C::N / C::R1;
+                put(C::R1 == 16 ? q.v * STEP + 2 * t : q.v * STEP + t, lo(re[p]));
+                put(C::R1 == 16 ? q.v * STEP + 2 * t + 1 : (q.v + 16) * STEP + t, hi(re[p]));
+            });
+        return;
+    }
     store_row<C, float, HALF>(re, kt + h * n, t, n, (n & 1) == 0, live && r % share == 0);
 }
 
@@ -221,7 +238,8 @@ cudaError_t spectrum(const m2_plan* pl, const float* k, int64_t H, int64_t n, vo
     });
 }
 
-cudaError_t time_kernel(const m2_plan* pl, const void* kf, int parts, float scale, int64_t H, int64_t n, float* kt, cudaStream_t stream) {
+cudaError_t time_kernel(const m2_plan* pl, const void* kf, int parts, float scale, int64_t H, int64_t n, bool both, float* kt,
+                        cudaStream_t stream) {
     if (H == 0) return cudaSuccess;
     return dispatch(pl->N, [&](auto cfg) {
         using C = decltype(cfg);
@@ -231,9 +249,9 @@ cudaError_t time_kernel(const m2_plan* pl, const void* kf, int parts, float scal
         const unsigned grid = (unsigned)((H + per_block - 1) / per_block);
         auto go = [&](auto half) {
             return launch_early(fft_time_kernel<C, decltype(half)::v != 0>, grid, C::THREADS, conv_smem<C>(), stream, (const float4*)kf, parts,
-                                scale, kt, (const float4*)pl->d_fft, (int)H, (int)n, share);
+                                scale, kt, (const float4*)pl->d_fft, (int)H, (int)n, share, (int)both);
         };
-        return 2 * n <= C::N ? go(Ic<1>{}) : go(Ic<0>{});
+        return 2 * n <= C::N && !both ? go(Ic<1>{}) : go(Ic<0>{});
     });
 }
 

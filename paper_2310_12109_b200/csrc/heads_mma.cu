@@ -9,7 +9,9 @@
 // product's B operand (rows of an accumulator fragment = columns of a B fragment), so nothing goes through shared memory between the
 // two products and no warp waits for another.  (tcgen05 would put every tile through tensor memory, shared memory and two barriers for
 // 8 K multiply-adds.)  Kernel values lie reversed in shared memory, in two copies one element apart, so that the two values of a
-// fragment's column pair are one aligned 64-bit load for even and odd rows alike; lags below zero are stored as zeros.
+// fragment's column pair are one aligned 64-bit load for even and odd rows alike.  Lags below zero exist where the spectrum was
+// conjugated or its kernel is longer than N - n: a block that finds one that is not zero walks the tiles s > t too, with kernel values
+// from L2.
 //
 // Measured, one B200, 1536 heads of n = 256: 21.6 us (28.6 with index divisions in the copies and the two copies of the kernel in the
 // same banks) where 24 576 tensor-core convolution units of 16 rows took about 280 us.  Bound by instruction issue and the fragments'
@@ -43,7 +45,7 @@ __device__ __forceinline__ uint32_t weigh(float a, float b, float2 k) {
 
 __global__ void __launch_bounds__(kThreads)
     heads_kernel(const __nv_bfloat16* __restrict__ X1, const __nv_bfloat16* __restrict__ X2, const __nv_bfloat16* __restrict__ V,
-                 const float* __restrict__ kt, __nv_bfloat16* __restrict__ O, int heads, int n) {
+                 const float* __restrict__ kt, int period, __nv_bfloat16* __restrict__ O, int heads, int n) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int np = padded(n), ld = pitch(n), kc = kcopy(n);
@@ -55,10 +57,14 @@ __global__ void __launch_bounds__(kThreads)
     const size_t base = (size_t)blockIdx.x * kDh * n;   // the 16 channels of a head are consecutive rows
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    kt += (size_t)h * period;   // lag u at u mod period, |u| < n
+    auto value = [&](int lag) { return lag < n && lag > -n ? __ldg(kt + (lag < 0 ? period + lag : lag)) : 0.f; };
+    bool earlier = false;       // a lag below zero is not zero
+    for (int u = 1 + tid; u < n; u += kThreads) earlier |= value(-u) != 0.f;
     // copy p (p = 0, 1): the kernel value of a lag lies at np + 14 + p - lag
     for (int i = tid; i < kc; i += kThreads) {
         const int lag = np + 14 - i;
-        const float a = lag >= 0 && lag < n ? __ldg(kt + (size_t)h * n + lag) : 0.f;
+        const float a = value(lag);
         ks[i] = a;
         if (i + 1 < kc) ks[kc + i + 1] = a;
     }
@@ -79,7 +85,7 @@ __global__ void __launch_bounds__(kThreads)
 #pragma unroll
                 for (int q = 0; q < 3; ++q) xs1[q * kDh * ld + r * ld + c] = c < n ? src[q][(size_t)r * n + c] : __float2bfloat16_rn(0.f);
     }
-    __syncthreads();
+    earlier = __syncthreads_or(earlier);
     const int m = lane >> 3, r8 = lane & 7, g = lane >> 2, c2 = 2 * (lane & 3);
     // ldmatrix row addresses: A of the scores (X1, transposed on load), B of the scores (X2, transposed), A of the output (V)
     const uint32_t a1 = smem_addr(xs1 + ((m >> 1) * 8 + r8) * ld + (m & 1) * 8);
@@ -93,18 +99,26 @@ __global__ void __launch_bounds__(kThreads)
         uint32_t fa[4];
         ldsm4t(fa, a1 + ti * 32);
         float o[2][4] = {};
-        for (int si = 0; si <= ti; ++si) {
+        auto tile = [&](int si, float2 k0, float2 k8, float2 km) {   // the kernel at lags u, u + 8, u - 8 and the one below each
             uint32_t fb[4], fv[4];
             ldsm4t(fb, b2 + si * 32);
             ldsm4(fv, av + si * 32);
-            const float* kq = kp - (ti - si) * 16;
-            const float2 k0 = *reinterpret_cast<const float2*>(kq), k8 = *reinterpret_cast<const float2*>(kq - 8),
-                         km = *reinterpret_cast<const float2*>(kq + 8);   // lags u, u + 8, u - 8 and the one below each
             float s0[4] = {}, s1[4] = {};
             mma(s0, fa, fb[0], fb[1]);
             mma(s1, fa, fb[2], fb[3]);
             mma(o[0], fv, weigh(s0[0], s0[1], k0), weigh(s1[0], s1[1], km));
             mma(o[1], fv, weigh(s0[2], s0[3], k8), weigh(s1[2], s1[3], k0));
+        };
+        for (int si = 0; si <= ti; ++si) {
+            const float* kq = kp - (ti - si) * 16;
+            tile(si, *reinterpret_cast<const float2*>(kq), *reinterpret_cast<const float2*>(kq - 8), *reinterpret_cast<const float2*>(kq + 8));
+        }
+        if (earlier) {
+#pragma unroll 1
+            for (int si = ti + 1; si < tiles; ++si) {
+                const int u = g - c2 + 16 * (ti - si);
+                tile(si, make_float2(value(u), value(u - 1)), make_float2(value(u + 8), value(u + 7)), make_float2(value(u - 8), value(u - 9)));
+            }
         }
         __syncwarp();   // this tile's columns of X1 are read by this warp only: the result takes their place
 #pragma unroll
@@ -128,8 +142,8 @@ bool covered(const m2_plan* pl, int64_t n, int64_t d, int64_t dh) {
     return pl->dtype == M2_BF16 && m2f::covered(pl) && dh == kDh && d % kDh == 0 && n > 0 && n <= kMaxN;
 }
 
-int32_t heads_fwd(const m2_plan* pl, const void* X1, const void* X2, const void* V, const float* kt, void* O, int64_t B, int64_t d, int64_t n,
-                  cudaStream_t stream) {
+int32_t heads_fwd(const m2_plan* pl, const void* X1, const void* X2, const void* V, const float* kt, int64_t period, void* O, int64_t B, int64_t d,
+                  int64_t n, cudaStream_t stream) {
     const int64_t blocks = B * (d / kDh);
     if (blocks == 0) return M2_OK;
     if (blocks > 0x7fffffffLL) return M2_ERR_UNSUPPORTED;
@@ -146,7 +160,7 @@ int32_t heads_fwd(const m2_plan* pl, const void* X1, const void* X2, const void*
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, heads_kernel, (const __nv_bfloat16*)X1, (const __nv_bfloat16*)X2, (const __nv_bfloat16*)V, kt,
+    if (cudaLaunchKernelEx(&cfg, heads_kernel, (const __nv_bfloat16*)X1, (const __nv_bfloat16*)X2, (const __nv_bfloat16*)V, kt, (int)period,
                            (__nv_bfloat16*)O, (int)(d / kDh), (int)n) != cudaSuccess)
         return M2_ERR_CUDA;
     pl->launches += 1;

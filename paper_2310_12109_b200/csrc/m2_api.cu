@@ -284,7 +284,7 @@ int32_t m2_monarch_conv_bwd_kernel(const m2_plan* plan, const void* x_dev, const
         int parts = 0;
         st = m2u::conv_wgrad_partials(plan, x_dev, g_dev, ws_dev, B, H, n, mode, &parts, (cudaStream_t)stream);
         if (st == M2_OK) {
-            if (m2f::time_kernel(plan, ws_dev, parts, 1.0f / (float)plan->N, H, n, dk_dev, (cudaStream_t)stream) != cudaSuccess)
+            if (m2f::time_kernel(plan, ws_dev, parts, 1.0f / (float)plan->N, H, n, false, dk_dev, (cudaStream_t)stream) != cudaSuccess)
                 return M2_ERR_CUDA;
             plan->launches += 1;
             plan->last_kernel = "conv_wgrad_umma_o2_512";
@@ -694,10 +694,12 @@ int32_t m2_hyena_heads_fwd(const m2_plan* plan, const void* u_dev, const void* c
     unsigned char* sc = static_cast<unsigned char*>(scratch_dev);
     void *uT = sc, *P1 = sc + tb, *P2 = sc + 2 * tb, *P3 = sc + 3 * tb, *C1 = sc + 4 * tb, *C2 = sc + 5 * tb, *C3 = sc + 6 * tb;
     void *XV = sc + 7 * tb, *XVc = sc + (7 + dh) * tb;
-    // the fused head product wants the long kernels in the time domain, [d / dh][n] fp32: they wait in y, which is written last
-    float* kt = static_cast<float*>(y_dev);
-    if (hyena_heads_fused(plan, n, d, dh)) {
-        if (m2f::time_kernel(plan, kf_long_dev, 1, 1.0f, d / dh, n, kt, st) != cudaSuccess) return M2_ERR_CUDA;
+    // the fused head product wants the long kernels in the time domain, fp32, lags of either sign: part of the spectrum of short plans,
+    // otherwise [d / dh][2 n] values that wait in y, which is written last
+    const float* kt = m2t::has_time_kernel(plan) ? m2t::time_kernel(plan, kf_long_dev, d / dh) : static_cast<const float*>(y_dev);
+    const int64_t period = m2t::has_time_kernel(plan) ? plan->N : 2 * n;
+    if (hyena_heads_fused(plan, n, d, dh) && !m2t::has_time_kernel(plan)) {
+        if (m2f::time_kernel(plan, kf_long_dev, 1, 1.0f, d / dh, n, true, static_cast<float*>(y_dev), st) != cudaSuccess) return M2_ERR_CUDA;
         plan->launches += 1;
     }
     // channel-first from here on: every projection, convolution and head product works on rows of n positions
@@ -717,7 +719,7 @@ int32_t m2_hyena_heads_fwd(const m2_plan* plan, const void* u_dev, const void* c
     }
     if (rc != M2_OK) return rc;
     if (hyena_heads_fused(plan, n, d, dh)) {
-        rc = m2h::heads_fwd(plan, C1, C2, C3, kt, P1, B, d, n, st);
+        rc = m2h::heads_fwd(plan, C1, C2, C3, kt, period, P1, B, d, n, st);
         if (rc != M2_OK) return rc;
     } else {
         if (m2g::launch_heads_outer(C2, C3, XV, B, (int)d, (int)dh, (int)n, bf, st) != cudaSuccess) return M2_ERR_CUDA;

@@ -918,6 +918,38 @@ def test_hyena_head_product_tiles(B, n, d, dims):
     plan.close()
 
 
+@pytest.mark.parametrize("B,n,d,dims,long_kernel", [(2, 256, 32, (32, 16), "conjugated"), (1, 77, 64, (32, 16), "full"), (3, 100, 16, (16, 16), "full"),
+                                                     (1, 512, 32, (32, 32), "conjugated"), (2, 200, 32, (64, 64), "full"), (1, 1000, 16, (64, 32), "conjugated")])
+def test_hyena_head_product_with_lags_below_zero(B, n, d, dims, long_kernel):
+    """Long kernels that reach backwards: a conjugated spectrum (the transposed convolution) and a kernel as long as the plan.  The fused
+    head product multiplies by the same circular kernel as the convolutions do."""
+    if 2 * n > int(np.prod(dims)):
+        n = int(np.prod(dims)) // 2
+    N, heads = int(np.prod(dims)), d // 16
+    u = synth.round_bf16(synth.normal(synth.stream_id(20, n), (B, n, d)))
+    delta = np.zeros((d, n), dtype=np.float32)
+    delta[:, 0] = 1.0
+    plan = M.Plan(dims, dtype=M.M2_BF16, device=0)
+    kfd = M.m2_kernel_spectrum(plan, dev(delta))
+    k = np.zeros((heads, N), dtype=np.float32)
+    m = N if long_kernel == "full" else n
+    k[:, :m] = synth.normal(synth.stream_id(20, n + 1), (heads, m)) / np.sqrt(n)
+    kfl = M.m2_kernel_spectrum(plan, dev(k[:, :m]))
+    if long_kernel == "conjugated":
+        kfl = M.m2_spectrum_conjugate(plan, kfl, heads)
+        k = np.roll(k[:, ::-1], 1, axis=1)
+    eye = torch.eye(d, dtype=torch.bfloat16, device="cuda")
+    y = M.m2_hyena_heads_fwd(plan, dev(u.astype(np.float32), torch.bfloat16), [eye] * 4, kfd, kfd, kfd, kfl, 16)
+    torch.cuda.synchronize()
+    assert plan.device_status() == 0 and plan.last_kernel() == "hyena_heads_fwd_fused"
+    uh = u.astype(np.float64).reshape(B, n, heads, 16)
+    T = k.astype(np.float64)[:, (np.arange(n)[:, None] - np.arange(n)[None]) % N]   # [heads, t, s]
+    want = np.einsum("hts,bths,bshj->bthj", T, np.einsum("bthi,bshi->bths", uh, uh), uh, optimize=True).reshape(B, n, d)
+    got = host(y)   # weighed scores and the result are rounded to bf16, the unit-kernel convolutions round too
+    assert np.linalg.norm(got - want) <= TOL_BF16 / 2 * np.linalg.norm(want)
+    plan.close()
+
+
 def test_m2_hyena_heads_full_size_sampled():
     """The layer at the benchmark shape (B = 32, n = 256, d = 768, heads of 16: 24 576 units of the fused kernel, many rounds per
     pipeline); batch entries are independent, so the first and the last one are compared with the oracle run on them alone."""
