@@ -628,7 +628,7 @@ int32_t m2_bert_mixer_fwd(const m2_plan* plan, const void* x_dev, const void* co
     for (int i = 0; i < 3; ++i)
         if (!w_short[i]) return M2_ERR_INVALID_ARG;
     if (!x_dev || !kf_dev || !kf_res_dev || !y_dev || !scratch_dev) return M2_ERR_INVALID_ARG;
-    if (!aligned16(x_dev) || !aligned16(y_dev) || !aligned16(scratch_dev)) return M2_ERR_ALIGNMENT;
+    if (!aligned16(x_dev) || !aligned16(y_dev) || !aligned16(scratch_dev) || !aligned16(kf_dev) || !aligned16(kf_res_dev)) return M2_ERR_ALIGNMENT;
     if (scratch_bytes < m2_bert_mixer_scratch_bytes(plan, B, d)) return M2_ERR_INVALID_ARG;
     DeviceGuard g(plan->device);
     if (!g.ok) return M2_ERR_CUDA;
@@ -684,7 +684,9 @@ int32_t m2_hyena_heads_fwd(const m2_plan* plan, const void* u_dev, const void* c
     for (int i = 0; i < 4; ++i)
         if (!W[i] || !aligned16(W[i])) return W[i] ? M2_ERR_ALIGNMENT : M2_ERR_INVALID_ARG;
     if (!u_dev || !kf1_dev || !kf2_dev || !kf3_dev || !kf_long_dev || !y_dev || !scratch_dev) return M2_ERR_INVALID_ARG;
-    if (!aligned16(u_dev) || !aligned16(y_dev) || !aligned16(scratch_dev)) return M2_ERR_ALIGNMENT;
+    if (!aligned16(u_dev) || !aligned16(y_dev) || !aligned16(scratch_dev) || !aligned16(kf1_dev) || !aligned16(kf2_dev) || !aligned16(kf3_dev) ||
+        !aligned16(kf_long_dev))
+        return M2_ERR_ALIGNMENT;
     if (scratch_bytes < m2_hyena_scratch_bytes(plan, B, n, d, dh)) return M2_ERR_INVALID_ARG;
     DeviceGuard g(plan->device);
     if (!g.ok) return M2_ERR_CUDA;

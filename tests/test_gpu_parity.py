@@ -950,6 +950,25 @@ def test_hyena_head_product_with_lags_below_zero(B, n, d, dims, long_kernel):
     plan.close()
 
 
+def test_layers_refuse_misaligned_spectra():
+    """Every spectrum of the Hyena layer and of the M2-BERT mixer is read in 16-byte pieces on some route: an address off that boundary is
+    refused before anything is enqueued, whichever route the shape takes."""
+    lib, s, d, n, B = M.lib(), torch.cuda.current_stream().cuda_stream, 32, 256, 1
+    buf = torch.zeros(1 << 22, dtype=torch.uint8, device="cuda")
+    p = buf.data_ptr()
+    W, w3 = (ctypes.c_void_p * 4)(p, p, p, p), (ctypes.c_void_p * 3)(p, p, p)
+    for dims, dtype in (((32, 16), M.M2_BF16), ((32, 32), M.M2_BF16), ((32, 16), M.M2_FP32)):
+        plan = M.Plan(dims, dtype=dtype, device=0)
+        for bad in range(4):
+            kf = [p + 4 * (i == bad) for i in range(4)]
+            st = lib.m2_hyena_heads_fwd(plan.handle, p, W, *kf, p, B, n, d, 16, p, buf.numel(), s)
+            assert st == M.M2_ERR_ALIGNMENT and plan.launch_count() == 0
+        for bad in range(2):
+            st = lib.m2_bert_mixer_fwd(plan.handle, p, W, w3, p + 8 * (bad == 0), p + 8 * (bad == 1), p, B, d, p, buf.numel(), s)
+            assert st == M.M2_ERR_ALIGNMENT and plan.launch_count() == 0
+        plan.close()
+
+
 def test_m2_hyena_heads_full_size_sampled():
     """The layer at the benchmark shape (B = 32, n = 256, d = 768, heads of 16: 24 576 units of the fused kernel, many rounds per
     pipeline); batch entries are independent, so the first and the last one are compared with the oracle run on them alone."""
