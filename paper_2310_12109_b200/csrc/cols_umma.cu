@@ -277,7 +277,6 @@ static int32_t stage(const m2_plan* pl, int64_t N, const void* W, const void* V,
         g.k = b;
         g.kmul = {Kmul, d, b, so * d, nb, d, 1, 0};
         g.relu = relu;
-        pl->launches -= 1;   // (the caller counts its stages)
         return gemm_pair(pl, g, stream);
     }
     const int m = b == 64 ? 64 : 128;
@@ -318,6 +317,7 @@ static int32_t stage(const m2_plan* pl, int64_t N, const void* W, const void* V,
     if (cudaLaunchKernelEx(&cfg, monarch_cols_stage_kernel, mw, mv, mo, (const __nv_bfloat16*)Kmul, relu, b, nb, (int)so, (int)d, nc, m,
                            (int)tiles, pl->d_status) != cudaSuccess)
         return M2_ERR_CUDA;
+    pl->launches += 1;
     return M2_OK;
 }
 
@@ -333,7 +333,6 @@ int32_t apply(const m2_plan* pl, const void* X, const void* L, const void* R, co
     st = stage(pl, pl->N, L, ws, Y, Kmul, relu, Bt, d, N2, N1, 1, N2, N1, stream);           // y[k2*N1 + k1]: N1 blocks L[k1] on the rows k1*N2 + n2
     if (st != M2_OK) return st;
     pl->last_kernel = "monarch_cols_umma";
-    pl->launches += 2;
     return M2_OK;
 }
 

@@ -950,6 +950,25 @@ def test_hyena_head_product_with_lags_below_zero(B, n, d, dims, long_kernel):
     plan.close()
 
 
+@pytest.mark.parametrize("dims", [(64, 64), (128, 256), (256, 256)])
+def test_monarch_cols_counts_what_it_launches(dims):
+    """Two launches a call whichever kernel a stage takes; a call that is refused (more tiles than the kernel can number, and too long for the
+    CUDA-core kernel) launches nothing and counts nothing."""
+    N, d = int(np.prod(dims)), 64
+    plan = M.Plan(dims, dtype=M.M2_BF16, device=0)
+    buf = torch.zeros(1, N, d, dtype=torch.bfloat16, device="cuda")
+    w = torch.zeros(max(dims) ** 3, dtype=torch.bfloat16, device="cuda")
+    L, R = w[:dims[0] * dims[1] ** 2].view(dims[0], dims[1], dims[1]), w[:dims[1] * dims[0] ** 2].view(dims[1], dims[0], dims[0])
+    M.m2_monarch_cols(plan, buf, L, R)
+    torch.cuda.synchronize()
+    assert plan.device_status() == 0 and plan.launch_count() == 2
+    if dims == (256, 256):
+        p = buf.data_ptr()
+        st = M.lib().m2_monarch_cols(plan.handle, p, p, p, None, 0, p, 1, 0x7ffffff8, p, 1 << 50, torch.cuda.current_stream().cuda_stream)
+        assert st == M.M2_ERR_UNSUPPORTED and plan.launch_count() == 2
+    plan.close()
+
+
 def test_layers_refuse_misaligned_spectra():
     """Every spectrum of the Hyena layer and of the M2-BERT mixer is read in 16-byte pieces on some route: an address off that boundary is
     refused before anything is enqueued, whichever route the shape takes."""
