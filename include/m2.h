@@ -379,7 +379,8 @@ const char* m2_status_string(int32_t status);
 int32_t m2_last_device_status(const m2_plan* plan, int32_t* out);
 
 /* Which implementation the last hot call on this plan dispatched to (a static string such as
- * "conv_generic_fp32" or "conv_umma_o2"); for tests and the benchmark's report. */
+ * "conv_fft_fp32" or "conv_umma_o2_512_pairs"); for tests and the benchmark's report.  ("conv_wgrad_generic" is every kernel gradient
+ * in fp32, by the transform kernels for powers of two from 256 to 8192 and by the dense stages otherwise.) */
 const char* m2_last_kernel_name(const m2_plan* plan);
 
 /* Number of kernels the library has launched on this plan since creation. */

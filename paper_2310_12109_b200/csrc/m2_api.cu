@@ -245,7 +245,7 @@ int32_t m2_kernel_spectrum(const m2_plan* plan, const float* k_dev, int64_t H, i
     if (e == cudaErrorInvalidValue) return M2_ERR_UNSUPPORTED;
     if (e != cudaSuccess) return M2_ERR_CUDA;
     if (m2u::relayout_spectrum(plan, kf_dev, H, (cudaStream_t)stream) != cudaSuccess) return M2_ERR_CUDA;
-    plan->last_kernel = "spectrum_generic_fp32";
+    plan->last_kernel = m2f::covered(plan) ? "spectrum_fft_fp32" : "spectrum_generic_fp32";
     plan->launches += (H > 0) * (m2u::has_private_spectrum(plan) && !priv512 ? 2 : 1);
     return M2_OK;
 }
@@ -356,7 +356,8 @@ static int32_t conv_fwd_grouped(const m2_plan* plan, const void* x_dev, const vo
                               : m2g::launch_conv(s, plan->dtype == M2_BF16, x_dev, kf_dev, y_dev, nullptr, (cudaStream_t)stream);
     if (e == cudaErrorInvalidValue) return M2_ERR_UNSUPPORTED;
     if (e != cudaSuccess) return M2_ERR_CUDA;
-    plan->last_kernel = plan->dtype == M2_BF16 ? "conv_generic_bf16io" : "conv_generic_fp32";
+    const bool bf = plan->dtype == M2_BF16;
+    plan->last_kernel = m2f::covered(plan) ? (bf ? "conv_fft_bf16io" : "conv_fft_fp32") : (bf ? "conv_generic_bf16io" : "conv_generic_fp32");
     plan->launches += 1;
     return M2_OK;
 }

@@ -200,6 +200,20 @@ def test_kernel_gradient_adds_its_parts(B, H, n, causal):
     plan.close()
 
 
+@pytest.mark.parametrize("dims,n,dtype,want", [((16, 16), 256, M.M2_FP32, "fft_fp32"), ((16, 16), 256, M.M2_BF16, "fft_bf16io"), ((16, 32), 512, M.M2_BF16, "fft_bf16io"),
+                                               ((128, 128), 16384, M.M2_FP32, "fft_fp32"), ((16, 8), 128, M.M2_FP32, "generic_fp32"),
+                                               ((16, 8), 128, M.M2_BF16, "generic_bf16io"), ((3, 100), 300, M.M2_FP32, "generic_fp32")])
+def test_which_fp32_kernels_run(dims, n, dtype, want):
+    """The transform kernels answer with names of their own, so that a plan that falls back to the dense stages shows."""
+    plan = M.Plan(dims, dtype=dtype, device=0)
+    kf = M.m2_kernel_spectrum(plan, torch.ones(2, n, device="cuda"))
+    assert plan.last_kernel() == "spectrum_" + want.split("_")[0] + "_fp32"
+    M.m2_monarch_conv_fwd(plan, torch.ones(1, 2, n, device="cuda", dtype=plan.torch_dtype), kf, M.M2_CIRCULAR)
+    torch.cuda.synchronize()
+    assert plan.device_status() == 0 and plan.last_kernel() == "conv_" + want
+    plan.close()
+
+
 @pytest.mark.parametrize("n,causal,B", [(1024, False, 3), (1024, False, 2), (512, True, 5), (510, True, 3)])
 def test_bf16_rows_of_32_point_columns(n, causal, B):
     """N = 1024 in bf16: whole rows (loaded without a bound) and shorter ones, batches with and without a second row in the last pair."""
