@@ -146,53 +146,58 @@ int32_t m2_plan_create(m2_plan** out, int64_t N, int32_t p, const int32_t* facto
     if (prod != N) return M2_ERR_INVALID_ARG;
     m2_plan* pl = new (std::nothrow) m2_plan();
     if (!pl) return M2_ERR_INVALID_ARG;
-    pl->N = N;
-    pl->p = p;
-    for (int a = 0; a < p; ++a) pl->dims[a] = factors[a];
-    pl->dtype = dtype;
-    pl->sign = sign;
-    pl->device = device;
-    build_tables(pl);
-    if (device >= 0) {
-        DeviceGuard g(device);
-        bool ok = g.ok;
-        // one device block, one copy: status word | roots of every factor | twiddle factors of the fp32 transform kernels
-        const std::vector<float4>* fft = m2f::host_table(pl);
-        size_t off_roots[4], bytes = 256;
-        for (int a = 0; a < p; ++a) {
-            off_roots[a] = bytes;
-            bytes += ((size_t)pl->dims[a] * sizeof(float2) + 255) / 256 * 256;
-        }
-        const size_t off_fft = bytes;
-        if (fft) bytes += fft->size() * sizeof(float4);
-        std::vector<unsigned char> block(bytes, 0);
-        for (int a = 0; a < p; ++a) {
-            const int Na = pl->dims[a];
-            float2* r = reinterpret_cast<float2*>(block.data() + off_roots[a]);
-            for (int j = 0; j < Na; ++j) {
-                const double ang = 2.0 * M_PI * (double)j / (double)Na;
-                r[j] = make_float2((float)std::cos(ang), (float)(sign * std::sin(ang)));
+    try {   // (host tables are vectors: no exception leaves the library)
+        pl->N = N;
+        pl->p = p;
+        for (int a = 0; a < p; ++a) pl->dims[a] = factors[a];
+        pl->dtype = dtype;
+        pl->sign = sign;
+        pl->device = device;
+        build_tables(pl);
+        if (device >= 0) {
+            DeviceGuard g(device);
+            bool ok = g.ok;
+            // one device block, one copy: status word | roots of every factor | twiddle factors of the fp32 transform kernels
+            const std::vector<float4>* fft = m2f::host_table(pl);
+            size_t off_roots[4], bytes = 256;
+            for (int a = 0; a < p; ++a) {
+                off_roots[a] = bytes;
+                bytes += ((size_t)pl->dims[a] * sizeof(float2) + 255) / 256 * 256;
+            }
+            const size_t off_fft = bytes;
+            if (fft) bytes += fft->size() * sizeof(float4);
+            std::vector<unsigned char> block(bytes, 0);
+            for (int a = 0; a < p; ++a) {
+                const int Na = pl->dims[a];
+                float2* r = reinterpret_cast<float2*>(block.data() + off_roots[a]);
+                for (int j = 0; j < Na; ++j) {
+                    const double ang = 2.0 * M_PI * (double)j / (double)Na;
+                    r[j] = make_float2((float)std::cos(ang), (float)(sign * std::sin(ang)));
+                }
+            }
+            if (fft) std::memcpy(block.data() + off_fft, fft->data(), fft->size() * sizeof(float4));
+            if (ok) ok = cudaMalloc(&pl->d_block, bytes) == cudaSuccess;
+            if (ok) ok = cudaMemcpy(pl->d_block, block.data(), bytes, cudaMemcpyHostToDevice) == cudaSuccess;
+            if (ok) {
+                unsigned char* base = static_cast<unsigned char*>(pl->d_block);
+                pl->d_status = reinterpret_cast<int32_t*>(base);
+                for (int a = 0; a < p; ++a) pl->d_roots[a] = reinterpret_cast<float2*>(base + off_roots[a]);
+                if (fft) pl->d_fft = reinterpret_cast<float4*>(base + off_fft);
+                ok = m2f::prepare(pl) == cudaSuccess;
+            }
+            if (ok) ok = m2u::create_tables(pl) == cudaSuccess;
+            if (ok) ok = m2u3::create_tables(pl) == cudaSuccess;
+            if (ok) ok = m2mm::prepare(pl) == cudaSuccess;
+            if (ok) ok = cudaDeviceSynchronize() == cudaSuccess;
+            if (!ok) {
+                cudaGetLastError();
+                m2_plan_destroy(pl);
+                return M2_ERR_CUDA;
             }
         }
-        if (fft) std::memcpy(block.data() + off_fft, fft->data(), fft->size() * sizeof(float4));
-        if (ok) ok = cudaMalloc(&pl->d_block, bytes) == cudaSuccess;
-        if (ok) ok = cudaMemcpy(pl->d_block, block.data(), bytes, cudaMemcpyHostToDevice) == cudaSuccess;
-        if (ok) {
-            unsigned char* base = static_cast<unsigned char*>(pl->d_block);
-            pl->d_status = reinterpret_cast<int32_t*>(base);
-            for (int a = 0; a < p; ++a) pl->d_roots[a] = reinterpret_cast<float2*>(base + off_roots[a]);
-            if (fft) pl->d_fft = reinterpret_cast<float4*>(base + off_fft);
-            ok = m2f::prepare(pl) == cudaSuccess;
-        }
-        if (ok) ok = m2u::create_tables(pl) == cudaSuccess;
-        if (ok) ok = m2u3::create_tables(pl) == cudaSuccess;
-        if (ok) ok = m2mm::prepare(pl) == cudaSuccess;
-        if (ok) ok = cudaDeviceSynchronize() == cudaSuccess;
-        if (!ok) {
-            cudaGetLastError();
-            m2_plan_destroy(pl);
-            return M2_ERR_CUDA;
-        }
+    } catch (...) {
+        m2_plan_destroy(pl);
+        return M2_ERR_INVALID_ARG;
     }
     *out = pl;
     return M2_OK;

@@ -3,6 +3,8 @@ bit-exact integer tables, and rejects bad arguments before touching a device."""
 import ctypes
 import os
 import re
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -103,3 +105,22 @@ def test_matmul_workspace_covers_whole_token_tiles():
         assert int(lib.m2_matmul_workspace_bytes(pl.handle, T)) == tiles * 128 * 4096 * 2
     assert int(lib.m2_matmul_workspace_bytes(host_plan((8, 8)).handle, 100)) == 0
     assert int(lib.m2_matmul_workspace_bytes(host_plan((64, 64)).handle, 100)) == 0   # fp32 plan: CUDA-core kernels
+
+
+def test_plan_creation_out_of_memory_is_a_status():
+    """No exception leaves the library: a plan whose host tables do not fit (address space limited to 150 MB more than the process has;
+    N = 2^24 wants four tables of 64 MB) is refused with a status, and the library goes on working."""
+    code = f"""
+import ctypes, resource
+lib = ctypes.CDLL({M.lib()._name!r})
+h, f = ctypes.c_void_p(), (ctypes.c_int32 * 2)(4096, 4096)
+lib.m2_plan_create.argtypes = [ctypes.c_void_p, ctypes.c_int64, ctypes.c_int32, ctypes.c_void_p] + [ctypes.c_int32] * 3
+lib.m2_plan_destroy.argtypes = [ctypes.c_void_p]
+used = int(open("/proc/self/statm").read().split()[0]) * resource.getpagesize()
+resource.setrlimit(resource.RLIMIT_AS, (used + (150 << 20), resource.getrlimit(resource.RLIMIT_AS)[1]))
+assert lib.m2_plan_create(ctypes.byref(h), 1 << 24, 2, f, 0, 1, -1) == {M.M2_ERR_INVALID_ARG} and not h.value
+assert lib.m2_plan_create(ctypes.byref(h), 512, 2, (ctypes.c_int32 * 2)(32, 16), 0, 1, -1) == {M.M2_OK}
+assert lib.m2_plan_destroy(h) == {M.M2_OK}
+"""
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True)
+    assert r.returncode == 0, (r.returncode, r.stderr[-500:])
