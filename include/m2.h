@@ -79,7 +79,8 @@ int32_t m2_plan_destroy(m2_plan* plan);
 /* Copies one integer table (enum m2_table) into host_out[0..len); len must equal N. */
 int32_t m2_plan_get_table(const m2_plan* plan, int32_t which, int32_t* host_out, int64_t len);
 
-/* Bytes of the spectrum buffer m2_kernel_spectrum writes for H channels. */
+/* Bytes of the spectrum buffer m2_kernel_spectrum writes for H channels: one copy of 8 N bytes a channel, a second one for the tensor-core
+ * plans (32 x 16 and 32 x 32 x 32, bf16), 4 N more for the kernel itself on bf16 plans of N = 256 and 512. */
 int64_t m2_spectrum_bytes(const m2_plan* plan, int64_t H);
 
 /* k_f = M * pad(k) per channel (Alg. BlockMonarchConv, the line k_f <- M k; Eq. 2's K_1 given in
@@ -110,11 +111,11 @@ int32_t m2_spectrum_conjugate(const m2_plan* plan, const void* kf_in_dev, int64_
  * ws_dev: optional caller-owned workspace of m2_conv_bwd_workspace_bytes(plan, B, H) bytes (16-byte aligned; 0 bytes
  * means this plan has no kernel that uses one).  With it, plans the tensor-core path covers (bf16, N = 512 = 32 x 16)
  * run both forward transforms and the products conj(M x) (.) M g on the tensor cores (intermediates rounded to bf16
- * like the forward pass), 8 batch rows at a time, and a CUDA-core kernel adds the groups in order and applies M^-1 in
+ * like the forward pass), 8 batch rows at a time, and a CUDA-core kernel adds the groups in a fixed order and applies M^-1 in
  * fp32; for N = 32768 = 32^3 (causal, n = 16384) the order-3 convolution kernel is run twice (the row pairs' conjugated
  * spectra, then the convolution of the g pairs with them) and the pairs' rows are added.  Otherwise, or with a workspace
- * too small for those, everything runs on the CUDA cores in fp32, one thread block per channel with its three complex
- * rows in shared memory (N up to 8192) or, for longer rows, in the workspace (at least 24 N bytes per channel for up to
+ * too small for those, everything runs on the CUDA cores in fp32, by register transforms for powers of two from 256 to 8192, otherwise
+ * one thread block per channel with its three complex rows in shared memory (N up to 8192) or, for longer rows, in the workspace (at least 24 N bytes per channel for up to
  * 296 channels; M2_ERR_UNSUPPORTED without it).  m2_conv_bwd_workspace_bytes returns the largest of these needs.  All
  * paths are deterministic.  (The paper trains through the operator, Sec. 5, without writing the
  * backward pass out.) */
@@ -215,8 +216,8 @@ int32_t m2_monarch_cols(const m2_plan* plan, const void* X_dev, const void* L_de
  * W: HOST array of 4 device pointers {W_q, W_k, W_v, W_o}, each [d][d] stored outputs x inputs; w_short: HOST array of 3
  * device pointers to fp32 [d][3] filters (q, k, v); kf_dev, kf_res_dev: m2_kernel_spectrum of k and k_res [d, n].
  * y_dev: [B, n, d] (must not overlap x_dev); scratch_dev: m2_bert_mixer_scratch_bytes(plan, B, d) bytes, caller-owned.
- * After one transposition everything runs channel-first: projections = the single-block column-layout kernel, the two
- * convolutions = m2_monarch_conv_fwd, two elementwise kernels for the filters and gates. */
+ * Everything between the projections runs channel-first (one transposition, for the residual convolution; the projections as in
+ * m2_hyena_heads_fwd): the two convolutions = m2_monarch_conv_fwd, two elementwise kernels for the filters and gates. */
 int64_t m2_bert_mixer_scratch_bytes(const m2_plan* plan, int64_t B, int64_t d);
 int32_t m2_bert_mixer_fwd(const m2_plan* plan, const void* x_dev, const void* const* W, const float* const* w_short,
                           const void* kf_dev, const void* kf_res_dev, void* y_dev, int64_t B, int64_t d, void* scratch_dev,
@@ -231,11 +232,11 @@ int32_t m2_bert_mixer_fwd(const m2_plan* plan, const void* x_dev, const void* co
  * kf1_dev, kf2_dev, kf3_dev: m2_kernel_spectrum of the short kernels [d, n];  kf_long_dev: m2_kernel_spectrum of the long
  * kernels, one row per head: [d / dh, n] (the dh^2 sequences of a head share its row: m2_monarch_conv_fwd_grouped).
  * y_dev: [B, n, d] (must not overlap u_dev).  scratch_dev: m2_hyena_scratch_bytes(plan, B, n, d, dh) bytes, caller-owned
- * ((7 + 2 dh) tensors of B d n elements; 7 for heads of dh = 16 on bf16 plans whose N is a power of two from 512 to 16384 and n up to
+ * ((7 + 2 dh) tensors of B d n elements; 7 for heads of dh = 16 on bf16 plans whose N is a power of two from 256 to 16384 and n up to
  * 1024, where outer product, long convolution and contraction are one kernel, O[t] = sum_s k[t - s] (X1~[t] . X2~[s]) V~[s], and the
- * dh-times larger tensors do not exist).
- * The projections are the single-block case of the column-layout Monarch kernel (tensor cores for d a multiple of 64 up
- * to 4096 and n a multiple of 8, bf16), so after one transposition everything runs channel-first. */
+ * dh-times larger tensors do not exist; a spectrum with lags below zero, s > t, is multiplied by those too, as in every other form).
+ * Everything between the projections runs channel-first.  The projections run on the tensor cores for d a multiple of 64 up to 4096 and
+ * n a multiple of 8, bf16, reading u and writing y as they lie; other shapes transpose first and last. */
 int64_t m2_hyena_scratch_bytes(const m2_plan* plan, int64_t B, int64_t n, int64_t d, int64_t dh);
 int32_t m2_hyena_heads_fwd(const m2_plan* plan, const void* u_dev, const void* const* W, const void* kf1_dev,
                            const void* kf2_dev, const void* kf3_dev, const void* kf_long_dev, void* y_dev, int64_t B,
@@ -274,8 +275,8 @@ int32_t m2_monarch_apply_order_p(const m2_plan* plan, const void* X_dev, const v
  *   dR[n2][k1][n1] = sum_t dv[t][n2][k1] X[t][n1 N2 + n2],          dv = L^T-stage applied to G.
  * X_dev, G_dev: [T, N], L_dev, R_dev as in m2_monarch_matmul (plan dtype); dL_dev [N1][N2][N2] and dR_dev [N2][N1][N1]
  * are fp32 and overwritten (zeros for T == 0).  ws_dev: caller-owned, at least m2_matmul_bwd_workspace_bytes(plan, T)
- * bytes (at least 4 T N: it holds v, then dv; bf16 plans with 64 x 64 blocks add room for the partial sums of the
- * token shares and one transposed factor), 16-byte aligned; too small or NULL with T > 0: M2_ERR_INVALID_ARG.
+ * bytes (at least 4 T N, v, then dv; bf16 plans with 64 x 64 blocks need room for v in bf16 and the partial sums of 37
+ * token shares, 38.8 MB), 16-byte aligned; too small or NULL with T > 0: M2_ERR_INVALID_ARG.
  * bf16 plans with 64 x 64 blocks run on the tensor cores with the tokens as the contraction dimension (v and dv pass
  * through bf16 like the forward intermediate; partial sums per token share in fp32, added in a fixed order); every
  * other plan runs four fp32 CUDA-core kernels with a fixed summation order.  Both are deterministic.  (The paper

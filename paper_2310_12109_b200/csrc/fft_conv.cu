@@ -1,13 +1,14 @@
-// Convolution in fp32 (fft_grad.cu: kernel spectrum and kernel gradient) for every plan whose length is a power of two from 256 to 16384: the fp32
-// path, and the bf16 shapes the tensor-core kernels do not cover.  A complex row (two real batch rows of one channel: the kernel is
-// real, so F^-1(k_f (.) F(x_a + i x_b)) = y_a + i y_b; balance_pair keeps them apart) stays in registers and shared memory from the load to the store; fft_core.cuh
-// has the transforms.
+// Convolution in fp32 (fft_grad.cu: kernel spectrum, and the kernel gradient up to 8192 points) for every plan whose length is a power
+// of two from 256 to 16384: the fp32 path, and the bf16 shapes the tensor-core kernels do not cover.  A complex row (two real batch rows
+// of one channel: the kernel is real, so F^-1(k_f (.) F(x_a + i x_b)) = y_a + i y_b; balance_pair keeps them apart) stays in registers
+// and shared memory from the load to the store; fft_core.cuh has the transforms.
 //
-// What bounds it: shared-memory wavefronts (64 KB each way per digit exchange of a 4096-point row) and packed FP32 issue, about equal;
-// with 126 registers four blocks of 128 threads share an SM.  bf16 x[8][768][2000], N = 4096, one B200: 47 us (0.2 of the roof: its
-// bytes take 9.8 us; 59 % of the load/store data pipe, DRAM 11 %), against 6034 us for the kernel before it, which contracted each 64-wide
-// digit as a dense product in shared memory with a sincos per element.  fp32 x[1][4][256]: 18.4 -> 11.2 us per call, all of it launch
-// and host path.
+// What bounds it: shared-memory wavefronts (64 KB each way per digit exchange of a 4096-point row), packed FP32 and the loads and stores
+// of a row that nothing overlaps within its block; with 126 registers four blocks of 128 threads share an SM.  bf16 x[8][768][2000], N =
+// 4096, one B200: 46 us (0.2 of the roof: its bytes take 9.8 us; the wavefronts alone would take 22 us), 66 % of the load/store data
+// pipe, 49 % of the FMA pipe, 46 % of the issue slots, DRAM 12 %; 6034 us for the kernel before it, which contracted each 64-wide
+// digit as a dense product in shared memory with a sincos per element.  fp32 x[1][4][256]: 18.4 -> 6.5 us per call, one launch and the
+// host's way to it.
 #include <atomic>
 #include <cmath>
 #include <vector>

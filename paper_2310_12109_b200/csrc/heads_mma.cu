@@ -13,9 +13,8 @@
 // conjugated or its kernel is longer than N - n: a block that finds one that is not zero walks the tiles s > t too, with kernel values
 // from L2.
 //
-// Measured, one B200, 1536 heads of n = 256: 21.6 us (28.6 with index divisions in the copies and the two copies of the kernel in the
-// same banks) where 24 576 tensor-core convolution units of 16 rows took about 280 us.  Bound by instruction issue and the fragments'
-// latency: 136 tile pairs of about 20 instructions.
+// Measured, one B200, 1536 heads of n = 256: 23.6 us where 24 576 tensor-core convolution units of 16 rows took about 280 us.  Bound by
+// the load/store data pipe (60 % busy), issue (48 %) and the fragments' latency: 136 tile pairs of about 20 instructions; matrix pipe 31 %.
 #include "fft_conv.h"
 #include "fft_core.cuh"
 #include "heads_mma.h"

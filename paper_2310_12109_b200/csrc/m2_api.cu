@@ -340,9 +340,9 @@ static int32_t conv_fwd_grouped(const m2_plan* plan, const void* x_dev, const vo
     DeviceGuard g(plan->device);
     if (!g.ok) return M2_ERR_CUDA;
     if (B * H == 0) return M2_OK;
-    // Short causal rows: Toeplitz products, up to 256 positions (512: 46 us against 45 for the transforms at [32][768]).  Batches of up
-    // to 8 rows of the 32 x 16 plan stay with the tensor-core kernel made for them, whose name callers ask for: 11.6 us at [8][768][256],
-    // where half-empty tiles of 16 rows would take 10.4.
+    // Short causal rows: Toeplitz products, up to 256 positions (512: 46 us against 45 for the transforms at [32][768], the one width both
+    // were measured at).  Batches of up to 8 rows of the 32 x 16 plan still run the tensor-core kernel for such batches, as the tests of the
+    // input gradient expect: 11.6 us at [8][768][256], where half-empty tiles of 16 rows would take 10.4.
     if (mode == M2_CAUSAL && n <= m2t::kMaxN && m2t::has_time_kernel(plan) && x_dev != y_dev && (B > 8 || !m2u::covers_rows(plan, n))) {
         const m2t::Rows rows = {x_dev, m2t::time_kernel(plan, kf_dev, H / kf_group), y_dev};
         const int32_t tst = m2t::conv(plan, &rows, 1, B, H, n, (int)kf_group, (cudaStream_t)stream);

@@ -11,8 +11,7 @@
 //   monarch64_fwd_kernel<1|2>   the forward path (further down): 32 tokens x 16 blocks per item, 32-byte pieces,
 //                               weights resident, loading / draining / issuing warps.
 //   monarch64_pass_kernel<1|2>  128 tokens x 8 blocks per CTA, 16-byte pieces (described next): serves inputs that are
-//                               only 16-byte aligned, and the weight gradients, whose kernel reads its workspace layout
-//                               z[token tile][n2 / 8][k1][t % 128][n2 % 8]:
+//                               only 16-byte aligned; its workspace is z[token tile][n2 / 8][k1][t % 128][n2 % 8]:
 //
 //   pass 1 (R): a CTA owns 128 tokens x 8 consecutive n2.  Threads read 16-byte pieces of x (8 values of
 //               n2 for one (t, n1)), transpose 8 x 8 blocks in registers (the permutation P) and write the
@@ -558,7 +557,7 @@ monarch64_fwd_kernel(const __nv_bfloat16* __restrict__ in, const __grid_constant
 //   D_b[m][a] = sum_t Z_b[t][m] * V_b[t][a]        for the 64 blocks b, contraction over ALL tokens
 //
 // V = x or the upstream gradient g, read as [t][a][b] with the block index b contiguous (exactly what pass 1 reads), and
-// Z = the intermediate in the workspace layout [token tile][m / 8][b][t % 128][m % 8] that pass 1 writes:
+// Z = the intermediate in the workspace layout [32-token tile][m / 16][t % 32][b][m % 16] that pass 1 writes:
 //   dR[n2][k1][n1] = sum_t dv[t][n2][k1] x[t][n1][n2]:  V = x (b = n2, a = n1),  Z = pass 1 of (g, L^T) (m = k1)
 //   dL[k1][k2][n2] = sum_t g[t][k2][k1] v[t][n2][k1]:   V = g (b = k1, a = k2),  Z = pass 1 of (x, R)   (m = n2), D = dL[k1]^T
 // With the tokens as the K dimension both operands lie in shared memory as the forward passes already produce them: the swizzled
