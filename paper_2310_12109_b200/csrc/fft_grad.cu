@@ -174,16 +174,18 @@ __global__ void __launch_bounds__(C::THREADS, wgrad_blocks<C>())
         const long long oa = has_a ? ((long long)b * H + h) * n : 0, ob = oa + (long long)H * n;
         load_row<C, IO, HALF>(re, x + oa, t, n, vec, has_a);
         load_row<C, IO, HALF>(im, x + ob, t, n, vec, has_b);
-        uint32_t ta, tb;   // x / 2^e and 2^e g: the cross terms of a pair are then no larger than the pair's share of the sum
+        uint32_t ta, tb;
+        int ea, eb;   // x / 2^e and 2^e g: the cross terms of a pair are then no larger than the pair's share of the sum
         pair_tops<C, HALF>(re, im, slot, t, r, ta, tb);
-        scale_row<HALF>(re, scale_down(ta));
-        scale_row<HALF>(im, scale_down(tb));
+        pair_exponents(ta, tb, ea, eb);
+        scale_row<HALF>(re, scale_down(ea));
+        scale_row<HALF>(im, scale_down(eb));
         forward<C, HALF>(re, im, sr, si, tab, t, r);
         unroll<16>([&](auto s) { zs[s.v * C::THREADS] = make_float4(lo(re[s.v]), hi(re[s.v]), lo(im[s.v]), hi(im[s.v])); });
         load_row<C, IO, HALF>(re, g + oa, t, n, vec, has_a);
         load_row<C, IO, HALF>(im, g + ob, t, n, vec, has_b);
-        scale_row<HALF>(re, scale_up(ta));
-        scale_row<HALF>(im, scale_up(tb));
+        scale_row<HALF>(re, scale_up(ea));
+        scale_row<HALF>(im, scale_up(eb));
         row_sync<C>(r);
         forward<C, HALF>(re, im, sr, si, tab, t, r);
         unroll<16>([&](auto s) {   // += conj(z) w

@@ -110,8 +110,9 @@ __device__ __forceinline__ void store_row(const u64* v, IO* row, int t, int n, b
 
 // ---- two real rows as one complex row ----
 // The rounding error of a transform is relative to the norm of the complex row, and a value that is not finite reaches all of it, so the
-// two rows are made alike first: each is brought to a largest magnitude in [1, 2) by a power of two, which is exact and is taken back
-// when the row leaves (without the factors a row beside one 1e4 times as large is about 1e-3 off).  One B200, without and with them: bf16
+// two rows are made alike first: each is multiplied by a power of two, which is exact and is taken back when the row leaves.  The first
+// row's brings its largest magnitude to [1, 2), the second's comes nearest to the same, so that rows of one distribution keep the ratio
+// they have (with both in [1, 2) they ended up a factor of two apart now and then, and the errors 5 % larger);  (without the factors a row beside one 1e4 times as large is about 1e-3 off).  One B200, without and with them: bf16
 // x[8][768][2000] 44.9 and 46.3 us, [16][768][1024] 21.3 and 23.4, fp32 [4][768][2048] 26.2 and 26.9.
 template <class C>
 __host__ __device__ constexpr int scale_words() { return 2 * (C::TP > 32 ? C::TP / 32 + 1 : 1); }   // per row pair: its warps' maxima, the factors
@@ -153,10 +154,14 @@ __device__ __forceinline__ void pair_tops(const u64* re, const u64* im, uint32_t
         }
     }
 }
-// 2^e for a largest magnitude in [2^e, 2^(e+1)), and its inverse; both normal numbers
-__device__ __forceinline__ uint32_t top_exponent(uint32_t top) { return min(max(top >> 23, 1u), 253u); }
-__device__ __forceinline__ float scale_up(uint32_t top) { return __uint_as_float(top_exponent(top) << 23); }
-__device__ __forceinline__ float scale_down(uint32_t top) { return __uint_as_float((254u - top_exponent(top)) << 23); }
+// exponent fields of the rows' powers of two (the power and its inverse are normal numbers); a row that is not finite counts as zeros
+__device__ __forceinline__ void pair_exponents(uint32_t ta, uint32_t tb, int& ea, int& eb) {
+    const int a = ta >= kInfBits ? 0 : (int)ta, b = tb >= kInfBits ? 0 : (int)tb;
+    ea = min(max(a >> 23, 1), 253);
+    eb = min(max(ea - ((a - b + (1 << 22)) >> 23), 1), 253);   // the bits of a float are its logarithm, nearly
+}
+__device__ __forceinline__ float scale_up(int e) { return __uint_as_float((uint32_t)e << 23); }
+__device__ __forceinline__ float scale_down(int e) { return __uint_as_float((uint32_t)(254 - e) << 23); }
 template <bool HALF>
 __device__ __forceinline__ void scale_row(u64* v, float f) {   // as load_row leaves it
     const u64 w = dup2(f);
@@ -168,13 +173,15 @@ template <class C, bool HALF>
 __device__ __forceinline__ void balance_pair(u64* re, u64* im, uint32_t* slot, int t, int r) {
     uint32_t ta, tb;
     pair_tops<C, HALF>(re, im, slot, t, r, ta, tb);
-    auto one = [&](u64* v, uint32_t top, uint32_t* back) {
+    int ea, eb;
+    pair_exponents(ta, tb, ea, eb);
+    auto one = [&](u64* v, uint32_t top, int e, uint32_t* back) {
         if (top >= kInfBits) unroll<(HALF ? 8 : 16)>([&](auto j) { v[j.v] = 0ull; });
-        else scale_row<HALF>(v, scale_down(top));
-        if (t == 0) *back = top >= kInfBits ? 0x7fffffffu : top == 0 ? 0u : __float_as_uint(scale_up(top));
+        else scale_row<HALF>(v, scale_down(e));
+        if (t == 0) *back = top >= kInfBits ? 0x7fffffffu : top == 0 ? 0u : __float_as_uint(scale_up(e));
     };
-    one(re, ta, slot + scale_words<C>() - 2);
-    one(im, tb, slot + scale_words<C>() - 1);
+    one(re, ta, ea, slot + scale_words<C>() - 2);
+    one(im, tb, eb, slot + scale_words<C>() - 1);
 }
 // (the row's threads have met since)
 template <class C>
