@@ -122,7 +122,8 @@ template <int N, class F>
 M2_HD void unroll(F&& f) { unroll_from<0, N>(f); }
 
 // o+- = a +- w b in place (a, b <- o+, o-); ROT: the factor is i w.  PLUS_ONLY: o- is not needed.
-template <bool ROT, bool PLUS_ONLY>
+// P: o- as 2 a - o+, two FMAs and one rounding more (0), or directly, four: with constant factors (1), with all (2).
+template <bool ROT, bool PLUS_ONLY, int P>
 M2_HD void bfly(u64& ar, u64& ai, u64& br, u64& bi, u64 wr, u64 wi) {
     const u64 two = dup2(2.0f);
     u64 pr, pi;
@@ -133,7 +134,18 @@ M2_HD void bfly(u64& ar, u64& ai, u64& br, u64& bi, u64 wr, u64 wi) {
         pr = fma2(neg2(wi), br, fma2(neg2(wr), bi, ar));
         pi = fma2(wr, br, fma2(neg2(wi), bi, ai));
     }
-    if (!PLUS_ONLY) {
+    if constexpr (!PLUS_ONLY && P >= 2) {
+        u64 mr, mi;
+        if (!ROT) {
+            mr = fma2(neg2(wr), br, fma2(wi, bi, ar));
+            mi = fma2(neg2(wr), bi, fma2(neg2(wi), br, ai));
+        } else {
+            mr = fma2(wi, br, fma2(wr, bi, ar));
+            mi = fma2(neg2(wr), br, fma2(wi, bi, ai));
+        }
+        br = mr;
+        bi = mi;
+    } else if constexpr (!PLUS_ONLY) {
         br = fma2(two, ar, neg2(pr));
         bi = fma2(two, ai, neg2(pi));
     }
@@ -141,7 +153,7 @@ M2_HD void bfly(u64& ar, u64& ai, u64& br, u64& bi, u64 wr, u64 wi) {
     ai = pi;
 }
 // the same with the constant factor W_32^Q
-template <int Q, bool PLUS_ONLY>
+template <int Q, bool PLUS_ONLY, int P>
 M2_HD void bfly_const(u64& ar, u64& ai, u64& br, u64& bi) {
     if constexpr ((Q & 31) == 0) {
         const u64 pr = add2(ar, br), pi = add2(ai, bi);
@@ -163,7 +175,11 @@ M2_HD void bfly_const(u64& ar, u64& ai, u64& br, u64& bi) {
     } else {
         const float c = (float)W32<Q>::re, s = (float)W32<Q>::im;
         const u64 pr = fma2(dup2(c), br, fma2(dup2(-s), bi, ar)), pi = fma2(dup2(c), bi, fma2(dup2(s), br, ai));
-        if (!PLUS_ONLY) {
+        if constexpr (!PLUS_ONLY && P >= 1) {
+            const u64 mr = fma2(dup2(-c), br, fma2(dup2(s), bi, ar)), mi = fma2(dup2(-c), bi, fma2(dup2(-s), br, ai));
+            br = mr;
+            bi = mi;
+        } else if constexpr (!PLUS_ONLY) {
             br = fma2(dup2(2.0f), ar, neg2(pr));
             bi = fma2(dup2(2.0f), ai, neg2(pi));
         }
@@ -176,7 +192,7 @@ M2_HD void bfly_const(u64& ar, u64& ai, u64& br, u64& bi) {
 //   TW: factors from tw[v * stride] = (re0, re1, im0, im1), v = 0: S = 2, 1: S = 4, 2, 3: S = 8, 4 .. 7: S = 16
 //   BRIN = false: input j in slot j, output q in slot brev(q); BRIN = true: input j in slot brev(j), output q in slot q
 //   HALF_IN: inputs j >= R / 2 are zero (their slots are not read); HALF_OUT: only outputs q < R / 2 are computed
-template <int R, bool TW, bool BRIN, bool HALF_IN, bool HALF_OUT>
+template <int R, bool TW, bool BRIN, bool HALF_IN, bool HALF_OUT, int P>
 M2_HD void fft_packed(u64* re, u64* im, const float4* tw, int stride) {
     constexpr int LOG = R == 16 ? 4 : 3;
     auto slot = [](int pos) constexpr { return BRIN ? pos : brev<LOG>(pos); };
@@ -201,8 +217,8 @@ M2_HD void fft_packed(u64* re, u64* im, const float4* tw, int stride) {
                 }
                 unroll<R / S>([&](auto b) {
                     constexpr int p0 = slot(b.v * S + q.v), p1 = slot(b.v * S + q.v + HS);
-                    if constexpr (TW) bfly<rot, plus>(re[p0], im[p0], re[p1], im[p1], wr, wi);
-                    else bfly_const<q.v * (32 / S), plus>(re[p0], im[p0], re[p1], im[p1]);
+                    if constexpr (TW) bfly<rot, plus, P>(re[p0], im[p0], re[p1], im[p1], wr, wi);
+                    else bfly_const<q.v * (32 / S), plus, P>(re[p0], im[p0], re[p1], im[p1]);
                 });
             });
         }
@@ -211,9 +227,9 @@ M2_HD void fft_packed(u64* re, u64* im, const float4* tw, int stride) {
 
 // 32-point transform of one column: input slot m = (x[2m], x[2m+1]), output q, q + 16 in slot brev(q) = (X[q], X[q+16]).
 //   TW: tw[v * stride], v < 8: the 16-point factors of base w^2, both halves equal; v = 8 + q / 2: (re, im) of w W_32^q for q, q + 1
-template <bool TW, bool HALF_IN, bool HALF_OUT>
+template <bool TW, bool HALF_IN, bool HALF_OUT, int P>
 M2_HD void fft32_eo(u64* re, u64* im, const float4* tw, int stride) {
-    fft_packed<16, TW, false, HALF_IN, false>(re, im, tw, stride);
+    fft_packed<16, TW, false, HALF_IN, false, P>(re, im, tw, stride);
     unroll<16>([&](auto q) {   // last level: even part E[q] in the low half, odd part O[q] in the high half
         constexpr int p = brev<4>(q.v);
         constexpr bool rot = q.v >= 8;
@@ -232,8 +248,8 @@ M2_HD void fft32_eo(u64* re, u64* im, const float4* tw, int stride) {
         const float pr = fmaf(wr, orr, fmaf(-wi, oi, er)), pi = fmaf(wr, oi, fmaf(wi, orr, ei));
         float mr = 0.f, mi = 0.f;
         if constexpr (!HALF_OUT) {
-            mr = fmaf(2.0f, er, -pr);
-            mi = fmaf(2.0f, ei, -pi);
+            mr = P >= (TW ? 2 : 1) ? fmaf(-wr, orr, fmaf(wi, oi, er)) : fmaf(2.0f, er, -pr);
+            mi = P >= (TW ? 2 : 1) ? fmaf(-wr, oi, fmaf(-wi, orr, ei)) : fmaf(2.0f, ei, -pi);
         }
         re[p] = pk(pr, mr);
         im[p] = pk(pi, mi);
@@ -241,6 +257,7 @@ M2_HD void fft32_eo(u64* re, u64* im, const float4* tw, int stride) {
 }
 
 // 32-point transform without factors that takes what fft32_eo left: input slot brev(j) = (x[j], x[j+16]), output slot m = (X[2m], X[2m+1])
+template <int P>
 M2_HD void fft32_dif(u64* re, u64* im) {
     unroll<16>([&](auto j) {
         constexpr int p = brev<4>(j.v);
@@ -260,7 +277,7 @@ M2_HD void fft32_dif(u64* re, u64* im) {
             im[p] = pk(ui, fmaf(c, vi, s * vr));
         }
     });
-    fft_packed<16, false, true, false, false>(re, im, nullptr, 0);
+    fft_packed<16, false, true, false, false, P>(re, im, nullptr, 0);
 }
 
 // ---- factorisations ------------------------------------------------------------------------------------------------------------
@@ -345,10 +362,10 @@ M2_HD int spec_index_any(int logn, int k, bool imag) {
 // Each pass reads its columns from the registers or from shared memory, contracts one digit, and leaves the result in registers
 // (fft_*) or writes it (put_*); the caller places the barriers.
 
-template <class C, bool HALF_IN>
+template <class C, bool HALF_IN, int P>
 M2_HD void fft_first(u64* re, u64* im) {   // registers: input digit n1 of the thread's columns
-    if constexpr (C::R1 == 16) fft_packed<16, false, false, HALF_IN, false>(re, im, nullptr, 0);
-    else fft32_eo<false, HALF_IN, false>(re, im, nullptr, 0);
+    if constexpr (C::R1 == 16) fft_packed<16, false, false, HALF_IN, false, P>(re, im, nullptr, 0);
+    else fft32_eo<false, HALF_IN, false, P>(re, im, nullptr, 0);
 }
 template <class C>
 M2_HD void put_first(const u64* re, const u64* im, float* sr, float* si, int t) {
@@ -419,15 +436,15 @@ M2_HD void put_cols_natural(const u64* re, const u64* im, float* sr, float* si, 
         si[a1] = hi(im[s.v]);
     });
 }
-template <int R>
+template <int R, int P>
 M2_HD void fft_tw(u64* re, u64* im, const float4* tw, int stride) {
     if constexpr (R == 8) {
-        fft_packed<8, true, false, false, false>(re, im, tw, stride);
-        fft_packed<8, true, false, false, false>(re + 8, im + 8, tw + 4 * stride, stride);
+        fft_packed<8, true, false, false, false, P>(re, im, tw, stride);
+        fft_packed<8, true, false, false, false, P>(re + 8, im + 8, tw + 4 * stride, stride);
     } else if constexpr (R == 16) {
-        fft_packed<16, true, false, false, false>(re, im, tw, stride);
+        fft_packed<16, true, false, false, false, P>(re, im, tw, stride);
     } else {
-        fft32_eo<true, false, false>(re, im, tw, stride);
+        fft32_eo<true, false, false, P>(re, im, tw, stride);
     }
 }
 

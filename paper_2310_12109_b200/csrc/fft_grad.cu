@@ -148,6 +148,12 @@ __global__ void __launch_bounds__(C::THREADS, min_blocks<C>())
 // sum stays in registers, F z waits in shared memory in the thread's own slots, and the rows' sums are added in order at the end.
 // (One row per channel left most SMs idle at short lengths: bf16 [64][768][256] 319 -> 35 us, [32][768][512] 176 -> 35 us with the
 // loads of a row in flight together, too.)
+// Three transforms follow one another and a pair's cross terms cancel, so differences are taken directly where the other kernels save two
+// of eight FMAs (fft_core.cuh): in the inverse and with constant factors everywhere, with variable factors at N = 256, where the dense
+// stages of a 16 x 16 plan are the most accurate.  Distance from the exact gradient, fp32: N = 4096 causal 2.46e-7 without, 2.39e-7 so (16 x 16 x 16
+// dense stages: 2.40e-7), N = 256 causal 2.02e-7 and 1.90e-7 (1.92e-7); x, g [4][768][2048] 36.9 and 37.5 us.
+template <class C>
+constexpr int kGradDirect = C::N == 256 ? 2 : 1;
 template <class C>
 constexpr int wgrad_blocks() { return C::THREADS == 128 ? 2 : 1; }
 template <class C, typename IO, bool HALF>
@@ -180,14 +186,14 @@ __global__ void __launch_bounds__(C::THREADS, wgrad_blocks<C>())
         pair_exponents(ta, tb, ea, eb);
         scale_row<HALF>(re, scale_down(ea));
         scale_row<HALF>(im, scale_down(eb));
-        forward<C, HALF>(re, im, sr, si, tab, t, r);
+        forward<C, HALF, kGradDirect<C>>(re, im, sr, si, tab, t, r);
         unroll<16>([&](auto s) { zs[s.v * C::THREADS] = make_float4(lo(re[s.v]), hi(re[s.v]), lo(im[s.v]), hi(im[s.v])); });
         load_row<C, IO, HALF>(re, g + oa, t, n, vec, has_a);
         load_row<C, IO, HALF>(im, g + ob, t, n, vec, has_b);
         scale_row<HALF>(re, scale_up(ea));
         scale_row<HALF>(im, scale_up(eb));
         row_sync<C>(r);
-        forward<C, HALF>(re, im, sr, si, tab, t, r);
+        forward<C, HALF, kGradDirect<C>>(re, im, sr, si, tab, t, r);
         unroll<16>([&](auto s) {   // += conj(z) w
             const float4 z = zs[s.v * C::THREADS];
             const u64 zr = pk(z.x, z.y), zi = pk(z.z, z.w);
@@ -197,7 +203,7 @@ __global__ void __launch_bounds__(C::THREADS, wgrad_blocks<C>())
         row_sync<C>(r);
     }
     if (C::ROWS > 1 && share > 1) add_shares<C>(ar, ai, zall, share, r, t);
-    inverse<C, HALF>(ar, ai, sr, si, tab, t, r);
+    inverse<C, HALF, 2>(ar, ai, sr, si, tab, t, r);
     const u64 sc = dup2(1.0f / (float)C::N);
     unroll<16>([&](auto s) { ar[s.v] = mul2(ar[s.v], sc); });
     store_row<C, float, HALF>(ar, dk + h * n, t, n, vec, live && r % share == 0);

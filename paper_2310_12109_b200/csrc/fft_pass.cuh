@@ -195,9 +195,9 @@ __device__ __forceinline__ void unbalance_pair(u64* re, u64* im, const uint32_t*
 
 // registers (input digit of the first pass) -> registers (output of the last digit: q in slot brev(q); R = 32: q, q + 16).
 // The row's shared memory must be free on entry; afterwards other threads may still be reading it.
-template <class C, bool HALF>
+template <class C, bool HALF, int P = 0>
 __device__ __forceinline__ void forward(u64* re, u64* im, float* sr, float* si, const float4* __restrict__ tab, int t, int r) {
-    fft_first<C, HALF>(re, im);
+    fft_first<C, HALF, P>(re, im);
     put_first<C>(re, im, sr, si, t);
     row_sync<C>(r);
     if constexpr (C::THREE) {
@@ -205,19 +205,19 @@ __device__ __forceinline__ void forward(u64* re, u64* im, float* sr, float* si, 
         auto m2 = [&](int c, int j) { return mid2<C>(t, c, j); };
         get_cols<C::R2>(re, im, sr, si, m1);
         row_sync<C>(r);
-        fft_tw<C::R2>(re, im, tab + Tab<C>::F2 + t / C::R3, Tab<C>::K2);
+        fft_tw<C::R2, P>(re, im, tab + Tab<C>::F2 + t / C::R3, Tab<C>::K2);
         put_cols<C::R2>(re, im, sr, si, m2);
         row_sync<C>(r);
     }
     get_cols<C::RL>(re, im, sr, si, [&](int c, int j) { return last2<C>(t, c, j); });
-    fft_tw<C::RL>(re, im, tab + Tab<C>::FL + t, C::TP);
+    fft_tw<C::RL, P>(re, im, tab + Tab<C>::FL + t, C::TP);
 }
 // registers (as forward leaves them) -> registers (output digit n1 of the first-pass columns); re and im swapped by the caller's
 // choice of names: the inverse transform is the forward one on (im, re)
-template <class C, bool HALF>
+template <class C, bool HALF, int P = 0>
 __device__ __forceinline__ void inverse(u64* re, u64* im, float* sr, float* si, const float4* __restrict__ tab, int t, int r) {
-    if constexpr (C::RL == 16) fft_packed<16, false, true, false, false>(im, re, nullptr, 0);
-    else fft32_dif(im, re);
+    if constexpr (C::RL == 16) fft_packed<16, false, true, false, false, P>(im, re, nullptr, 0);
+    else fft32_dif<P>(im, re);
     put_cols_natural<C::RL>(re, im, sr, si, [&](int c, int j) { return last2<C>(t, c, j); });   // the thread's own columns: in place
     row_sync<C>(r);
     if constexpr (C::THREE) {
@@ -225,7 +225,7 @@ __device__ __forceinline__ void inverse(u64* re, u64* im, float* sr, float* si, 
         auto m2 = [&](int c, int j) { return mid2<C>(t, c, j); };
         get_cols<C::R2>(re, im, sr, si, m2);
         row_sync<C>(r);
-        fft_tw<C::R2>(im, re, tab + Tab<C>::I2 + t % C::R3, C::R3);
+        fft_tw<C::R2, P>(im, re, tab + Tab<C>::I2 + t % C::R3, C::R3);
         put_cols<C::R2>(re, im, sr, si, m1);
         row_sync<C>(r);
     }
@@ -239,10 +239,10 @@ __device__ __forceinline__ void inverse(u64* re, u64* im, float* sr, float* si, 
                 im[j.v] = pk(si[j.v * C::S1 + 2 * t], si[j.v * C::S1 + 2 * t + 1]);
             }
         });
-        fft_packed<16, true, false, false, HALF>(im, re, tab + Tab<C>::I1 + t, C::TP);
+        fft_packed<16, true, false, false, HALF, P>(im, re, tab + Tab<C>::I1 + t, C::TP);
     } else {
         get_cols<C::R1>(re, im, sr, si, [&](int, int j) { return j * C::S1 + t; });
-        fft32_eo<true, false, HALF>(im, re, tab + Tab<C>::I1 + t, C::TP);
+        fft32_eo<true, false, HALF, P>(im, re, tab + Tab<C>::I1 + t, C::TP);
     }
 }
 
