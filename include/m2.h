@@ -126,7 +126,10 @@ int32_t m2_monarch_conv_bwd_kernel(const m2_plan* plan, const void* x_dev, const
 /* y = Re( M^-1 ( k_f (.) M pad(x) ) )[0:n)  (Eq. 2 with M_1 = F, M_2 = F^-1; App. D.3).
  * x_dev, y_dev: [B, H, n] in the plan dtype; kf_dev from m2_kernel_spectrum with the same H.
  * mode M2_CAUSAL: n <= N/2, x zero padded to N, first n outputs kept (Thm 3 / App. D.3 review).
- * mode M2_CIRCULAR: n == N. */
+ * mode M2_CIRCULAR: n == N.
+ * A row's result depends on that row and its kernel alone, with one exception: the bf16 tensor-core kernels for N = 512 (more than 8 batch
+ * rows) and N = 32768 transform two batch rows as one complex row, so that the rounding between their stages is relative to the larger
+ * of the two and a value that is not finite reaches both. */
 int32_t m2_monarch_conv_fwd(const m2_plan* plan, const void* x_dev, const void* kf_dev, void* y_dev, int64_t B,
                             int64_t H, int64_t n, int32_t mode, void* stream);
 

@@ -110,10 +110,11 @@ __device__ __forceinline__ void store_row(const u64* v, IO* row, int t, int n, b
 
 // ---- two real rows as one complex row ----
 // The rounding error of a transform is relative to the norm of the complex row, and a value that is not finite reaches all of it, so the
-// two rows are made alike first: each is multiplied by a power of two, which is exact and is taken back when the row leaves.  The first
-// row's brings its largest magnitude to [1, 2), the second's comes nearest to the same, so that rows of one distribution keep the ratio
-// they have (with both in [1, 2) they ended up a factor of two apart now and then, and the errors 5 % larger);  (without the factors a row beside one 1e4 times as large is about 1e-3 off).  One B200, without and with them: bf16
-// x[8][768][2000] 44.9 and 46.3 us, [16][768][1024] 21.3 and 23.4, fp32 [4][768][2048] 26.2 and 26.9.
+// two rows are made alike first: each is multiplied by a power of two, which is exact and is taken back when the row leaves (without that
+// a row beside one 1e4 times as large is about 1e-3 off).  The first row's brings its largest magnitude to [1, 2), the second's comes
+// nearest to the same, so that rows of one distribution keep the ratio they have (with both in [1, 2) they ended up a factor of two apart
+// now and then, and the errors 5 % larger).  One B200, without and with the factors: bf16 x[8][768][2000] 44.9 and 46.3 us,
+// [16][768][1024] 21.3 and 23.4, fp32 [4][768][2048] 26.2 and 26.9.
 template <class C>
 __host__ __device__ constexpr int scale_words() { return 2 * (C::TP > 32 ? C::TP / 32 + 1 : 1); }   // per row pair: its warps' maxima, the factors
 template <class C>

@@ -880,13 +880,13 @@ def run_monarch_cols(N1, N2, Bt, d, dtype, withK):
     plan.close()
 
 
-@pytest.mark.parametrize("B,n,d,dh,dims,dtype", [(9, 256, 128, 16, (32, 16), M.M2_BF16),   # heads of 16: one fused tensor-core kernel
+@pytest.mark.parametrize("B,n,d,dh,dims,dtype", [(9, 256, 128, 16, (32, 16), M.M2_BF16),   # heads of 16: outer product, convolution and contraction in one kernel
                                                   (3, 112, 64, 16, (32, 16), M.M2_BF16),    # the same with a ragged sequence length
                                                   (2, 100, 64, 4, (32, 16), M.M2_BF16),     # other head sizes: three kernels
                                                   (2, 24, 12, 3, (8, 8), M.M2_FP32)])
 def test_m2_hyena_heads_fwd(B, n, d, dh, dims, dtype):
     """The M2 Hyena layer with heads: projections, short convolutions, head outer products through the long convolution, output
-    projection (all channel-first after one transposition)."""
+    projection (channel-first in between)."""
     tdt = torch.bfloat16 if dtype == M.M2_BF16 else torch.float32
     rnd = (lambda a: synth.round_bf16(a)) if dtype == M.M2_BF16 else (lambda a: a.astype(np.float32).astype(np.float64))
     p = {k: rnd(synth.normal(synth.stream_id(14, i), (d, d)) / np.sqrt(d)) for i, k in enumerate(("W_x1", "W_x2", "W_v", "W_o"))}
@@ -947,7 +947,8 @@ def test_hyena_head_product_tiles(B, n, d, dims):
 
 
 @pytest.mark.parametrize("B,n,d,dims,long_kernel", [(2, 256, 32, (32, 16), "conjugated"), (1, 77, 64, (32, 16), "full"), (3, 100, 16, (16, 16), "full"),
-                                                     (1, 512, 32, (32, 32), "conjugated"), (2, 200, 32, (64, 64), "full"), (1, 1000, 16, (64, 32), "conjugated")])
+                                                     (1, 512, 32, (32, 32), "conjugated"), (2, 200, 32, (64, 64), "full"), (1, 1000, 16, (64, 32), "conjugated"),
+                                                     (1, 90, 16, (32, 32, 8), "full"), (1, 1024, 16, (128, 128), "conjugated")])
 def test_hyena_head_product_with_lags_below_zero(B, n, d, dims, long_kernel):
     """Long kernels that reach backwards: a conjugated spectrum (the transposed convolution) and a kernel as long as the plan.  The fused
     head product multiplies by the same circular kernel as the convolutions do."""
@@ -1017,8 +1018,8 @@ def test_layers_refuse_misaligned_spectra():
 
 
 def test_m2_hyena_heads_full_size_sampled():
-    """The layer at the benchmark shape (B = 32, n = 256, d = 768, heads of 16: 24 576 units of the fused kernel, many rounds per
-    pipeline); batch entries are independent, so the first and the last one are compared with the oracle run on them alone."""
+    """The layer at the benchmark shape (B = 32, n = 256, d = 768, heads of 16: 1536 blocks of the fused kernel, 2304 items
+    of the Toeplitz kernel); batch entries are independent, so the first and the last one are compared with the oracle run on them alone."""
     B, n, d, dh, dims = 32, 256, 768, 16, (32, 16)
     rnd = synth.round_bf16
     p = {k: rnd(synth.normal(synth.stream_id(16, i), (d, d)) / np.sqrt(d)) for i, k in enumerate(("W_x1", "W_x2", "W_v", "W_o"))}
