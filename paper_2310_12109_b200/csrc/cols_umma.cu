@@ -14,7 +14,7 @@
 // the epilogue applies the optional factor K (.) and ReLU in fp32, rounds to bf16, stages the tile in the swizzled image of
 // the TMA store boxes and stores it to its rows.  One persistent CTA per SM with a producer warp, an issuing warp
 // and four epilogue warps; two accumulators in TMEM, so a tile's epilogue overlaps the next tile's UMMAs.  Block sizes are
-// 64 and 128 here, larger multiples of 64 in gemm_pair.cu (whose tile of 256 rows they fill), d a multiple of 8 (a ragged
+// multiples of 64 (those that fill the 256-row tiles of gemm_pair.cu go there), d a multiple of 8 (a ragged
 // last column tile is zero-filled on the way in and clipped on the way out).  All waits are bounded.
 #include <cuda.h>
 
@@ -267,7 +267,10 @@ cudaError_t prepare() {
 // one stage: nb blocks of b x b; out rows o*so + j = W[j] applied to the rows i*si + j*sj of V (N = rows per matrix of the batch)
 static int32_t stage(const m2_plan* pl, int64_t N, const void* W, const void* V, void* O, const void* Kmul, int relu, int64_t Bt, int64_t d,
                      int b, int nb, int64_t si, int64_t sj, int64_t so, cudaStream_t stream) {
-    if (b > 128) {   // a block fills both halves of a pair's tile (at 128 half of it would be padding)
+    // CTA pairs where a block's last tile of 256 rows needs its second half, and the columns fill the narrowest tile or the 128-row tiles
+    // here would be padded as well.  One product, us, here and on pairs: b = 256, d = 8 19.7 and 22.9, 128 26.4 and 26.0, 768 93.4 and 85.1; 192,
+    // d = 8 21.7 and 19.3; 448, 8 98 and 86, 768 386 and 354; against that 320, 8 34.7 and 48.3, 768 172 and 177; 576, 768 788 and 842; 640, 768 1001 and 1028.
+    if (b > 128 && (b + 127) / 128 % 2 == 0 && (d > 64 || b % 128 != 0)) {
         PairGemm g;
         g.a[0] = {W, b, b, b, nb, (int64_t)b * b, 1, 0};
         g.b = {V, d, b, si * d, nb, sj * d, Bt, N * d};

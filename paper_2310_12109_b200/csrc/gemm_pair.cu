@@ -1,6 +1,6 @@
 // Batched GEMM on CTA pairs (tcgen05 cta_group::2):  O[bt][j] = A[j] B[bt][j], a tile of 256 output rows x up to 256 columns per pair.
 //
-// Serves the column-layout Monarch stages with blocks larger than 128 (cols_umma.cu has the formulation; 64 and 128 stay there) and the
+// Serves the column-layout Monarch stages whose blocks fill its tiles of 256 rows (cols_umma.cu has the formulation and the rule) and the
 // dense projections of the Hyena layer and the M2-BERT mixer (up to three weights in one launch).  Operands are taken as they lie: A is
 // K-major (weights) or M-major (activations [k][m]), B is N-major ([k][n]) or K-major ([n][k]); tensor maps do the rest, so the
 // projections read x [positions][channels] without a transposition and the output projection writes that layout.

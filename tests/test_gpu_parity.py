@@ -836,6 +836,14 @@ def test_monarch_cols(b, Bt, d, dtype, withK):
     run_monarch_cols(b, b, Bt, d, dtype, withK)
 
 
+@pytest.mark.parametrize("N1,N2,Bt,d,withK", [(256, 64, 2, 72, True), (64, 256, 2, 64, True), (320, 64, 1, 136, True), (64, 320, 2, 8, False),
+                                             (448, 64, 1, 8, False), (64, 448, 1, 200, True), (512, 64, 1, 64, False)])
+def test_monarch_cols_on_either_side_of_the_pair_rule(N1, N2, Bt, d, withK):
+    """Blocks above 128: 256 with more and with no more than 64 columns, 320 (its last tile of 256 rows half empty), 448 (two tiles whatever the
+    columns), 512 with few columns; as the first factor's block and as the second's, with and without the factor."""
+    run_monarch_cols(N1, N2, Bt, d, M.M2_BF16, withK)
+
+
 @pytest.mark.parametrize("N1,N2,d", [(64, 128, 72), (128, 64, 256), (192, 64, 64)])
 def test_monarch_cols_rectangular(N1, N2, d):
     run_monarch_cols(N1, N2, 2, d, M.M2_BF16, True)
