@@ -307,6 +307,19 @@ def test_short_causal_convolution_as_toeplitz_product(B, H, n, dims, group):
     plan.close()
 
 
+@pytest.mark.parametrize("B,H,n,kernel", [(48, 600, 256, "conv_umma_o2_512_pairs"), (48, 500, 256, "conv_toeplitz_mma"), (64, 600, 256, "conv_toeplitz_mma"),
+                                          (17, 600, 224, "conv_toeplitz_mma"), (33, 1400, 192, "conv_toeplitz_mma"), (40, 1000, 224, "conv_umma_o2_512_pairs"),
+                                          (48, 1200, 160, "conv_toeplitz_mma")])
+def test_short_causal_rows_take_the_faster_kernel(B, H, n, kernel):
+    """Batches whose last 32-row item is half empty, many channels, n near 256: the row-pair kernel; everything around that: Toeplitz products."""
+    x = synth.round_bf16(synth.normal(770 + n, (B, H, n)))
+    k = (synth.normal(771 + n, (H, n)) / np.sqrt(n)).astype(np.float32)
+    y, name = run_conv((32, 16), x, k, True, M.M2_BF16)
+    assert name == kernel
+    want = np.fft.irfft(np.fft.rfft(x.astype(np.float64), 512) * np.fft.rfft(k.astype(np.float64), 512)[None], 512)[..., :n]
+    check(y, want, 4e-3 if "toeplitz" in kernel else TOL_BF16, name)
+
+
 @pytest.mark.parametrize("B", [5, 19])
 def test_bf16_causal_order2_and_ragged(B):
     for n in (256, 100, 48):
