@@ -199,6 +199,10 @@ const float* time_kernel(const m2_plan* pl, const void* kf, int64_t H) {
 
 int32_t conv(const m2_plan* pl, const Rows* sets, int count, int64_t B, int64_t H, int64_t n, int kf_group, cudaStream_t stream) {
     if (!has_time_kernel(pl) || n > kMaxN || 2 * n > pl->N || count < 1 || count > 3) return M2_ERR_UNSUPPORTED;
+    if (umma_pays(pl, count, B, H, n)) {
+        const int32_t rc = conv_umma(pl, sets, count, B, H, n, kf_group, stream);
+        if (rc != M2_ERR_UNSUPPORTED) return rc;
+    }
     Sets s;
     for (int i = 0; i < 3; ++i) s.r[i] = sets[i < count ? i : 0];
     const int rows = B <= 16 ? 16 : 32;

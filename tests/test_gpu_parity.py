@@ -307,6 +307,26 @@ def test_short_causal_convolution_as_toeplitz_product(B, H, n, dims, group):
     plan.close()
 
 
+@pytest.mark.parametrize("B,H,n,group", [(17, 296, 192, 1), (32, 300, 248, 3), (33, 150, 200, 1), (64, 160, 256, 2)])
+def test_toeplitz_products_of_long_items(B, H, n, group):
+    """The tcgen05 Toeplitz kernel (296 items of 32 rows and more, 192 to 256 positions): partial batch chunks, ragged last segments, two and
+    three items per block, channel groups; lags on one side, on the other (conjugated) and on both (a kernel of all 512 lags).  The kernel's
+    values keep 16 bits, the output is rounded once to bf16 (1.7e-3 in the 2-norm)."""
+    Hk = H // group
+    x = synth.round_bf16(synth.normal(780 + n, (B, H, n)))
+    plan = M.Plan((32, 16), dtype=M.M2_BF16, device=0)
+    xd = dev(x.astype(np.float32), torch.bfloat16)
+    fx = np.fft.rfft(x.astype(np.float64), 512)
+    for nk, conj in ((n, False), (n, True), (512, False)):
+        k = (synth.normal(781 + n, (Hk, nk)) / np.sqrt(n)).astype(np.float32)
+        kf = M.m2_kernel_spectrum(plan, dev(k))
+        fk = np.repeat(np.fft.rfft(k.astype(np.float64), 512), group, axis=0)[None]
+        y = M.m2_monarch_conv_fwd_grouped(plan, xd, M.m2_spectrum_conjugate(plan, kf, Hk) if conj else kf, M.M2_CAUSAL, group)
+        assert plan.device_status() == 0 and plan.last_kernel() == "conv_toeplitz_mma"
+        check(host(y), np.fft.irfft(fx * (np.conj(fk) if conj else fk), 512)[..., :n], 4e-3, f"{nk} lags, conjugated {conj}")
+    plan.close()
+
+
 @pytest.mark.parametrize("B,H,n,kernel", [(48, 600, 256, "conv_umma_o2_512_pairs"), (48, 500, 256, "conv_toeplitz_mma"), (64, 600, 256, "conv_toeplitz_mma"),
                                           (17, 600, 224, "conv_toeplitz_mma"), (33, 1400, 192, "conv_toeplitz_mma"), (40, 1000, 224, "conv_umma_o2_512_pairs"),
                                           (48, 1200, 160, "conv_toeplitz_mma")])
