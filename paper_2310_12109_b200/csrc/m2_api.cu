@@ -286,6 +286,9 @@ int32_t m2_monarch_conv_bwd_kernel(const m2_plan* plan, const void* x_dev, const
     m2g::ConvShape s = conv_shape(plan, B, H, n);
     const int64_t need = m2u::conv_wgrad_workspace_bytes(plan, B, H);
     if (need > 0 && B > 0 && ws_dev && ws_bytes >= need) {   // tensor-core transforms and products, CUDA-core sum + inverse
+        st = m2t::conv_grad(plan, x_dev, g_dev, dk_dev, B, H, n, mode == M2_CAUSAL, (cudaStream_t)stream);
+        if (st == M2_OK) plan->last_kernel = "conv_wgrad_umma_o2_512";
+        if (st != M2_ERR_UNSUPPORTED) return st;
         int parts = 0;
         st = m2u::conv_wgrad_partials(plan, x_dev, g_dev, ws_dev, B, H, n, mode, &parts, (cudaStream_t)stream);
         if (st == M2_OK) {

@@ -26,4 +26,8 @@ int32_t conv(const m2_plan* pl, const Rows* sets, int count, int64_t B, int64_t 
 bool umma_pays(const m2_plan* pl, int count, int64_t B, int64_t H, int64_t n);
 int32_t conv_umma(const m2_plan* pl, const Rows* sets, int count, int64_t B, int64_t H, int64_t n, int kf_group, cudaStream_t stream);
 
+// Kernel gradient dk[H][n] (fp32) of rows [B][H][n], N = 512, n = 512 circular or causal n <= 256, a multiple of 16 (toeplitz_grad.cu)
+bool grad_covers(const m2_plan* pl, int64_t B, int64_t H, int64_t n, bool causal);
+int32_t conv_grad(const m2_plan* pl, const void* x, const void* g, float* dk, int64_t B, int64_t H, int64_t n, bool causal, cudaStream_t stream);
+
 }  // namespace m2t
