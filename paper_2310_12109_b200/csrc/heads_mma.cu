@@ -4,8 +4,8 @@
 // Language Modeling").  In the second form the convolution is an n x n Toeplitz factor on the rank-16 scores: two contractions
 // with K = 16 and one product per (t, s), against 256 convolutions of 2 n points.
 //
-// One thread block per (batch entry, head); a warp owns tiles of 16 positions t and walks the tiles of 16 positions s <= t.  A tile pair
-// is four m16n8k16 MMAs on register fragments: the scores' accumulator, times the kernel values and rounded to bf16, IS the second
+// One thread block per (batch entry, head); a warp owns tiles of 16 positions t, one or two neighbouring ones at a time, and walks the tiles
+// of 16 positions s <= t.  A tile pair is four m16n8k16 MMAs on register fragments: the scores' accumulator, times the kernel values and rounded to bf16, IS the second
 // product's B operand (rows of an accumulator fragment = columns of a B fragment), so nothing goes through shared memory between the
 // two products and no warp waits for another.  (tcgen05 would put every tile through tensor memory, shared memory and two barriers for
 // 8 K multiply-adds.)  Kernel values lie reversed in shared memory, in two copies one element apart, so that the two values of a
@@ -13,8 +13,9 @@
 // conjugated or its kernel is longer than N - n: a block that finds one that is not zero walks the tiles s > t too, with kernel values
 // from L2.
 //
-// Measured, one B200, 1536 heads of n = 256: 23.6 us where 24 576 tensor-core convolution units of 16 rows took about 280 us.  Bound by
-// the load/store data pipe (60 % busy), issue (48 %) and the fragments' latency: 136 tile pairs of about 20 instructions; matrix pipe 31 %.
+// Measured, one B200, 1536 heads of n = 256: 23.6 us with one tile at a time, where 24 576 tensor-core convolution units of 16 rows took about
+// 280 us, and 20 us with two: bound by the load/store data pipe with one (60 % busy, issue 48 %: 14 wavefronts a tile pair), which two cut to 6
+// (they share the fragments of X2 and V, and a distance's kernel values serve the next one), and by the fragments' latency.
 #include "fft_conv.h"
 #include "fft_core.cuh"
 #include "heads_mma.h"
@@ -23,7 +24,7 @@
 
 namespace m2h {
 
-constexpr int kThreads = 256, kDh = 16, kMaxN = 1024;
+constexpr int kDh = 16, kMaxN = 1024;
 
 __host__ __device__ constexpr int padded(int n) { return (n + 15) / 16 * 16; }
 __host__ __device__ constexpr int pitch(int n) { return padded(n) + 8; }              // bf16 elements: rows 16 bytes apart mod 128
@@ -42,6 +43,7 @@ __device__ __forceinline__ uint32_t weigh(float a, float b, float2 k) {
     return bf2(m2f::lo(p), m2f::hi(p));
 }
 
+template <int kThreads, int T>   // T: tiles of 16 positions t that a warp takes at a time
 __global__ void __launch_bounds__(kThreads)
     heads_kernel(const __nv_bfloat16* __restrict__ X1, const __nv_bfloat16* __restrict__ X2, const __nv_bfloat16* __restrict__ V,
                  const float* __restrict__ kt, int period, __nv_bfloat16* __restrict__ O, int heads, int n) {
@@ -70,16 +72,22 @@ __global__ void __launch_bounds__(kThreads)
     if (tid == 0) ks[kc] = 0.f;   // (lag np + 15)
     const __nv_bfloat16* src[3] = {X1 + base, X2 + base, V + base};
     if (n % 8 == 0) {   // 16-byte pieces never straddle a row
-        for (int c = lane * 8; c < n; c += 256) {   // two rows of each tensor per warp, all six loads in flight
-            uint4 v[6];
+        constexpr int kW = kThreads / 32, kR = 3 * kDh / kW / 2;   // rows per warp, in two rounds of loads in flight
+        for (int c = lane * 8; c < n; c += 256)
 #pragma unroll
-            for (int q = 0; q < 6; ++q) v[q] = __ldg(reinterpret_cast<const uint4*>(src[q >> 1] + (size_t)(warp + 8 * (q & 1)) * n + c));
+            for (int z = 0; z < 2; ++z) {
+                uint4 v[kR];
 #pragma unroll
-            for (int q = 0; q < 6; ++q) *reinterpret_cast<uint4*>(xs1 + ((q >> 1) * kDh + warp + 8 * (q & 1)) * ld + c) = v[q];
-        }
+                for (int q = 0; q < kR; ++q) {
+                    const int r = warp + kW * (z * kR + q);   // row of the three tensors one after the other
+                    v[q] = __ldg(reinterpret_cast<const uint4*>((r < kDh ? src[0] : r < 2 * kDh ? src[1] : src[2]) + (size_t)(r % kDh) * n + c));
+                }
+#pragma unroll
+                for (int q = 0; q < kR; ++q) *reinterpret_cast<uint4*>(xs1 + (warp + kW * (z * kR + q)) * ld + c) = v[q];
+            }
         if (np != n && tid < 3 * kDh) *reinterpret_cast<uint4*>(xs1 + tid * ld + n) = make_uint4(0u, 0u, 0u, 0u);
     } else {
-        for (int r = warp; r < kDh; r += 8)
+        for (int r = warp; r < kDh; r += kThreads / 32)
             for (int c = lane; c < np; c += 32)
 #pragma unroll
                 for (int q = 0; q < 3; ++q) xs1[q * kDh * ld + r * ld + c] = c < n ? src[q][(size_t)r * n + c] : __float2bfloat16_rn(0.f);
@@ -91,48 +99,81 @@ __global__ void __launch_bounds__(kThreads)
     const uint32_t b2 = smem_addr(xs2 + ((m & 1) * 8 + r8) * ld + (m >> 1) * 8);
     const uint32_t av = smem_addr(vs + ((m & 1) * 8 + r8) * ld + (m >> 1) * 8);
     const float* kp = ks + (g & 1) * kc + np + 14 + (g & 1) - g + c2;   // lag g - c2; minus the tile distance
-    const int tiles = np / 16, nw = kThreads / 32;
-    const int front = nw * ((tiles + 2 * nw - 1) / (2 * nw));   // the first half of a warp's tiles in order, the second from the far end:
-    for (int it = warp; it < tiles; it += nw) {                 // every warp gets as many short tiles as long ones
-        const int ti = it < front ? it : tiles - 1 - (it - front);
-        uint32_t fa[4];
-        ldsm4t(fa, a1 + ti * 32);
-        float o[2][4] = {};
-        auto tile = [&](int si, float2 k0, float2 k8, float2 km) {   // the kernel at lags u, u + 8, u - 8 and the one below each
-            uint32_t fb[4], fv[4];
-            ldsm4t(fb, b2 + si * 32);
-            ldsm4(fv, av + si * 32);
+    const int tiles = np / 16, groups = (tiles + T - 1) / T, nw = kThreads / 32;
+    const int front = nw * ((groups + 2 * nw - 1) / (2 * nw));   // the first half of a warp's groups in order, the second from the far end:
+    for (int it = warp; it < groups; it += nw) {                 // every warp gets as many short ones as long ones
+        const int t0 = T * (it < front ? it : groups - 1 - (it - front));   // (t0 + 1 = tiles: nothing but the rows' padding, not stored)
+        uint32_t fa[T][4];
+#pragma unroll
+        for (int z = 0; z < T; ++z) ldsm4t(fa[z], a1 + (t0 + z) * 32);
+        float o[T][2][4] = {};
+        uint32_t fb[4] = {}, fv[4] = {};   // the tile si of X2 and of V
+        auto tile = [&](int z, float2 k0, float2 k8, float2 km) {   // the kernel at lags u, u + 8, u - 8 and the one below each
             float s0[4] = {}, s1[4] = {};
-            mma(s0, fa, fb[0], fb[1]);
-            mma(s1, fa, fb[2], fb[3]);
-            mma(o[0], fv, weigh(s0[0], s0[1], k0), weigh(s1[0], s1[1], km));
-            mma(o[1], fv, weigh(s0[2], s0[3], k8), weigh(s1[2], s1[3], k0));
+            mma(s0, fa[z], fb[0], fb[1]);
+            mma(s1, fa[z], fb[2], fb[3]);
+            mma(o[z][0], fv, weigh(s0[0], s0[1], k0), weigh(s1[0], s1[1], km));
+            mma(o[z][1], fv, weigh(s0[2], s0[3], k8), weigh(s1[2], s1[3], k0));
         };
-        for (int si = 0; si <= ti; ++si) {
-            const float* kq = kp - (ti - si) * 16;
-            tile(si, *reinterpret_cast<const float2*>(kq), *reinterpret_cast<const float2*>(kq - 8), *reinterpret_cast<const float2*>(kq + 8));
+        auto kernel = [&](const float* q) { return *reinterpret_cast<const float2*>(q); };
+        if constexpr (T == 1) {
+            for (int si = 0; si <= t0; ++si) {
+                const float* kq = kp - (t0 - si) * 16;
+                ldsm4t(fb, b2 + si * 32);
+                ldsm4(fv, av + si * 32);
+                tile(0, kernel(kq), kernel(kq - 8), kernel(kq + 8));
+            }
+        } else {
+            const float* kq = kp;   // one tile further away with every step down in s: what was 8 above is then 8 below
+            float2 k0 = kernel(kq), k8 = kernel(kq - 8), km = kernel(kq + 8);
+            if (t0 + 1 < tiles) {
+                ldsm4t(fb, b2 + t0 * 32 + 32);
+                ldsm4(fv, av + t0 * 32 + 32);
+                tile(1, k0, k8, km);
+            }
+            for (int si = t0; si >= 0; --si) {
+                kq -= 16;
+                const float2 n0 = kernel(kq), n8 = kernel(kq - 8);
+                ldsm4t(fb, b2 + si * 32);
+                ldsm4(fv, av + si * 32);
+                tile(0, k0, k8, km);
+                tile(1, n0, n8, k8);
+                km = k8;
+                k0 = n0;
+                k8 = n8;
+            }
         }
         if (earlier) {
 #pragma unroll 1
-            for (int si = ti + 1; si < tiles; ++si) {
-                const int u = g - c2 + 16 * (ti - si);
-                tile(si, make_float2(value(u), value(u - 1)), make_float2(value(u + 8), value(u + 7)), make_float2(value(u - 8), value(u - 9)));
+            for (int si = t0 + 1; si < tiles; ++si) {
+                ldsm4t(fb, b2 + si * 32);
+                ldsm4(fv, av + si * 32);
+#pragma unroll
+                for (int z = 0; z < T; ++z) {
+                    if (si <= t0 + z) continue;
+                    const int u = g - c2 + 16 * (t0 + z - si);
+                    tile(z, make_float2(value(u), value(u - 1)), make_float2(value(u + 8), value(u + 7)), make_float2(value(u - 8), value(u - 9)));
+                }
             }
         }
-        __syncwarp();   // this tile's columns of X1 are read by this warp only: the result takes their place
+        __syncwarp();   // these tiles' columns of X1 are read by this warp only: the result takes their place
 #pragma unroll
-        for (int x = 0; x < 2; ++x) {
-            *reinterpret_cast<uint32_t*>(xs1 + g * ld + ti * 16 + x * 8 + c2) = bf2(o[x][0], o[x][1]);
-            *reinterpret_cast<uint32_t*>(xs1 + (g + 8) * ld + ti * 16 + x * 8 + c2) = bf2(o[x][2], o[x][3]);
+        for (int z = 0; z < T; ++z) {
+            if (t0 + z >= tiles) break;
+#pragma unroll
+            for (int x = 0; x < 2; ++x) {
+                *reinterpret_cast<uint32_t*>(xs1 + g * ld + (t0 + z) * 16 + x * 8 + c2) = bf2(o[z][x][0], o[z][x][1]);
+                *reinterpret_cast<uint32_t*>(xs1 + (g + 8) * ld + (t0 + z) * 16 + x * 8 + c2) = bf2(o[z][x][2], o[z][x][3]);
+            }
         }
     }
     __syncthreads();
     if (n % 8 == 0) {
-        for (int r = warp; r < kDh; r += 8)
+        for (int r = warp; r < kDh; r += kThreads / 32)
             for (int c = lane * 8; c < n; c += 256)
                 *reinterpret_cast<uint4*>(O + base + (size_t)r * n + c) = *reinterpret_cast<const uint4*>(xs1 + r * ld + c);
     } else {
-        for (int r = warp; r < kDh; r += 8)
+        for (int r = warp; r < kDh; r += kThreads / 32)
             for (int c = lane; c < n; c += 32) O[base + (size_t)r * n + c] = xs1[r * ld + c];
     }
 }
@@ -147,11 +188,17 @@ int32_t heads_fwd(const m2_plan* pl, const void* X1, const void* X2, const void*
     if (blocks == 0) return M2_OK;
     if (blocks > 0x7fffffffLL) return M2_ERR_UNSUPPORTED;
     const int smem = smem_bytes((int)n);
-    if (smem > 48 * 1024 && cudaFuncSetAttribute(heads_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(kMaxN)) != cudaSuccess)
+    // Two tiles at a time halve the fragments and kernel values read per tile pair and leave a warp half as many groups.  Layer of d = 768, us,
+    // one tile and two: n = 1024, [8] (batch) 204.6 and 178.9, [1] 82.6 and 86.7; n = 512 [32] 261 and 242, [1] 66.2 and 59.9; 320 [8] 75.6 and 71.0;
+    // 256 [32] 89.4 and 85.7, [16] 61.9 and 60.6, [8] 49.1 and 49.8; 208 [24] 70.0 and 69.9, [8] 46.0 and 46.8.
+    const bool pairs = n > 512 ? blocks >= 64 : n > 256 || (n > 224 && blocks >= 768);
+    const int threads = pairs && n <= 256 ? 128 : 256;
+    auto kern = !pairs ? heads_kernel<256, 1> : n <= 256 ? heads_kernel<128, 2> : heads_kernel<256, 2>;
+    if (smem > 48 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(kMaxN)) != cudaSuccess)
         return M2_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)blocks);
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
@@ -159,7 +206,7 @@ int32_t heads_fwd(const m2_plan* pl, const void* X1, const void* X2, const void*
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, heads_kernel, (const __nv_bfloat16*)X1, (const __nv_bfloat16*)X2, (const __nv_bfloat16*)V, kt, (int)period,
+    if (cudaLaunchKernelEx(&cfg, kern, (const __nv_bfloat16*)X1, (const __nv_bfloat16*)X2, (const __nv_bfloat16*)V, kt, (int)period,
                            (__nv_bfloat16*)O, (int)(d / kDh), (int)n) != cudaSuccess)
         return M2_ERR_CUDA;
     pl->launches += 1;
