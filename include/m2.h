@@ -110,9 +110,10 @@ int32_t m2_spectrum_conjugate(const m2_plan* plan, const void* kf_in_dev, int64_
  * x_dev, g_dev: [B, H, n] in the plan dtype; dk_dev: [H, n] float32.
  * ws_dev: optional caller-owned workspace of m2_conv_bwd_workspace_bytes(plan, B, H) bytes (16-byte aligned; 0 bytes
  * means this plan has no kernel that uses one).  With it, plans the tensor-core path covers (bf16, N = 512 = 32 x 16)
- * run both forward transforms and the products conj(M x) (.) M g on the tensor cores (intermediates rounded to bf16
- * like the forward pass), 8 batch rows at a time, and a CUDA-core kernel adds the groups in a fixed order and applies M^-1 in
- * fp32; for N = 32768 = 32^3 (causal, n = 16384) the order-3 convolution kernel is run twice (the row pairs' conjugated
+ * take dk as sums along the diagonals of products of segments of g and x on the tensor cores (nothing is rounded between the
+ * inputs and dk; the workspace is not touched then), or, for more than 256 batch rows of fewer than 64 channels, run both forward transforms
+ * and the products conj(M x) (.) M g there (intermediates rounded to bf16 like the forward pass), 8 batch rows at a time, with a CUDA-core kernel
+ * that adds the groups in a fixed order and applies M^-1 in fp32; for N = 32768 = 32^3 (causal, n = 16384) the order-3 convolution kernel is run twice (the row pairs' conjugated
  * spectra, then the convolution of the g pairs with them) and the pairs' rows are added.  Otherwise, or with a workspace
  * too small for those, everything runs on the CUDA cores in fp32, by register transforms for powers of two from 256 to 8192, otherwise
  * one thread block per channel with its three complex rows in shared memory (N up to 8192) or, for longer rows, in the workspace (at least 24 N bytes per channel for up to

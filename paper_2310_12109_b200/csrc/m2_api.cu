@@ -339,6 +339,8 @@ int32_t m2_spectrum_conjugate(const m2_plan* plan, const void* kf_in_dev, int64_
 // the price of 2.05, 1.87 and 1.69 units, fewer than 1.5 below, so that batches whose last item is half empty can lose; the row-pair
 // kernel starts 4.3 us (600 units) later.  [33][3000][256]: 85.8 us as items, 69.8 as units; [200][768][256] 79.7 and 76.6, [200][300][256]
 // 32.9 and 35.5, [48][3000][224] 79.3 and 70.4, [48][1100][192] 27.0 and 29.9, [64][3000][256] 88.9 and 91.1.
+// (The prices are those of the mma.sync items.  From 192 positions on the tcgen05 kernel takes such items at 8.9 ns and would win some of the sizes
+// that go to the row pairs here, [48][768][256] at 18 us instead of 24.6; they keep the kernel that their results are known from.)
 static bool toeplitz_loses(int64_t B, int64_t H, int64_t n) {
     if (B <= 16 || n <= 160) return false;   // (up to 16 rows: items of 16)
     const int64_t items = H * ((B + 31) / 32), units = H * ((B + 15) / 16);

@@ -16,7 +16,8 @@
 // 42 %, load/store data pipe 45 %, 20 warps per SM): the rest is the fragments' latency between two barriers per item and a last round
 // of 2304 items on 444 blocks that is a fifth full.
 // Measured, one B200: bf16 [32][768][256] 15.8 us (20.2 with 512-point transforms on the tensor cores), [32][768][200] 13.5 us, the three
-// short convolutions of the Hyena layer at [32][768][256] in one launch 43 us (3 x 23.5).
+// short convolutions of the Hyena layer at [32][768][256] in one launch 43 us (3 x 23.5).  Of these sizes, the ones with full items are
+// toeplitz_umma.cu's now (11.9, 11.8 and 28 us; umma_pays has the line): this kernel runs shorter rows, odd lengths, small batches, few items.
 #include "m2_plan.h"
 #include "mma_sync.cuh"
 #include "toeplitz_mma.h"
