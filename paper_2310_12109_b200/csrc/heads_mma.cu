@@ -14,7 +14,7 @@
 // from L2.
 //
 // Measured, one B200, 1536 heads of n = 256: 23.6 us with one tile at a time, where 24 576 tensor-core convolution units of 16 rows took about
-// 280 us, and 20 us with two: bound by the load/store data pipe with one (60 % busy, issue 48 %: 14 wavefronts a tile pair), which two cut to 6
+// 280 us, and 22.2 us with two: bound by the load/store data pipe with one (60 % busy, issue 48 %: 14 wavefronts a tile pair), which two cut to 6
 // (they share the fragments of X2 and V, and a distance's kernel values serve the next one), and by the fragments' latency.
 #include "fft_conv.h"
 #include "fft_core.cuh"

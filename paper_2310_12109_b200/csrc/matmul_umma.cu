@@ -709,20 +709,25 @@ monarch64_wgrad_kernel(const __nv_bfloat16* __restrict__ in, const __grid_consta
 }
 
 // out = the sum of the shares, four values per thread (nshare = 0: zeros): warp y of a block adds the shares y, y + 8, .. in order, the
-// eight sums are added in order (one thread per value walking all shares: 11.1 us for 37 shares, now 9.7)
+// eight sums are added in order.  Bound by the shares' bytes (39 MB for 37 shares) once a warp's loads are in flight together: one thread per
+// value walking all shares 11.1 us, warps whose last loads came one by one 10.1, now 8.4 (cold); [5001] tokens forward and backward 166.6 -> 165.4.
 __global__ void __launch_bounds__(256) wgrad_reduce_kernel(const float4* __restrict__ partial, float4* __restrict__ out, int nshare) {
     __shared__ float4 part[8][32];
     const int lane = threadIdx.x & 31, y = threadIdx.x >> 5, e = blockIdx.x * 32 + lane;   // < 64 * 4096 / 4
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 5
-    for (int s = y; s < nshare; s += 8) {
-        const float4 v = __ldcg(partial + (size_t)s * 65536 + e);
-        acc.x += v.x;
-        acc.y += v.y;
-        acc.z += v.z;
-        acc.w += v.w;
+    for (int s0 = y; s0 < nshare; s0 += 40) {
+        float4 v[5];
+#pragma unroll
+        for (int q = 0; q < 5; ++q) v[q] = s0 + 8 * q < nshare ? __ldcg(partial + (size_t)(s0 + 8 * q) * 65536 + e) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int q = 0; q < 5; ++q) {
+            acc.x += v[q].x;
+            acc.y += v[q].y;
+            acc.z += v[q].z;
+            acc.w += v[q].w;
+        }
     }
     part[y][lane] = acc;
     __syncthreads();
