@@ -21,8 +21,19 @@ __global__ void __launch_bounds__(C::THREADS, min_blocks<C>())
     // rows of k are only as aligned as n floats make them; a pair needs 8 bytes
     load_row<C, float, HALF>(re, k + h * n, t, n, (n & 1) == 0 && (reinterpret_cast<uintptr_t>(k) & 7) == 0, live);
     unroll<16>([&](auto j) { im[j.v] = 0ull; });
-    if (kt != nullptr && live)
-        for (int i = t; i < C::N; i += C::TP) kt[h * C::N + i] = i < n ? k[h * n + i] : 0.f;
+    if (kt != nullptr && live) {   // a thread's 32 values, eight on their way together (one by one: conv_train [32][768][512] 72.9 us, so 69.7)
+#pragma unroll
+        for (int g = 0; g < 32; g += 8) {
+            float v[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const int i = t + (g + q) * C::TP;
+                v[q] = i < n ? __ldg(k + h * n + i) : 0.f;
+            }
+#pragma unroll
+            for (int q = 0; q < 8; ++q) kt[h * C::N + t + (g + q) * C::TP] = v[q];
+        }
+    }
     forward<C, HALF>(re, im, sr, si, tab, t, r);
     if (!live) return;
     const u64 sc = dup2(1.0f / (float)C::N);
