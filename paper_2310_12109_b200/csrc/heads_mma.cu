@@ -102,10 +102,10 @@ __global__ void __launch_bounds__(kThreads)
     const int tiles = np / 16, groups = (tiles + T - 1) / T, nw = kThreads / 32;
     const int front = nw * ((groups + 2 * nw - 1) / (2 * nw));   // the first half of a warp's groups in order, the second from the far end:
     for (int it = warp; it < groups; it += nw) {                 // every warp gets as many short ones as long ones
-        const int t0 = T * (it < front ? it : groups - 1 - (it - front));   // (t0 + 1 = tiles: nothing but the rows' padding, not stored)
+        const int t0 = T * (it < front ? it : groups - 1 - (it - front));
         uint32_t fa[T][4];
 #pragma unroll
-        for (int z = 0; z < T; ++z) ldsm4t(fa[z], a1 + (t0 + z) * 32);
+        for (int z = 0; z < T; ++z) ldsm4t(fa[z], a1 + min(t0 + z, tiles - 1) * 32);   // (past the last tile: that tile again, its products are not stored)
         float o[T][2][4] = {};
         uint32_t fb[4] = {}, fv[4] = {};   // the tile si of X2 and of V
         auto tile = [&](int z, float2 k0, float2 k8, float2 km) {   // the kernel at lags u, u + 8, u - 8 and the one below each
@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(kThreads)
                 }
             }
         }
-        __syncwarp();   // these tiles' columns of X1 are read by this warp only: the result takes their place
+        __syncwarp();   // these tiles' columns of X1 are read by this warp alone, above: the result takes their place
 #pragma unroll
         for (int z = 0; z < T; ++z) {
             if (t0 + z >= tiles) break;

@@ -1041,6 +1041,22 @@ def test_hyena_head_product_two_tiles_at_a_time(B, n, d, dims):
     test_hyena_head_product_with_lags_below_zero(B, n, d, dims, "full")
 
 
+@pytest.mark.parametrize("n,d,dims", [(264, 512, (32, 32)), (400, 256, (32, 32)), (1000, 1024, (64, 32))])
+def test_hyena_head_product_of_an_odd_number_of_tiles_repeats(n, d, dims):
+    """Two tiles at a time and an odd number of them: the last group has one tile, and nothing that another warp writes is read for the
+    missing one.  Results of 30 calls are the same, bit for bit."""
+    plan = M.Plan(dims, dtype=M.M2_BF16, device=0)
+    u = dev(synth.normal(synth.stream_id(21, n), (1, n, d)), torch.bfloat16)
+    W = [dev(synth.normal(synth.stream_id(21, n + 1 + i), (d, d)) / np.sqrt(d), torch.bfloat16) for i in range(4)]
+    kf = [M.m2_kernel_spectrum(plan, dev((synth.normal(synth.stream_id(21, n + 5 + i), (h, n)) / np.sqrt(n)).astype(np.float32))) for i, h in enumerate((d, d, d, d // 16))]
+    first = M.m2_hyena_heads_fwd(plan, u, W, *kf, 16)
+    assert plan.last_kernel() == "hyena_heads_fwd_fused"
+    for _ in range(30):
+        assert torch.equal(M.m2_hyena_heads_fwd(plan, u, W, *kf, 16), first)
+    assert plan.device_status() == 0
+    plan.close()
+
+
 @pytest.mark.parametrize("dims", [(64, 64), (128, 256), (256, 256)])
 def test_monarch_cols_counts_what_it_launches(dims):
     """Two launches a call whichever kernel a stage takes; a call that is refused (more tiles than the kernel can number, and too long for the
