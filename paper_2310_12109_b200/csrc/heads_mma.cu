@@ -44,7 +44,7 @@ __device__ __forceinline__ uint32_t weigh(float a, float b, float2 k) {
 }
 
 template <int kThreads, int T>   // T: tiles of 16 positions t that a warp takes at a time
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, T == 1 ? 5 : kThreads == 128 ? 7 : 0)   // (blocks per SM: 48, 72 and 80 registers, no spills)
     heads_kernel(const __nv_bfloat16* __restrict__ X1, const __nv_bfloat16* __restrict__ X2, const __nv_bfloat16* __restrict__ V,
                  const float* __restrict__ kt, int period, __nv_bfloat16* __restrict__ O, int heads, int n) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -143,16 +143,37 @@ __global__ void __launch_bounds__(kThreads)
                 k8 = n8;
             }
         }
-        if (earlier) {
+        if (earlier && t0 + 1 < tiles) {
+            auto below = [&](int lag) { return lag > -n ? __ldg(kt + period + lag) : 0.f; };   // (every lag of these tiles is below zero)
+            auto pair = [&](int lag) { return make_float2(below(lag), below(lag - 1)); };
+            if constexpr (T == 1) {
+                float2 k8 = pair(g - c2 - 8);
 #pragma unroll 1
-            for (int si = t0 + 1; si < tiles; ++si) {
-                ldsm4t(fb, b2 + si * 32);
-                ldsm4(fv, av + si * 32);
-#pragma unroll
-                for (int z = 0; z < T; ++z) {
-                    if (si <= t0 + z) continue;
-                    const int u = g - c2 + 16 * (t0 + z - si);
-                    tile(z, make_float2(value(u), value(u - 1)), make_float2(value(u + 8), value(u + 7)), make_float2(value(u - 8), value(u - 9)));
+                for (int si = t0 + 1; si < tiles; ++si) {
+                    const int u = g - c2 + 16 * (t0 - si);
+                    const float2 k0 = pair(u), km = pair(u - 8);
+                    ldsm4t(fb, b2 + si * 32);
+                    ldsm4(fv, av + si * 32);
+                    tile(0, k0, k8, km);
+                    k8 = km;   // (what was 8 below is 8 above a step later)
+                }
+            } else {
+                int u = g - c2 - 16;
+                float2 k0 = pair(u), k8 = pair(u + 8), km = pair(u - 8), l0 = {}, l8 = {}, lm = {};   // this step's, the step's before: one tile further away
+#pragma unroll 1
+                for (int si = t0 + 1; si < tiles; ++si) {
+                    u -= 16;
+                    const float2 n0 = pair(u), nm = pair(u - 8);   // the next step's, on their way while this one is multiplied
+                    ldsm4t(fb, b2 + si * 32);
+                    ldsm4(fv, av + si * 32);
+                    tile(0, k0, k8, km);
+                    if (si > t0 + 1) tile(1, l0, l8, lm);
+                    l0 = k0;
+                    l8 = k8;
+                    lm = km;
+                    k8 = km;
+                    k0 = n0;
+                    km = nm;
                 }
             }
         }
