@@ -22,6 +22,8 @@
 #include "m2_plan.h"
 #include "mma_sync.cuh"
 
+#include <type_traits>
+
 namespace m2h {
 
 constexpr int kDh = 16, kMaxN = 1024;
@@ -44,7 +46,7 @@ __device__ __forceinline__ uint32_t weigh(float a, float b, float2 k) {
 }
 
 template <int kThreads, int T>   // T: tiles of 16 positions t that a warp takes at a time
-__global__ void __launch_bounds__(kThreads, T == 1 ? 5 : kThreads == 128 ? 7 : 0)   // (blocks per SM: 48, 72 and 80 registers, no spills)
+__global__ void __launch_bounds__(kThreads, T == 1 ? 5 : 0)   // (T = 1: five blocks per SM, 48 registers without spills)
     heads_kernel(const __nv_bfloat16* __restrict__ X1, const __nv_bfloat16* __restrict__ X2, const __nv_bfloat16* __restrict__ V,
                  const float* __restrict__ kt, int period, __nv_bfloat16* __restrict__ O, int heads, int n) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -101,63 +103,65 @@ __global__ void __launch_bounds__(kThreads, T == 1 ? 5 : kThreads == 128 ? 7 : 0
     const float* kp = ks + (g & 1) * kc + np + 14 + (g & 1) - g + c2;   // lag g - c2; minus the tile distance
     const int tiles = np / 16, groups = (tiles + T - 1) / T, nw = kThreads / 32;
     const int front = nw * ((groups + 2 * nw - 1) / (2 * nw));   // the first half of a warp's groups in order, the second from the far end:
-    for (int it = warp; it < groups; it += nw) {                 // every warp gets as many short ones as long ones
-        const int t0 = T * (it < front ? it : groups - 1 - (it - front));
-        uint32_t fa[T][4];
+    auto walk = [&](auto both) {   // (two tiles at a time, both sides of the diagonal: a loop of its own, so that the other stays as it is)
+        for (int it = warp; it < groups; it += nw) {                 // every warp gets as many short ones as long ones
+            const int t0 = T * (it < front ? it : groups - 1 - (it - front));
+            uint32_t fa[T][4];
 #pragma unroll
-        for (int z = 0; z < T; ++z) ldsm4t(fa[z], a1 + min(t0 + z, tiles - 1) * 32);   // (past the last tile: that tile again, its products are not stored)
-        float o[T][2][4] = {};
-        uint32_t fb[4] = {}, fv[4] = {};   // the tile si of X2 and of V
-        auto tile = [&](int z, float2 k0, float2 k8, float2 km) {   // the kernel at lags u, u + 8, u - 8 and the one below each
-            float s0[4] = {}, s1[4] = {};
-            mma(s0, fa[z], fb[0], fb[1]);
-            mma(s1, fa[z], fb[2], fb[3]);
-            mma(o[z][0], fv, weigh(s0[0], s0[1], k0), weigh(s1[0], s1[1], km));
-            mma(o[z][1], fv, weigh(s0[2], s0[3], k8), weigh(s1[2], s1[3], k0));
-        };
-        auto kernel = [&](const float* q) { return *reinterpret_cast<const float2*>(q); };
-        if constexpr (T == 1) {
-            for (int si = 0; si <= t0; ++si) {
-                const float* kq = kp - (t0 - si) * 16;
-                ldsm4t(fb, b2 + si * 32);
-                ldsm4(fv, av + si * 32);
-                tile(0, kernel(kq), kernel(kq - 8), kernel(kq + 8));
-            }
-        } else {
-            const float* kq = kp;   // one tile further away with every step down in s: what was 8 above is then 8 below
-            float2 k0 = kernel(kq), k8 = kernel(kq - 8), km = kernel(kq + 8);
-            if (t0 + 1 < tiles) {
-                ldsm4t(fb, b2 + t0 * 32 + 32);
-                ldsm4(fv, av + t0 * 32 + 32);
-                tile(1, k0, k8, km);
-            }
-            for (int si = t0; si >= 0; --si) {
-                kq -= 16;
-                const float2 n0 = kernel(kq), n8 = kernel(kq - 8);
-                ldsm4t(fb, b2 + si * 32);
-                ldsm4(fv, av + si * 32);
-                tile(0, k0, k8, km);
-                tile(1, n0, n8, k8);
-                km = k8;
-                k0 = n0;
-                k8 = n8;
-            }
-        }
-        if (earlier && t0 + 1 < tiles) {
-            auto below = [&](int lag) { return lag > -n ? __ldg(kt + period + lag) : 0.f; };   // (every lag of these tiles is below zero)
-            auto pair = [&](int lag) { return make_float2(below(lag), below(lag - 1)); };
+            for (int z = 0; z < T; ++z) ldsm4t(fa[z], a1 + min(t0 + z, tiles - 1) * 32);   // (past the last tile: that tile again, its products are not stored)
+            float o[T][2][4] = {};
+            uint32_t fb[4] = {}, fv[4] = {};   // the tile si of X2 and of V
+            auto tile = [&](int z, float2 k0, float2 k8, float2 km) {   // the kernel at lags u, u + 8, u - 8 and the one below each
+                float s0[4] = {}, s1[4] = {};
+                mma(s0, fa[z], fb[0], fb[1]);
+                mma(s1, fa[z], fb[2], fb[3]);
+                mma(o[z][0], fv, weigh(s0[0], s0[1], k0), weigh(s1[0], s1[1], km));
+                mma(o[z][1], fv, weigh(s0[2], s0[3], k8), weigh(s1[2], s1[3], k0));
+            };
+            auto kernel = [&](const float* q) { return *reinterpret_cast<const float2*>(q); };
             if constexpr (T == 1) {
-                float2 k8 = pair(g - c2 - 8);
-#pragma unroll 1
-                for (int si = t0 + 1; si < tiles; ++si) {
-                    const int u = g - c2 + 16 * (t0 - si);
-                    const float2 k0 = pair(u), km = pair(u - 8);
+                for (int si = 0; si <= t0; ++si) {
+                    const float* kq = kp - (t0 - si) * 16;
+                    ldsm4t(fb, b2 + si * 32);
+                    ldsm4(fv, av + si * 32);
+                    tile(0, kernel(kq), kernel(kq - 8), kernel(kq + 8));
+                }
+            } else {
+                const float* kq = kp;   // one tile further away with every step down in s: what was 8 above is then 8 below
+                float2 k0 = kernel(kq), k8 = kernel(kq - 8), km = kernel(kq + 8);
+                if (t0 + 1 < tiles) {
+                    ldsm4t(fb, b2 + t0 * 32 + 32);
+                    ldsm4(fv, av + t0 * 32 + 32);
+                    tile(1, k0, k8, km);
+                }
+                for (int si = t0; si >= 0; --si) {
+                    kq -= 16;
+                    const float2 n0 = kernel(kq), n8 = kernel(kq - 8);
                     ldsm4t(fb, b2 + si * 32);
                     ldsm4(fv, av + si * 32);
                     tile(0, k0, k8, km);
-                    k8 = km;   // (what was 8 below is 8 above a step later)
+                    tile(1, n0, n8, k8);
+                    km = k8;
+                    k0 = n0;
+                    k8 = n8;
                 }
-            } else {
+            }
+            if constexpr (T == 1) {
+                if (earlier) {
+                    auto below = [&](int lag) { return lag > -n ? __ldg(kt + period + lag) : 0.f; };   // (every lag of these tiles is below zero)
+                    auto pair = [&](int lag) { return make_float2(below(lag), below(lag - 1)); };
+                    float2 k8 = pair(g - c2 - 8);
+#pragma unroll 1
+                    for (int d = 16; d < np - 16 * t0; d += 16) {
+                        const float2 k0 = pair(g - c2 - d), km = pair(g - c2 - d - 8);
+                        ldsm4t(fb, b2 + t0 * 32 + 2 * d);
+                        ldsm4(fv, av + t0 * 32 + 2 * d);
+                        tile(0, k0, k8, km);
+                        k8 = km;   // (what was 8 below is 8 above a step later)
+                    }
+                }
+            } else if constexpr (decltype(both)::value) {
+                auto pair = [&](int lag) { return make_float2(value(lag), value(lag - 1)); };
                 int u = g - c2 - 16;
                 float2 k0 = pair(u), k8 = pair(u + 8), km = pair(u - 8), l0 = {}, l8 = {}, lm = {};   // this step's, the step's before: one tile further away
 #pragma unroll 1
@@ -176,18 +180,22 @@ __global__ void __launch_bounds__(kThreads, T == 1 ? 5 : kThreads == 128 ? 7 : 0
                     km = nm;
                 }
             }
-        }
-        __syncwarp();   // these tiles' columns of X1 are read by this warp alone, above: the result takes their place
+            __syncwarp();   // these tiles' columns of X1 are read by this warp alone, above: the result takes their place
 #pragma unroll
-        for (int z = 0; z < T; ++z) {
-            if (t0 + z >= tiles) break;
+            for (int z = 0; z < T; ++z) {
+                if (t0 + z >= tiles) break;
 #pragma unroll
-            for (int x = 0; x < 2; ++x) {
-                *reinterpret_cast<uint32_t*>(xs1 + g * ld + (t0 + z) * 16 + x * 8 + c2) = bf2(o[z][x][0], o[z][x][1]);
-                *reinterpret_cast<uint32_t*>(xs1 + (g + 8) * ld + (t0 + z) * 16 + x * 8 + c2) = bf2(o[z][x][2], o[z][x][3]);
+                for (int x = 0; x < 2; ++x) {
+                    *reinterpret_cast<uint32_t*>(xs1 + g * ld + (t0 + z) * 16 + x * 8 + c2) = bf2(o[z][x][0], o[z][x][1]);
+                    *reinterpret_cast<uint32_t*>(xs1 + (g + 8) * ld + (t0 + z) * 16 + x * 8 + c2) = bf2(o[z][x][2], o[z][x][3]);
+                }
             }
         }
-    }
+    };
+    if (T > 1 && earlier)
+        walk(std::true_type{});
+    else
+        walk(std::false_type{});
     __syncthreads();
     if (n % 8 == 0) {
         for (int r = warp; r < kDh; r += kThreads / 32)
