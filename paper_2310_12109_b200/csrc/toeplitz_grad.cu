@@ -4,22 +4,25 @@
 // With t = 128 p + t' and x cut into blocks of 64 positions, the products that share p, t' and the distance rho = 2 p - block are one matrix
 // product over K = (p, b): D[t'][64 m + j'] = sum over p, b of g[b][128 p + t'] x[b][64 (2 p - top + m) + j'], and an element belongs to
 // d = 64 top + t' - (64 m + j'): dk is the sum of D along its diagonals.  Both operands are taken as the TMA delivers them (blocks of
-// [32 batch rows][64 positions], 128-byte swizzle, M/N-major: K runs over slots and rows); blocks before the row are zeros (causal) or come a
-// second time from L2 (circular).  n = 512: two accumulators of 256 columns (distances 0 .. 3 and 4 .. 7); causal n <= 256: one, the two
-// halves of tensor memory taking channels in turn.
-// Products of bf16 values are exact and everything after them is fp32: nothing is rounded between the inputs and dk, no partial sums go
-// through memory and no inverse transform follows.
+// [32 or 16 batch rows][64 positions], 128-byte swizzle, M/N-major: K runs over slots and rows); blocks before the row are zeros (causal); a
+// circular row's first two blocks come a second time from L2, so that every run of four lies in consecutive slots.  n = 512: two accumulators of
+// 256 columns (distances 0 .. 3 and 4 .. 7); causal n <= 256: one, the two halves of tensor memory taking channels in turn.
+// Products of bf16 values are exact and their sums fp32: no operand and no partial sum is rounded to bf16, no partial sums go through memory and no
+// inverse transform follows.  An accumulator is one chain over all batch rows, and the tensor core drops what lies below its last bit: the distance
+// from 64 bits is 1.4e-7 for 32 rows of 512, 1.0e-6 for 256, 4.4e-6 for 1024 (fp32 transforms, the call without a workspace: 2.0e-7 to 2.9e-7).
 //
 // Diagonal sums: a warp reads its 32 rows x 128 columns as 8 x 8 blocks, each lane holding the same two places of every block
-// (tcgen05.ld 16x256b), so the blocks along a diagonal are added without leaving the lane: 64 blocks become 19 bands, which 55 shuffles fold into
+// (tcgen05.ld 16x256b), so the blocks along a diagonal are added without leaving the lane: 64 blocks become 19 bands, which 35 shuffles fold into
 // 160 consecutive lags.  The warps' windows of lags are added through shared memory in a fixed order: results do not vary between calls.  Two
-// sets of eight warps take the channels in turn: the chain of a channel (waits, two accumulators, one exchange) is longer than its products.
+// sets of eight warps: circular, each has an accumulator of every channel; causal, they take the channels in turn.  A channel's windows are added
+// after the next one's accumulator has been read, when every warp's have long arrived.
 //
-// Measured, one B200 (call with its host work): [32][768][512] circular 31.6 -> 16.5 us, [32][768][256] causal 30.4 -> 11.4, [256][768][256] 181 ->
-// 37.7, against bf16 transforms of both operands, partial spectra and an inverse transform; distance from 64 bits 3.0e-3 -> 1.4e-7.  Bound by a
-// block's copies (88 KB a channel of 32 rows, of which 24 from L2) and its 16 UMMAs of 128 cycles, both ~2000 cycles of the ~2600 it takes; short
-// calls by launch and host.  With one shuffle per element instead of the bands the same took 22.5 us, with bands whose cross-warp sum waited
-// twice per accumulator 30.
+// Measured, one B200, us a launch, against bf16 transforms of both operands, partial spectra and an inverse transform (distance from 64 bits 3.0e-3):
+// [32][768][512] circular 30.0 and 14.0, [8][768] 13.2 and 11.1, [8][4096] 34.5 and 38.8; causal [32][768][256] 29.1 and 7.3, [8][4096] 33.1
+// and 23.  Up to 16 rows a channel costs the summing warps ~2400 cycles, whatever its rows (its 8 UMMAs take 1024): short batches of more than ~1500
+// channels are where the transforms were faster.  With 32 rows the copies (72 KB a channel) and 16 UMMAs of 128 cycles come to as much.
+// Sets that took whole channels in turn, each with both accumulators, a chain of two reads, two folds and an exchange: 15.5, 14.3, 52 us; the x row
+// twice over (14 slots): 15.7 and 44 at [32][768] and [8][4096]; eight slots and UMMAs of 128 columns where a run wraps: 14.8 and 39.3.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -36,23 +39,23 @@ using namespace sm100;
 
 namespace {
 
-constexpr int kGRows = 32, kGSlot = kGRows * 128;
 constexpr int kSumWarps = 8, kSets = 2, kLoadWarp = kSets * kSumWarps, kIssueWarp = kLoadWarp + 1, kGradThreads = 32 * (kIssueWarp + 1);
 constexpr int kBands = 19, kWindow = 8 * (kBands + 1);   // diagonals of 8 x 8 blocks in 32 rows x 128 columns; the lags they hold
 constexpr int kRed = kSumWarps * kWindow * 4;            // one accumulator's windows of a set's warps
 
-template <bool CIRC>   // circular n = 512, or causal n <= 256
+template <bool CIRC, int ROWS>   // circular n = 512, or causal n <= 256; batch rows per chunk
 struct GCfg {
+    static constexpr int SLOT = ROWS * 128;
     static constexpr int P = CIRC ? 4 : 2;                 // groups of 128 positions t
-    static constexpr int GS = 2 * P, XS = CIRC ? 14 : 6;   // slots of g and x
+    static constexpr int GS = 2 * P, XS = CIRC ? 10 : 6;   // slots of g and x
     static constexpr int GROUPS = CIRC ? 2 : 1;            // accumulators per channel
-    static constexpr int STAGE = (GS + XS) * kGSlot;
-    static constexpr int STAGES = CIRC ? 2 : 4;
+    static constexpr int STAGE = (GS + XS) * SLOT;
+    static constexpr int STAGES = CIRC ? (ROWS == 32 ? 2 : 5) : 4 * 32 / ROWS;
     static constexpr int OFF_RED = STAGES * STAGE;
-    static constexpr int OFF_BAR = OFF_RED + 2 * kSets * GROUPS * kRed;   // two per set: a warp may be a channel ahead
+    static constexpr int OFF_BAR = OFF_RED + 2 * kSets * kRed;   // two per set: a warp may be a channel ahead
     static constexpr int SMEM = OFF_BAR + 256;
 };
-static_assert(GCfg<true>::SMEM <= 232448 && GCfg<false>::SMEM <= 232448, "shared memory budget");
+static_assert(GCfg<true, 32>::SMEM <= 232448 && GCfg<false, 32>::SMEM <= 232448 && GCfg<true, 16>::SMEM <= 232448 && GCfg<false, 16>::SMEM <= 232448, "shared memory budget");
 
 // 16 rows x 32 columns: registers 4 n .. 4 n + 3 are (row, column) (l / 4, 8 n + 2 (l % 4)), the next column, and both again 8 rows below
 __device__ __forceinline__ void tmem_ld_16x32(uint32_t taddr, float* v) {
@@ -65,15 +68,15 @@ __device__ __forceinline__ void tmem_ld_16x32(uint32_t taddr, float* v) {
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-template <bool CIRC>
+template <bool CIRC, int ROWS>
 __global__ void __launch_bounds__(kGradThreads, 1)
     toeplitz_grad_kernel(const __grid_constant__ CUtensorMap mx, const __grid_constant__ CUtensorMap mg, float* __restrict__ dk, int H, int n,
                          int chunks, int32_t* __restrict__ status) {
-    using C = GCfg<CIRC>;
+    using C = GCfg<CIRC, ROWS>;
     extern __shared__ __align__(1024) unsigned char smem[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t s0 = smem_u32(smem);
-    const uint32_t bar_f = s0 + C::OFF_BAR, bar_e = bar_f + 8 * C::STAGES, bar_df = bar_e + 8 * C::STAGES, bar_de = bar_df + 8 * kSets * C::GROUPS, bar_r = bar_de + 16,
+    const uint32_t bar_f = s0 + C::OFF_BAR, bar_e = bar_f + 8 * C::STAGES, bar_df = bar_e + 8 * C::STAGES, bar_de = bar_df + 16, bar_r = bar_de + 16,
                    s_tptr = bar_r + 8 * kSets;
     volatile uint32_t* tptr = reinterpret_cast<volatile uint32_t*>(smem + (s_tptr - s0));
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + (s_tptr - s0) + 4);
@@ -82,16 +85,18 @@ __global__ void __launch_bounds__(kGradThreads, 1)
             mbar_init(bar_f + 8 * s, 1);
             mbar_init(bar_e + 8 * s, 1);
         }
-        for (int z = 0; z < kSets * C::GROUPS; ++z) mbar_init(bar_df + 8 * z, 1);   // per set: neither waits on a phase of the other's
-        for (int a = 0; a < 2; ++a) mbar_init(bar_de + 8 * a, kSumWarps);
-        for (int z = 0; z < kSets; ++z) mbar_init(bar_r + 8 * z, kSumWarps);
+        for (int a = 0; a < 2; ++a) {   // an accumulator is one set's
+            mbar_init(bar_df + 8 * a, 1);
+            mbar_init(bar_de + 8 * a, kSumWarps);
+            mbar_init(bar_r + 8 * a, CIRC ? kSets * kSumWarps : kSumWarps);
+        }
         *abort_flag = 0;
         fence_barrier_init();
     }
     if (!CIRC) {   // the blocks before a row are zero for good
-        for (int i = tid; i < C::STAGES * 2 * (kGSlot / 16); i += kGradThreads) {
-            const int st = i / (2 * (kGSlot / 16)), r = i % (2 * (kGSlot / 16));
-            *reinterpret_cast<uint4*>(smem + st * C::STAGE + C::GS * kGSlot + r * 16) = make_uint4(0, 0, 0, 0);
+        for (int i = tid; i < C::STAGES * 2 * (C::SLOT / 16); i += kGradThreads) {
+            const int st = i / (2 * (C::SLOT / 16)), r = i % (2 * (C::SLOT / 16));
+            *reinterpret_cast<uint4*>(smem + st * C::STAGE + C::GS * C::SLOT + r * 16) = make_uint4(0, 0, 0, 0);
         }
         fence_proxy_async();
     }
@@ -115,20 +120,20 @@ __global__ void __launch_bounds__(kGradThreads, 1)
                         ok = false;
                         break;
                     }
-                    const uint32_t ga = s0 + s * C::STAGE, xa = ga + C::GS * kGSlot, bar = bar_f + 8 * s;
-                    mbar_expect_tx(bar, (uint32_t)((C::GS + (CIRC ? C::XS : 4)) * kGSlot));
-                    for (int j = 0; j < C::GS; ++j) tma_load_4d(ga + j * kGSlot, &mg, 64 * j, h, ch * kGRows, 0, bar);
+                    const uint32_t ga = s0 + s * C::STAGE, xa = ga + C::GS * C::SLOT, bar = bar_f + 8 * s;
+                    mbar_expect_tx(bar, (uint32_t)((C::GS + (CIRC ? C::XS : 4)) * C::SLOT));
+                    for (int j = 0; j < C::GS; ++j) tma_load_4d(ga + j * C::SLOT, &mg, 64 * j, h, ch * ROWS, 0, bar);
                     if (CIRC) {
-                        for (int j = 0; j < C::XS; ++j) tma_load_4d(xa + j * kGSlot, &mx, 64 * ((j + 1) & 7), h, ch * kGRows, 0, bar);
+                        for (int j = 0; j < C::XS; ++j) tma_load_4d(xa + j * C::SLOT, &mx, 64 * ((j + 1) & 7), h, ch * ROWS, 0, bar);
                     } else {
-                        for (int j = 0; j < 4; ++j) tma_load_4d(xa + (j + 2) * kGSlot, &mx, 64 * j, h, ch * kGRows, 0, bar);
+                        for (int j = 0; j < 4; ++j) tma_load_4d(xa + (j + 2) * C::SLOT, &mx, 64 * j, h, ch * ROWS, 0, bar);
                     }
                 }
             for (int i = v > C::STAGES ? v - C::STAGES : 0; i < v && ok; ++i) ok = mbar_wait(bar_e + 8 * (i % C::STAGES), (i / C::STAGES) & 1);
         }
     } else if (warp == kIssueWarp) {
         constexpr uint32_t idesc = instr_desc_bf16(128, 256, true, true);
-        const uint64_t da0 = smem_desc_sw128(s0, kGSlot, 1024), db0 = smem_desc_sw128(s0 + C::GS * kGSlot, kGSlot, 1024);
+        const uint64_t da0 = smem_desc_sw128(s0, C::SLOT, 1024), db0 = smem_desc_sw128(s0 + C::GS * C::SLOT, C::SLOT, 1024);
         int v = 0, it = 0;
         for (int h = blockIdx.x; h < H && ok; h += gridDim.x, ++it)
             for (int ch = 0; ch < chunks && ok; ++ch, ++v) {
@@ -143,96 +148,107 @@ __global__ void __launch_bounds__(kGradThreads, 1)
                     if (!ok) break;
                     tc_fence_after();
                     if (elect_one()) {
-                        const uint64_t da = da0 + (uint32_t)(s * C::STAGE >> 4), db = db0 + (uint32_t)((s * C::STAGE + (C::GROUPS == 2 ? 4 - 4 * gr : 0) * kGSlot) >> 4);
+                        const uint64_t da = da0 + (uint32_t)(s * C::STAGE >> 4), db = db0 + (uint32_t)(s * C::STAGE >> 4);
 #pragma unroll
                         for (int p = 0; p < C::P; ++p)
 #pragma unroll
-                            for (int ks = 0; ks < 2; ++ks)
-                                umma_f16(tmem + a * 256, da + (uint32_t)((2 * p * kGSlot + ks * 2048) >> 4), db + (uint32_t)((2 * p * kGSlot + ks * 2048) >> 4), idesc,
+                            for (int ks = 0; ks < ROWS / 16; ++ks) {
+                                const int sl = C::GROUPS == 2 ? (2 * p + 4 - 4 * gr) & 7 : 2 * p;   // the first of the four slots that meet segment p
+                                umma_f16(tmem + a * 256, da + (uint32_t)((2 * p * C::SLOT + ks * 2048) >> 4), db + (uint32_t)((sl * C::SLOT + ks * 2048) >> 4), idesc,
                                          ch != 0 || p != 0 || ks != 0);
-                        if (ch == chunks - 1) umma_commit(bar_df + 8 * (it % kSets * C::GROUPS + gr));
+                            }
+                        if (ch == chunks - 1) umma_commit(bar_df + 8 * a);
                         if (gr == C::GROUPS - 1) umma_commit(bar_e + 8 * s);
                     }
                     __syncwarp();
                 }
             }
     } else {
-        const int set = warp / kSumWarps, sw = warp % kSumWarps, q = warp & 3, hc = sw >> 2;   // rows 32 q .. of the accumulators, columns 128 hc ..
-        const int r = lane >> 2, m = lane & 3;
-        int it = set;
-        for (int h = blockIdx.x + set * gridDim.x; h < H && ok; h += kSets * gridDim.x, it += kSets) {
-            float* red = reinterpret_cast<float*>(smem + C::OFF_RED) + (set * 2 + ((it / kSets) & 1)) * C::GROUPS * kSumWarps * kWindow;
-#pragma unroll 1
-            for (int gr = 0; gr < C::GROUPS; ++gr) {
-                const int a = C::GROUPS == 2 ? gr : it & 1;
-                ok = mbar_wait(bar_df + 8 * (set * C::GROUPS + gr), (it / kSets) & 1);
-                ok = __all_sync(0xffffffffu, ok && *abort_flag == 0);
-                if (!ok) break;
-                tc_fence_after();
-                float2 band[kBands];   // block (R, k) of 8 x 8 adds to band R - k + 15
+        const int set = warp / kSumWarps, sw = warp % kSumWarps, q = warp & 3, hc = sw >> 2;   // rows 32 q .. of the set's accumulator, columns 128 hc ..
+        const int r = lane >> 2, m = lane & 3, from1 = ((r + (m & 1 ? -2 : 2)) & 7) << 2 | (m ^ 1), from2 = (r ^ 4) << 2 | (m ^ 2);
+        // circular: both sets take every channel, an accumulator each; causal: they take the channels in turn
+        const int step = CIRC ? gridDim.x : kSets * gridDim.x;
+        const uint32_t bar_set = bar_r + (CIRC ? 0 : 8 * set);
+        float* const red = reinterpret_cast<float*>(smem + C::OFF_RED) + (CIRC ? 0 : 2 * set) * kSumWarps * kWindow;
+        constexpr int kBuf = (CIRC ? kSets : 1) * kSumWarps * kWindow;   // the windows of a channel; two buffers
+        // dk of the channel hp, the j-th of this warp.  The window of (set, q, hc) begins at lag 64 top + 32 q - 128 hc - 128, top = 3 and 7 (circular,
+        // modulo 512), 2 (causal), and holds five times 32 lags: 32 lags lie in the windows q = c - 4 .. c of each hc, whose block c - q of 32 they
+        // are; circular, c < 8 in one of the sets.
+        auto finish = [&](int hp, int j) {
+            bool done = mbar_wait(bar_set, j & 1);
+            if (!__all_sync(0xffffffffu, done && *abort_flag == 0)) return false;
+            const int d = 32 * (CIRC ? warp : sw) + lane;
+            float sum = 0.f;
 #pragma unroll
-                for (int z = 0; z < kBands; ++z) band[z] = make_float2(0.f, 0.f);
-                const uint32_t tcol = tmem + ((uint32_t)(q * 32) << 16) + a * 256 + hc * 128;
+            for (int hz = 0; hz < 2; ++hz) {
+                int c = (CIRC ? warp - 2 : sw) + 4 * hz;
+                const int z = CIRC ? (c >> 3) & 1 : 0;
+                if (CIRC) c &= 7;
+                const float* w = red + (j & 1) * kBuf + (z * kSumWarps + 4 * hz) * kWindow + 32 * c + lane;
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    float v[2][16];
-                    tmem_ld_16x32(tcol + 32 * c, v[0]);
-                    tmem_ld_16x32(tcol + (16u << 16) + 32 * c, v[1]);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int z = 0; z < 4; ++z) tmem_ld_fence8(&v[0][0] + 8 * z);
-#pragma unroll
-                    for (int R = 0; R < 4; ++R)
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            float2& b = band[R - (4 * c + k) + 15];
-                            b.x += v[R >> 1][4 * k + 2 * (R & 1)];
-                            b.y += v[R >> 1][4 * k + 2 * (R & 1) + 1];
-                        }
-                }
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bar_de + 8 * a);
-                // lags 8 z + 0 .. 7 of the window: places with row - column = i of band z - 1 and i - 8 of band z; lane (r, m) gets lag 8 (4 j + m) + r
-#pragma unroll
-                for (int j = 0; j < 5; ++j) {
-                    float t[4];
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const int z = 4 * j + e;
-                        const float2 lo = z > 0 ? band[z - 1] : make_float2(0.f, 0.f), up = z < kBands ? band[z] : make_float2(0.f, 0.f);
-                        const float v0 = r >= 2 * m ? lo.x : up.x, v1 = r > 2 * m ? lo.y : up.y;
-                        t[e] = v0 + __shfl_sync(0xffffffffu, v1, lane + 4);   // (row r + 1, column 2 m + 1) joins (row r, column 2 m)
-                        t[e] = __shfl_sync(0xffffffffu, t[e], lane + 8 * m);   // i = r - 2 m: the four columns' rows side by side
-                    }
-                    const float s01 = (m & 1 ? t[1] : t[0]) + __shfl_xor_sync(0xffffffffu, m & 1 ? t[0] : t[1], 1);
-                    const float s23 = (m & 1 ? t[3] : t[2]) + __shfl_xor_sync(0xffffffffu, m & 1 ? t[2] : t[3], 1);
-                    red[(gr * kSumWarps + sw) * kWindow + 32 * j + 8 * m + r] = (m & 2 ? s23 : s01) + __shfl_xor_sync(0xffffffffu, m & 2 ? s01 : s23, 2);
-                }
+                for (int qz = 0; qz < 4; ++qz)
+                    if (c - qz >= 0 && c - qz <= 4) sum += w[qz * (kWindow - 32)];
             }
-            if (!ok) break;
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar_r + 8 * set);
-            ok = mbar_wait(bar_r + 8 * set, (it / kSets) & 1);
+            if (d < n) dk[(size_t)hp * n + d] = sum;
+            return true;
+        };
+        int j = 0;
+        for (int h = blockIdx.x + (CIRC ? 0 : set * gridDim.x); h < H; h += step, ++j) {
+            ok = mbar_wait(bar_df + 8 * set, j & 1);
             ok = __all_sync(0xffffffffu, ok && *abort_flag == 0);
             if (!ok) break;
-            // the window of (gr, q, hc) begins at lag 64 top + 32 q - 128 hc - 128, top = 3 and 7 (circular, modulo 512), 2 (causal).  (The set's
-            // next channel goes to the other buffer; this one is written again when every warp of the set has passed here.)
+            tc_fence_after();
+            uint64_t band[kBands];   // block (R, k) of 8 x 8 adds to band R - k + 15
 #pragma unroll
-            for (int z = 0; z < (CIRC ? 2 : 1); ++z) {
-                const int d = 32 * sw + lane + 256 * z;
-                float sum = 0.f;
+            for (int z = 0; z < kBands; ++z) band[z] = 0ull;
+            const uint32_t tcol = tmem + ((uint32_t)(q * 32) << 16) + set * 256 + hc * 128;
 #pragma unroll
-                for (int gr = 0; gr < C::GROUPS; ++gr)
+            for (int c = 0; c < 4; ++c) {
+                float v[2][16];
+                tmem_ld_16x32(tcol + 32 * c, v[0]);
+                tmem_ld_16x32(tcol + (16u << 16) + 32 * c, v[1]);
+                tmem_ld_wait();
 #pragma unroll
-                    for (int w = 0; w < kSumWarps; ++w) {
-                        int o = d - 64 * (CIRC ? 3 + 4 * gr : 2) - 32 * (w & 3) + 128 * (w >> 2) + 128;
-                        if (CIRC) o &= 511;
-                        if (o >= 0 && o < kWindow) sum += red[(gr * kSumWarps + w) * kWindow + o];
+                for (int z = 0; z < 4; ++z) tmem_ld_fence8(&v[0][0] + 8 * z);
+#pragma unroll
+                for (int R = 0; R < 4; ++R)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        uint64_t& b = band[R - (4 * c + k) + 15];
+                        b = add2(b, pk2(v[R >> 1][4 * k + 2 * (R & 1)], v[R >> 1][4 * k + 2 * (R & 1) + 1]));
                     }
-                if (d < n) dk[(size_t)h * n + d] = sum;
             }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_de + 8 * set);
+            if (j > 0) {   // the channel before: its windows have had this one's wait and loads to arrive in
+                ok = finish(h - step, j - 1);
+                if (!ok) break;
+            }
+            // lags 8 z + 0 .. 7 of the window: places with row - column = i of band z - 1 and i - 8 of band z; lane (r, m) gets lag 8 (4 y + m) + (r - 2 m mod 8).
+            // (The buffer was read two channels ago; every warp has been through that when the barrier of the last one, just waited for, completed.)
+            float* win = red + (j & 1) * kBuf + (CIRC ? warp : sw) * kWindow;
+#pragma unroll
+            for (int y = 0; y < 5; ++y) {
+                float t[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int z = 4 * y + e;
+                    float lox = 0.f, loy = 0.f, upx = 0.f, upy = 0.f;
+                    if (z > 0) upk2(band[z - 1], lox, loy);
+                    if (z < kBands) upk2(band[z], upx, upy);
+                    const float v0 = r >= 2 * m ? lox : upx, v1 = r > 2 * m ? loy : upy;
+                    t[e] = v0 + __shfl_sync(0xffffffffu, v1, lane + 4);   // (row r + 1, column 2 m + 1) joins (row r, column 2 m): i = r - 2 m
+                }
+                // the same i is two rows further down a column pair to the right, four rows two of them
+                const float s01 = (m & 1 ? t[1] : t[0]) + __shfl_sync(0xffffffffu, m & 1 ? t[0] : t[1], from1);
+                const float s23 = (m & 1 ? t[3] : t[2]) + __shfl_sync(0xffffffffu, m & 1 ? t[2] : t[3], from1);
+                win[32 * y + 8 * m + ((r - 2 * m) & 7)] = (m & 2 ? s23 : s01) + __shfl_sync(0xffffffffu, m & 2 ? s01 : s23, from2);
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_set);
         }
+        if (ok && j > 0) ok = finish(blockIdx.x + (CIRC ? 0 : set * gridDim.x) + (j - 1) * step, j - 1);
     }
     if (!ok && lane == 0) {
         *abort_flag = 1;
@@ -256,37 +272,41 @@ bool grad_covers(const m2_plan* pl, int64_t B, int64_t H, int64_t n, bool causal
 
 int32_t conv_grad(const m2_plan* pl, const void* x, const void* g, float* dk, int64_t B, int64_t H, int64_t n, bool causal, cudaStream_t stream) {
     if (!grad_covers(pl, B, H, n, causal) || B > 0x7fffffffLL || H > 0x7fffffffLL) return M2_ERR_UNSUPPORTED;
+    // Up to 16 batch rows: chunks of 16, half the copies and UMMAs (K = 16 is the least): [8][4096][512] circular 52 -> 47 us with the kernel as it was
+    const int rows = B <= 16 ? 16 : 32;
+    auto kern = causal ? (rows == 16 ? toeplitz_grad_kernel<false, 16> : toeplitz_grad_kernel<false, 32>)
+                       : (rows == 16 ? toeplitz_grad_kernel<true, 16> : toeplitz_grad_kernel<true, 32>);
+    const int smem = causal ? (rows == 16 ? GCfg<false, 16>::SMEM : GCfg<false, 32>::SMEM) : (rows == 16 ? GCfg<true, 16>::SMEM : GCfg<true, 32>::SMEM);
     alignas(64) CUtensorMap m[2];
     const void* const src[2] = {x, g};
-    for (int i = 0; i < 2; ++i) {   // box: 64 positions of 32 batch rows
+    for (int i = 0; i < 2; ++i) {   // box: 64 positions of a chunk's batch rows
         const cuuint64_t gdim[4] = {(cuuint64_t)n, (cuuint64_t)H, (cuuint64_t)B, 1};
         const cuuint64_t gstr[3] = {(cuuint64_t)n * 2, (cuuint64_t)H * n * 2, (cuuint64_t)B * H * n * 2};
-        const cuuint32_t box[4] = {64, 1, (cuuint32_t)kGRows, 1};
+        const cuuint32_t box[4] = {64, 1, (cuuint32_t)rows, 1};
         if (!tma_host::encode_sw128_bf16(&m[i], src[i], 4, gdim, gstr, box)) return M2_ERR_UNSUPPORTED;
     }
-    static std::atomic<bool> done[64];
+    static std::atomic<uint32_t> done[64];   // bit per kernel
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return M2_ERR_CUDA;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const bool known = dev >= 0 && dev < 64;
-    if (!known || !done[dev].load(std::memory_order_acquire)) {
-        if (cudaFuncSetAttribute(toeplitz_grad_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, GCfg<true>::SMEM) != cudaSuccess ||
-            cudaFuncSetAttribute(toeplitz_grad_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, GCfg<false>::SMEM) != cudaSuccess)
-            return M2_ERR_CUDA;
-        if (known) done[dev].store(true, std::memory_order_release);
+    const uint32_t bit = 1u << ((causal ? 2 : 0) + (rows == 16 ? 1 : 0));
+    if (!known || !(done[dev].load(std::memory_order_acquire) & bit)) {
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return M2_ERR_CUDA;
+        if (known) done[dev].fetch_or(bit, std::memory_order_release);
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(H < sms ? H : sms));
     cfg.blockDim = dim3(kGradThreads);
-    cfg.dynamicSmemBytes = causal ? GCfg<false>::SMEM : GCfg<true>::SMEM;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const int chunks = (int)((B + kGRows - 1) / kGRows);
-    if (cudaLaunchKernelEx(&cfg, causal ? toeplitz_grad_kernel<false> : toeplitz_grad_kernel<true>, m[0], m[1], dk, (int)H, (int)n, chunks, pl->d_status) != cudaSuccess)
+    const int chunks = (int)((B + rows - 1) / rows);
+    if (cudaLaunchKernelEx(&cfg, kern, m[0], m[1], dk, (int)H, (int)n, chunks, pl->d_status) != cudaSuccess)
         return M2_ERR_CUDA;
     pl->launches += 1;
     return M2_OK;

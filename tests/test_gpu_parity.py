@@ -200,11 +200,13 @@ def test_kernel_gradient_adds_its_parts(B, H, n, causal):
     plan.close()
 
 
-@pytest.mark.parametrize("B,H,n", [(1, 1, 512), (33, 297, 512), (31, 150, 256), (64, 5, 144), (3, 4, 16), (300, 3, 512)])
+@pytest.mark.parametrize("B,H,n", [(1, 1, 512), (33, 297, 512), (31, 150, 256), (64, 5, 144), (3, 4, 16), (300, 3, 512),
+                                    (16, 600, 512), (7, 1250, 256), (17, 2, 512)])
 def test_kernel_gradient_of_products_of_segments(B, H, n):
     """N = 512 with a workspace: one and three channels per block (both sets of summing warps), whole and partial batch chunks accumulated in
     place, causal lengths that fill one and both groups of 128 positions.  Products of bf16 values are exact and the sums fp32, B n terms: a few
-    times 2^-24 (1.4e-7 to 4e-7 measured).  The last size stays with the bf16 transforms."""
+    times 2^-24 (1.4e-7 to 4e-7 measured).  Chunks of 16 rows up to that many, with every stage, accumulator and exchange buffer used again.  More
+    than 256 rows of few channels stay with the bf16 transforms."""
     x, g = synth.round_bf16(synth.normal(790 + n, (B, H, n))).astype(np.float64), synth.round_bf16(synth.normal(791 + n, (B, H, n))).astype(np.float64)
     plan = M.Plan((32, 16), dtype=M.M2_BF16, device=0)
     dk = M.m2_monarch_conv_bwd_kernel(plan, dev(x, torch.bfloat16), dev(g, torch.bfloat16), M.M2_CIRCULAR if n == 512 else M.M2_CAUSAL)
