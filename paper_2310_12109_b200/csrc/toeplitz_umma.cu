@@ -44,7 +44,7 @@ constexpr int kKBuf = 2048;   // a kernel row: up to 512 fp32 values
 constexpr int kKRows = 2;     // ... of which this many are on their way
 constexpr int kImages = 2;
 
-constexpr int kDiags = 5 * S / 8 - 1, kAllDiags = 8 * S / 8 - 1;   // core matrices of one part: lags above -64, and those further below zero
+constexpr int kOwnDiag = 3 * S / 8, kDiags = 5 * S / 8 - 1, kAllDiags = 8 * S / 8 - 1;   // core matrices of one part: the first of a segment with itself; lags above -64; all
 constexpr int kAcc = 512 / (2 * S);                                // accumulators of 2 S columns
 
 constexpr int kSlots = 10, kStages = 3;                            // segments -3 .. 3, and up to 6 for lags below zero
@@ -205,7 +205,6 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) toeplitz_umma_kernel(const __
                 dst[0] = make_uint4(hi[0], hi[1], hi[2], hi[3]);
                 dst[8] = make_uint4(lo[0], lo[1], lo[2], lo[3]);
             };
-            for (int w = bt; w < 8 * kDiags; w += 32 * kBuildWarps) window(w);
             bool later = false, earlier = false;   // (every building warp looks at all lags: they need not meet)
 #pragma unroll
             for (int u = 1 + lane; u < 256; u += 32) {
@@ -215,8 +214,8 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) toeplitz_umma_kernel(const __
             later = __any_sync(0xffffffffu, later);
             earlier = __any_sync(0xffffffffu, earlier);
             if (bt == 0) flags[b] = (later ? 1u : 0u) | (earlier ? 2u : 0u);
-            if (earlier)
-                for (int w = 8 * kDiags + bt; w < 8 * kAllDiags; w += 32 * kBuildWarps) window(w);
+            // the diagonals that the walked segments reach
+            for (int w = (later ? 0 : 8 * kOwnDiag) + bt; w < 8 * (earlier ? kAllDiags : kDiags); w += 32 * kBuildWarps) window(w);
             fence_proxy_async();
             __syncwarp();
             if (lane == 0) {
