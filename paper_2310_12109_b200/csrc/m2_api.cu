@@ -287,7 +287,6 @@ int32_t m2_monarch_conv_bwd_kernel(const m2_plan* plan, const void* x_dev, const
     const int64_t need = m2u::conv_wgrad_workspace_bytes(plan, B, H);
     if (need > 0 && B > 0 && ws_dev && ws_bytes >= need) {   // tensor-core transforms and products, CUDA-core sum + inverse
         st = m2t::conv_grad(plan, x_dev, g_dev, dk_dev, B, H, n, mode == M2_CAUSAL, (cudaStream_t)stream);
-        if (st == M2_OK) plan->last_kernel = "conv_wgrad_umma_o2_512";
         if (st != M2_ERR_UNSUPPORTED) return st;
         int parts = 0;
         st = m2u::conv_wgrad_partials(plan, x_dev, g_dev, ws_dev, B, H, n, mode, &parts, (cudaStream_t)stream);
@@ -363,7 +362,6 @@ static int32_t conv_fwd_grouped(const m2_plan* plan, const void* x_dev, const vo
         (!m2u::covers_rows(plan, n) || (B > 8 && !toeplitz_loses(B, H, n)))) {
         const m2t::Rows rows = {x_dev, m2t::time_kernel(plan, kf_dev, H / kf_group), y_dev};
         const int32_t tst = m2t::conv(plan, &rows, 1, B, H, n, (int)kf_group, (cudaStream_t)stream);
-        if (tst == M2_OK) plan->last_kernel = "conv_toeplitz_mma";
         if (tst != M2_ERR_UNSUPPORTED) return tst;
     }
     // tensor-core path where a kernel exists for the shape, CUDA-core path otherwise

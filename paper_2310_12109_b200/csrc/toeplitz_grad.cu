@@ -308,6 +308,7 @@ int32_t conv_grad(const m2_plan* pl, const void* x, const void* g, float* dk, in
     const int chunks = (int)((B + rows - 1) / rows);
     if (cudaLaunchKernelEx(&cfg, kern, m[0], m[1], dk, (int)H, (int)n, chunks, pl->d_status) != cudaSuccess)
         return M2_ERR_CUDA;
+    pl->last_kernel = "conv_wgrad_toeplitz";
     pl->launches += 1;
     return M2_OK;
 }

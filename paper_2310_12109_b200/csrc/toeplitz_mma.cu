@@ -229,6 +229,7 @@ int32_t conv(const m2_plan* pl, const Rows* sets, int count, int64_t B, int64_t 
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if (cudaLaunchKernelEx(&cfg, kern, s, (int)items, (int)B, (int)H, (int)n, (int)pl->N, kf_group) != cudaSuccess) return M2_ERR_CUDA;
+    pl->last_kernel = "conv_toeplitz_mma";
     pl->launches += 1;
     return M2_OK;
 }

@@ -334,6 +334,7 @@ int32_t conv_umma(const m2_plan* pl, const Rows* sets, int count, int64_t B, int
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if (cudaLaunchKernelEx(&cfg, toeplitz_umma_kernel, A, pl->d_status) != cudaSuccess) return M2_ERR_CUDA;
+    pl->last_kernel = "conv_toeplitz_umma";
     pl->launches += 1;
     return M2_OK;
 }
