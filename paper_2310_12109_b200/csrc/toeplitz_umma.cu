@@ -291,11 +291,14 @@ bool map_rows(CUtensorMap* m, const void* p, int64_t B, int64_t H, int64_t n) {
 }  // namespace
 
 // With the machine full an item takes 8.9 ns here, whatever n and the rows it holds; the mma.sync kernel's items of 32 rows take 12.7 (n =
-// 256), 12.0 (200), 10.9 (192) and 8.7 ns (136), its items of 16 rows half of that.  One set, us, there and here: [32][768][256] 15.7 and 11.9,
-// [17] 14.4 and 11.5, [16] 9.6 and 11.5, [33][768][200] 22.4 and 17.9, [32][768][192] 13.0 and 11.7, [136] 10.3 and 11.6.  Few items: both are one
-// launch, this one with its set-up and its tensor maps.
+// 256), 12.0 (200), 10.9 (192) and 8.7 ns (136), its items of 16 rows half of that.  One set, us, there and here: [32][768][256] 14.4 and 11.5,
+// [33][768][216] 21.5 and 17.7, [32][768][192] 11.9 and 11.4, [16][768][256] 9.6 and 11.5.  This kernel starts 1.5 to 2 us later (set-up, tensor maps), and the
+// other takes up to three items per SM, 444 in all, in one round; what its fourth to sixth cost grows with n.  Items, there and here, n = 256:
+// [300] 7.5 and 7.3, [444] 7.6 and 8.2, [445] 9.5 and 8.6; 224: [444] 7.0 and 8.2, [445] 8.6 both, [520] 9.6 and 9.0; 192: [296] 5.0 and 6.9, [444] 6.4 and 8.1,
+// [520] 8.8 and 8.9, [592] 10.8 and 9.4.
 bool umma_pays(const m2_plan* pl, int count, int64_t B, int64_t H, int64_t n) {
-    return has_time_kernel(pl) && pl->N == 512 && n >= 192 && n <= 256 && n % 8 == 0 && B > 16 && count * H * ((B + kRowsPerItem - 1) / kRowsPerItem) >= 296;
+    return has_time_kernel(pl) && pl->N == 512 && n >= 192 && n <= 256 && n % 8 == 0 && B > 16 &&
+           count * H * ((B + kRowsPerItem - 1) / kRowsPerItem) >= 445 + (256 - n) * 3 / 2;
 }
 
 int32_t conv_umma(const m2_plan* pl, const Rows* sets, int count, int64_t B, int64_t H, int64_t n, int kf_group, cudaStream_t stream) {
