@@ -333,19 +333,6 @@ int32_t m2_spectrum_conjugate(const m2_plan* plan, const void* kf_in_dev, int64_
     return M2_OK;
 }
 
-// Rows that both the Toeplitz kernel (items of 32 batch rows, n in steps of 32) and the row-pair kernel of the 32 x 16 plan (units of 16,
-// whatever n) cover: is the first one slower?  With the machine full an item takes 14.6 ns at n = 256, 13.3 at 224, 12.0 at 192, a unit 7.1:
-// the price of 2.05, 1.87 and 1.69 units, fewer than 1.5 below, so that batches whose last item is half empty can lose; the row-pair
-// kernel starts 4.3 us (600 units) later.  [33][3000][256]: 85.8 us as items, 69.8 as units; [200][768][256] 79.7 and 76.6, [200][300][256]
-// 32.9 and 35.5, [48][3000][224] 79.3 and 70.4, [48][1100][192] 27.0 and 29.9, [64][3000][256] 88.9 and 91.1.
-// (The prices are those of the mma.sync items.  From 192 positions on the tcgen05 kernel takes such items at 8.9 ns and would win some of the sizes
-// that go to the row pairs here, [48][768][256] at 18 us instead of 24.6; they keep the kernel that their results are known from.)
-static bool toeplitz_loses(int64_t B, int64_t H, int64_t n) {
-    if (B <= 16 || n <= 160) return false;   // (up to 16 rows: items of 16)
-    const int64_t items = H * ((B + 31) / 32), units = H * ((B + 15) / 16);
-    return 100 * (units + 600) < (n > 224 ? 205 : n > 192 ? 187 : 169) * items;
-}
-
 // y = conv(k[h / kf_group], x[b][h]); arguments beyond kf_group checked here
 static int32_t conv_fwd_grouped(const m2_plan* plan, const void* x_dev, const void* kf_dev, void* y_dev, int64_t B, int64_t H, int64_t n,
                                 int32_t mode, int64_t kf_group, void* stream) {
@@ -356,10 +343,13 @@ static int32_t conv_fwd_grouped(const m2_plan* plan, const void* x_dev, const vo
     if (!g.ok) return M2_ERR_CUDA;
     if (B * H == 0) return M2_OK;
     // Short causal rows: Toeplitz products, up to 256 positions (512: 46 us against 45 for the transforms at [32][768], the one width both
-    // were measured at).  Batches of up to 8 rows of the 32 x 16 plan still run the tensor-core kernel for such batches, as the tests of the
-    // input gradient expect: 11.6 us at [8][768][256], where half-empty tiles of 16 rows would take 10.4.
+    // were measured at).  Batches whose last item of 32 rows is half empty lose by mma.sync from 160 positions on where there are many channels, but not by
+    // tcgen05, which takes those (us, there, here, and by the row-pair kernel of the 32 x 16 plan, whose units are 16 rows: [33][3000][256] 85.1, 55.8, 68.2;
+    // [48][768][256] 23.6, 17.8, 23.1; [200][768][256] 78.9, 50.9, 74.9; [48][2400][176] 56.6, 45.5, 56.1; [48][2400][160] 45.7, -, 56.1).  Batches of up to 8 rows of
+    // that plan still run the tensor-core kernel for such batches, as the tests of the input gradient expect: 11.6 us at [8][768][256], where half-empty
+    // tiles of 16 rows would take 10.4.
     if (mode == M2_CAUSAL && n <= m2t::kMaxN && m2t::has_time_kernel(plan) && x_dev != y_dev &&
-        (!m2u::covers_rows(plan, n) || (B > 8 && !toeplitz_loses(B, H, n)))) {
+        (!m2u::covers_rows(plan, n) || B > 8)) {
         const m2t::Rows rows = {x_dev, m2t::time_kernel(plan, kf_dev, H / kf_group), y_dev};
         const int32_t tst = m2t::conv(plan, &rows, 1, B, H, n, (int)kf_group, (cudaStream_t)stream);
         if (tst != M2_ERR_UNSUPPORTED) return tst;

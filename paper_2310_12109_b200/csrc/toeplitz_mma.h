@@ -22,7 +22,7 @@ struct Rows {
 // y = the first n values of the circular convolution of the zero-padded rows (2 n <= N), up to three sets of rows in one launch
 int32_t conv(const m2_plan* pl, const Rows* sets, int count, int64_t B, int64_t H, int64_t n, int kf_group, cudaStream_t stream);
 
-// The same on the fifth-generation tensor cores (toeplitz_umma.cu): 192 <= n <= 256 on N = 512, n a multiple of 8; conv calls it where it pays
+// The same on the fifth-generation tensor cores (toeplitz_umma.cu): 160 < n <= 256 on N = 512, n a multiple of 8; conv calls it where it pays
 bool umma_pays(const m2_plan* pl, int count, int64_t B, int64_t H, int64_t n);
 int32_t conv_umma(const m2_plan* pl, const Rows* sets, int count, int64_t B, int64_t H, int64_t n, int kf_group, cudaStream_t stream);
 

@@ -1,4 +1,4 @@
-// Short causal convolutions (bf16, 192 <= n <= 256) as Toeplitz products on the fifth-generation tensor cores:
+// Short causal convolutions (bf16, 160 < n <= 256) as Toeplitz products on the fifth-generation tensor cores:
 //   y[b][t] = sum_j k[t - j] x[b][j] per channel.
 //
 // A channel's T(k) is n x n, but only its diagonals differ.  Rows are cut into four segments of S = 64 positions and the UMMA's M index is
@@ -295,10 +295,11 @@ bool map_rows(CUtensorMap* m, const void* p, int64_t B, int64_t H, int64_t n) {
 // [33][768][216] 21.5 and 17.7, [32][768][192] 11.9 and 11.4, [16][768][256] 9.6 and 11.5.  This kernel starts 1.5 to 2 us later (set-up, tensor maps), and the
 // other takes up to three items per SM, 444 in all, in one round; what its fourth to sixth cost grows with n.  Items, there and here, n = 256:
 // [300] 7.5 and 7.3, [444] 7.6 and 8.2, [445] 9.5 and 8.6; 224: [444] 7.0 and 8.2, [445] 8.6 both, [520] 9.6 and 9.0; 192: [296] 5.0 and 6.9, [444] 6.4 and 8.1,
-// [520] 8.8 and 8.9, [592] 10.8 and 9.4.
+// [520] 8.8 and 8.9, [592] 10.8 and 9.4.  Shorter rows: two rounds of the other's, [888] 11.6 and 12.1, [1500] 19.8 and 17.7 (n = 168 .. 184); down to 160, where
+// an item costs the same in both ([48][2400] 45.7 and 45.5).
 bool umma_pays(const m2_plan* pl, int count, int64_t B, int64_t H, int64_t n) {
-    return has_time_kernel(pl) && pl->N == 512 && n >= 192 && n <= 256 && n % 8 == 0 && B > 16 &&
-           count * H * ((B + kRowsPerItem - 1) / kRowsPerItem) >= 445 + (256 - n) * 3 / 2;
+    return has_time_kernel(pl) && pl->N == 512 && n > 160 && n <= 256 && n % 8 == 0 && B > 16 &&
+           count * H * ((B + kRowsPerItem - 1) / kRowsPerItem) >= (n >= 192 ? 445 + (256 - n) * 3 / 2 : 889);
 }
 
 int32_t conv_umma(const m2_plan* pl, const Rows* sets, int count, int64_t B, int64_t H, int64_t n, int kf_group, cudaStream_t stream) {

@@ -333,9 +333,9 @@ def test_short_causal_convolution_as_toeplitz_product(B, H, n, dims, group):
     plan.close()
 
 
-@pytest.mark.parametrize("B,H,n,group", [(17, 541, 192, 1), (32, 459, 248, 3), (33, 265, 200, 1), (64, 224, 256, 2)])
+@pytest.mark.parametrize("B,H,n,group", [(17, 541, 192, 1), (32, 459, 248, 3), (33, 265, 200, 1), (64, 224, 256, 2), (48, 445, 168, 1), (20, 892, 184, 4)])
 def test_toeplitz_products_of_long_items(B, H, n, group):
-    """The tcgen05 Toeplitz kernel (445 items of 32 rows and more for 256 positions, 541 for 192): partial batch chunks, ragged last segments, three
+    """The tcgen05 Toeplitz kernel (445 items of 32 rows and more for 256 positions, 889 for 168): partial batch chunks, ragged last segments, three
     and four items per block, channel groups; lags on one side, on the other (conjugated) and on both (a kernel of all 512 lags).  The kernel's
     values keep 16 bits, the output is rounded once to bf16 (1.7e-3 in the 2-norm)."""
     Hk = H // group
@@ -353,12 +353,13 @@ def test_toeplitz_products_of_long_items(B, H, n, group):
     plan.close()
 
 
-@pytest.mark.parametrize("B,H,n,kernel", [(48, 600, 256, "conv_umma_o2_512_pairs"), (48, 500, 256, "conv_toeplitz_umma"), (64, 600, 256, "conv_toeplitz_umma"),
-                                          (17, 600, 224, "conv_toeplitz_umma"), (33, 1400, 192, "conv_toeplitz_umma"), (40, 1000, 224, "conv_umma_o2_512_pairs"),
+@pytest.mark.parametrize("B,H,n,kernel", [(48, 600, 256, "conv_toeplitz_umma"), (48, 500, 256, "conv_toeplitz_umma"), (64, 600, 256, "conv_toeplitz_umma"),
+                                          (17, 600, 224, "conv_toeplitz_umma"), (33, 1400, 192, "conv_toeplitz_umma"), (40, 1000, 224, "conv_toeplitz_umma"), (48, 2400, 176, "conv_toeplitz_umma"),
                                           (48, 1200, 160, "conv_toeplitz_mma"), (32, 540, 192, "conv_toeplitz_mma"), (32, 541, 192, "conv_toeplitz_umma"), (17, 444, 256, "conv_toeplitz_mma"),
-                                          (17, 445, 256, "conv_toeplitz_umma"), (32, 296, 200, "conv_toeplitz_mma")])
+                                          (17, 445, 256, "conv_toeplitz_umma"), (32, 296, 200, "conv_toeplitz_mma"), (33, 445, 168, "conv_toeplitz_umma"), (32, 888, 176, "conv_toeplitz_mma")])
 def test_short_causal_rows_take_the_faster_kernel(B, H, n, kernel):
-    """Batches whose last 32-row item is half empty, many channels, n near 256: the row-pair kernel; everything around that: Toeplitz products."""
+    """Toeplitz products: on tcgen05 beyond 160 positions where the items are more than one round of the mma.sync kernel (batches whose last 32-row item
+    is half empty among them), by mma.sync otherwise."""
     x = synth.round_bf16(synth.normal(770 + n, (B, H, n)))
     k = (synth.normal(771 + n, (H, n)) / np.sqrt(n)).astype(np.float32)
     y, name = run_conv((32, 16), x, k, True, M.M2_BF16)
