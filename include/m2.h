@@ -110,8 +110,9 @@ int32_t m2_spectrum_conjugate(const m2_plan* plan, const void* kf_in_dev, int64_
  * x_dev, g_dev: [B, H, n] in the plan dtype; dk_dev: [H, n] float32.
  * ws_dev: optional caller-owned workspace of m2_conv_bwd_workspace_bytes(plan, B, H) bytes (16-byte aligned; 0 bytes
  * means this plan has no kernel that uses one).  With it, plans the tensor-core path covers (bf16, N = 512 = 32 x 16)
- * take dk as sums along the diagonals of products of segments of g and x on the tensor cores (nothing is rounded between the
- * inputs and dk; the workspace is not touched then), or, for more than 256 batch rows of fewer than 64 channels, run both forward transforms
+ * take dk as sums along the diagonals of products of segments of g and x on the tensor cores (exact products, fp32 sums, one chain of additions
+ * over all batch rows in each accumulator: 1.4e-7 from 64 bits for 32 rows of 512 positions, 1e-6 for 256, 4.4e-6 for 1024, where the fp32 transforms of a
+ * call without a workspace have 2.0e-7 to 2.9e-7; the workspace is not touched then), or, for more than 256 batch rows of fewer than 64 channels, run both forward transforms
  * and the products conj(M x) (.) M g there (intermediates rounded to bf16 like the forward pass), 8 batch rows at a time, with a CUDA-core kernel
  * that adds the groups in a fixed order and applies M^-1 in fp32; for N = 32768 = 32^3 (causal, n = 16384) the order-3 convolution kernel is run twice (the row pairs' conjugated
  * spectra, then the convolution of the g pairs with them) and the pairs' rows are added.  Otherwise, or with a workspace
@@ -128,9 +129,11 @@ int32_t m2_monarch_conv_bwd_kernel(const m2_plan* plan, const void* x_dev, const
  * x_dev, y_dev: [B, H, n] in the plan dtype; kf_dev from m2_kernel_spectrum with the same H.
  * mode M2_CAUSAL: n <= N/2, x zero padded to N, first n outputs kept (Thm 3 / App. D.3 review).
  * mode M2_CIRCULAR: n == N.
- * A row's result depends on that row and its kernel alone, with one exception: the bf16 tensor-core kernels for N = 512 (more than 8 batch
- * rows) and N = 32768 transform two batch rows as one complex row, so that the rounding between their stages is relative to the larger
- * of the two and a value that is not finite reaches both. */
+ * A row's result depends on that row and its kernel alone, with one exception: the bf16 tensor-core kernels for N = 512 (circular, or causal with
+ * y_dev = x_dev; more than 8 batch rows) and N = 32768 transform two batch rows as one complex row, so that the rounding between their
+ * stages is relative to the larger of the two and a value that is not finite reaches both.  Within its row such a value reaches earlier positions
+ * too, in causal mode as well: all of them where the row is transformed, up to 31 or 63 of them, the ones in its segment of 32 or 64 positions, where the
+ * row is multiplied by the Toeplitz matrix (causal bf16 rows of up to 256 positions on plans of N = 256 and 512): a zero of the matrix times it is NaN. */
 int32_t m2_monarch_conv_fwd(const m2_plan* plan, const void* x_dev, const void* kf_dev, void* y_dev, int64_t B,
                             int64_t H, int64_t n, int32_t mode, void* stream);
 

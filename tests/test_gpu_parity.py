@@ -353,6 +353,23 @@ def test_toeplitz_products_of_long_items(B, H, n, group):
     plan.close()
 
 
+@pytest.mark.parametrize("B,H,n,reach,kernel", [(17, 541, 200, 64, "conv_toeplitz_umma"), (33, 5, 200, 32, "conv_toeplitz_mma")])
+def test_values_that_are_not_finite_in_toeplitz_products(B, H, n, reach, kernel):
+    """A value that is not finite stays in its row and, going back, in its segment of positions (a zero of the Toeplitz matrix times it is NaN)."""
+    x = synth.round_bf16(synth.normal(785, (B, H, n)))
+    k = (synth.normal(786, (H, n)) / np.sqrt(n)).astype(np.float32)
+    want = np.fft.irfft(np.fft.rfft(x.astype(np.float64), 512) * np.fft.rfft(k.astype(np.float64), 512)[None], 512)[..., :n]
+    bad = {0: (np.nan, 0), 4: (np.inf, 101), 5: (-np.inf, 199), 16: (np.nan, 128)}
+    for b, (v, t) in bad.items():
+        x[b, H // 2, t] = v
+    y, name = run_conv((32, 16), x, k, True, M.M2_BF16)
+    assert name == kernel
+    for b, (v, t) in bad.items():
+        assert not np.isfinite(y[b, H // 2, t:]).any()
+        y[b, H // 2, t // reach * reach:], want[b, H // 2, t // reach * reach:] = 0, 0
+    check(y, want, 4e-3, name)
+
+
 @pytest.mark.parametrize("B,H,n,kernel", [(48, 600, 256, "conv_toeplitz_umma"), (48, 500, 256, "conv_toeplitz_umma"), (64, 600, 256, "conv_toeplitz_umma"),
                                           (17, 600, 224, "conv_toeplitz_umma"), (33, 1400, 192, "conv_toeplitz_umma"), (40, 1000, 224, "conv_toeplitz_umma"), (48, 2400, 176, "conv_toeplitz_umma"),
                                           (48, 1200, 160, "conv_toeplitz_mma"), (32, 540, 192, "conv_toeplitz_mma"), (32, 541, 192, "conv_toeplitz_umma"), (17, 444, 256, "conv_toeplitz_mma"),
