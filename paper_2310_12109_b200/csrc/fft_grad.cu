@@ -21,7 +21,7 @@ __global__ void __launch_bounds__(C::THREADS, min_blocks<C>())
     // rows of k are only as aligned as n floats make them; a pair needs 8 bytes
     load_row<C, float, HALF>(re, k + h * n, t, n, (n & 1) == 0 && (reinterpret_cast<uintptr_t>(k) & 7) == 0, live);
     unroll<16>([&](auto j) { im[j.v] = 0ull; });
-    if (kt != nullptr && live) {   // a thread's 32 values, eight on their way together (one by one: conv_train [32][768][512] 72.9 us, so 69.7)
+    if (kt != nullptr && live) {   // a thread's 32 values, eight on their way together (spectrum, forward and both gradients of [32][768][512]: 72.9 us one by one, 69.7 in eights)
 #pragma unroll
         for (int g = 0; g < 32; g += 8) {
             float v[8];

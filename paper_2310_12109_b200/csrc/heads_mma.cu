@@ -14,8 +14,9 @@
 // from L2.
 //
 // Measured, one B200, 1536 heads of n = 256: 23.6 us with one tile at a time, where 24 576 tensor-core convolution units of 16 rows took about
-// 280 us, and 22.2 us with two: bound by the load/store data pipe with one (60 % busy, issue 48 %: 14 wavefronts a tile pair), which two cut to 6
-// (they share the fragments of X2 and V, and a distance's kernel values serve the next one), and by the fragments' latency.
+// 280 us, and 22.4 us with two.  Two share the fragments of X2 and V, and a distance's kernel values serve the next one: 6 wavefronts a tile pair instead
+// of 14, load/store data pipe 60 -> 40 % busy, issue 48 -> 38 %, for 5 % of the time.  Bound by the latency of a tile pair's chain (fragments, scores,
+// weights, second product) with 37 and now 21 warps per SM; matrix pipe 31 -> 34 % of active cycles.
 #include "fft_conv.h"
 #include "fft_core.cuh"
 #include "heads_mma.h"
