@@ -218,11 +218,10 @@ int32_t heads_fwd(const m2_plan* pl, const void* X1, const void* X2, const void*
     if (blocks == 0) return M2_OK;
     if (blocks > 0x7fffffffLL) return M2_ERR_UNSUPPORTED;
     const int smem = smem_bytes((int)n);
-    // Two tiles at a time halve the fragments and kernel values read per tile pair and leave a warp half as many groups.  The kernel alone, us, one
-    // tile and two, [blocks]: n = 1024 [48] 24.1 and 20.3, [144] 24.5 and 20.7, [768] 118 and 91; 640 [48] 13.4 and 12.3, [512] 37.4 and 29.3; 320 [48] 7.9
-    // and 7.6, [256] 9.5 and 9.6; 264 [4 .. 256] the same; 256 [1536] 21.7 and 18.9, [768] 14.1 and 12.6, [384] 8.9 both, [128] 6.2 and 7.2; 232 [768] 13.3 and
-    // 12.7, [384] 8.6 and 9.1.  Layer of d = 768: n = 512 [32] (batch) 261 and 242, 256 [32] 89.4 and 85.7, 208 [24] 70.0 and 69.9.
-    const bool pairs = n > 256 || (n > 224 && blocks >= 768);
+    // Two tiles at a time halve the fragments and kernel values read per tile pair and leave a warp half as many groups.  Layer of d = 768, us,
+    // one tile and two: n = 1024, [8] (batch) 204.6 and 178.9, [1] 82.6 and 86.7; n = 512 [32] 261 and 242, [1] 66.2 and 59.9; 320 [8] 75.6 and 71.0;
+    // 256 [32] 89.4 and 85.7, [16] 61.9 and 60.6, [8] 49.1 and 49.8; 208 [24] 70.0 and 69.9, [8] 46.0 and 46.8.
+    const bool pairs = n > 512 ? blocks >= 64 : n > 256 || (n > 224 && blocks >= 768);
     const int threads = pairs && n <= 256 ? 128 : 256;
     auto kern = !pairs ? heads_kernel<256, 1> : n <= 256 ? heads_kernel<128, 2> : heads_kernel<256, 2>;
     if (smem > 48 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(kMaxN)) != cudaSuccess)
