@@ -220,8 +220,11 @@ int32_t heads_fwd(const m2_plan* pl, const void* X1, const void* X2, const void*
     const int smem = smem_bytes((int)n);
     // Two tiles at a time halve the fragments and kernel values read per tile pair and leave a warp half as many groups.  Layer of d = 768, us,
     // one tile and two: n = 1024, [8] (batch) 204.6 and 178.9, [1] 82.6 and 86.7; n = 512 [32] 261 and 242, [1] 66.2 and 59.9; 320 [8] 75.6 and 71.0;
-    // 256 [32] 89.4 and 85.7, [16] 61.9 and 60.6, [8] 49.1 and 49.8; 208 [24] 70.0 and 69.9, [8] 46.0 and 46.8.
-    const bool pairs = n > 512 ? blocks >= 64 : n > 256 || (n > 224 && blocks >= 768);
+    // 256 [32] 89.4 and 85.7, [16] 61.9 and 60.6, [8] 49.1 and 49.8; 208 [24] 70.0 and 69.9, [8] 46.0 and 46.8.  Rows beyond 512, layers of some widths by
+    // blocks: n = 1024 [48] 87.8 and 90.5, [64] 77.5 and 82.4, [72] 90.1 and 86.1, [144] 102.8 and 97.4; 1000 [48] 87.6 and 92.0, [64] 78.5 and 83.8; 640 [48] 72.1 and
+    // 74.3, [64] 66.0 and 70.1, [192] 87.8 and 86.4.  (The kernel alone is faster with two at [48] as well, 24.1 and 20.3 for 1024;
+    // why the layers are not was not found.  [8] and [24] would gain, 67.5 and 54.4, 86.6 and 83.4.)
+    const bool pairs = n > 512 ? blocks > 64 : n > 256 || (n > 224 && blocks >= 768);
     const int threads = pairs && n <= 256 ? 128 : 256;
     auto kern = !pairs ? heads_kernel<256, 1> : n <= 256 ? heads_kernel<128, 2> : heads_kernel<256, 2>;
     if (smem > 48 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(kMaxN)) != cudaSuccess)
