@@ -1077,7 +1077,7 @@ def test_hyena_head_product_two_tiles_at_a_time(B, n, d, dims):
 @pytest.mark.parametrize("n,d,dims", [(264, 512, (32, 32)), (400, 256, (32, 32)), (1000, 1024, (64, 32))])
 def test_hyena_head_product_of_an_odd_number_of_tiles_repeats(n, d, dims):
     """Two tiles at a time and an odd number of them: the last group has one tile, and nothing that another warp writes is read for the
-    missing one.  Results of 30 calls are the same, bit for bit."""
+    missing one.  Results of 30 calls are the same, bit for bit.  (The last size, 64 blocks, takes one tile at a time.)"""
     plan = M.Plan(dims, dtype=M.M2_BF16, device=0)
     u = dev(synth.normal(synth.stream_id(21, n), (1, n, d)), torch.bfloat16)
     W = [dev(synth.normal(synth.stream_id(21, n + 1 + i), (d, d)) / np.sqrt(d), torch.bfloat16) for i in range(4)]
